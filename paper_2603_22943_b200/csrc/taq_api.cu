@@ -103,6 +103,37 @@ static taq_status run_linear(const LinearArgs& a, int n_z, cudaStream_t st) {
     return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "dequant-GEMM launch");
 }
 
+static taq_status run_linear_i8(const LinearArgs& a, cudaStream_t st) {
+    count_launch(TAQ_KERNEL_LINEAR_TENSOR);
+    if (!sm100_linear_supported(a))
+        return fail(TAQ_ERR_UNSUPPORTED, "integer-activation GEMM: needs k_in a multiple of 16, group 0 or 128, n_out a multiple of 64 or 80 (per-head output: head width 40, 64, 80 or 160)");
+    cudaError_t e = launch_linear_sm100(a, 1, st);
+    return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "integer-activation GEMM launch");
+}
+
+// K/V projection with Eq. 2.  On the tensor cores one launch computes both and writes the operand images as well; the generic
+// kernel takes a launch for each, and the images are built from its rows afterwards.  (The dispatch counter counts
+// projections, so that a merged launch reads 2.)
+static taq_status run_kv_projection(const taq_layer_desc& d, LinearArgs a, const void* Wk, const void* Wv, int n_blocks, int n_z, cudaStream_t st) {
+    a.w = Wk; a.w2 = Wv;
+    LinearArgs t = a;                      // there a row tile is one sequence: z = sequence or request
+    t.rows = d.n_ctx;
+    if (sm100_linear_supported(t)) {
+        count_launch(TAQ_KERNEL_LINEAR_TENSOR);
+        count_launch(TAQ_KERNEL_LINEAR_TENSOR);
+        cudaError_t e = launch_linear_sm100(t, n_blocks, st);
+        return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "K/V projection launch");
+    }
+    for (int which = 0; which < 2; ++which) {
+        a.w = which ? Wv : Wk;
+        a.which = a.kv_which = which;
+        taq_status s = a.xq ? run_linear_i8(a, st) : run_linear(a, n_z, st);
+        if (s != TAQ_OK) return s;
+    }
+    cudaError_t e = launch_kv_operands(d, a.y, a.reqs, n_blocks, st);
+    return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "K/V operand image launch");
+}
+
 static taq_status run_attention(const AttnArgs& a, int n_z, cudaStream_t st) {
     cudaError_t e;
     // C = 320 / 8 heads: up to one wave of CTAs the head-parallel kernel (four heads of a row tile at once) is the shorter
@@ -215,16 +246,7 @@ static taq_status kv_project_impl(const taq_layer_desc* d, const taq_request* re
     a.heads = d->heads; a.n_ctx = d->n_ctx; a.max_trigger = d->max_trigger;
     a.epi = EPI_KV; a.kv_qmax = d->kv_bits == 4 ? 7 : 127;
     a.status = status;
-    for (int which = 0; which < 2; ++which) {
-        a.w = which ? Wv : Wk;
-        a.which = which;
-        a.kv_which = which;
-        s = run_linear(a, n_z, st);
-        if (s != TAQ_OK) return s;
-    }
-    // the same rows once more as MMA-ready operand images for the attention kernel
-    cudaError_t e = launch_kv_operands(*d, kv, reqs, reqs ? n_z : d->batch, st);
-    return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "K/V operand image launch");
+    return run_kv_projection(*d, a, Wk, Wv, reqs ? n_z : d->batch, n_z, st);
 }
 
 taq_status taq_kv_project(const taq_layer_desc* d, const void* ctx_f16_dev, const void* Wk_packed_dev, const void* Wv_packed_dev,
@@ -381,7 +403,6 @@ static taq_status layer_forward_impl(const taq_layer_desc* d, const taq_request*
     o.y = y;
     o.rows = (long long)d->batch * d->n_query; o.n_out = d->channels; o.k_in = d->channels; o.bits = d->w_bits; o.group = d->w_group;
     o.heads = 1; o.epi = EPI_F16; o.status = status;
-    o.early_weights = 1;        // the kernel before it in the stream is the attention above, which writes O only
     return run_linear(o, n_req, st);
 }
 
@@ -416,14 +437,6 @@ taq_status taq_quantize_rows_f16(const void* x_f16_dev, int64_t rows, int32_t co
     TAQ_REQUIRE_PTR(scales_dev);
     cudaError_t e = launch_quantize_rows_f16((const __half*)x_f16_dev, rows, cols, codes_dev, scales_dev, (cudaStream_t)stream);
     return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "quantize_rows_f16 launch");
-}
-
-static taq_status run_linear_i8(const LinearArgs& a, cudaStream_t st) {
-    count_launch(TAQ_KERNEL_LINEAR_TENSOR);
-    if (!sm100_linear_supported(a))
-        return fail(TAQ_ERR_UNSUPPORTED, "integer-activation GEMM: needs k_in a multiple of 16, group 0 or 128, n_out a multiple of 64 or 80 (per-head output: head width 40, 64, 80 or 160)");
-    cudaError_t e = launch_linear_sm100(a, 1, st);
-    return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "integer-activation GEMM launch");
 }
 
 taq_status taq_quantized_linear_i8(const taq_weight_desc* d, const int8_t* x_codes_dev, const float* x_scales_dev, int64_t rows,
@@ -519,7 +532,6 @@ taq_status taq_layer_forward_a8(const taq_layer_desc* d, const void* x_f16_dev, 
     q.heads = d->q_bits == 8 ? d->heads : 1;
     q.epi = d->q_bits == 8 ? EPI_Q8_HEAD : EPI_F16;
     q.status = status;
-    q.early_weights = 1;        // the kernel before it in the stream is the quantizer above, which writes xq / xs only
     s = run_linear_i8(q, st);
     if (s != TAQ_OK) return s;
     AttnArgs at = attn_args(d, status);
@@ -535,7 +547,6 @@ taq_status taq_layer_forward_a8(const taq_layer_desc* d, const void* x_f16_dev, 
     o.y = y_f16_dev;
     o.rows = rows; o.n_out = d->channels; o.k_in = d->channels; o.bits = d->w_bits; o.group = d->w_group;
     o.heads = 1; o.epi = EPI_F16; o.status = status;
-    o.early_weights = 1;
     return run_linear_i8(o, st);
 }
 
@@ -580,15 +591,7 @@ taq_status taq_kv_project_a8(const taq_layer_desc* d, const void* ctx_f16_dev, c
     a.heads = d->heads; a.n_ctx = d->n_ctx; a.max_trigger = d->max_trigger;
     a.epi = EPI_KV; a.kv_qmax = d->kv_bits == 4 ? 7 : 127;
     a.status = status;
-    for (int which = 0; which < 2; ++which) {
-        a.w = which ? Wv_packed_dev : Wk_packed_dev;
-        a.which = which;
-        a.kv_which = which;
-        s = run_linear_i8(a, st);
-        if (s != TAQ_OK) return s;
-    }
-    e = launch_kv_operands(*d, kv_packed_dev, nullptr, d->batch, st);
-    return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "K/V operand image launch");
+    return run_kv_projection(*d, a, Wk_packed_dev, Wv_packed_dev, d->batch, 1, st);
 }
 
 // ---- Eq. 3's M_A chosen independently of Eq. 2's M_KV; the token-sensitivity sweep of Eq. 1 -------------------------

@@ -17,6 +17,7 @@
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
 #include "taq_sm100_parts.cuh"
+#include <cstddef>
 #include <cstring>
 
 namespace taq {
@@ -30,7 +31,10 @@ using namespace parts;
 constexpr int ROWS = 128;
 constexpr int ROW_WARPS = 8;         // two threads per query row
 constexpr int MMA_WARP = 8, COPY_WARP = 9;
-constexpr int ATT_THREADS = 320;
+// Three warpgroups: two of row warps, and one of the MMA and copy warps with two idle ones, which gives registers to the rows where
+// two CTAs share an SM (384 threads launched with 80 each = 128 x (2 x 104 + 32); with 96 for everybody the softmax spilled).
+constexpr int ATT_THREADS = 384;
+constexpr int R_ROWS = 104, R_REST = 32;
 
 template <int D>
 struct Cfg {
@@ -77,7 +81,8 @@ struct Misc {
     volatile int abort_flag;
     float2 xchg[2][2][ROWS];     // [head parity][half][row]: (max, sum) of a thread's half of the softmax
 };
-static_assert(sizeof(Misc) <= 4096 + 128, "misc block");
+constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
+static_assert(sizeof(Misc) <= 4096 + 128 && N_BARS <= 32, "misc block");
 static_assert(sizeof(OperandConsts) % 16 == 0 && sizeof(OperandConsts) <= 384, "constants slot");
 
 // Half of the query codes (or fp16 values) of one row and head, held in registers between the global load and
@@ -132,19 +137,12 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(126); }
-    if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&misc->kv_full[i], 1);
-            ptx::mbar_init(&misc->kv_free[i], 1);
-            ptx::mbar_init(&misc->s_full[i], 1);
-            ptx::mbar_init(&misc->o_full[i], 1);
-        }
-        ptx::mbar_init(&misc->q_full, ROW_WARPS);      // one arrival per row warp
-        ptx::mbar_init(&misc->p_full, ROW_WARPS);
-        ptx::mbar_init(&misc->drain, 1);
-        ptx::mbar_init(&misc->qraw_full, 1);
-        misc->abort_flag = 0;
+    if (warp == COPY_WARP) {                          // one lane per barrier
+        uint64_t* all = misc->kv_full;
+        if (lane < N_BARS) ptx::mbar_init(all + lane, all + lane == &misc->q_full || all + lane == &misc->p_full ? ROW_WARPS : 1);     // (one arrival per row warp)
+        if (lane == 0) misc->abort_flag = 0;
         ptx::mbar_fence_init();
+        if (C::TMA_IO && lane == 0) { ptx::tma_prefetch_desc(&tmap_q); ptx::tma_prefetch_desc(&tmap_o); }
     }
     if (warp == MMA_WARP) ptx::tmem_alloc(&misc->tmem_base, C::TMEM_COLS);
     ptx::tc_fence_before_sync();
@@ -155,6 +153,9 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
 
     const taq_kv_layout KL = kv_layout(H, T, D, a.max_trigger);
 
+    constexpr bool REG_SPLIT = C::CTAS_PER_SM == 2;
+    if (warp >= MMA_WARP) {
+    if constexpr (REG_SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_REST));
     if (warp == COPY_WARP) {
         // ---------------- K~/V~ operand images, one head ahead ----------------
         if (lane == 0) {
@@ -199,9 +200,10 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
         }
     } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer ----------------
-        // All 32 lanes walk the control flow (warp-uniform loop state and descriptor words); one elected lane issues.
-        const bool leader = ptx::elect_one();
-        auto wait = [&](uint64_t* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity) && !misc->abort_flag) != 0; };
+        // One elected thread walks it alone (a wait on a complete barrier costs it 60 cycles; a vote of the whole warp and a poll
+        // of the abort flag made it 190).
+        if (ptx::elect_one()) {
+        auto wait = [&](uint64_t* bar, uint32_t parity) -> bool { return ptx::mbar_wait(bar, parity); };
         constexpr uint32_t HI = ptx::kDescHiSw128;
         const uint32_t q_lo0 = ptx::desc_lo(ptx::smem_u32(smem + C::OFF_Q)), p_lo0 = ptx::desc_lo(ptx::smem_u32(smem + C::OFF_P));
         const uint32_t kv_lo0 = ptx::desc_lo(ptx::smem_u32(smem + C::OFF_KV));
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             const int buf = hi % C::KVBUF;
             if (!wait(&misc->kv_full[buf], C::SPLIT_KV ? (hi & 1) : (hi / C::KVBUF) & 1) || !wait(&misc->q_full, hi & 1)) return false;
             ptx::tc_fence_after_sync();
-            if (leader) {
+            {
                 if (hi < 8) TAQ_PROF(80 + hi);
                 const uint32_t k_lo = kv_lo0 + buf * (C::HEAD_BYTES >> 4);
 #pragma unroll
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             if (C::SPLIT_KV && !wait(&misc->kv_full[1], hi & 1)) return false;
             if (!wait(&misc->p_full, hi & 1)) return false;
             ptx::tc_fence_after_sync();
-            if (leader) {
+            {
                 if (hi < 8) TAQ_PROF(96 + hi);
                 const uint32_t vt_lo = kv_lo0 + ((buf * C::HEAD_BYTES + C::K_BYTES) >> 4);
 #pragma unroll
@@ -243,23 +245,29 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 if (hi + 1 < HG) ok = issue_s(hi + 1);
                 if (ok) ok = issue_pv(hi);
             } else {
-                // one image buffer: the next head's K~ arrives some time after this head's S; its S goes first if K~
-                // and Q~ are there already (it then runs under this head's softmax), else after this head's PV
-                const bool early = hi + 1 < HG && __all_sync(0xffffffffu, ptx::mbar_try_wait(&misc->kv_full[0], (hi + 1) & 1) && ptx::mbar_try_wait(&misc->q_full, (hi + 1) & 1)) != 0;
-                if (early) ok = issue_s(hi + 1);
+                // one image buffer: the next head's K~ arrives some time after this head's S; its S goes as soon as K~ and Q~
+                // are there (it then runs under this head's softmax), at the latest after this head's PV
+                bool s_next = hi + 1 >= HG;
+                for (const long long t0 = clock64(); ok;) {
+                    if (!s_next && ptx::mbar_try_wait(&misc->kv_full[0], (hi + 1) & 1) && ptx::mbar_try_wait(&misc->q_full, (hi + 1) & 1)) ok = s_next = issue_s(hi + 1);
+                    if (ptx::mbar_try_wait(&misc->p_full, hi & 1)) break;
+                    if (clock64() - t0 > ptx::kWaitCycles) ok = false;
+                }
                 if (ok) ok = issue_pv(hi);
-                if (ok && !early && hi + 1 < HG) ok = issue_s(hi + 1);
+                if (ok && !s_next) ok = issue_s(hi + 1);
             }
         }
         if (!ok) {                        // wait (bounded) for whatever was issued before TMEM is given back
-            if (leader) {
-                raise_status(a.status, TAQ_ERR_TIMEOUT);
-                misc->abort_flag = 1;
-                ptx::mma_commit(&misc->drain);
-            }
+            raise_status(a.status, TAQ_ERR_TIMEOUT);
+            misc->abort_flag = 1;
+            ptx::mma_commit(&misc->drain);
             (void)ptx::mbar_wait(&misc->drain, 0);
         }
+        }
+        __syncwarp();
+    }
     } else {
+        if constexpr (REG_SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_ROWS));
         // ---------------- row threads: two per query row (TMEM lane), each with half of the keys ----------------
         const int q4 = warp & 3, half = warp >> 2;
         const int r = q4 * 32 + lane;
@@ -297,7 +305,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             auto stage_q_u = [&](int hi) {
                 static_assert(D % 8 == 0 && (ROWS * (D / 8)) % 256 == 0, "chunks per thread");
                 constexpr int CPR = D / 8;                   // chunks per row
-                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->qraw_full, hi & 1) && !misc->abort_flag);
+                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->qraw_full, hi & 1));
                 if (alive) {
                     uint4 t16[ROWS * CPR / 256];
 #pragma unroll
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 const uint32_t ph = hi & 1;
                 const bool more = hi + 1 < HG;
                 if (Q8 && more) sq_next = valid ? __ldg(a.q_scales + grow * H + h_begin + hi + 1) : 0.f;
-                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[ph], (hi >> 1) & 1) && !misc->abort_flag);
+                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[ph], (hi >> 1) & 1));
                 if (tid == 0 && hi < 8) TAQ_PROF(16 + hi);
                 float e[HK];
                 float k255 = 0.f;
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 all256();                                    // the raw tile has been read by everybody, U by the store
                 if (SEPQ && tid == 0 && hi + 2 < HG && alive) load_q(hi + 2);
                 if (hi > 0) {                                // O of the previous head: TMEM -> U -> global (TMA store)
-                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) % C::OBUF], ((hi - 1) / C::OBUF) & 1) && !misc->abort_flag);
+                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) % C::OBUF], ((hi - 1) / C::OBUF) & 1));
                     if (alive) {
                         ptx::tc_fence_after_sync();
                         stage_o_u(hi - 1);
@@ -424,7 +432,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 }
                 sq = sq_next;
             }
-            alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(HG - 1) % C::OBUF], ((HG - 1) / C::OBUF) & 1) && !misc->abort_flag);
+            alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(HG - 1) % C::OBUF], ((HG - 1) / C::OBUF) & 1));
             if (SEPQ) {                                      // the store of the head before must have read U
                 if (tid == 0) ptx::bulk_store_wait_read();
                 all256();
@@ -487,7 +495,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 qr.load(a.q, grow * Cch + (size_t)(h_begin + hi + 1) * D, valid, half);
                 if (Q8) sq_next = valid ? a.q_scales[grow * H + h_begin + hi + 1] : 0.f;
             }
-            alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[ph], (hi >> 1) & 1) && !misc->abort_flag);
+            alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[ph], (hi >> 1) & 1));
             if (!alive) break;
             if (tid == 0 && hi < 8) TAQ_PROF(16 + hi);
             ptx::tc_fence_after_sync();
@@ -524,7 +532,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             if (tid == 0 && hi < 8) TAQ_PROF(32 + hi);
             // the P tile is free once the previous head's PV has completed
             if (hi > 0) {
-                alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) % C::OBUF], ((hi - 1) / C::OBUF) & 1) && !misc->abort_flag);
+                alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) % C::OBUF], ((hi - 1) / C::OBUF) & 1));
                 if (!alive) break;
                 ptx::tc_fence_after_sync();
                 if (C::OBUF == 1) store_o(hi - 1);   // one O accumulator: empty it before the next PV may start
@@ -542,7 +550,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             sq = sq_next;
         }
         if (alive) {
-            alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(HG - 1) % C::OBUF], ((HG - 1) / C::OBUF) & 1) && !misc->abort_flag);
+            alive = __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(HG - 1) % C::OBUF], ((HG - 1) / C::OBUF) & 1));
             if (alive) {
                 ptx::tc_fence_after_sync();
                 store_o(HG - 1);
@@ -579,14 +587,23 @@ EncodeTiledFn encode_tiled_fn3() {
 
 template <int D>
 int pick_heads_per_cta(const AttnArgs& a, int n_z) {
-    // The largest head group that still fills the GPU's CTA slots to about three quarters.
+    // One CTA per SM: the head group with the shortest estimated time, a CTA's start and end counted as two heads and a last wave in
+    // full (180 CTAs of two heads take longer than 90 of four).  Two CTAs per SM: the largest group that still fills the
+    // places to about three quarters (there the second CTA of an SM hides the first one's gaps, and fewer, longer CTAs lose).
     const long long tiles = (long long)((a.n_query + ROWS - 1) / ROWS) * n_z;
-    const long long want = (long long)148 * Cfg<D>::CTAS_PER_SM * 3 / 4;
-    for (int hg = a.heads; hg > 1; --hg) {
+    int best = 1;
+    double best_cost = 1e30;
+    for (int hg = 1; hg <= a.heads; ++hg) {
         if (a.heads % hg) continue;
-        if (tiles * (a.heads / hg) >= want) return hg;
+        const long long ctas = tiles * (a.heads / hg);
+        if (Cfg<D>::CTAS_PER_SM == 2) {
+            if (ctas >= 222) best = hg;
+            continue;
+        }
+        const double cost = (double)((ctas + 147) / 148) * (2.0 + hg);
+        if (cost <= best_cost) { best_cost = cost; best = hg; }
     }
-    return 1;
+    return best;
 }
 
 template <int D, bool Q8, bool TAIL_ONLY>

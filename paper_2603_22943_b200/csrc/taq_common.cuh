@@ -126,6 +126,7 @@ struct LinearArgs {
     const int8_t* xq;           // integer-activation variant: int8 codes [z][rows][k_in] instead of x ...
     const float* x_scales;      // ... and one fp32 scale per row [z][rows]
     const void* w;              // packed blob (single problem)
+    const void* w2;             // EPI_KV on the tensor cores: the V projection's blob (w: the K projection's); one launch does both
     const taq_request* reqs;    // nullable
     int which;                  // 0: reqs[z].Wq, 1: reqs[z].Wout
     void* y;                    // F16/F32/int8 [z][rows][n_out]; for EPI_KV: kv blocks (single problem)
@@ -135,17 +136,9 @@ struct LinearArgs {
     int n_out, k_in, bits, group;
     int heads;                  // EPI_Q8_HEAD / EPI_KV
     int n_ctx, max_trigger;     // EPI_KV: rows = batch * n_ctx
-    int kv_which;               // EPI_KV: 0 = K, 1 = V
+    int kv_which;               // EPI_KV on CUDA cores: 0 = K, 1 = V
     int kv_qmax;                // EPI_KV: 127 (int8 rows) or 7 (4-bit rows); 0 is read as 127
     int epi;
-    int w_direct;               // (set by the launcher) 1: int8 activations and 8-bit weights: the weight codes are the B
-                                // operand as they are and go from the blob into the ring by TMA, no staging or expansion;
-                                // 2: fp16 activations and 8-bit weights too large to stage whole: a slice of the codes per
-                                // k-block by TMA, expanded by the workers; 0: all codes staged once
-    int early_weights;          // the previous kernel in the stream is known not to write the weights: fetch and expand
-                                // them before waiting for it
-    int head_pair;              // (set by the launcher) EPI_Q8_HEAD with heads twice as wide as the tile: the two CTAs whose
-                                // tiles make up a head exchange their rows' absmax through the cluster
     int* status;
 };
 

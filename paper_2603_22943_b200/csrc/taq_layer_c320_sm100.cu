@@ -4,7 +4,7 @@
 //
 // A CTA owns 128 query rows of one sequence and four heads (160 channels); the two CTAs that share a row tile form a
 // cluster and exchange their halves of O through distributed shared memory.  Warps: 0 producer (TMA / bulk copies),
-// 1 MMA issuer, 2..17 workers.  A worker thread is (row r, head hi) from start to end:
+// 1 MMA issuer, 4..19 workers.  A worker thread is (row r, head hi) from start to end:
 //   phase 1  Q = X Wq^T for the CTA's 160 channels: workers expand the packed 4-bit codes to fp16-integer operand tiles
 //            (all five K blocks, before X has arrived), one TMEM accumulator per scale group, folded into registers with
 //            the group's scales;
@@ -25,6 +25,7 @@
 #include "taq_sm100.cuh"
 #include "taq_sm100_parts.cuh"
 #include "taq_prof.cuh"
+#include <cstddef>
 #include <type_traits>
 
 TAQ_PROF_DEFINE(layer)
@@ -39,7 +40,12 @@ constexpr int D = 40, DP = 48, HG = 4;          // head width, padded width, hea
 constexpr int NQ = HG * D;                      // 160 channels per CTA
 constexpr int KIN = 320, BK = 64, NKB = KIN / BK;
 constexpr int ROWS = 128;
-constexpr int NWORK = 512, NTHREADS = 64 + NWORK;
+constexpr int NWORK = 512, FIRST_WORKER = 4, NTHREADS = 32 * FIRST_WORKER + NWORK;
+// A worker holds a row's 80 scores: the first warpgroup (producer, MMA issuer, two idle warps) gives registers to the four of the
+// workers.  640 threads launched with 96 each = 128 x (32 + 4 x 112); with 96 for everybody the softmax spilled 33 registers, and
+// beside this much shared memory a spill is a trip to L2.
+constexpr int R_FIRST = 32, R_WORK = 112;
+static_assert(128 * (R_FIRST + 4 * R_WORK) == NTHREADS * 96, "register split");
 constexpr int MAX_GROUPS = 3;
 
 constexpr int A_TILE = ROWS * 128;              // 16 KB: a 64-wide K block of X, a head's Q~ tile, keys 0..63 of P
@@ -91,6 +97,7 @@ struct Misc {
     uint32_t tmem_base;
     volatile int abort_flag;
 };
+constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
 constexpr int TOTAL = OFF_MISC + (int)sizeof(Misc) + 1024;
 static_assert(TOTAL <= 232448, "shared memory budget");
 
@@ -285,32 +292,39 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(30); }
-    if (tid == 0) {
-        for (int i = 0; i < NKB; ++i) { ptx::mbar_init(&misc->a_full[i], 1); ptx::mbar_init(&misc->b1_full[i], NWORK / 32); }
-        ptx::mbar_init(&misc->w_full, 1);
-        ptx::mbar_init(&misc->w2_full, 1);
-        ptx::mbar_init(&misc->kc_full, 1);
-        ptx::mbar_init(&misc->vt_full, 1);
-        for (int i = 0; i < NKB; ++i) ptx::mbar_init(&misc->b4_full[i], NEXP / 32);
-        for (int i = 0; i < NS4; ++i) ptx::mbar_init(&misc->b4_empty[i], 1);
-        for (int i = 0; i < MAX_GROUPS; ++i) ptx::mbar_init(&misc->acc_full[i], 1);
-        ptx::mbar_init(&misc->q_all, NWORK / 32);
-        for (int i = 0; i < HG; ++i) {
-            ptx::mbar_init(&misc->s_full[i], 1);
-            ptx::mbar_init(&misc->p_full[i], NWORK / 32 / HG);     // the four warps of the head
-            ptx::mbar_init(&misc->o_full[i], 1);
+    if (warp == 0) {
+        // One lane per barrier (45 in a row by one thread take a while); then, still in front of the CTA's first barrier, the packed
+        // weights: they are written by taq_pack_weights, which never lets its successor start early, so they are complete
+        // before this kernel can run at all and are fetched (and expanded) under the previous kernel's tail.
+        uint64_t* all = misc->a_full;
+        for (int i = lane; i < N_BARS; i += 32) {
+            const uint64_t* bar = all + i;
+            uint32_t count = 1;
+            if (bar >= misc->b1_full && bar < misc->b4_full) count = NWORK / 32;
+            else if (bar >= misc->b4_full && bar < misc->b4_empty) count = NEXP / 32;
+            else if (bar >= misc->tile_done && bar < misc->acc_full) {   // the warps of the one or two heads that write the tile
+                const int lt = (int)(bar - misc->tile_done);
+                count = (lt == 0 || lt == HG ? 1 : 2) * (NWORK / 32 / HG);
+            }
+            else if (bar == &misc->q_all) count = NWORK / 32;
+            else if (bar >= misc->p_full && bar < misc->o_full) count = NWORK / 32 / HG;      // the four warps of the head
+            ptx::mbar_init(all + i, count);
         }
-        for (int lt = 0; lt < N_OTILE / 2; ++lt)                   // the warps of the one or two heads that write the tile
-            ptx::mbar_init(&misc->tile_done[lt], (lt == 0 || lt == HG ? 1 : 2) * (NWORK / 32 / HG));
-        ptx::mbar_init(&misc->o_all, 1);
-        ptx::mbar_init(&misc->peer_ready, 1);
-        ptx::mbar_init(&misc->peer_got, 1);
-        ptx::mbar_init(&misc->drain, 1);
-        misc->abort_flag = 0;
         ptx::mbar_fence_init();
-        if (FUSE_OUT) ptx::mbar_arrive_expect_tx(&misc->o_all, (N_OTILE / 2) * O_TILE);     // the partner's five tiles
-        ptx::tma_prefetch_desc(&tmap_x);
-        ptx::tma_prefetch_desc(&tmap_y);
+        __syncwarp();
+        if (lane == 0) {
+            misc->abort_flag = 0;
+            if (FUSE_OUT) ptx::mbar_arrive_expect_tx(&misc->o_all, (N_OTILE / 2) * O_TILE);     // the partner's five tiles
+            if (!Q_IN) {
+                const uint32_t scale_bytes = (uint32_t)(NQ * n_groups * 4);
+                const uint8_t* blob = (const uint8_t*)(a.reqs ? a.reqs[zb].Wq : a.wq);
+                ptx::mbar_arrive_expect_tx(&misc->w_full, RAW_BYTES + scale_bytes);
+                ptx::bulk_load(smem + OFF_RAW, blob + L.off_codes + (size_t)col0 * L.row_bytes, RAW_BYTES, &misc->w_full);
+                ptx::bulk_load(smem + OFF_SC, blob + L.off_scales + (size_t)col0 * n_groups * 4, scale_bytes, &misc->w_full);
+            }
+            ptx::tma_prefetch_desc(&tmap_x);
+            ptx::tma_prefetch_desc(&tmap_y);
+        }
     }
     if (warp == 1) ptx::tmem_alloc(&misc->tmem_base, TMEM_COLS);
     ptx::tc_fence_before_sync();
@@ -327,18 +341,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
     const taq_kv_layout KL = kv_layout(H, T, D, a.max_trigger);
     auto give_up = [&]() { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; };
 
+    if (warp < FIRST_WORKER) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_FIRST));
     if (warp == 0) {
         // ---------------- producer ----------------
         if (lane == 0) {
-            // Packed weights are written by taq_pack_weights, which never lets its successor start early: they are complete
-            // before this kernel can run at all and are fetched (and expanded) under the previous kernel's tail.
             const uint32_t scale_bytes = (uint32_t)(NQ * n_groups * 4);
-            if (!Q_IN) {
-                const uint8_t* blob = (const uint8_t*)(a.reqs ? a.reqs[zb].Wq : a.wq);
-                ptx::mbar_arrive_expect_tx(&misc->w_full, RAW_BYTES + scale_bytes);
-                ptx::bulk_load(smem + OFF_RAW, blob + L.off_codes + (size_t)col0 * L.row_bytes, RAW_BYTES, &misc->w_full);
-                ptx::bulk_load(smem + OFF_SC, blob + L.off_scales + (size_t)col0 * n_groups * 4, scale_bytes, &misc->w_full);
-            }
             ptx::pdl_wait();                              // X and the K~/V~ block may come from the previous kernel
             TAQ_PROF(1); TAQ_GPROF(28);
             for (int kb = 0; kb < NKB && !Q_IN; ++kb) {   // the whole X tile at once: every K block has its own buffer
@@ -403,23 +411,23 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        // All 32 lanes walk the control flow (waits, loop state and descriptor words stay warp-uniform); one elected lane
-        // issues the MMAs and commits.  Its waits are bounded but do not poll the abort flag: the path between two MMAs is
-        // kept as short as possible.
+        // One elected thread walks it alone: a wait on a complete barrier costs it 60 cycles (a vote of the whole warp made it
+        // about 150), an MMA 45, so that a 64-wide K block stays at the tensor core's own 320 cycles.
         const bool leader = ptx::elect_one();
         bool ok = true;
-        auto wait = [&](uint64_t* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity, WL)) != 0; };
+        auto wait = [&](uint64_t* bar, uint32_t parity) -> bool { return ptx::mbar_wait(bar, parity, WL); };
         constexpr uint32_t idesc = ptx::idesc_f16_m128(NQ);
         constexpr uint32_t HI128 = ptx::kDescHiSw128, HI64 = ptx::kDescHiSw64, HI32 = ptx::kDescHiSw32;
         const uint32_t r0_lo = ptx::desc_lo(ptx::smem_u32(smem + OFF_R0)), r1_lo = ptx::desc_lo(ptx::smem_u32(smem + OFF_R1));
         const uint32_t pb_lo = ptx::desc_lo(ptx::smem_u32(smem + OFF_PB)), k_lo = ptx::desc_lo(ptx::smem_u32(smem + OFF_K));
+        if (leader) {
         if (!Q_IN) {   // phase 1: one accumulation pass per scale group; every weight tile was expanded before X arrived
             int kb = 0;
             for (int g = 0; g < n_groups && ok; ++g) {
                 const int kb_end = min(NKB, kb + kb_per_group);
                 for (bool first = true; kb < kb_end && ok; ++kb) {
                     if (!wait(&misc->b1_full[kb], 0) || !wait(&misc->a_full[kb], 0)) { ok = false; break; }
-                    if (leader) {
+                    {
                         TAQ_PROF(2 + kb);
                         const uint32_t a_lo = r0_lo + kb * (A_TILE >> 4), b_lo = ptx::desc_lo(ptx::smem_u32(smem + stage1_offset(kb)));
 #pragma unroll
@@ -435,7 +443,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         // phase-1 accumulators, whose columns S and O reuse, are ordered before that arrival)
         ok = ok && wait(&misc->kc_full, 0) && wait(&misc->q_all, 0);
         ptx::tc_fence_after_sync();
-        if (ok && leader) {
+        if (ok) {
             TAQ_PROF(10);
 #pragma unroll
             for (int hi = 0; hi < HG; ++hi) {
@@ -450,7 +458,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         for (int hi = 0; hi < HG && ok; ++hi) {
             if (!wait(&misc->p_full[hi], 0)) { ok = false; break; }
             ptx::tc_fence_after_sync();
-            if (leader) {
+            {
                 TAQ_PROF(11 + hi);
                 const uint32_t p_lo = r0_lo + hi * (A_TILE >> 4), pt_lo = pb_lo + hi * (PB_TILE >> 4), v_lo = r1_lo + hi * (VT_BYTES >> 4);
 #pragma unroll
@@ -460,8 +468,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
                 ptx::mma_commit(&misc->o_full[hi]);
             }
         }
-        if (FUSE_OUT) {
-            ptx::cluster_wait();                          // the partner's barriers exist (peer_got below)
+        }
+        __syncwarp();
+        if (FUSE_OUT) ptx::cluster_wait();                // the partner's barriers exist (peer_got below)
+        if (FUSE_OUT && leader) {
             // phase 4: Y = O Wout^T for this CTA's 160 output channels, in six steps (see walk_block): three over this CTA's
             // own O tiles, each as soon as the heads that write its tiles have stored them, then three over the partner's.
             // The accumulators reuse the columns of S (all read long ago) and, for the third scale group, of O: both
@@ -495,13 +505,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
                     if (i == 3) {
                         ok = ok && wait(&misc->o_all, 0);
                         // the partner's copies have landed: it may leave without waiting for this CTA any longer
-                        if (ok && leader) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&misc->peer_got), peer));
-                        if (leader) TAQ_PROF(38);
+                        if (ok) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&misc->peer_got), peer));
+                        TAQ_PROF(38);
                     } else {
                         // (block 2 returns at step 3 with the tile it already has)
                         ok = ok && wait(&misc->b4_full[walk_order(R, kb)], 0);
                     }
-                    if (ok && leader) {
+                    if (ok) {
                         TAQ_PROF(40 + i);
                         const uint32_t b_lo = ptx::desc_lo(ptx::smem_u32(smem + stage4_offset(st)));
                         bool acc = !((first_mask >> i) & 1u);
@@ -524,17 +534,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             };
             if (rank == 0) phase4(std::integral_constant<int, 0>{}); else phase4(std::integral_constant<int, 1>{});
         }
-        if (!ok) {
-            if (leader) {
-                give_up();
-                ptx::mma_commit(&misc->drain);               // wait (bounded) for whatever was issued before TMEM is given back
-            }
+        if (leader && !ok) {
+            give_up();
+            ptx::mma_commit(&misc->drain);                   // wait (bounded) for whatever was issued before TMEM is given back
             (void)ptx::mbar_wait(&misc->drain, 0, WL);
         }
+        __syncwarp();
     } else {
-        // ---------------- workers (warps 2..17): thread = (row r, head hi) ----------------
-        const int wt = tid - 64;
-        const int q4 = warp & 3, hi = (warp - 2) >> 2;       // TMEM lane quarter; head
+        if (FUSE_OUT) ptx::cluster_wait();
+    }
+    } else {
+        // ---------------- workers (warps 4..19): thread = (row r, head hi) ----------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_WORK));
+        const int wt = tid - 32 * FIRST_WORKER;
+        const int q4 = warp & 3, hi = (warp - FIRST_WORKER) >> 2;       // TMEM lane quarter; head
         const int r = q4 * 32 + lane;
         const int n = row0 + r;
         const bool valid = n < a.n_query;
@@ -562,7 +575,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             for (int c = 0; c < D; ++c) y[c] = 0.f;
             for (int gi = 0; gi < n_groups && ok; ++gi) {
                 const int g = descending ? n_groups - 1 - gi : gi;
-                ok = ptx::mbar_wait(&misc->acc_full[g], parity, WL) && !misc->abort_flag;
+                ok = ptx::mbar_wait(&misc->acc_full[g], parity, WL);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const float* sg = scales_t + g * NQ + cb;
@@ -665,7 +678,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         if (wt == 0) TAQ_PROF(8);
 
         // ---- phase 3: the 80 scores of (row, head): softmax, Eq. 3, P ----
-        ok = ok && ptx::mbar_wait(&misc->kc_full, 0, WL) && ptx::mbar_wait(&misc->s_full[hi], 0, WL) && !misc->abort_flag;
+        ok = ok && ptx::mbar_wait(&misc->kc_full, 0, WL) && ptx::mbar_wait(&misc->s_full[hi], 0, WL);
         if (lane == 0 && q4 == 0) TAQ_PROF(16 + hi);           // S seen
         const float pmax = a.p_bits == 4 ? 15.0f : 255.0f;     // probabilities are held in units of 1 / pmax (uint8 or 4-bit codes)
         if (ok) {
@@ -697,7 +710,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             // The first Wout tile of the walk goes into a K~ buffer (dead once every S product is complete) while this
             // head's PV product runs; the second follows after the head's O has been stored.  The warps of the last head,
             // whose probabilities are the last to be complete, take no part in the expansion.
-            ok = ok && ptx::mbar_wait(&misc->s_full[HG - 1], 0, WL) && ptx::mbar_wait(&misc->w2_full, 0, WL) && !misc->abort_flag;
+            ok = ok && ptx::mbar_wait(&misc->s_full[HG - 1], 0, WL) && ptx::mbar_wait(&misc->w2_full, 0, WL);
             for (int i = wt; i < NQ * n_groups; i += NWORK) scales_t[(i % n_groups) * NQ + i / n_groups] = wscales[i];     // (last read in phase 1)
             if (wt < NEXP) {
                 if (ok) expand_block_by<NEXP>(raw, walk_tile(rank, 0), smem + stage4_offset(0), wt);
@@ -707,7 +720,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         }
 
         // ---- O of (row, head): the accumulator in units of 1 / pmax -> fp16, as soon as this head's PV product is complete ----
-        ok = ok && ptx::mbar_wait(&misc->o_full[hi], 0, WL) && !misc->abort_flag;
+        ok = ok && ptx::mbar_wait(&misc->o_full[hi], 0, WL);
         if (ok) {
             ptx::tc_fence_after_sync();
             const float inv = 1.0f / pmax;
@@ -753,10 +766,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             if (wt < NEXP) {
                 if (ok) expand_block_by<NEXP>(raw, walk_tile(rank, 1), smem + stage4_offset(1), wt);
                 tile_built(&misc->b4_full[1]);
-                ok = ok && ptx::mbar_wait(&misc->o_full[HG - 1], 0, WL) && !misc->abort_flag;
+                ok = ok && ptx::mbar_wait(&misc->o_full[HG - 1], 0, WL);
                 for (int i = 2; i < NKB; ++i) {
                     const int s = i < NS4 ? i : walk_reuse_stage(rank);
-                    if (i >= NS4 && ok) ok = ptx::mbar_wait(&misc->b4_empty[s], 0, WL) && !misc->abort_flag;
+                    if (i >= NS4 && ok) ok = ptx::mbar_wait(&misc->b4_empty[s], 0, WL);
                     if (ok) expand_block_by<NEXP>(raw, walk_tile(rank, i), smem + stage4_offset(s), wt);
                     tile_built(&misc->b4_full[i]);
                 }

@@ -1,25 +1,34 @@
 // Dequant-GEMM on the Blackwell tensor cores: y = x W^T with W^ = code * scale.
 //
-// The tensor cores never see a scale: the B operand holds the integer codes as fp16 (exact), every scale group
-// (128 fan-in elements for W4, the whole row for W8) is accumulated in its own pass into one of two TMEM
-// accumulators, and the worker threads fold each finished group into fp32 registers, y += scale[n][g] * acc_g,
-// while the tensor core is already on the next group.
+// The tensor cores never see a scale: the B operand holds the integer codes as fp16 (exact; int8 in the integer-activation
+// variant), every scale group (128 fan-in elements for W4, the whole row for W8) is accumulated on its own in TMEM, and
+// each finished group is folded into fp32 registers, y += scale[n][g] * acc_g, while the tensor core is already on the
+// next groups.
 //
-// One CTA computes a 128-row x BN-column tile.  The packed codes of its BN output channels (a contiguous slice of
-// the blob), their scales and biases are fetched once with three bulk copies; K is walked in blocks of 64 through
-// a ring of shared-memory stages.  Roles:
-//   warp 0       one thread issues the bulk copies and the TMA loads of the fp16 activation tile (128 x 64,
-//                128-byte swizzle);
-//   warp 1       owns the TMEM allocation; one thread issues tcgen05.mma (M=128, N=BN, K=16) and commits;
-//   warps 2..9   workers, two threads per accumulator row (TMEM lane), each owning half of the tile's columns:
-//                they expand the 4/8-bit codes from shared memory into the fp16 weight tile (BN x 64, swizzled
-//                K-major), fold finished groups into registers, and run the epilogue: bias / fp16 conversion, or
-//                the per-(row, head) int8 quantization Q_a of Eq. 2, or the mixed int8 / fp16 K~,V~ of Eq. 2.
-// The packed weights stay packed in HBM and are read once per CTA.
+// A CTA computes tiles of 128 rows x BN columns.  K is walked in pairs of blocks of 64 elements (128 for int8) through two
+// rings of shared-memory stages: activation tiles (128 rows x 128 bytes per block, by TMA) and expanded weight tiles (BN rows
+// x 128 bytes per block), both in the 128-byte swizzle.  Every step has warps of its own, so that none of them is behind
+// another one in program order:
+//   producer  one thread issues the TMA loads of the activation tiles;
+//   MMA       owns the TMEM allocation; one thread issues tcgen05.mma (M=128, N=BN, K=32 bytes) and commits;
+//   builders  (4 or 8 warps) fetch the packed codes straight from global memory into registers, one pair of blocks ahead,
+//             and expand them into the weight tiles; they also bring the scales and biases of a tile;
+//   folders   (4 or 8 warps) one thread per row (TMEM lane) and HC = 80 or 64 columns: fold finished groups into registers
+//             and run the epilogue: bias / fp16 conversion, or the per-(row, head) int8 quantization Q_a of Eq. 2, or the
+//             mixed int8 / fp16 K~, V~ of Eq. 2 together with the attention kernel's operand images.
+// Launches of more tiles than SMs are persistent: a CTA walks several tiles, and the epilogue of one runs under the K loop of
+// the next.  The packed weights stay packed in HBM.
+//
+// What bounds it.  A 64-wide K block of a 160-column tile is 320 cycles of tensor time; the MMA thread needs 60 cycles per wait
+// on a complete barrier, 60 per commit and 45 per MMA (measured), hence barriers per pair of blocks, looked at one pair ahead.
+// Nothing in the loops may spill: beside 200 KB of shared memory there is next to no L1, and a spilled register is a
+// round trip to L2 (a first version with 120 bytes of spills ran at half the speed), hence the register split.
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
 #include "taq_sm100_parts.cuh"
 #include "taq_prof.cuh"
+#include <cstddef>
+#include <cstring>
 #include <type_traits>
 
 TAQ_PROF_DEFINE(linear)
@@ -32,593 +41,775 @@ using namespace parts;
 
 constexpr int BM = 128;
 constexpr int BK = 64;                     // fp16 elements per 128-byte operand row; the int8 variant has 2 BK
-constexpr int MAX_STAGE = 6;
-constexpr int MAX_PREBUILT = 12;           // k-blocks per CTA whose expanded weight tiles may all be resident at once
-constexpr int MAX_ACC = 8;                  // TMEM accumulators (scale groups in flight) per CTA
-constexpr int NWORK = 256;                  // worker threads: two per accumulator row
-constexpr int NTHREADS = 64 + NWORK;
-constexpr int A_TILE_BYTES = BM * BK * 2;   // 16 KB
+constexpr int A_TILE_BYTES = BM * 128;     // 16 KB
+constexpr int MAX_STAGE = 6;               // ring depths, in pairs of k-blocks
+constexpr int MAX_SLOT = 4;                // accumulators in TMEM
 constexpr int SMEM_LIMIT = 227 * 1024;
 
-template <int BN>
+// Tile shapes: 160 columns (a multiple of every SD head width), 80 for launches with few rows, 128 and 64 for heads of 64 channels
+// and matrices that are no multiple of 80.  One CTA per SM: what a launch costs beyond its K loop is the latency of a few
+// hand-overs between warps, and more warps per role shorten it more than a second CTA hides it.
+template <int BN_>
 struct Tile {
-    static constexpr int HC = BN / 2;                                         // columns per worker thread
-    static constexpr int B_TILE_BYTES = ((BN * BK * 2 + 1023) / 1024) * 1024;
-    static constexpr int STAGE_BYTES = A_TILE_BYTES + B_TILE_BYTES;
-    static constexpr uint32_t TMEM_COLS = 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;
-    static constexpr int CTAS_PER_SM = TMEM_COLS <= 256 ? 2 : 1;
-    static_assert(HC % 8 == 0, "a worker's columns come in groups of 8");
+    static constexpr int BN = BN_;
+    static constexpr int NCG = 2;                                             // column groups: folder threads per row
+    static constexpr int HC = BN / NCG;                                       // columns per folder thread
+    static constexpr int NF = 4 * NCG, NFOLD = 32 * NF;                       // folder warps, threads
+    static constexpr int NB = 16, NBUILD = 32 * NB;                           // builder warps, threads
+    // Warpgroups keep one role each, and registers go where they are needed.  What the block is launched with covers it:
+    //   896 threads x 72 = 128 x (56 + 2 x 128 + 4 x 48)
+    static constexpr int NTHREADS = 128 + NFOLD + NBUILD;
+    static constexpr int W_PROD = 0, W_MMA = 1, W_AUX = 2, W_FOLD = 4, W_BUILD = W_FOLD + NF;
+    static constexpr int R_FOLD = 128, R_BUILD = 48, R_REST = 56;
+    static_assert(128 * (R_REST + NF / 4 * R_FOLD + NB / 4 * R_BUILD) == NTHREADS * 72, "register split");
+    static constexpr uint32_t TMEM_COLS = BN >= 128 ? 512 : 256;
+    static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 or 4
+    static constexpr int B_TILE = BN * 128;                                   // one k-block
+    static constexpr int NCH = BN * 16 / (NBUILD / 2);                        // 16-byte tile chunks per builder thread and pair of k-blocks
+    static constexpr int PART_ROW = HC * 4 + 16;                              // a thread's partial sums in transit, padded against bank conflicts
+    static constexpr int PIECE = 32 * PART_ROW;                               // ... of one warp
+    static_assert(BN * 16 % (NBUILD / 2) == 0 && HC % 8 == 0 && NSLOT <= MAX_SLOT && NSLOT >= 3, "tile shape");
 };
 
 struct Bars {
-    uint64_t full_a[MAX_STAGE];
-    uint64_t full_b[MAX_PREBUILT];
-    uint64_t empty[MAX_STAGE];
-    uint64_t w_full;
-    uint64_t acc_full[MAX_ACC];
-    uint64_t acc_free[MAX_ACC];
-    uint64_t part_full[8], part_got[8], peer_ready;   // K loop split over a CTA pair: hand-over of the second CTA's partial sums
-    uint64_t pair_full[4], pair_got[4];               // head split over two column tiles: the rows' absmax from / to the other tile's CTA
+    uint64_t full_a[MAX_STAGE], empty_a[MAX_STAGE], full_b[MAX_STAGE], empty_b[MAX_STAGE];
+    uint64_t acc_full[MAX_SLOT], acc_free[MAX_SLOT];
+    uint64_t scale_full[2], scale_free[2];
+    uint64_t tmem_ready, peer_ready, part_full[8], pair_full[4];
     uint32_t tmem_base;
     volatile int abort_flag;
 };
+constexpr int N_BARS = 4 * MAX_STAGE + 2 * MAX_SLOT + 4 + 2 + 8 + 4;        // the barriers above, one after the other
+static_assert(offsetof(Bars, tmem_base) == N_BARS * 8, "barriers are contiguous");
+
+// How a launch is laid out: CTAs that share the K loop of a tile, ring depths in pairs of k-blocks, bytes of an output staging area
+// of its own (several tiles per CTA), heads of 160 channels on two tiles, tiles.
+struct LinearLayout { int nsplit, nsa, nsb, staging, head_pair, row_tiles, n_tiles; };
 
 // Shared-memory plan of one launch (host and device agree through these numbers).
-struct Plan {
-    int raw_bytes, scale_bytes, bias_bytes;   // BN rows of codes / scales / bias
-    int stage_bytes;                          // one ring stage: the activation tile, plus the weight tile unless prebuilt
-    int off_ball;                             // prebuilt: the CTA's expanded weight tiles, one per k-block
-    int off_raw, off_scales, off_scales_t, off_bias, off_xchg, off_bars, total;
-};
+struct Plan { int ring_bytes, off_scales, scale_bytes, off_bias, off_xchg, off_staging, off_bars, total; };
 
-// prebuilt = number of k-blocks of the CTA when all of its expanded weight tiles are resident at once (0: the tiles go
-// through the ring with the activations).
+// nsa, nsb: pairs of k-blocks in the rings; staging: bytes of an output staging area of its own (0: the epilogue stages in the
+// rings, which are free by then unless the CTA walks several tiles).
 template <int BN>
-__host__ __device__ inline Plan make_plan(int k_in, int bits, int group, int nstage, int mode, int prebuilt = 0) {
-    const WeightLayout L = weight_layout(BN, k_in, bits, group);
+__host__ __device__ inline Plan make_plan(int n_groups, int nsa, int nsb, int staging) {
     Plan p;
-    p.stage_bytes = prebuilt ? A_TILE_BYTES : Tile<BN>::STAGE_BYTES;
-    p.off_ball = nstage * p.stage_bytes;
-    // codes of the BN channels over the whole fan-in; mode 1: none (the codes are the B operand); mode 2: one 64-byte slice
-    // per channel and ring stage
-    p.raw_bytes = mode == 1 ? 0 : mode == 2 ? nstage * BN * BK : (int)(L.row_bytes * BN);
-    p.scale_bytes = BN * L.n_groups * 4;
-    p.bias_bytes = BN * 4;
-    p.off_raw = p.off_ball + prebuilt * Tile<BN>::B_TILE_BYTES;
-    p.off_scales = p.off_raw + (p.raw_bytes + 127) / 128 * 128;
-    p.off_scales_t = p.off_scales + (p.scale_bytes + 127) / 128 * 128;        // [n_groups][BN]
-    p.off_bias = p.off_scales_t + (p.scale_bytes + 127) / 128 * 128;
-    p.off_xchg = p.off_bias + (p.bias_bytes + 127) / 128 * 128;              // float [2][128]
-    p.off_bars = p.off_xchg + 2048;           // float [2][128] exchange between a row's two threads, [128] out and [128] in for the head pair
-    p.total = p.off_bars + 1024 + 1024;       // barriers + slack to align the base to 1024
+    p.ring_bytes = 2 * (nsa * A_TILE_BYTES + nsb * Tile<BN>::B_TILE);
+    p.off_staging = p.ring_bytes;
+    p.off_scales = p.off_staging + staging;                                   // two buffers of float [n_groups][BN], then bias [BN]
+    p.scale_bytes = (n_groups + 1) * BN * 4;
+    p.off_bias = p.off_scales + n_groups * BN * 4;
+    p.off_xchg = p.off_scales + (staging ? 2 : 1) * p.scale_bytes;            // (one tile per CTA: one buffer) float [4][128]
+    p.off_bars = p.off_xchg + 4 * 128 * 4 + 128;           // (K~/V~: the slots and the bitmap use the second half)
+    p.total = p.off_bars + 1024 + 1024;                                       // barriers + slack to align the base to 1024
     return p;
+}
+
+__device__ __forceinline__ void ffma2(unsigned long long& acc, uint32_t lo, uint32_t hi, unsigned long long s) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(v), "l"(s));
+}
+
+// Packed codes of one 16-byte chunk of a weight tile, as they lie in the blob.
+template <bool I8, bool W8> struct Code { using T = typename std::conditional<I8 && W8, uint4, typename std::conditional<I8 || W8, uint2, uint32_t>::type>::type; };
+template <bool I8, bool W8>
+__device__ __forceinline__ uint4 expand_chunk(const typename Code<I8, W8>::T& p) {
+    if constexpr (I8 && W8) return p;
+    else if constexpr (I8) { const uint2 lo = codes_w4_to_i8(p.x), hi = codes_w4_to_i8(p.y); return make_uint4(lo.x, lo.y, hi.x, hi.y); }
+    else if constexpr (W8) return codes_w8_to_half(p);
+    else return codes_w4_to_half(p);
+}
+template <bool I8, bool W8>
+__device__ __forceinline__ typename Code<I8, W8>::T zero_codes() {
+    if constexpr (I8 && W8) return make_uint4(0, 0, 0, 0);
+    else if constexpr (I8) return make_uint2(0x88888888u, 0x88888888u);      // nibble 8 = code 0
+    else if constexpr (W8) return make_uint2(0, 0);
+    else return 0x88888888u;
 }
 
 // I8: the integer-activation variant (the literal W/A reading of Table 1).  The A operand is the int8 codes of the
 // per-token-quantized activations, the B operand the int8 weight codes, the accumulators are exact int32; a K block is
 // 128 elements (one W4 scale group), and the row's activation scale multiplies the folded sum at the end.
-// SPLIT: for launches with few tiles and a long K loop, two CTAs (a cluster of two along x) share one output tile: the first
-// takes the lower half of the scale groups (of the k-blocks, when there is one group), the second the upper half; then
-// they exchange folded fp32 partial sums through bulk copies between the two shared memories, the first CTA adding and
-// storing rows 0..63 of the tile, the second rows 64..127.
-template <int BN, bool I8, bool SPLIT>
-__global__ void __launch_bounds__(NTHREADS, Tile<BN>::CTAS_PER_SM) linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_y, const LinearArgs a, const int nstage, const int prebuilt) {
+// KV: the K~/V~ epilogue.  The K and the V projection are one launch: the first half of the column tiles is K's.
+// nsplit > 1: for launches with few tiles and a long K loop, two or four CTAs (a cluster) share one output tile: each
+// takes a share of the scale groups (of the k-blocks, when there is one group); then they exchange folded fp32 partial sums
+// through bulk copies between the shared memories, every CTA adding and storing its share of the tile's rows.
+template <int BN, bool I8, bool W8, bool KV>
+__global__ void __launch_bounds__(Tile<BN>::NTHREADS, 1)
+linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_y, const LinearArgs a, const LinearLayout lay) {
     using TL = Tile<BN>;
+    using CodeT = typename Code<I8, W8>::T;
+    constexpr int HC = TL::HC, NCG = TL::NCG, NSLOT = TL::NSLOT, NCH = TL::NCH;
     constexpr int BKE = I8 ? 2 * BK : BK;             // elements per K block
-    constexpr int HC = TL::HC;
+    constexpr int FC = HC == 80 ? 16 : HC == 64 ? 32 : HC;      // columns in flight while a group is folded
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* smem = smem_dyn + ((1024u - (ptx::smem_u32(smem_dyn) & 1023u)) & 1023u);   // 1024-byte aligned, still provably shared
-    const Plan P = make_plan<BN>(a.k_in, a.bits, a.group, nstage, a.w_direct, prebuilt);
-    static_assert(sizeof(Bars) <= 1024, "barrier block");
-    Bars* bars = reinterpret_cast<Bars*>(smem + P.off_bars);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int z = blockIdx.z;
-    const int rank = SPLIT ? (int)(blockIdx.x & 1) : 0;
-    const int row0 = (SPLIT ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * BM;
-    const int col0 = blockIdx.y * BN;
-    const int n_kb = (a.k_in + BKE - 1) / BKE;          // (int8: the last block may be ragged; TMA and the expansion zero-fill)
-    const uint8_t* blob = (const uint8_t*)(a.reqs ? (a.which == 0 ? a.reqs[z].Wq : a.reqs[z].Wout) : a.w);
+    const int nsplit = lay.nsplit, nsa = lay.nsa, nsb = lay.nsb;
+    const int rank = nsplit > 1 ? (int)(blockIdx.x % (unsigned)nsplit) : 0;
     const WeightLayout L = weight_layout(a.n_out, a.k_in, a.bits, a.group);
     const int n_groups = L.n_groups;
-    const int kb_per_group = n_groups == 1 ? n_kb : L.group_len / BKE;   // k-blocks in a full group (the last group may be shorter)
-    // this CTA's share of the K loop: all of it, one half of the scale groups, or (one scale per output channel) one half
-    // of the k-blocks of the only group
-    const bool split_kb = SPLIT && n_groups == 1;
-    const int g_begin = SPLIT && !split_kb && rank ? n_groups / 2 : 0, g_end = SPLIT && !split_kb && !rank ? n_groups / 2 : n_groups;
-    const int kb_begin = split_kb ? (rank ? n_kb / 2 : 0) : g_begin * kb_per_group;
-    const int kb_stop = split_kb ? (rank ? n_kb : n_kb / 2) : min(n_kb, g_end * kb_per_group);
-    // Accumulators: two (the workers fold one while the tensor core fills the other), or, when the weight tiles are all
-    // built before the first fold (prebuilt), one per scale group of the CTA as far as TMEM holds them, so that no MMA
-    // waits for a fold.
-    const int n_acc = prebuilt ? max(1, min(min(g_end - g_begin, 512 / BN), MAX_ACC)) : 2;
-    uint32_t tmem_cols = TL::TMEM_COLS;
-    if (prebuilt) for (tmem_cols = 32; tmem_cols < (uint32_t)(n_acc * BN); tmem_cols *= 2) {}
-    constexpr uint32_t PART_ROW = (uint32_t)BN * 2u + 16u;           // a thread's fp32 partial sums (BN / 2 columns), padded against bank conflicts
+    const Plan P = make_plan<BN>(n_groups, nsa, nsb, lay.staging);
+    static_assert(sizeof(Bars) <= 1024, "barrier block");
+    Bars* bars = reinterpret_cast<Bars*>(smem + P.off_bars);
+    const int n_kb_all = (a.k_in + BKE - 1) / BKE;      // (int8: the last block may be ragged; TMA and the expansion zero-fill)
+    const int kb_per_group = n_groups == 1 ? n_kb_all : L.group_len / BKE;   // k-blocks in a full group (the last group may be shorter)
+    // this CTA's share of the K loop: a run of whole scale groups, or (one scale per output channel) of k-blocks
+    int g_begin = 0, g_end = n_groups, kb_begin = 0, kb_stop = n_kb_all;
+    if (nsplit > 1) {
+        if (n_groups == 1) {
+            kb_begin = n_kb_all * rank / nsplit; kb_stop = n_kb_all * (rank + 1) / nsplit;
+        } else {
+            g_begin = n_groups * rank / nsplit; g_end = n_groups * (rank + 1) / nsplit;
+            kb_begin = g_begin * kb_per_group; kb_stop = min(n_kb_all, g_end * kb_per_group);
+        }
+    }
+    const int n_kb = kb_stop - kb_begin;
+    const bool clustered = nsplit > 1;
+    const bool with_bias = !KV && a.epi != EPI_Q8_HEAD && (I8 || rank == 0);   // (of CTAs that share a tile one starts from the bias)
+    // Tiles: column tile fastest, so that the CTAs running at one time share rows of x; then row tile, then z.
+    const int n_col = a.n_out / BN, n_cols = KV ? 2 * n_col : n_col, n_rows = lay.row_tiles;
+    const int tile0 = (int)(blockIdx.x / (unsigned)nsplit), tile_step = (int)(gridDim.x / (unsigned)nsplit);
+    auto tile_of = [&](int t, int& z, int& row0, int& col0, int& kv_which) {
+        const int cz = t / n_cols;
+        int c = t - cz * n_cols;
+        z = cz / n_rows;
+        row0 = (cz - z * n_rows) * BM;
+        kv_which = KV && c >= n_col ? 1 : 0;
+        if (kv_which) c -= n_col;
+        col0 = c * BN;
+    };
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(30); }
-    if (tid == 0) {
-        for (int s = 0; s < MAX_STAGE; ++s) {
-            ptx::mbar_init(&bars->full_a[s], 1);
-            ptx::mbar_init(&bars->empty[s], 1);
+    if (warp == TL::W_PROD) {
+        // (one lane per barrier: fifty in a row by one thread took a fifth of a small launch's start)
+        uint64_t* all = bars->full_a;
+        for (int i = lane; i < N_BARS; i += 32) {
+            const uint64_t* bar = all + i;
+            const uint32_t count = bar >= bars->full_b && bar < bars->empty_b ? TL::NB / 2 : bar >= bars->acc_free && bar < bars->scale_full ? TL::NF :
+                                   bar >= bars->scale_full && bar < bars->scale_free ? 2 : bar >= bars->scale_free && bar < &bars->tmem_ready ? TL::NF :
+                                   bar == &bars->peer_ready && clustered ? nsplit - 1 : 1;
+            ptx::mbar_init(all + i, count);
         }
-        for (int s = 0; s < MAX_PREBUILT; ++s) ptx::mbar_init(&bars->full_b[s], NWORK / 32);    // one arrival per worker warp
-        ptx::mbar_init(&bars->w_full, 1);
-        for (int i = 0; i < MAX_ACC; ++i) {
-            ptx::mbar_init(&bars->acc_full[i], 1);
-            ptx::mbar_init(&bars->acc_free[i], NWORK / 32);
-        }
-        for (int i = 0; i < 8; ++i) { ptx::mbar_init(&bars->part_full[i], 1); ptx::mbar_init(&bars->part_got[i], 1); }
-        ptx::mbar_init(&bars->peer_ready, 1);
-        for (int i = 0; i < 4; ++i) { ptx::mbar_init(&bars->pair_full[i], 1); ptx::mbar_init(&bars->pair_got[i], 1); }
-        bars->abort_flag = 0;
         ptx::mbar_fence_init();
-        if (SPLIT)                                          // the worker warps whose rows this CTA finishes receive a piece each
-            for (int i = 0; i < 8; ++i)
-                if (((i & 3) >> 1) == rank) ptx::mbar_arrive_expect_tx(&bars->part_full[i], 32u * PART_ROW);
-        if (SPLIT && a.head_pair)                           // the TMEM lane quarters whose rows this CTA finishes: (q + 2) & 3 of worker warp q
-            for (int ww = 0; ww < 4; ++ww)
-                if ((ww >> 1) == rank) ptx::mbar_arrive_expect_tx(&bars->pair_full[(ww + 2) & 3], 128u);
-        ptx::tma_prefetch_desc(&tmap_x);
-    }
-    if (warp == 1) ptx::tmem_alloc(&bars->tmem_base, tmem_cols);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
-    const uint32_t tmem_base = bars->tmem_base;
-    ptx::pdl_trigger();
-    if (SPLIT) ptx::cluster_sync_all();                    // the partner's barriers exist before anything arrives on them
-
-    if (warp == 0) {
-        // ---------------- producer: packed weights once, then activation tiles ----------------
+        __syncwarp();
         if (lane == 0) {
-            if (!a.early_weights) ptx::pdl_wait();        // in general the weights may come from the previous kernel
-            const int staged = a.w_direct ? 0 : P.raw_bytes;
-            ptx::mbar_arrive_expect_tx(&bars->w_full, (uint32_t)(staged + P.scale_bytes + P.bias_bytes));
-            if (staged) ptx::bulk_load(smem + P.off_raw, blob + L.off_codes + (size_t)col0 * L.row_bytes, (uint32_t)P.raw_bytes, &bars->w_full);
-            ptx::bulk_load(smem + P.off_scales, blob + L.off_scales + (size_t)col0 * n_groups * 4, (uint32_t)P.scale_bytes, &bars->w_full);
-            ptx::bulk_load(smem + P.off_bias, blob + L.off_bias + (size_t)col0 * 4, (uint32_t)P.bias_bytes, &bars->w_full);
-            if (a.early_weights) ptx::pdl_wait();         // the activations come from the previous kernel
-            TAQ_PROF(1); TAQ_GPROF(28);
-            int issued = 0, s = 0;
-            uint32_t ph = 0;                               // parity of the ring pass
-            for (int kb = kb_begin; kb < kb_stop; ++kb) {
-                if (kb - kb_begin >= nstage && !ptx::mbar_wait(&bars->empty[s], ph ^ 1)) { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; }
-                if (bars->abort_flag) break;
-                ptx::mbar_arrive_expect_tx(&bars->full_a[s], A_TILE_BYTES + (a.w_direct == 1 ? BN * 128 : a.w_direct == 2 ? BN * BK : 0));
-                ptx::tma_load_3d(smem + s * P.stage_bytes, &tmap_x, &bars->full_a[s], kb * BKE, row0, z);
-                if (a.w_direct == 1) ptx::tma_load_3d(smem + s * P.stage_bytes + A_TILE_BYTES, &tmap_w, &bars->full_a[s], kb * BKE, col0, 0);
-                if (a.w_direct == 2) ptx::tma_load_3d(smem + P.off_raw + s * (BN * BK), &tmap_w, &bars->full_a[s], kb * BK, col0, 0);
-                issued = kb - kb_begin + 1;
-                if (++s == nstage) { s = 0; ph ^= 1; }
-            }
-            if (bars->abort_flag) {   // give copies that are still in flight a bounded chance to land before the CTA exits
-                (void)ptx::mbar_wait(&bars->w_full, 0);
-                for (int kb = issued > nstage ? issued - nstage : 0; kb < issued; ++kb) (void)ptx::mbar_wait(&bars->full_a[kb % nstage], (kb / nstage) & 1);
+            bars->abort_flag = 0;
+            if (clustered) {
+                const int per_cta = 4 / nsplit;              // lane quarters whose rows a CTA finishes
+                for (int cg = 0; cg < NCG; ++cg)             // the warps of those quarters receive a piece from every other CTA
+                    for (int i = 0; i < per_cta; ++i) ptx::mbar_arrive_expect_tx(&bars->part_full[cg * 4 + rank * per_cta + i], (uint32_t)((nsplit - 1) * TL::PIECE));
+                if (lay.head_pair)
+                    for (int i = 0; i < per_cta; ++i) ptx::mbar_arrive_expect_tx(&bars->pair_full[rank * per_cta + i], 128u);
             }
         }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer: one accumulation pass per scale group ----------------
-        // All 32 lanes walk the control flow, so that loop state and descriptor words stay warp-uniform; one elected lane
-        // issues.  The path between two MMAs is kept short: this warp shares its scheduler with worker warps.
-        const bool leader = ptx::elect_one();
-        auto wait = [&](uint64_t* bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, ptx::mbar_wait(bar, parity) && !bars->abort_flag) != 0; };
-        constexpr uint32_t idesc = I8 ? ptx::idesc_i8_m128(BN) : ptx::idesc_f16_m128(BN);
-        constexpr uint32_t HI = ptx::kDescHiSw128;
-        const uint32_t lo0 = ptx::desc_lo(ptx::smem_u32(smem));
-        int s = 0, kb = kb_begin;
-        uint32_t ph = 0;
-        bool ok = true;
-        for (int g = g_begin; g < g_end && ok; ++g) {
-            const int gl = g - g_begin;
-            const int buf = gl % n_acc;
-            if (gl >= n_acc) {                              // the workers have emptied this accumulator
-                if (!wait(&bars->acc_free[buf], (gl / n_acc - 1) & 1)) { ok = false; break; }
-                ptx::tc_fence_after_sync();
-            }
-            const int kb_end = min(kb_stop, kb + kb_per_group);
-            for (bool first = true; kb < kb_end && ok; ++kb) {
-                // (prebuilt: every weight tile has its own barrier, complete long before its activations arrive)
-                if ((a.w_direct != 1 && !wait(&bars->full_b[prebuilt ? kb - kb_begin : s], prebuilt ? 0u : ph)) || !wait(&bars->full_a[s], ph)) { ok = false; break; }
-                if (leader) {
-                    if (kb < 20) TAQ_PROF(40 + kb);
-                    const uint32_t a_lo = lo0 + s * (P.stage_bytes >> 4);
-                    const uint32_t b_lo = prebuilt ? lo0 + ((P.off_ball + (kb - kb_begin) * TL::B_TILE_BYTES) >> 4) : a_lo + (A_TILE_BYTES >> 4);
+    } else if (warp == TL::W_AUX && lane == 0) {
+        ptx::tma_prefetch_desc(&tmap_x);
+        ptx::tma_prefetch_desc(&tmap_y);
+    }
+    // Every role passes this barrier before it touches another role's state; the builders do so with their first codes under way.
+    auto start = [&]() {
+        __syncthreads();
+        ptx::pdl_trigger();
+        if (clustered) ptx::cluster_arrive();                // waited for right before the first operation on another CTA
+    };
+    auto blob_of = [&](int z, int kv_which) { return (const uint8_t*)(a.reqs ? ((KV ? kv_which : a.which) == 0 ? a.reqs[z].Wq : a.reqs[z].Wout) : kv_which ? a.w2 : a.w); };
+    auto give_up = [&]() { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; };
+
+    // K~/V~, second half: all folders and builders, once the fp32 tile and the scales of its rows are in shared memory.  Short loops
+    // over 8-element chunks, neighbouring lanes on neighbouring chunks, write everything in runs.  (With a row per lane straight
+    // from the registers this epilogue took 15 000 - 24 000 cycles: 32 sectors per store, 20 KB of unrolled code that runs
+    // once.  With the eight folder warps alone these loops took 9 000: two warps on a scheduler hide no latency.)
+    const int kv_staging_off = clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0;
+    constexpr int KV_STRIDE = BN + 1;                        // floats (odd: a row per lane is free of bank conflicts)
+    auto kv_store = [&](int w) {
+        constexpr int NT = TL::NFOLD + TL::NBUILD, NC8 = BN / 8;
+        int z, row0, col0, kv_which;
+        tile_of(tile0, z, row0, col0, kv_which);
+        const int T = a.n_ctx, d = a.n_out / a.heads, nh = BN / d, head0 = col0 / d;
+        const taq_kv_layout KL = kv_layout(a.heads, T, d, a.max_trigger);
+        uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * KL.block_bytes;
+        OperandGeom G;
+        const bool images = operand_geom(d, T, &G);
+        uint8_t* img0 = blk + KL.off_operands + (size_t)head0 * G.head_bytes;
+        const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 256;
+        const float* ys = reinterpret_cast<const float*>(smem + kv_staging_off);
+        const float2* hs = reinterpret_cast<const float2*>(smem + kv_staging_off + 128 * KV_STRIDE * 4);
+        const int own_shift = nsplit == 1 ? 7 : nsplit == 2 ? 6 : 5;         // (CTAs that share the tile finish the rows of some lane quarters each)
+        auto own = [&](int key) { return key >> own_shift == rank; };
+        {                                                    // codes, trigger rows and K~'s image: 8 channels of a token
+            const int c = (w % NC8) * 8, hl = c / d, ch = c - hl * d, h = head0 + hl;
+            uint8_t* codes = blk + (kv_which ? KL.off_v_codes : KL.off_k_codes) + (size_t)h * T * d + ch;
+            uint8_t* trigs = blk + (kv_which ? KL.off_v_trigger : KL.off_k_trigger) + ((size_t)h * d + ch) * 2;
+            uint8_t* k_img = img0 + (size_t)hl * G.head_bytes + (ch >> 6) * (kOperandKeys * 128);
+            for (int t = w / NC8; t < T && w < NT / NC8 * NC8; t += NT / NC8) {
+                if (!own(t)) continue;
+                const int slot = slots[t];
+                const float rs = hs[hl * 128 + t].y;
+                float f[8];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {            // four 32-byte K slices per 128-byte operand row
-                        if (I8) ptx::mma_i8_ss(tmem_base + buf * BN, ptx::desc_join(HI, a_lo + 2 * k), ptx::desc_join(HI, b_lo + 2 * k), idesc, !(first && k == 0));
-                        else ptx::mma_f16_ss(tmem_base + buf * BN, ptx::desc_join(HI, a_lo + 2 * k), ptx::desc_join(HI, b_lo + 2 * k), idesc, !(first && k == 0));
-                    }
-                    ptx::mma_commit(&bars->empty[s]);       // frees the stage once these MMAs have read it
-                    if (kb + 1 == kb_end) ptx::mma_commit(&bars->acc_full[buf]);
+                for (int e = 0; e < 8; ++e) f[e] = ys[t * KV_STRIDE + c + e];
+                const uint2 code = slot == -1 ? quant8(f, rs) : make_uint2(0, 0);
+                *reinterpret_cast<uint2*>(codes + t * d) = code;
+                uint4 k8 = codes_w8_to_half(code);
+                if (slot >= 0) {
+                    k8 = pack8(f);
+                    *reinterpret_cast<uint4*>(trigs + (size_t)slot * a.n_out * 2) = k8;
                 }
-                first = false;
-                if (++s == nstage) { s = 0; ph ^= 1; }
+                if (images && !kv_which) *reinterpret_cast<uint4*>(k_img + ptx::sw128_offset(t, (ch >> 3) & 7)) = k8;
             }
         }
-        if (!ok && leader) {
-            raise_status(a.status, TAQ_ERR_TIMEOUT);
-            bars->abort_flag = 1;
-            for (int i = 0; i < n_acc; ++i) ptx::mma_commit(&bars->acc_full[i]);        // wake the workers; they see the abort flag
-        }
-    } else {
-        // ---------------- workers (warps 2..9) ----------------
-        const int wt = tid - 64;                          // 0..255
-        const int q = warp & 3;                           // TMEM lane quarter this warp may read
-        const int half = (warp - 2) >> 2;                 // which half of the tile's columns this thread owns
-        const int r = q * 32 + lane;
-        long long row = (long long)row0 + r;
-        const int cb = half * HC;                         // first owned column inside the tile
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + cb;
-        const unsigned char* raw = smem + P.off_raw;
-        const float* wscales = reinterpret_cast<const float*>(smem + P.off_scales);
-        float* scales_t = reinterpret_cast<float*>(smem + P.off_scales_t);
-        const float* bias = reinterpret_cast<const float*>(smem + P.off_bias);
-        float* xchg = reinterpret_cast<float*>(smem + P.off_xchg);
-        const int row_bytes = (int)L.row_bytes;
-        bool ok = ptx::mbar_wait(&bars->w_full, 0);
-        if (wt == 0) TAQ_PROF(2);
-        if (!ok) { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; }
-        // scales [BN][n_groups] -> [n_groups][BN], so that a group's scales of consecutive columns are contiguous
-        for (int i = wt; i < BN * n_groups; i += NWORK) scales_t[(i % n_groups) * BN + i / n_groups] = wscales[i];
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-
-        float y[HC];
+        if (!images) return;
+        if (!kv_which) {                                     // K~'s padding: keys T..79, and the channels behind the head's last
+            const int ncc = G.kbq * 8;
+            for (int line = w >> 3; line < nh * kOperandKeys; line += NT / 8) {
+                const int hl = line / kOperandKeys, t = line - hl * kOperandKeys;
+                if (!own(t)) continue;
+                for (int cc = (w & 7) + (t >= T || d >= 64 ? 0 : d / 8 & ~7); cc < ncc; cc += 8)
+                    if (t >= T || cc * 8 >= d) *reinterpret_cast<uint4*>(img0 + (size_t)hl * G.head_bytes + (cc >> 3) * (kOperandKeys * 128) + ptx::sw128_offset(t, cc & 7)) = make_uint4(0, 0, 0, 0);
+            }
+        } else {
+            // V~^T: 8 keys of a channel per lane; a warp takes 8 channels x 4 chunks of keys (reads of the fp32 tile without bank
+            // conflicts, stores of 64 contiguous bytes).
+            const int wl = w & 31;
+            for (int u = w >> 5; u < nh * (G.dp >> 3) * 4; u += NT / 32) {
+                const int jc = (u & 3) * 4 + (wl >> 3), line = (u >> 2) * 8 + (wl & 7), hl = line / G.dp, ch = line - hl * G.dp;
+                if (!own(jc * 8)) continue;
+                const float* col = ys + jc * 8 * KV_STRIDE + hl * d + ch;
+                const int n_real = ch < d ? min(8, T - jc * 8) : 0;
+                __half v[8];
 #pragma unroll
-        for (int c = 0; c < HC; ++c) y[c] = 0.f;
-
-        // y += scale[g] * accumulator of group g (this thread's HC columns of its row)
-        auto fold_group = [&](int g) -> bool {
-            const int buf = (g - g_begin) % n_acc;
-            if (!ptx::mbar_wait(&bars->acc_full[buf], ((g - g_begin) / n_acc) & 1) || bars->abort_flag) return false;
-            ptx::tc_fence_after_sync();
-            const float* sg = scales_t + g * BN + cb;
-#pragma unroll
-            for (int c0 = 0; c0 < HC; c0 += 40) {
-                constexpr int N8MAX = 5;
-                uint32_t v[N8MAX][8];
-#pragma unroll
-                for (int i = 0; i < N8MAX; ++i)
-                    if (c0 + i * 8 < HC) ptx::tmem_ld8(taddr + buf * BN + c0 + i * 8, v[i]);
-                ptx::tmem_ld_wait(v[0]);
-#pragma unroll
-                for (int i = 1; i < N8MAX; ++i) ptx::reg_fence8(v[i]);
-#pragma unroll
-                for (int i = 0; i < N8MAX; ++i)
-                    if (c0 + i * 8 < HC) {
-                        const float4 s0 = *reinterpret_cast<const float4*>(sg + c0 + i * 8), s1 = *reinterpret_cast<const float4*>(sg + c0 + i * 8 + 4);
-                        float* yy = y + c0 + i * 8;
-                        float f[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) f[e] = I8 ? __int2float_rn((int)v[i][e]) : __uint_as_float(v[i][e]);
-                        yy[0] = fmaf(f[0], s0.x, yy[0]); yy[1] = fmaf(f[1], s0.y, yy[1]);
-                        yy[2] = fmaf(f[2], s0.z, yy[2]); yy[3] = fmaf(f[3], s0.w, yy[3]);
-                        yy[4] = fmaf(f[4], s1.x, yy[4]); yy[5] = fmaf(f[5], s1.y, yy[5]);
-                        yy[6] = fmaf(f[6], s1.z, yy[6]); yy[7] = fmaf(f[7], s1.w, yy[7]);
+                for (int e = 0; e < 8; ++e) {
+                    float x = 0.f;
+                    if (e < n_real) {
+                        x = col[e * KV_STRIDE];
+                        const float2 sc = hs[hl * 128 + jc * 8 + e];
+                        if (slots[jc * 8 + e] < 0) x = __fmul_rn(fmaf(x, sc.y, 12582912.0f) - 12582912.0f, sc.x);
                     }
+                    v[e] = __float2half_rn(x);
+                }
+                *reinterpret_cast<uint4*>(img0 + (size_t)hl * G.head_bytes + G.k_bytes + (jc >> 3) * (G.dp * 128) + ptx::sw128_offset(ch, jc & 7)) = *reinterpret_cast<const uint4*>(v);
             }
+        }
+    };
+    // The folders hand registers to the builders on the way, 128 x (56 + 2 x 80 + 4 x 72) = 896 x 72: they give theirs back before
+    // the barrier, the builders ask behind it.  (A builder that asked as soon as it ran out of work could be given what the
+    // folders' first request was still waiting for, and neither would ever go on.)
+    auto kv_together = [&](bool folder, int w) {
+        if (folder) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        asm volatile("bar.sync 15, %0;" ::"n"(TL::NFOLD + TL::NBUILD) : "memory");
+        if (!folder) asm volatile("setmaxnreg.inc.sync.aligned.u32 72;");
+        if (!bars->abort_flag) kv_store(w);
+    };
+
+    if (warp >= TL::W_FOLD && warp < TL::W_BUILD) {
+        // ---------------- folders ----------------
+        start();
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::R_FOLD));
+        const int ft = tid - 32 * TL::W_FOLD;
+        const int q = warp & 3;                              // TMEM lane quarter this warp may read
+        const int cg = (warp - TL::W_FOLD) >> 2;             // column group
+        const int fw = cg * 4 + q;
+        const int r = q * 32 + lane;
+        const int cb = cg * HC;                              // first owned column inside the tile
+        int slot = 0, sbuf = 0;
+        uint32_t ph_acc = 0, ph_scale = 0;
+        bool joined = false;                                 // has waited for the cluster's first barrier
+        uint32_t tmem_base = 0;
+        if (ptx::mbar_wait(&bars->tmem_ready, 0)) tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base); else give_up();
+        for (int tile = tile0; tile < lay.n_tiles; tile += tile_step) {
+            int z, row0, col0, kv_which;
+            tile_of(tile, z, row0, col0, kv_which);
+            const float* scales = reinterpret_cast<const float*>(smem + P.off_scales + sbuf * P.scale_bytes) + cb;
+            const float* bias = scales + n_groups * BN;
+            unsigned long long y2[HC / 2];
+            bool ok = ptx::mbar_wait(&bars->scale_full[sbuf], ph_scale);
+#pragma unroll
+            for (int c = 0; c < HC; c += 4) {                // the sums start from the bias (zero where there is none; int8: added last)
+                const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(bias + c);
+                y2[c / 2] = I8 ? 0ull : b4.x; y2[c / 2 + 1] = I8 ? 0ull : b4.y;
+            }
+            // y += scale[g] * accumulator of group g (this thread's HC columns of its row)
+            for (int g = g_begin; g < g_end && ok; ++g) {
+                ok = ptx::mbar_wait(&bars->acc_full[slot], ph_acc);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + slot * BN + cb;
+                const float* sg = scales + g * BN;
+#pragma unroll
+                for (int c0 = 0; c0 < HC; c0 += FC) {
+                    uint32_t v[FC / 8][8];
+#pragma unroll
+                    for (int i = 0; i < FC / 8; ++i) ptx::tmem_ld8(taddr + c0 + i * 8, v[i]);
+                    ptx::tmem_ld_wait(v[0]);
+#pragma unroll
+                    for (int i = 1; i < FC / 8; ++i) ptx::reg_fence8(v[i]);
+                    if (c0 + FC == HC) {                     // the accumulator is in registers: the tensor core may have it back
+                        ptx::tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive(&bars->acc_free[slot]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < FC / 8; ++i) {
+                        const ulonglong2 s0 = *reinterpret_cast<const ulonglong2*>(sg + c0 + i * 8), s1 = *reinterpret_cast<const ulonglong2*>(sg + c0 + i * 8 + 4);
+                        if (I8) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) v[i][e] = __float_as_uint(__int2float_rn((int)v[i][e]));
+                        }
+                        unsigned long long* yy = y2 + (c0 + i * 8) / 2;
+                        ffma2(yy[0], v[i][0], v[i][1], s0.x); ffma2(yy[1], v[i][2], v[i][3], s0.y);
+                        ffma2(yy[2], v[i][4], v[i][5], s1.x); ffma2(yy[3], v[i][6], v[i][7], s1.y);
+                    }
+                }
+                if (++slot == NSLOT) { slot = 0; ph_acc ^= 1; }
+            }
+            if (!ok) give_up();
+            if (tile == tile0) ptx::pdl_wait();              // (already satisfied: the activations have arrived) orders the stores below
+            if (ft == 0) TAQ_PROF(7);
+            asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");         // every folder gets here; the decision below is uniform
+            if (bars->abort_flag) break;
+            if (!I8 && lane == 0) ptx::mbar_arrive(&bars->scale_free[sbuf]);     // scales and biases of this tile have been read
+
+            float y[HC];
+#pragma unroll
+            for (int c = 0; c < HC / 2; ++c) asm("mov.b64 {%0, %1}, %2;" : "=f"(y[2 * c]), "=f"(y[2 * c + 1]) : "l"(y2[c]));
+
+            bool mine = true;                                // this CTA finishes the warp's rows
+            if (clustered) {
+                // All of this CTA's MMAs are complete (every group was folded), so its rings are free: they hold the partial
+                // sums in transit.  CTA `owner` of the cluster finishes the rows of 4 / nsplit lane quarters: a folder warp
+                // either hands its 32 rows to that CTA (one bulk copy between the shared memories) or receives a piece from
+                // every other CTA and adds them in rank order, so that every output is the same sum whoever computes it.
+                const int per_cta = 4 / nsplit, owner = q / per_cta;
+                const uint32_t base = ptx::cluster_ctarank() - (uint32_t)rank;        // ranks along x are consecutive
+                mine = owner == rank;
+                ptx::cluster_wait();                         // the other CTAs' barriers exist
+                joined = true;
+                if (ft < nsplit && ft != rank) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), base + (uint32_t)ft));
+                const int n_send = NCG * (4 - per_cta);
+                if (!mine) {
+                    unsigned char* piece = smem + (cg * (4 - per_cta) + (q < rank * per_cta ? q : q - per_cta)) * TL::PIECE;
+                    float* out = reinterpret_cast<float*>(piece + lane * TL::PART_ROW);
+#pragma unroll
+                    for (int c = 0; c < HC; c += 4) *reinterpret_cast<float4*>(out + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (ptx::mbar_wait(&bars->peer_ready, 0)) {                      // the other CTAs' rings are free, too
+                            const int src_idx = rank < owner ? rank : rank - 1;
+                            const int dst = (n_send + (cg * per_cta + q - owner * per_cta) * (nsplit - 1) + src_idx) * TL::PIECE;
+                            ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(smem + dst), base + (uint32_t)owner), piece, (uint32_t)TL::PIECE,
+                                                  ptx::map_to_cta(ptx::smem_u32(&bars->part_full[fw]), base + (uint32_t)owner));
+                        } else give_up();
+                    }
+                } else if (!ptx::mbar_wait(&bars->part_full[fw], 0)) {
+                    give_up();
+                } else {
+                    const unsigned char* in = smem + (n_send + (cg * per_cta + q - rank * per_cta) * (nsplit - 1)) * TL::PIECE + lane * TL::PART_ROW;
+                    if (nsplit == 2) {
+#pragma unroll
+                        for (int c = 0; c < HC; c += 4) {
+                            const float4 p4 = *reinterpret_cast<const float4*>(in + c * 4);
+                            y[c] += p4.x; y[c + 1] += p4.y; y[c + 2] += p4.z; y[c + 3] += p4.w;
+                        }
+                    } else {
+                        // rank order: ((p0 + p1) + p2) + p3, this CTA's own sum in its place
+#pragma unroll
+                        for (int c = 0; c < HC; c += 4) {
+                            float4 p[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                p[k] = k == rank ? make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]) : *reinterpret_cast<const float4*>(in + (k < rank ? k : k - 1) * TL::PIECE + c * 4);
+                            y[c] = ((p[0].x + p[1].x) + p[2].x) + p[3].x; y[c + 1] = ((p[0].y + p[1].y) + p[2].y) + p[3].y;
+                            y[c + 2] = ((p[0].z + p[1].z) + p[2].z) + p[3].z; y[c + 3] = ((p[0].w + p[1].w) + p[2].w) + p[3].w;
+                        }
+                    }
+                }
+                asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");     // pieces read: the epilogue stages output where they were ...
+                if (ft == 0) TAQ_PROF(10);
+                if (bars->abort_flag) break;
+            }
+            // ... but not over this CTA's outgoing pieces, which may still be in flight: the staging area begins behind them
+            unsigned char* staging = smem + (lay.staging ? P.off_staging : clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0);
+
+            const long long row = (long long)row0 + r;
+            const bool live = mine && row < a.rows;
+            if (I8) {                                        // x~ = code * s_x: the row's activation scale
+                const float sx = live ? a.x_scales[(size_t)z * a.rows + row] : 0.f;
+#pragma unroll
+                for (int c = 0; c < HC; c += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(bias + c);
+                    y[c] = fmaf(y[c], sx, b4.x); y[c + 1] = fmaf(y[c + 1], sx, b4.y); y[c + 2] = fmaf(y[c + 2], sx, b4.z); y[c + 3] = fmaf(y[c + 3], sx, b4.w);
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&bars->scale_free[sbuf]);
+            }
+
+            // ---------------- epilogue on this thread's HC columns ----------------
+            // Dense outputs are staged per warp in shared memory as boxes of 32 rows and leave by TMA stores (the tensor map
+            // clips rows beyond the matrix).  A box row is 80 bytes (an odd number of 16-byte units) or swizzled, so that
+            // the row-per-lane writes are free of bank conflicts.
+            const bool store_rows = mine && (long long)row0 + q * 32 < a.rows;
+            if (!KV && a.epi != EPI_Q8_HEAD) {
+                auto dense = [&](auto f16_c) {
+                    constexpr bool F16 = decltype(f16_c)::value;
+                    constexpr bool B80 = HC % 40 == 0;
+                    constexpr int BOX = B80 ? (F16 ? 40 : 20) : 32;                  // columns
+                    constexpr int BOX_BYTES = B80 ? 2560 : F16 ? 2048 : 4096, NBOX = HC / BOX;
+                    // (several tiles per CTA: one box buffer per warp; else every box has a place of its own in the rings)
+                    unsigned char* st = staging + (size_t)fw * (lay.staging ? 1 : NBOX) * BOX_BYTES;
+#pragma unroll
+                    for (int b = 0; b < NBOX; ++b) {
+                        if (lay.staging) {                                           // the previous store has read the buffer
+                            if (lane == 0) ptx::bulk_store_wait_read();
+                            __syncwarp();
+                        }
+#pragma unroll
+                        for (int c = 0; c < BOX; c += F16 ? 8 : 4) {
+                            const int k = b * BOX + c;
+                            if (F16) {
+                                float f[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) f[e] = y[(k + e) % HC];
+                                *reinterpret_cast<uint4*>(B80 ? st + lane * 80 + c * 2 : st + ptx::sw64_offset(lane, c / 8)) = pack8(f);
+                            } else {
+                                *reinterpret_cast<float4*>(B80 ? st + lane * 80 + c * 4 : st + ptx::sw128_offset(lane, c / 4)) =
+                                    make_float4(y[k], y[(k + 1) % HC], y[(k + 2) % HC], y[(k + 3) % HC]);
+                            }
+                        }
+                        ptx::fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0 && store_rows) {
+                            ptx::tma_store_3d(&tmap_y, st, col0 + cb + b * BOX, row0 + q * 32, z);
+                            ptx::bulk_store_commit();
+                        }
+                        if (!lay.staging) st += BOX_BYTES;
+                    }
+                };
+                if (a.epi == EPI_F16) dense(std::true_type{}); else dense(std::false_type{});
+            } else {
+                // Per-(row, head) symmetric int8.  A thread's columns are whole heads (two of 40, or one), or half of what the row
+                // has of a head in this tile.
+                const int d = a.n_out / a.heads;
+                const int colg = col0 + cb;
+                const int h0 = colg / d;
+                constexpr int SPLIT_AT = HC == 80 ? 40 : HC;  // two heads of 40: columns 0..39 are head h0, the rest h0 + 1
+                const bool two = HC == 80 && d == 40;
+                float am0 = 0.f, am1 = 0.f;
+#pragma unroll
+                for (int c = 0; c < HC; ++c) { if (c < SPLIT_AT) am0 = fmaxf(am0, fabsf(y[c])); else am1 = fmaxf(am1, fabsf(y[c])); }
+                if (!two) { am0 = fmaxf(am0, am1); am1 = am0; }
+                if (d > HC) {
+                    float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [2][128]
+                    xc[cg * 128 + r] = am0;
+                    asm volatile("bar.sync %0, 64;" ::"r"(2 + q) : "memory");
+                    am0 = fmaxf(am0, xc[(cg ^ 1) * 128 + r]);
+                    if (!KV && lay.head_pair && mine) {
+                        // The head's other columns belong to a CTA of the same cluster (same rows, same share of the K loop):
+                        // each sends its rows' absmax over, one 128-byte copy between the shared memories per 32 rows.
+                        const uint32_t me = ptx::cluster_ctarank();
+                        const uint32_t other = me < (uint32_t)nsplit ? me + nsplit : me - nsplit;
+                        if (cg == 0) {
+                            xc[256 + r] = am0;
+                            ptx::fence_proxy_async_smem();
+                            __syncwarp();
+                            if (lane == 0)
+                                ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(xc + 384 + q * 32), other), xc + 256 + q * 32, 128u, ptx::map_to_cta(ptx::smem_u32(&bars->pair_full[q]), other));
+                        }
+                        if (ptx::mbar_wait(&bars->pair_full[q], 0)) am0 = fmaxf(am0, xc[384 + r]);
+                        else give_up();
+                        __syncwarp();
+                    }
+                    am1 = am0;
+                }
+                const float qmax = KV && a.kv_qmax ? (float)a.kv_qmax : 127.f;
+                const float s0 = quant_scale(am0, qmax), s1 = two ? quant_scale(am1, qmax) : s0;
+                const float r0 = s0 > 0.f ? __frcp_rn(s0) : 0.f, r1 = s1 > 0.f ? __frcp_rn(s1) : 0.f;
+                if constexpr (!KV) {
+                    // Q~ = Q_a(Q), Eq. 2 third line.  Boxes of 80 columns (one warp's, or 40 of each of the row's two threads),
+                    // 64 or 32.
+                    constexpr bool SHARED_BOX = HC == 40;
+                    unsigned char* st = staging + (SHARED_BOX ? (size_t)q * 2560 : (size_t)fw * 32 * HC);
+                    if (tile != tile0) {                     // the previous tile's store has read the box
+                        if (lane == 0) ptx::bulk_store_wait_read();
+                        if (SHARED_BOX) asm volatile("bar.sync %0, 64;" ::"r"(6 + q) : "memory"); else __syncwarp();
+                    }
+#pragma unroll
+                    for (int c = 0; c < HC; c += 8)
+                        *reinterpret_cast<uint2*>(HC == 80 ? st + lane * 80 + c : HC == 40 ? st + lane * 80 + cg * 40 + c :
+                                                  HC == 64 ? st + ptx::sw64_offset(lane, c / 16) + (c & 8) : st + ptx::sw32_offset(lane, c / 16) + (c & 8)) = quant8(y + c, c < SPLIT_AT ? r0 : r1);
+                    ptx::fence_proxy_async_smem();
+                    if (SHARED_BOX) asm volatile("bar.sync %0, 64;" ::"r"(6 + q) : "memory"); else __syncwarp();
+                    if (lane == 0 && store_rows && (!SHARED_BOX || cg == 0)) {
+                        ptx::tma_store_3d(&tmap_y, st, SHARED_BOX ? col0 : colg, row0 + q * 32, z);
+                        ptx::bulk_store_commit();
+                    }
+                    if (live) {
+                        float* sc = a.scales + ((size_t)z * a.rows + row) * a.heads;
+                        if (colg == h0 * d) sc[h0] = s0;
+                        if (two) sc[h0 + 1] = s1;
+                    }
+                } else {
+                    // Eq. 2 for K or V of one sequence (a row tile is one sequence; rows beyond its T tokens are the padding keys of
+                    // the images): rows of ordinary tokens -> int8 codes + scale, rows of trigger tokens -> fp16; and the same
+                    // rows once more as the attention kernel's operand images (taq_kv_operands.cu rebuilds them for blocks
+                    // that were not written here): K~ as a row of fp16 integers, V~ as a column of fp16(code * scale).  The
+                    // fp32 tile goes through shared memory to kv_store below.
+                    const int T = a.n_ctx;
+                    const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 256;      // [128] and the bitmap [4], by the scales' warps
+                    const taq_kv_layout KL = kv_layout(a.heads, T, d, a.max_trigger);
+                    uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * KL.block_bytes;
+                    OperandGeom G;
+                    const bool images = operand_geom(d, T, &G);
+                    const int head0 = col0 / d;
+                    float* ys = reinterpret_cast<float*>(staging);                   // [128][KV_STRIDE]
+                    float2* hs = reinterpret_cast<float2*>(staging + 128 * KV_STRIDE * 4);   // [nh][128] scale and its reciprocal
+                    if (mine) {
+                        const int slot = slots[r];           // >= 0: trigger row, -1: ordinary (or padding), -2: a trigger row beyond the capacity
+                        const bool plain = r < T && slot == -1;
+#pragma unroll
+                        for (int c = 0; c < HC; ++c) ys[r * KV_STRIDE + cb + c] = y[c];
+                        const float logit_unit = 1.4426950408889634f / sqrtf((float)d);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            if (k == 1 && !two) break;
+                            const int h = h0 + k;
+                            const float s = plain ? (k ? s1 : s0) : 0.f;
+                            if (k == 0 && colg != h * d) continue;           // the head's first column is another thread's (or CTA's)
+                            hs[(h - head0) * 128 + r] = make_float2(s, plain ? (k ? r1 : r0) : 0.f);
+                            if (r < T) reinterpret_cast<float*>(blk + (kv_which ? KL.off_v_scales : KL.off_k_scales))[(size_t)h * T + r] = s;
+                            if (!kv_which && h == 0) reinterpret_cast<int32_t*>(blk + KL.off_trig_slot)[r] = slot >= 0 ? slot : -1;
+                            if (!kv_which && images && r < kOperandKeys) {
+                                OperandConsts* cst = reinterpret_cast<OperandConsts*>(blk + KL.off_operands + (size_t)h * G.head_bytes + G.k_bytes + G.vt_bytes);
+                                cst->logit_factor[r] = (slot >= 0 ? 1.0f : s) * logit_unit;
+                                if (r < 4) cst->trig_bits[r] = (uint32_t)slots[128 + r];
+                            }
+                        }
+                    }
+                }
+            }
+            sbuf ^= 1;
+            if (sbuf == 0) ph_scale ^= 1;
+        }
+        if (lane == 0) ptx::bulk_store_wait_read();          // shared memory is given back only after the stores have read it
+        __syncwarp();
+        if constexpr (KV) kv_together(true, ft);
+        if (clustered && !joined) ptx::cluster_wait();
+    } else if (warp >= TL::W_BUILD && warp < TL::W_BUILD + TL::NB) {
+        // ---------------- builders ----------------
+        const int bt = (tid - 32 * TL::W_BUILD) & (TL::NBUILD / 2 - 1), group = (warp - TL::W_BUILD) / (TL::NB / 2);
+        unsigned char* b_ring = smem + 2 * nsa * A_TILE_BYTES;
+        // The two halves of the builders take the pairs of k-blocks in turn: a pair costs its warps about 900 cycles of latency
+        // (barrier, expansion, proxy fence), half of which is somebody else's turn.  16 chunks per weight row; sixteen
+        // consecutive lanes take one row, so that a warp's loads are two runs of 64 (128) consecutive bytes and its stores
+        // of a tile row hit all banks.
+        constexpr int CB = (int)sizeof(CodeT);
+        const int c16 = bt & 15, n0 = bt >> 4;
+        const uint32_t row_step = (uint32_t)(TL::NBUILD / 2 / 16) * (uint32_t)L.row_bytes;
+        const int n_pair = (n_kb + 1) / 2;
+        // Codes are fetched one turn ahead, across tile boundaries: all of a pair's chunks where they take at most ten registers
+        // (more would spill), else half of them, the rest when they are needed.
+        constexpr int NPRE = NCH * (CB / 4) <= 10 ? NCH : (NCH + 1) / 2;
+        CodeT pw[NPRE];
+        const uint8_t* src = nullptr;                        // codes of the fetched pair
+        int tile = tile0, pair = group;                      // the fetched pair
+        // (Packed weights are written by taq_pack_weights, which never lets its successor start early: they are complete
+        // before this kernel can run at all and are fetched and expanded under the previous kernel's tail.)
+        auto load = [&](int j) {
+            const int i = 2 * pair + (c16 >> 3);
+            const bool have = i < n_kb && (!I8 || (kb_begin + 2 * pair) * BKE + c16 * 16 < a.k_in);
+            return have ? __ldg(reinterpret_cast<const CodeT*>(src + (uint32_t)j * row_step)) : zero_codes<I8, W8>();
+        };
+        auto fetch = [&](bool new_tile) {
+            while (pair >= n_pair) { pair -= n_pair; tile += tile_step; new_tile = true; }
+            if (tile >= lay.n_tiles) return;
+            if (new_tile) {
+                int z, row0, col0, kv_which;
+                tile_of(tile, z, row0, col0, kv_which);
+                src = blob_of(z, kv_which) + L.off_codes + (size_t)(col0 + n0) * L.row_bytes + (size_t)(kb_begin + 2 * pair) * (8 * CB) + c16 * CB;
+            }
+#pragma unroll
+            for (int j = 0; j < NPRE; ++j) pw[j] = load(j);
+        };
+        fetch(true);
+        start();
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_BUILD));
+        int s = group;
+        uint32_t ph = 1;
+        bool passed = false, ok = true;                      // passed: the ring has been passed once
+        while (tile < lay.n_tiles) {
+            while (s >= nsb) { s -= nsb; ph ^= 1; passed = true; }
+            if (passed && !ptx::mbar_wait(&bars->empty_b[s], ph)) { ok = false; break; }
+            unsigned char* tile_b = b_ring + (2 * s + (c16 >> 3)) * TL::B_TILE;
+            if (c16 < 8 || 2 * pair + 1 < n_kb) {
+#pragma unroll
+                for (int j = 0; j < NPRE; ++j) *reinterpret_cast<uint4*>(tile_b + ptx::sw128_offset(n0 + j * (TL::NBUILD / 32), c16 & 7)) = expand_chunk<I8, W8>(pw[j]);
+                if constexpr (NPRE < NCH) {
+#pragma unroll
+                    for (int j = NPRE; j < NCH; ++j) pw[j - NPRE] = load(j);
+#pragma unroll
+                    for (int j = NPRE; j < NCH; ++j) *reinterpret_cast<uint4*>(tile_b + ptx::sw128_offset(n0 + j * (TL::NBUILD / 32), c16 & 7)) = expand_chunk<I8, W8>(pw[j - NPRE]);
+                }
+            }
+            if (bt == 0 && pair < 10) TAQ_PROF(60 + 2 * pair);
+            pair += 2; src += 32 * CB;
+            fetch(false);
+            ptx::fence_proxy_async_smem();                   // make the generic-proxy writes visible to the tensor core
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&bars->full_b[s]);
+            s += 2;
+        }
+        if (!ok) give_up();
+        __syncwarp();
+        if constexpr (KV) kv_together(false, TL::NFOLD + tid - 32 * TL::W_BUILD);
+        if (clustered) ptx::cluster_wait();
+    } else {
+        start();
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_REST));
+        if (warp == TL::W_PROD) {
+            // ---------------- producer: activation tiles ----------------
+            if (lane == 0) {
+                ptx::pdl_wait();                             // the activations may come from the previous kernel
+                TAQ_PROF(1); TAQ_GPROF(28);
+                int s = 0, issued = 0;
+                uint32_t ph = 1;
+                bool passed = false, ok = true;
+                for (int tile = tile0; tile < lay.n_tiles && ok; tile += tile_step) {
+                    int z, row0, col0, kv_which;
+                    tile_of(tile, z, row0, col0, kv_which);
+                    for (int i = 0; i < n_kb; i += 2) {
+                        if (passed && !ptx::mbar_wait(&bars->empty_a[s], ph)) { give_up(); ok = false; break; }
+                        unsigned char* dst = smem + 2 * s * A_TILE_BYTES;
+                        const bool two = i + 1 < n_kb;
+                        ptx::mbar_arrive_expect_tx(&bars->full_a[s], two ? 2 * A_TILE_BYTES : A_TILE_BYTES);
+                        ptx::tma_load_3d(dst, &tmap_x, &bars->full_a[s], (kb_begin + i) * BKE, row0, z);
+                        if (two) ptx::tma_load_3d(dst + A_TILE_BYTES, &tmap_x, &bars->full_a[s], (kb_begin + i + 1) * BKE, row0, z);
+                        ++issued;
+                        if (++s == nsa) { s = 0; ph ^= 1; passed = true; }
+                    }
+                }
+                if (bars->abort_flag)                        // give copies that are still in flight a bounded chance to land before the CTA exits
+                    for (int k = issued > nsa ? issued - nsa : 0; k < issued; ++k) (void)ptx::mbar_wait(&bars->full_a[k % nsa], (k / nsa) & 1);
+            }
+        } else if (warp == TL::W_MMA) {
+            // ---------------- MMA issuer ----------------
+            // (The allocation may have to wait for a predecessor on the same SM to give its TMEM back; only this warp waits.)
+            ptx::tmem_alloc(&bars->tmem_base, TL::TMEM_COLS);
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&bars->acc_free[buf]);
-            return true;
-        };
-
-        // expand the weight tiles of group g's k-blocks
-        int s = 0, kb = kb_begin;
-        uint32_t ph = 0;
-        auto build_group = [&](int g) -> bool {
-            const int kb_end = min(kb_stop, kb + kb_per_group);
-            for (; kb < kb_end; ++kb) {
-                if (!prebuilt && kb - kb_begin >= nstage && !ptx::mbar_wait(&bars->empty[s], ph ^ 1)) return false;
-                if (bars->abort_flag) return false;
-                if (a.w_direct == 2 && !ptx::mbar_wait(&bars->full_a[s], ph)) return false;    // this k-block's slice of the codes has arrived
-                unsigned char* b_tile = prebuilt ? smem + P.off_ball + (kb - kb_begin) * TL::B_TILE_BYTES : smem + s * P.stage_bytes + A_TILE_BYTES;
-                // 16-byte chunks of the fp16 tile: 8 per weight row; this thread owns chunk c of rows n0, n0 + 32, ...
-                constexpr int NCH = (BN * 8 + NWORK - 1) / NWORK;
-                const int n0 = wt >> 3, c = wt & 7;
-                if (I8) {
-                    // int8 tile: a chunk is 16 fan-in elements; chunks at or beyond k_in (ragged last block) are zero
-                    const int k0 = kb * BKE + c * 16;
-                    uint4 cw[NCH];
+            if (ptx::elect_one()) {
+                ptx::mbar_arrive(&bars->tmem_ready);
+                ptx::tc_fence_after_sync();
+                const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
+                constexpr uint32_t idesc = I8 ? ptx::idesc_i8_m128(BN) : ptx::idesc_f16_m128(BN);
+                constexpr uint32_t HI = ptx::kDescHiSw128;
+                const uint32_t a_lo0 = ptx::desc_lo(ptx::smem_u32(smem)), b_lo0 = ptx::desc_lo(ptx::smem_u32(smem + 2 * nsa * A_TILE_BYTES));
+                int sa = 0, sb = 0, slot = 0;
+                uint32_t pha = 0, phb = 0, ph_free = 1, a_lo = a_lo0, b_lo = b_lo0;
+                bool ok = true, recycled = false;            // recycled: every accumulator has been used once
+                bool next_a = false, next_b = false;         // the next pair was seen complete already
+                for (int tile = tile0; tile < lay.n_tiles && ok; tile += tile_step) {
+                    int left = 0;                            // k-blocks left in the current group
+                    uint32_t d_tmem = 0;
+                    for (int i = 0; i < n_kb; i += 2) {
+                        if (!next_b && !ptx::mbar_wait(&bars->full_b[sb], phb)) { ok = false; break; }
+                        if (!next_a && !ptx::mbar_wait(&bars->full_a[sa], pha)) { ok = false; break; }
+                        if (i < 20) TAQ_PROF(40 + i);
 #pragma unroll
-                    for (int i = 0; i < NCH; ++i) {
-                        const int n = n0 + (NWORK / 8) * i;
-                        cw[i] = make_uint4(0, 0, 0, 0);
-                        if (((BN * 8) % NWORK == 0 || n < BN) && k0 < a.k_in) {
-                            if (a.bits == 4) {
-                                const uint2 p = *reinterpret_cast<const uint2*>(raw + n * row_bytes + (k0 >> 1));
-                                const uint2 lo = codes_w4_to_i8(p.x), hi = codes_w4_to_i8(p.y);
-                                cw[i] = make_uint4(lo.x, lo.y, hi.x, hi.y);
-                            } else {
-                                cw[i] = *reinterpret_cast<const uint4*>(raw + n * row_bytes + k0);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < NCH; ++i) {
-                        const int n = n0 + (NWORK / 8) * i;
-                        if ((BN * 8) % NWORK == 0 || n < BN) *reinterpret_cast<uint4*>(b_tile + ptx::sw128_offset(n, c)) = cw[i];
-                    }
-                } else {
-                uint2 pw[NCH];
-#pragma unroll
-                for (int i = 0; i < NCH; ++i) {
-                    const int n = n0 + (NWORK / 8) * i;
-                    pw[i] = make_uint2(0, 0);
-                    if ((BN * 8) % NWORK == 0 || n < BN) {
-                        if (a.bits == 4) pw[i].x = *reinterpret_cast<const uint32_t*>(raw + n * row_bytes + kb * (BK / 2) + c * 4);
-                        else if (a.w_direct == 2) pw[i] = *reinterpret_cast<const uint2*>(raw + s * (BN * BK) + n * BK + c * 8);
-                        else pw[i] = *reinterpret_cast<const uint2*>(raw + n * row_bytes + kb * BK + c * 8);
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < NCH; ++i) {
-                    const int n = n0 + (NWORK / 8) * i;
-                    if ((BN * 8) % NWORK == 0 || n < BN)
-                        *reinterpret_cast<uint4*>(b_tile + ptx::sw128_offset(n, c)) = a.bits == 4 ? codes_w4_to_half(pw[i].x) : codes_w8_to_half(pw[i]);
-                }
-                }
-                ptx::fence_proxy_async_smem();            // make the generic-proxy writes visible to the tensor core
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bars->full_b[prebuilt ? kb - kb_begin : s]);
-                if (wt == 0 && kb < 20) TAQ_PROF(60 + kb);
-                if (++s == nstage) { s = 0; ph ^= 1; }
-            }
-            return true;
-        };
-
-        // prebuilt (fp16 activations, codes staged): two tiles per pass, all loads before the conversions and the stores, one
-        // proxy fence for both
-        auto build_pair = [&](int kb0, int ntile) {
-            constexpr int NCH = (BN * 8 + NWORK - 1) / NWORK;
-            const int n0 = wt >> 3, c = wt & 7;
-            uint2 pw[2][NCH];
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int i = 0; i < NCH; ++i) {
-                    const int n = n0 + (NWORK / 8) * i;
-                    pw[t][i] = make_uint2(0, 0);
-                    if (t < ntile && ((BN * 8) % NWORK == 0 || n < BN)) {
-                        if (a.bits == 4) pw[t][i].x = *reinterpret_cast<const uint32_t*>(raw + n * row_bytes + (kb0 + t) * (BK / 2) + c * 4);
-                        else pw[t][i] = *reinterpret_cast<const uint2*>(raw + n * row_bytes + (kb0 + t) * BK + c * 8);
-                    }
-                }
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                unsigned char* b_tile = smem + P.off_ball + (kb0 + t - kb_begin) * TL::B_TILE_BYTES;
-#pragma unroll
-                for (int i = 0; i < NCH; ++i) {
-                    const int n = n0 + (NWORK / 8) * i;
-                    if (t < ntile && ((BN * 8) % NWORK == 0 || n < BN))
-                        *reinterpret_cast<uint4*>(b_tile + ptx::sw128_offset(n, c)) = a.bits == 4 ? codes_w4_to_half(pw[t][i].x) : codes_w8_to_half(pw[t][i]);
-                }
-            }
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane < ntile) ptx::mbar_arrive(&bars->full_b[kb0 + lane - kb_begin]);
-            if (wt == 0 && kb0 < 20) TAQ_PROF(60 + kb0);
-        };
-
-        if (prebuilt) {            // every weight tile first (nothing to wait for), then the folds as the groups complete
-            if (!I8)
-                for (int k2 = kb_begin; k2 < kb_stop && !bars->abort_flag; k2 += 2) build_pair(k2, min(2, kb_stop - k2));
-            ok = !bars->abort_flag;
-            for (int g = g_begin; g < g_end && ok; ++g) ok = fold_group(g);
-        } else {
-            for (int g = g_begin; g < g_end && ok; ++g) {
-                ok = a.w_direct == 1 ? true : build_group(g);
-                if (ok && g > g_begin) ok = fold_group(g - 1);
-            }
-            if (ok) ok = fold_group(g_end - 1);
-        }
-        if (!ok) { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; }
-        asm volatile("bar.sync 1, 256;" ::: "memory");       // every worker gets here; the decision below is uniform
-        ok = !bars->abort_flag;
-        ptx::pdl_wait();                                     // (already satisfied: the activations have arrived) orders the stores below
-        if (wt == 0) TAQ_PROF(7);
-        if (SPLIT) {
-            // All of this CTA's MMAs are complete (every group was folded), so its ring is free: it holds the partial sums
-            // in transit, each thread's piece at the same place in both CTAs.  The first CTA finishes rows 0..63 of the
-            // tile, the second rows 64..127: a worker warp either hands its 32 rows over (one bulk copy between the shared
-            // memories, one barrier per warp) or receives the partner's piece and adds it, so both directions of the
-            // exchange run at once and each CTA stores half of the tile.
-            const int ww = wt >> 5, wl = wt & 31;
-            const uint32_t peer = ptx::cluster_ctarank() ^ 1u;   // (clusters are two CTAs along x, times two along y for a head pair)
-            const bool keep = ((ww & 3) >> 1) == rank;
-            unsigned char* warp_part = smem + (size_t)ww * 32 * PART_ROW;
-            float* piece = reinterpret_cast<float*>(warp_part + (size_t)wl * PART_ROW);
-            if (wt == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), peer));
-            if (!keep) {
-#pragma unroll
-                for (int c = 0; c < HC; c += 4) *reinterpret_cast<float4*>(piece + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (wl == 0) {
-                    if (ww == 2) TAQ_PROF(11);
-                    bool go = ptx::mbar_wait(&bars->peer_ready, 0) && !bars->abort_flag;         // the partner's ring is free, too
-                    if (ww == 2) TAQ_PROF(12);
-                    if (go) {
-                        ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(warp_part), peer), warp_part, 32u * PART_ROW,
-                                              ptx::map_to_cta(ptx::smem_u32(&bars->part_full[ww]), peer));
-                        go = ptx::mbar_wait(&bars->part_got[ww], 0);     // this CTA's shared memory is the source: stay until it was read
-                    }
-                    if (!go) { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; }
-                }
-                row = a.rows;                                // these rows are stored by the partner
-            } else {
-                if (!ptx::mbar_wait(&bars->part_full[ww], 0)) {
-                    raise_status(a.status, TAQ_ERR_TIMEOUT);
-                    bars->abort_flag = 1;
-                } else {
-#pragma unroll
-                    for (int c = 0; c < HC; c += 4) {
-                        const float4 p4 = *reinterpret_cast<const float4*>(piece + c);
-                        y[c] += p4.x; y[c + 1] += p4.y; y[c + 2] += p4.z; y[c + 3] += p4.w;
-                    }
-                }
-                __syncwarp();
-                if (wl == 0) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->part_got[ww]), peer));
-            }
-            asm volatile("bar.sync 1, 256;" ::: "memory");   // pieces read, outgoing copies done: the epilogue stages output there
-            ok = !bars->abort_flag;
-            if (wt == 0) TAQ_PROF(10);
-        }
-        if (I8 && ok) {                                      // x~ = code * s_x: the row's activation scale
-            const float sx = row < a.rows ? a.x_scales[(size_t)z * a.rows + row] : 0.f;
-#pragma unroll
-            for (int c = 0; c < HC; ++c) y[c] *= sx;
-        }
-
-        // ---------------- epilogue on this thread's HC columns ----------------
-        // Dense outputs (fp16, fp32, int8 codes) are staged in shared memory as the plain [128][BN] tile (the ring is free
-        // now) and leave by one TMA store per 32 rows, issued as soon as the two warps that own those rows have written
-        // them; the tensor map clips rows beyond the matrix.
-        const bool stores_rows = !SPLIT || (((warp - 2) & 3) >> 1) == rank;
-        auto store_quarter = [&](int esz) {
-            ptx::fence_proxy_async_smem();
-            asm volatile("bar.sync %0, 64;" ::"r"(3 + q) : "memory");
-            if (half == 0 && lane == 0 && stores_rows && (long long)row0 + q * 32 < a.rows) {
-                ptx::tma_store_3d(&tmap_y, smem + (size_t)q * 32 * BN * esz, col0, row0 + q * 32, z);
-                ptx::bulk_store_commit();
-                ptx::bulk_store_wait_read();
-            }
-        };
-        if (ok) {
-            if (a.epi == EPI_F16 || a.epi == EPI_F32) {
-                const int esz = a.epi == EPI_F16 ? 2 : 4;
-                unsigned char* seg = smem + ((size_t)r * BN + cb) * esz;
-#pragma unroll
-                for (int c = 0; c < HC; c += 8) {
-                    float f[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) f[e] = y[c + e] + bias[cb + c + e];
-                    if (a.epi == EPI_F16) {
-                        *reinterpret_cast<uint4*>(seg + c * 2) = pack8(f);
-                    } else {
-                        *reinterpret_cast<float4*>(seg + c * 4) = make_float4(f[0], f[1], f[2], f[3]);
-                        *reinterpret_cast<float4*>(seg + c * 4 + 16) = make_float4(f[4], f[5], f[6], f[7]);
-                    }
-                }
-                store_quarter(esz);
-            } else {
-                // Per-(row, head) symmetric int8.  A thread's columns are either whole heads (HC a multiple of d) or half
-                // of the tile's single head (d = BN); in the second case the row's two threads exchange their absmax.
-                const int d = a.n_out / a.heads;
-                const bool whole_heads = HC % d == 0;
-                const int dd = whole_heads ? d : HC;                  // columns of one head held by this thread
-                int slot = -1;
-                bool trig = false;
-                int t = 0;
-                uint8_t* blk = nullptr;
-                taq_kv_layout KL;
-                if (a.epi == EPI_KV && row < a.rows) {
-                    const int b = a.reqs ? 0 : (int)(row / a.n_ctx);
-                    t = (int)(row % a.n_ctx);
-                    const uint8_t* mask = a.reqs ? a.reqs[z].trig_mask : a.mask + (size_t)b * a.n_ctx;
-                    KL = kv_layout(a.heads, a.n_ctx, d, a.max_trigger);
-                    blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)b * KL.block_bytes;
-                    trig = mask[t] != 0;
-                    if (trig) {
-                        slot = 0;
-                        for (int u = 0; u < t; ++u) slot += mask[u] != 0;
-                        if (slot >= a.max_trigger) { raise_status(a.status, TAQ_ERR_SHAPE); slot = -2; }
-                    }
-                }
-#pragma unroll
-                for (int hc = 0; hc < HC; hc += 40) {                 // heads are 40, 64, 80 or 160 wide: steps of 40 or the whole of HC
-                    if (hc % dd != 0) continue;
-                    const int h = (col0 + cb + hc) / d;
-                    const int ch = (col0 + cb + hc) - h * d;          // first column of this piece inside the head
-                    float amax = 0.f;
-#pragma unroll
-                    for (int c = 0; c < HC; ++c)
-                        if (c >= hc && c < hc + dd) amax = fmaxf(amax, fabsf(y[c]));
-                    if (!whole_heads) {
-                        xchg[half * 128 + r] = amax;
-                        asm volatile("bar.sync 2, 256;" ::: "memory");
-                        amax = fmaxf(amax, xchg[(half ^ 1) * 128 + r]);
-                        if (SPLIT && a.head_pair && stores_rows) {
-                            // The head's other 80 channels belong to the CTA next to this one along y (same rows, same
-                            // half of the K loop): each sends its rows' absmax over (one 128-byte copy between the shared
-                            // memories per 32 rows), waits for the other's, and confirms, so that the source outlives the copy.
-                            float* out = xchg + 256, * in = xchg + 384;
-                            const uint32_t other = ptx::cluster_ctarank() ^ 2u;
-                            bool got = true;
-                            if (half == 0) {
-                                out[r] = amax;
-                                ptx::fence_proxy_async_smem();
-                                __syncwarp();
-                                if (lane == 0)
-                                    ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(in + q * 32), other), out + q * 32, 128u,
-                                                          ptx::map_to_cta(ptx::smem_u32(&bars->pair_full[q]), other));
-                            }
-                            got = ptx::mbar_wait(&bars->pair_full[q], 0);
-                            if (got) amax = fmaxf(amax, in[r]);
-                            asm volatile("bar.sync %0, 64;" ::"r"(7 + q) : "memory");      // both warps of the quarter have read the piece
-                            if (half == 0 && lane == 0) {
-                                ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->pair_got[q]), other));
-                                got = ptx::mbar_wait(&bars->pair_got[q], 0) && got;
-                            }
-                            if (!got) { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; }
-                        }
-                    }
-                    const float s = quant_scale(amax, a.epi == EPI_KV && a.kv_qmax ? (float)a.kv_qmax : 127.f);
-                    const float rs = s > 0.f ? __frcp_rn(s) : 0.f;
-                    const bool owner = whole_heads || half == 0;      // writes the head's scale
-                    if (a.epi == EPI_Q8_HEAD) {
-                        // Q~ = Q_a(Q), Eq. 2 third line
-                        unsigned char* seg = smem + (size_t)r * BN + cb;
-#pragma unroll
-                        for (int c = 0; c < HC; c += 8)
-                            if (c >= hc && c < hc + dd) *reinterpret_cast<uint2*>(seg + c) = quant8(y + c, rs);
-                        if (hc + dd >= HC) store_quarter(1);  // last head of the piece
-                        if (row < a.rows && owner) a.scales[((size_t)z * a.rows + row) * a.heads + h] = s;
-                    } else if (row < a.rows) {
-                        // Eq. 2 for K or V: rows of ordinary tokens -> int8 codes + scale, rows of trigger tokens -> fp16
-                        int8_t* cq = (int8_t*)(blk + (a.kv_which ? KL.off_v_codes : KL.off_k_codes)) + ((size_t)h * a.n_ctx + t) * d + ch;
-#pragma unroll
-                        for (int c = 0; c < HC; c += 8)
-                            if (c >= hc && c < hc + dd) *reinterpret_cast<uint2*>(cq + c - hc) = trig ? make_uint2(0, 0) : quant8(y + c, rs);
-                        if (slot >= 0) {
-                            __half* tr = (__half*)(blk + (a.kv_which ? KL.off_v_trigger : KL.off_k_trigger)) + ((size_t)slot * a.heads + h) * d + ch;
-#pragma unroll
-                            for (int c = 0; c < HC; c += 8)
-                                if (c >= hc && c < hc + dd) {
-                                    float f[8];
-#pragma unroll
-                                    for (int e = 0; e < 8; ++e) f[e] = y[c + e];
-                                    *reinterpret_cast<uint4*>(tr + c - hc) = pack8(f);
+                        for (int h = 0; h < 2; ++h) {
+                            if (h == 1 && i + 1 >= n_kb) break;
+                            uint32_t acc = 1;
+                            if (left == 0) {                 // a new group: the next accumulator, emptied by the folders if it was in use
+                                left = min(kb_per_group, n_kb - i - h);
+                                if (recycled) {
+                                    if (!ptx::mbar_wait(&bars->acc_free[slot], ph_free)) { ok = false; break; }
+                                    ptx::tc_fence_after_sync();
                                 }
+                                d_tmem = tmem_base + slot * BN;
+                                acc = 0;
+                            }
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {    // four 32-byte K slices per 128-byte operand row
+                                const uint64_t da = ptx::desc_join(HI, a_lo + h * (A_TILE_BYTES >> 4) + 2 * k), db = ptx::desc_join(HI, b_lo + h * (TL::B_TILE >> 4) + 2 * k);
+                                if (I8) ptx::mma_i8_ss(d_tmem, da, db, idesc, acc | k);
+                                else ptx::mma_f16_ss(d_tmem, da, db, idesc, acc | k);
+                            }
+                            if (--left == 0) {
+                                ptx::mma_commit(&bars->acc_full[slot]);
+                                if (++slot == NSLOT) { slot = 0; recycled = true; ph_free ^= 1; }
+                            }
                         }
-                        if (owner) {
-                            ((float*)(blk + (a.kv_which ? KL.off_v_scales : KL.off_k_scales)))[(size_t)h * a.n_ctx + t] = trig ? 0.f : s;
-                            if (h == 0 && a.kv_which == 0) ((int32_t*)(blk + KL.off_trig_slot))[t] = slot >= 0 ? slot : -1;
-                        }
+                        if (!ok) break;
+                        ptx::mma_commit(&bars->empty_a[sa]); // these free the stages once the MMAs have read them
+                        ptx::mma_commit(&bars->empty_b[sb]);
+                        a_lo += 2 * A_TILE_BYTES >> 4;
+                        b_lo += 2 * TL::B_TILE >> 4;
+                        if (++sa == nsa) { sa = 0; pha ^= 1; a_lo = a_lo0; }
+                        if (++sb == nsb) { sb = 0; phb ^= 1; b_lo = b_lo0; }
+                        next_b = ptx::mbar_try_wait(&bars->full_b[sb], phb);
+                        next_a = ptx::mbar_try_wait(&bars->full_a[sa], pha);
                     }
                 }
-                if (a.epi == EPI_KV && a.kv_which == 0 && blockIdx.x == 0 && blockIdx.y == 0) {   // slot table beyond T
-                    const int nb = a.reqs ? 1 : (int)(a.rows / a.n_ctx);
-                    const taq_kv_layout K2 = kv_layout(a.heads, a.n_ctx, d, a.max_trigger);
-                    for (int i = wt; i < nb * (kMaxCtx - a.n_ctx); i += NWORK) {
-                        const int bb = i / (kMaxCtx - a.n_ctx), tt = a.n_ctx + i % (kMaxCtx - a.n_ctx);
-                        uint8_t* bk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)bb * K2.block_bytes;
-                        ((int32_t*)(bk + K2.off_trig_slot))[tt] = -1;
-                    }
-                }
+                if (!ok) give_up();
             }
         }
+        else if (warp < TL::W_AUX + 2) {
+            // ---------------- scales and biases, one tile ahead ----------------
+            int sbuf = 0, it = 0;
+            uint32_t ph = 1;
+            for (int tile = tile0; tile < lay.n_tiles; tile += tile_step, ++it) {
+                int z, row0, col0, kv_which;
+                tile_of(tile, z, row0, col0, kv_which);
+                const uint8_t* blob = blob_of(z, kv_which);
+                const float* gs = reinterpret_cast<const float*>(blob + L.off_scales) + (size_t)col0 * n_groups;
+                const float* gb = reinterpret_cast<const float*>(blob + L.off_bias) + col0;
+                if (it >= 2 && !ptx::mbar_wait(&bars->scale_free[sbuf], ph)) { give_up(); break; }
+                float* sc = reinterpret_cast<float*>(smem + P.off_scales + sbuf * P.scale_bytes);
+                // [BN][n_groups] -> [n_groups][BN], so that a group's scales of consecutive columns are contiguous
+                for (int n = (warp - TL::W_AUX) * 32 + lane; n < BN; n += 64) {
+#pragma unroll 4
+                    for (int g = g_begin; g < g_end; ++g) sc[g * BN + n] = __ldg(gs + (size_t)n * n_groups + g);
+                    sc[n_groups * BN + n] = with_bias ? __ldg(gb + n) : 0.f;
+                }
+                if (KV && warp == TL::W_AUX) {               // slot of every token of the sequence among its trigger tokens, and their bitmap
+                    const uint8_t* mask = a.reqs ? a.reqs[z].trig_mask : a.mask + (size_t)z * a.n_ctx;
+                    int* slots = reinterpret_cast<int*>(smem + P.off_xchg) + 256;
+                    int before = 0;
+                    for (int k = 0; k < 4; ++k) {
+                        const int t = 32 * k + lane;
+                        const bool trig = t < a.n_ctx && mask[t] != 0;
+                        const uint32_t w = __ballot_sync(0xffffffffu, trig);
+                        int slot = trig ? before + __popc(w & ((1u << lane) - 1u)) : -1;
+                        if (slot >= a.max_trigger) { raise_status(a.status, TAQ_ERR_SHAPE); slot = -2; }
+                        before += __popc(w);
+                        slots[t] = slot;
+                        const uint32_t kept = __ballot_sync(0xffffffffu, slot >= 0);
+                        if (lane == 0) slots[128 + k] = (int)kept;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&bars->scale_full[sbuf]);
+                sbuf ^= 1;
+                if (sbuf == 0) ph ^= 1;
+            }
+        }
+        __syncwarp();
+        if (clustered) ptx::cluster_wait();
     }
 
     // ---------------- teardown ----------------
-    if (tid == 64) TAQ_PROF(8);
     ptx::tc_fence_before_sync();
+    // (No CTA of a cluster may leave while a copy out of its shared memory is in flight: by this barrier every copy has
+    // been received.  Every thread arrives, whatever happened to its waits.)
+    if (clustered) { ptx::cluster_arrive(); ptx::cluster_wait(); }
     __syncthreads();
     if (tid == 0) { TAQ_PROF(9); TAQ_GPROF(29); }
-    if (warp == 1) {
+    if (warp == TL::W_MMA) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, tmem_cols);
+        ptx::tmem_dealloc(*reinterpret_cast<volatile uint32_t*>(&bars->tmem_base), TL::TMEM_COLS);
     }
 }
 
@@ -638,225 +829,194 @@ EncodeTiledFn encode_tiled_fn() {
     return fn;
 }
 
-// How the kernel gets at the weight codes: 0 = all codes of the tile's channels staged in shared memory once; 1 = int8
-// activations and 8-bit weights: the codes are the B operand, by TMA per k-block; 2 = fp16 activations and 8-bit weights whose
-// staged codes would not fit beside a two-stage ring (a 160-wide tile at a fan-in of 1280): a 64-byte slice per channel
-// arrives by TMA with every k-block's activations and the workers expand from it.
-template <int BN>
-int weight_mode(const LinearArgs& a) {
-    if (a.bits != 8) return 0;
-    if (a.xq) return a.reqs ? 0 : 1;      // (per-request blobs have no common tensor map: their codes are staged)
-    return make_plan<BN>(a.k_in, a.bits, a.group, 2, 0).total > SMEM_LIMIT ? (a.reqs ? 0 : 2) : 0;
+// How a launch is laid out.
+struct Choice { int bn, grid; LinearLayout lay; int total, ring, staged; };      // grid in CTAs; staged: bytes the epilogue stages in the rings
+
+struct Problem {                       // what the choice depends on
+    int n_groups, group_len, bke, n_kb, d, ncols_factor;
+    bool i8;
+    long long row_tiles;
+};
+Problem problem_of(const LinearArgs& a) {
+    const WeightLayout L = weight_layout(a.n_out, a.k_in, a.bits, a.group);
+    Problem p;
+    p.i8 = a.xq != nullptr;
+    p.bke = p.i8 ? 2 * BK : BK;
+    p.n_groups = L.n_groups; p.group_len = L.group_len;
+    p.n_kb = (a.k_in + p.bke - 1) / p.bke;
+    p.d = a.epi == EPI_Q8_HEAD || a.epi == EPI_KV ? a.n_out / a.heads : 0;
+    p.ncols_factor = a.epi == EPI_KV ? 2 : 1;
+    p.row_tiles = (a.rows + BM - 1) / BM;
+    return p;
+}
+// k-blocks of the longest share when the K loop is split
+int share_of(const Problem& p, int nsplit) {
+    if (nsplit == 1) return p.n_kb;
+    if (p.n_groups == 1) return (p.n_kb + nsplit - 1) / nsplit;
+    const int kbs = ((p.n_groups + nsplit - 1) / nsplit) * (p.group_len / p.bke);
+    return kbs < p.n_kb ? kbs : p.n_kb;
 }
 
-// Bytes of the ring that the epilogue reuses to stage a tile's output before the TMA stores: the dense [128][BN] tile.
+// Ring depths of a tile width, or false when it does not fit: as many of a tile's weight blocks as shared memory holds (they are
+// expanded before the activations arrive), activations two pairs of blocks deep, or three.
 template <int BN>
-int epilogue_staging_bytes(const LinearArgs& a) {
-    if (a.epi == EPI_F16) return BM * BN * 2;
-    if (a.epi == EPI_F32) return BM * BN * 4;
-    if (a.epi == EPI_Q8_HEAD) return BM * BN;
-    return 0;
-}
-
-// Ring depth: as deep as the K loop needs, but no deeper than three stages when that keeps two CTAs on an SM, and never
-// shallower than the epilogue's staging area (which lives in the ring).  0: this tile width does not fit.
-template <int BN>
-int pick_nstage(const LinearArgs& a) {
-    const int bke = a.xq ? 2 * BK : BK;
-    const int direct = weight_mode<BN>(a);
-    const int n_kb = (a.k_in + bke - 1) / bke;
-    const int half_sm = Tile<BN>::CTAS_PER_SM == 2 ? SMEM_LIMIT / 2 : SMEM_LIMIT;
-    const int ns_min = (epilogue_staging_bytes<BN>(a) + Tile<BN>::STAGE_BYTES - 1) / Tile<BN>::STAGE_BYTES;
-    const int ns_max = n_kb < 2 ? 2 : n_kb;
-    int best = 0;
-    for (int ns = 1; ns <= MAX_STAGE && ns <= (ns_max > ns_min ? ns_max : ns_min); ++ns) {
-        const int total = make_plan<BN>(a.k_in, a.bits, a.group, ns, direct).total;
-        if (total > SMEM_LIMIT) break;
-        if (ns > 3 && ns > ns_min && total + 1024 > half_sm && make_plan<BN>(a.k_in, a.bits, a.group, 3, direct).total + 1024 <= half_sm) break;
-        best = ns;
+bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, bool persistent, Choice& c) {
+    using TL = Tile<BN>;
+    const int n_pair = (share_of(p, nsplit) + 1) / 2;
+    int staging = 0, staged = 0;
+    const int tile_bytes = a.epi == EPI_F16 ? BM * BN * 2 : a.epi == EPI_F32 ? BM * BN * 4 : a.epi == EPI_Q8_HEAD ? BM * BN : 128 * (BN + 1) * 4 + BN / p.d * 1024;      // (K~/V~: the fp32 tile and the rows' scales)
+    if (persistent) {
+        staging = TL::NF * (TL::HC % 40 == 0 ? 2560 : a.epi == EPI_F32 ? 4096 : 2048);
+    } else if (nsplit == 1) {
+        staged = tile_bytes;
+    } else {
+        const int send = (TL::NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024;         // (as many pieces come in as go out)
+        staged = 2 * send > send + tile_bytes ? 2 * send : send + tile_bytes;
     }
-    return best >= ns_min ? best : 0;
+    int nsa = n_pair < 2 ? 1 : 2, nsb = n_pair < 2 ? 1 : 2;
+    while (make_plan<BN>(p.n_groups, nsa, nsb, staging).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
+    auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, staging).total <= SMEM_LIMIT; };
+    while (nsb < (persistent ? MAX_STAGE : n_pair) && nsb < MAX_STAGE && fits(nsa, nsb + 1)) ++nsb;
+    while (nsa < 3 && nsa < n_pair && fits(nsa + 1, nsb)) ++nsa;
+    const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, staging);
+    if (P.total > SMEM_LIMIT || P.ring_bytes < staged) return false;
+    c.bn = BN;
+    c.lay.nsplit = nsplit; c.lay.nsa = nsa; c.lay.nsb = nsb; c.lay.staging = staging; c.lay.head_pair = head_pair;
+    c.total = P.total; c.ring = P.ring_bytes; c.staged = staged;
+    return true;
 }
-
-int nstage_for(const LinearArgs& a, int bn) {
+bool rings_of(const LinearArgs& a, const Problem& p, int bn, int nsplit, int head_pair, bool persistent, Choice& c) {
     switch (bn) {
-        case 64: return pick_nstage<64>(a);
-        case 80: return pick_nstage<80>(a);
-        case 160: return pick_nstage<160>(a);
+        case 64: return rings<64>(a, p, nsplit, head_pair, persistent, c);
+        case 80: return rings<80>(a, p, nsplit, head_pair, persistent, c);
+        case 128: return rings<128>(a, p, nsplit, head_pair, persistent, c);
+        case 160: return rings<160>(a, p, nsplit, head_pair, persistent, c);
     }
-    return 0;
+    return false;
 }
 
-// EPI_Q8_HEAD with heads of 160 channels: instead of one 160-wide tile per head (whose expanded weight tiles do not fit
-// resident) two 80-wide tiles whose CTAs exchange the rows' absmax, when that launch is one wave of split tiles with
-// resident weight tiles (clusters of 2 x 2: halves of the K loop along x, halves of the head along y).
-bool head_pair_mode(const LinearArgs& a, int n_z);
-
-int pick_bn(const LinearArgs& a, int n_z = 1) {
-    // Every column tile re-reads the activation rows, so tiles are as wide as the row count allows while the grid
-    // still covers most of the SMs; a width whose ring and staging do not fit shared memory is passed over.
-    const long long row_tiles = (a.rows + BM - 1) / BM;
-    auto fits = [&](int bn) { return nstage_for(a, bn) >= 2; };
-    if (a.epi == EPI_Q8_HEAD || a.epi == EPI_KV) {
-        const int d = a.n_out / a.heads;
-        if (d == 40 && a.heads % 4 == 0 && row_tiles * (a.n_out / 160) >= 96 && fits(160)) return 160;   // two heads per worker thread
-        if (d == 40 && a.heads % 2 == 0) return fits(80) ? 80 : 0;     // one head per worker thread
-        if (d == 160 && a.epi == EPI_Q8_HEAD && head_pair_mode(a, n_z)) return 80;
-        if (d == 64 || d == 80 || d == 160) return fits(d) ? d : 0;   // one head per tile, split between the row's two threads
-        return 0;
+// Whether a tile of bn columns can carry the epilogue: per-head outputs want a thread's 80 or 64 columns to be whole heads, or a
+// head of 160 channels on the two threads of a row.
+bool tile_carries(const LinearArgs& a, const Problem& p, int bn) {
+    if (a.n_out % bn) return false;
+    switch (p.d) {
+        case 0: return true;
+        case 40: return bn == 160 || bn == 80;
+        case 80: return bn == 160 || bn == 80;
+        case 160: return bn == 160;                      // (80: head pairs, below)
+        case 64: return bn == 128 || bn == 64;
     }
-    if (a.n_out % 160 == 0 && row_tiles * (a.n_out / 160) >= 96 && fits(160)) return 160;
-    if (a.n_out % 80 == 0 && fits(80)) return 80;
-    if (a.n_out % 64 == 0 && fits(64)) return 64;
-    return 0;
+    return false;
 }
 
-// How a launch is laid out: ring depth, whether two CTAs share a tile (split of the K loop), and whether every CTA keeps
-// all of its expanded weight tiles resident (`prebuilt` = its number of k-blocks, else 0).
-struct Choice { int ns, prebuilt; bool split; };
-
-template <int BN>
+// The cheapest layout by a small model of a CTA's life in SM cycles: a fixed part (launch, barriers, first loads, epilogue), the K
+// loop at the pace of the tensor core, and the exchange of partial sums when the loop is split; a persistent CTA pays
+// the fixed part once and the K loop per tile.
 Choice choose(const LinearArgs& a, int n_z) {
-    const bool i8 = a.xq != nullptr;
-    const int mode = weight_mode<BN>(a);
-    Choice c{pick_nstage<BN>(a), 0, false};
-    const WeightLayout Lw = weight_layout(a.n_out, a.k_in, a.bits, a.group);
-    const int bke = i8 ? 2 * BK : BK;
-    const int n_kb = (a.k_in + bke - 1) / bke;
-    const long long tiles = ((a.rows + BM - 1) / BM) * (a.n_out / BN) * (long long)n_z;
-    const int staging = epilogue_staging_bytes<BN>(a);
-    const int part = NWORK * (BN * 2 + 16);          // fp32 partial sums in transit between the two CTAs of a split tile
-    // few tiles and a long K loop: two CTAs per tile, each with half of the scale groups (or of the k-blocks of a single
-    // group: not for integer activations, where a group's sum stays one exact int32 accumulation)
-    const bool want_split = (Lw.n_groups >= 2 || !i8) && tiles <= 74 * Tile<BN>::CTAS_PER_SM && n_kb >= 6;
-    c.split = want_split && (long long)c.ns * Tile<BN>::STAGE_BYTES >= part;
-    // One wave at one CTA per SM, codes staged once, fp16 activations: expand every weight tile of the CTA before the
-    // activations arrive (under the previous kernel's tail when the weights are known early), so that the K loop waits
-    // for the TMA loads only.
-    if (mode == 0 && !i8 && tiles <= 148) {
-        for (int with_split = (want_split && 2 * tiles <= 148) ? 1 : 0; with_split >= 0; --with_split) {
-            int n_cta = n_kb;
-            if (with_split) {
-                if (Lw.n_groups == 1) n_cta = n_kb - n_kb / 2;
-                else { const int kbg = Lw.group_len / bke, lo = (Lw.n_groups / 2) * kbg; n_cta = lo > n_kb - lo ? lo : n_kb - lo; }
-            }
-            // the activation ring as deep as shared memory allows: with the weight tiles resident the K loop's pace is
-            // the latency of the activation loads divided by the loads in flight
-            bool found = false;
-            for (int ns = n_cta < MAX_STAGE ? (n_cta < 2 ? 2 : n_cta) : MAX_STAGE; ns >= (n_cta < 3 ? 2 : 3) && !found; --ns) {
-                const Plan P = make_plan<BN>(a.k_in, a.bits, a.group, ns, 0, n_cta);
-                if (n_cta <= MAX_PREBUILT && P.total <= SMEM_LIMIT && P.off_raw >= staging && (!with_split || P.off_raw >= part)) {
-                    c.ns = ns; c.prebuilt = n_cta; c.split = with_split != 0;
-                    found = true;
-                }
-            }
-            if (found) break;
+    const Problem p = problem_of(a);
+    Choice best{};
+    auto finish = [&](Choice& c, long long tiles, long long ctas) {
+        c.lay.row_tiles = (int)p.row_tiles; c.lay.n_tiles = (int)tiles;
+        c.grid = (int)ctas;
+        return c;
+    };
+    // Heads of 160 channels in a launch of few rows: two 80-wide tiles per head whose CTAs exchange the rows' absmax.
+    if (a.epi == EPI_Q8_HEAD && p.d == 160 && !p.i8 && !a.reqs && a.bits == 4 && p.n_groups >= 2) {
+        const long long tiles = p.row_tiles * (a.n_out / 80) * (long long)n_z;
+        Choice c{};
+        if (tiles * 2 <= 148 && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);
+    }
+    double best_cost = 1e30;
+    for (int bn : {160, 128, 80, 64}) {
+        if (!tile_carries(a, p, bn)) continue;
+        const long long tiles = p.row_tiles * (a.n_out / bn) * p.ncols_factor * (long long)n_z;
+        if (tiles > (1 << 30)) continue;
+        const double kb = bn == 160 ? 380 : bn == 128 ? 340 : 260;
+        for (int ns : {1, 2, 4}) {
+            if (ns > 1 && ((p.i8 && p.n_groups == 1) || (p.n_groups == 1 ? p.n_kb : p.n_groups) < ns || tiles * ns > 148)) continue;    // (integer activations: a group's sum stays one exact int32 accumulation)
+            const bool persistent = a.epi != EPI_KV && tiles * ns > 148;           // (K~/V~ tiles are assembled in the rings: one per CTA)
+            Choice c{};
+            if (!rings_of(a, p, bn, ns, 0, persistent, c)) continue;
+            const long long per = (tiles * ns + 147) / 148;                                            // tiles per CTA
+            const long long ctas = persistent ? (tiles + per - 1) / per : tiles * ns;
+            const double cost = (persistent ? 1 : per) * (5000 + bn * (a.epi == EPI_KV ? 20 : 5)) + (double)per * (share_of(p, ns) * kb + (persistent ? 300 : 0)) + (ns > 1 ? 1000 + 300 * ns : 0);
+            if (cost < best_cost) { best_cost = cost; best = finish(c, tiles, ctas); }
         }
     }
-    return c;
-}
-
-bool head_pair_mode(const LinearArgs& a, int n_z) {
-    if (a.epi != EPI_Q8_HEAD || a.heads <= 0 || a.n_out != a.heads * 160 || a.xq || a.reqs) return false;
-    if (nstage_for(a, 80) < 2) return false;
-    const Choice c = choose<80>(a, n_z);
-    return c.split && c.prebuilt > 0;
+    return best;
 }
 
 template <int BN>
-cudaError_t launch_bn(const CUtensorMap& tmap, EncodeTiledFn enc, LinearArgs a, int n_z, cudaStream_t stream) {
-    const bool i8 = a.xq != nullptr;
-    const Choice ch = choose<BN>(a, n_z);
-    const int ns = ch.ns;
-    const bool split = ch.split;
-    void (*kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const LinearArgs, const int, const int) =
-        split ? (i8 ? linear_sm100_kernel<BN, true, true> : linear_sm100_kernel<BN, false, true>)
-              : (i8 ? linear_sm100_kernel<BN, true, false> : linear_sm100_kernel<BN, false, false>);
-    a.w_direct = weight_mode<BN>(a);
-    a.head_pair = (BN == 80 && a.epi == EPI_Q8_HEAD && a.n_out == a.heads * 160) ? 1 : 0;
-    if (a.head_pair && !(split && ch.prebuilt)) return cudaErrorNotSupported;
-    CUtensorMap tmap_w = tmap;                        // (unused unless w_direct)
-    if (a.w_direct) {                                 // the codes section of the blob as an int8 matrix [n_out][k_in]
-        const WeightLayout L = weight_layout(a.n_out, a.k_in, a.bits, a.group);
-        const cuuint64_t dims[3] = {(cuuint64_t)a.k_in, (cuuint64_t)a.n_out, 1};
-        const cuuint64_t strides[2] = {(cuuint64_t)L.row_bytes, (cuuint64_t)L.row_bytes * (cuuint64_t)a.n_out};
-        const cuuint32_t box[3] = {(cuuint32_t)(a.w_direct == 1 ? 2 * BK : BK), BN, 1}, estr[3] = {1, 1, 1};    // mode 2: plain rows of 64 codes
-        CUresult r = enc(&tmap_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void*)((const uint8_t*)a.w + L.off_codes), dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, a.w_direct == 1 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    }
+cudaError_t launch_bn(const CUtensorMap& tmap, EncodeTiledFn enc, const LinearArgs& a, int n_z, const Choice& ch, cudaStream_t stream) {
+    using TL = Tile<BN>;
+    const bool i8 = a.xq != nullptr, w8 = a.bits == 8;
+    void (*kern)(const CUtensorMap, const CUtensorMap, const LinearArgs, const LinearLayout) =
+        a.epi == EPI_KV ? (i8 ? (w8 ? linear_sm100_kernel<BN, true, true, true> : linear_sm100_kernel<BN, true, false, true>)
+                              : (w8 ? linear_sm100_kernel<BN, false, true, true> : linear_sm100_kernel<BN, false, false, true>))
+                        : (i8 ? (w8 ? linear_sm100_kernel<BN, true, true, false> : linear_sm100_kernel<BN, true, false, false>)
+                              : (w8 ? linear_sm100_kernel<BN, false, true, false> : linear_sm100_kernel<BN, false, false, false>));
     CUtensorMap tmap_y = tmap;                        // (unused by the K~/V~ epilogue, which scatters into the cache block)
-    if (a.epi == EPI_F16 || a.epi == EPI_F32 || a.epi == EPI_Q8_HEAD) {   // the output matrix [n_z][rows][n_out] in boxes of 32 rows x BN
+    if (a.epi != EPI_KV) {                            // the output matrix [n_z][rows][n_out] in the epilogue's boxes of 32 rows
         const cuuint64_t esz = a.epi == EPI_F16 ? 2 : a.epi == EPI_F32 ? 4 : 1;
         const cuuint64_t dims[3] = {(cuuint64_t)a.n_out, (cuuint64_t)a.rows, (cuuint64_t)n_z};
         const cuuint64_t strides[2] = {(cuuint64_t)a.n_out * esz, (cuuint64_t)a.n_out * esz * (cuuint64_t)a.rows};
-        const cuuint32_t box[3] = {BN, 32, 1}, estr[3] = {1, 1, 1};
+        const bool b80 = TL::HC % 40 == 0;            // boxes of 80 bytes per row, or 32 (int8: HC) columns in the swizzle of that row length
+        const cuuint32_t box[3] = {(cuuint32_t)(b80 ? 80 / esz : esz == 1 ? TL::HC : 32), 32, 1}, estr[3] = {1, 1, 1};
         CUresult r = enc(&tmap_y, a.epi == EPI_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : a.epi == EPI_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT8,
-                         3, a.y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                         3, a.y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         b80 ? CU_TENSOR_MAP_SWIZZLE_NONE : esz == 4 ? CU_TENSOR_MAP_SWIZZLE_128B : esz == 1 && TL::HC == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
+                         CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
     {   // (the attribute belongs to the current device's copy of the function: set on every launch, it is cheap)
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
         if (e != cudaSuccess) return e;
     }
-    const Plan P = make_plan<BN>(a.k_in, a.bits, a.group, ns, a.w_direct, ch.prebuilt);
-    dim3 grid((unsigned)((a.rows + BM - 1) / BM) * (split ? 2u : 1u), a.n_out / BN, n_z);
-    if (split) return launch_pdl_cluster(kern, grid, dim3(2, a.head_pair ? 2 : 1, 1), dim3(NTHREADS), (size_t)P.total, stream, tmap, tmap_w, tmap_y, a, ns, ch.prebuilt);
-    return launch_pdl(kern, grid, dim3(NTHREADS), (size_t)P.total, stream, tmap, tmap_w, tmap_y, a, ns, ch.prebuilt);
+    if (ch.lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(ch.grid), dim3(ch.lay.nsplit * (ch.lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
+    return launch_pdl(kern, dim3(ch.grid), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
+}
+
+// Shapes the tensor-core kernel takes at all (before looking for a layout).
+bool takes_shape(const LinearArgs& a) {
+    if (a.xq) {       // int8 activations: rows of 16-byte granularity, a scale group = one 128-element K block
+        if (a.k_in % 16) return false;
+        if (a.group != 0 && a.group != 2 * BK && a.group < a.k_in) return false;
+    } else {
+        if (a.k_in % BK) return false;
+        if (a.group != 0 && a.group % BK) return false;
+    }
+    return a.rows >= 1 && a.rows <= (1LL << 31) - 1;
 }
 
 }  // namespace
 
 bool sm100_linear_supported(const LinearArgs& a) {
-    if (a.xq) {       // int8 activations: rows of 16-byte granularity, a scale group = one 128-element K block
-        if (a.k_in % 16) return false;
-        if (a.group != 0 && a.group != 2 * BK && a.group < a.k_in) return false;
-        if (reinterpret_cast<uintptr_t>(a.xq) & 15u) return false;
-    } else {
-        if (a.k_in % BK) return false;
-        if (a.group != 0 && a.group % BK) return false;
-        if (reinterpret_cast<uintptr_t>(a.x) & 15u) return false;
-    }
+    if (!takes_shape(a)) return false;
+    if ((a.xq ? reinterpret_cast<uintptr_t>(a.xq) : reinterpret_cast<uintptr_t>(a.x)) & 15u) return false;
     if (a.epi != EPI_KV && (reinterpret_cast<uintptr_t>(a.y) & 15u)) return false;   // the output leaves by TMA stores
-    if (a.rows < 1 || a.rows > (1LL << 31) - 1) return false;
-    const int bn = pick_bn(a);
-    if (bn == 0) return false;
-    if (nstage_for(a, bn) < 2) return false;
-    return encode_tiled_fn() != nullptr;
+    return choose(a, 1).bn != 0 && encode_tiled_fn() != nullptr;
 }
 
-// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed): tile width, ring depth, how the codes
-// reach the CTA, and the byte ranges of shared memory that the ring, the epilogue's staging area and the fixed sections
-// occupy.  out: {bn, nstage, mode, ring_bytes, staging_bytes, off_raw, off_bias, off_bars, total, limit}.  bn = 0: the
-// tensor-core kernel does not take this problem.
+// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed): tile width, ring depth in k-blocks, how the
+// codes reach the CTA (0: from global memory through registers), and the byte ranges of shared memory that the rings,
+// the epilogue's staging area in them and the fixed sections occupy.  out: {bn, nstage, mode, ring_bytes, staging_bytes,
+// off_raw (the first fixed section), off_bias, off_bars, total, limit}.  bn = 0: the tensor-core kernel does not take it.
 void linear_plan_of(const LinearArgs& a, int out[10]) {
     for (int i = 0; i < 10; ++i) out[i] = 0;
     out[9] = SMEM_LIMIT;
-    bool ok = a.rows >= 1;
-    if (a.xq) ok = ok && a.k_in % 16 == 0 && (a.group == 0 || a.group == 2 * BK || a.group >= a.k_in);
-    else ok = ok && a.k_in % BK == 0 && (a.group == 0 || a.group % BK == 0);
-    if (!ok) return;
-    const int bn = pick_bn(a);
-    if (bn == 0) return;
-    if (nstage_for(a, bn) < 2) return;
-    Plan P;
-    int ring = 0, staging = 0, mode = 0, ns = 0;
-    auto fill = [&](auto bn_c) {
-        constexpr int B = decltype(bn_c)::value;
-        const Choice c = choose<B>(a, 1);
-        mode = weight_mode<B>(a); ns = c.ns;
-        P = make_plan<B>(a.k_in, a.bits, a.group, c.ns, mode, c.prebuilt);
-        ring = P.off_raw;                          // ring stages (and resident weight tiles): what the epilogue may reuse
-        staging = epilogue_staging_bytes<B>(a);
-        if (c.split && staging < NWORK * (B * 2 + 16)) staging = NWORK * (B * 2 + 16);
-    };
-    switch (bn) {
-        case 64: fill(std::integral_constant<int, 64>{}); break;
-        case 80: fill(std::integral_constant<int, 80>{}); break;
-        default: fill(std::integral_constant<int, 160>{}); break;
+    if (!takes_shape(a)) return;
+    const Choice c = choose(a, 1);
+    if (c.bn == 0) return;
+    const int n_groups = weight_layout(a.n_out, a.k_in, a.bits, a.group).n_groups;
+    Plan P{};
+    switch (c.bn) {
+        case 64: P = make_plan<64>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
+        case 80: P = make_plan<80>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
+        case 128: P = make_plan<128>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
+        default: P = make_plan<160>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
     }
-    out[0] = bn; out[1] = ns; out[2] = mode; out[3] = ring; out[4] = staging;
-    out[5] = P.off_raw; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
+    out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = 0; out[3] = P.ring_bytes; out[4] = c.staged;
+    out[5] = P.off_staging; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
 }
 
 cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t stream) {
@@ -874,10 +1034,12 @@ cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t strea
                      i8 ? (void*)const_cast<int8_t*>(a.xq) : (void*)const_cast<__half*>(a.x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    switch (pick_bn(a, n_z)) {
-        case 64: return launch_bn<64>(tmap, enc, a, n_z, stream);
-        case 80: return launch_bn<80>(tmap, enc, a, n_z, stream);
-        case 160: return launch_bn<160>(tmap, enc, a, n_z, stream);
+    const Choice c = choose(a, n_z);
+    switch (c.bn) {
+        case 64: return launch_bn<64>(tmap, enc, a, n_z, c, stream);
+        case 80: return launch_bn<80>(tmap, enc, a, n_z, c, stream);
+        case 128: return launch_bn<128>(tmap, enc, a, n_z, c, stream);
+        case 160: return launch_bn<160>(tmap, enc, a, n_z, c, stream);
     }
     return cudaErrorNotSupported;
 }
