@@ -1,11 +1,14 @@
 """ctypes binding of ``libtaq.so``: the same entry points as ``include/taq.h``, taking torch CUDA tensors.
 
 Only argument marshalling happens here (pointers, sizes, the current CUDA stream); every step of the TAQ
-cross-attention path runs in the library's kernels.  There is no CPU path: a missing library raises.
+cross-attention path runs in the library's kernels.  There is no CPU path: a missing library raises.  The calls of a
+running program (packing, projections, attention, layer passes) go through ``_taq_call``, a C++ extension module that
+unpacks the tensors (``csrc/taq_pymodule.cpp``); the rest goes through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -13,6 +16,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libtaq.so")
+CALL_PATH = os.path.join(_PKG, "_taq_call.so")
 
 TAQ_OK = 0
 TAQ_ERR_INVALID_ARG, TAQ_ERR_SHAPE, TAQ_ERR_ALIGNMENT, TAQ_ERR_BUFFER_TOO_SMALL = 1, 2, 3, 4
@@ -67,6 +71,22 @@ class Request(C.Structure):
 
 
 _lib = None
+_call_module = None
+
+
+def _call():
+    """The native call path, bound to the loaded library on first use."""
+    global _call_module
+    if _call_module is None:
+        L = lib()
+        if not os.path.exists(CALL_PATH):
+            raise RuntimeError(f"{CALL_PATH} is missing: build it with `python -m paper_2603_22943_b200.build`")
+        spec = importlib.util.spec_from_file_location("_taq_call", CALL_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.init(*[C.cast(getattr(L, n), C.c_void_p).value for n in m.names()])
+        _call_module = m
+    return _call_module
 
 
 def lib() -> C.CDLL:
@@ -187,7 +207,7 @@ def taq_pack_weights(desc: WeightDesc, W: torch.Tensor, bias: Optional[torch.Ten
         if nbytes == 0:
             _check(lib().taq_pack_weights(C.byref(desc), _ptr(W), _ptr(bias), None, 0, _stream(stream)))
         packed = torch.zeros(nbytes, dtype=torch.uint8, device=W.device)
-    _check(lib().taq_pack_weights(C.byref(desc), _ptr(W), _ptr(bias), _ptr(packed), packed.numel(), _stream(stream)))
+    _check((_call_module or _call()).pack_weights(desc, W, bias, packed, stream))
     return packed
 
 
@@ -223,8 +243,7 @@ def taq_kv_project(desc: LayerDesc, ctx: torch.Tensor, Wk_packed: torch.Tensor, 
                    trig_mask: torch.Tensor, kv: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     if kv is None:
         kv = torch.zeros(max(taq_kv_bytes(desc), 16), dtype=torch.uint8, device=ctx.device)
-    _check(lib().taq_kv_project(C.byref(desc), _ptr(ctx), _ptr(Wk_packed), _ptr(Wv_packed), _ptr(trig_mask), _ptr(kv),
-                                kv.numel(), _stream(stream)))
+    _check((_call_module or _call()).kv_project(desc, ctx, Wk_packed, Wv_packed, trig_mask, kv, stream))
     return kv
 
 
@@ -242,7 +261,7 @@ def taq_quantized_linear(desc: WeightDesc, x: torch.Tensor, W_packed: torch.Tens
         y = torch.empty((rows, desc.n_out), dtype=dt, device=x.device)
     if out_kind == TAQ_OUT_INT8_HEAD_ROWS and scales is None:
         scales = torch.empty((rows, heads), dtype=torch.float32, device=x.device)
-    _check(lib().taq_quantized_linear(C.byref(desc), _ptr(x), rows, _ptr(W_packed), _ptr(y), out_kind, heads, _ptr(scales), _stream(stream)))
+    _check((_call_module or _call()).quantized_linear(desc, x, rows, W_packed, y, out_kind, heads, scales, stream))
     return (y, scales) if out_kind == TAQ_OUT_INT8_HEAD_ROWS else y
 
 
@@ -252,7 +271,7 @@ def taq_quantize_rows_f16(x: torch.Tensor, stream=None):
     rows = x.numel() // cols
     codes = torch.empty(x.shape, dtype=torch.int8, device=x.device)
     scales = torch.empty(x.shape[:-1], dtype=torch.float32, device=x.device)
-    _check(lib().taq_quantize_rows_f16(_ptr(x), rows, cols, _ptr(codes), _ptr(scales), _stream(stream)))
+    _check((_call_module or _call()).quantize_rows_f16(x, rows, cols, codes, scales, stream))
     return codes, scales
 
 
@@ -266,8 +285,7 @@ def taq_quantized_linear_i8(desc: WeightDesc, x_codes: torch.Tensor, x_scales: t
         y = torch.empty((rows, desc.n_out), dtype=dt, device=x_codes.device)
     if out_kind == TAQ_OUT_INT8_HEAD_ROWS and scales is None:
         scales = torch.empty((rows, heads), dtype=torch.float32, device=x_codes.device)
-    _check(lib().taq_quantized_linear_i8(C.byref(desc), _ptr(x_codes), _ptr(x_scales), rows, _ptr(W_packed), _ptr(y), out_kind, heads,
-                                         _ptr(scales), _stream(stream)))
+    _check((_call_module or _call()).quantized_linear_i8(desc, x_codes, x_scales, rows, W_packed, y, out_kind, heads, scales, stream))
     return (y, scales) if out_kind == TAQ_OUT_INT8_HEAD_ROWS else y
 
 
@@ -283,8 +301,7 @@ def taq_layer_forward_a8(desc: LayerDesc, x: torch.Tensor, Wq_packed: torch.Tens
         y = torch.empty((desc.batch, desc.n_query, desc.channels), dtype=torch.float16, device=x.device)
     if workspace is None:
         workspace = torch.empty(max(taq_workspace_bytes_a8(desc), 128), dtype=torch.uint8, device=x.device)
-    _check(lib().taq_layer_forward_a8(C.byref(desc), _ptr(x), _ptr(Wq_packed), _ptr(Wout_packed), _ptr(kv), _ptr(trig_mask), _ptr(y),
-                                      _ptr(workspace), workspace.numel(), _stream(stream)))
+    _check((_call_module or _call()).layer_forward_a8(desc, x, Wq_packed, Wout_packed, kv, trig_mask, y, workspace, stream))
     return y
 
 
@@ -296,8 +313,7 @@ def taq_kv_project_a8(desc: LayerDesc, ctx: torch.Tensor, Wk_packed: torch.Tenso
         kv = torch.zeros(max(taq_kv_bytes(desc), 16), dtype=torch.uint8, device=ctx.device)
     if workspace is None:
         workspace = torch.empty(max(lib().taq_kv_project_a8_workspace_bytes(C.byref(desc)), 128), dtype=torch.uint8, device=ctx.device)
-    _check(lib().taq_kv_project_a8(C.byref(desc), _ptr(ctx), _ptr(Wk_packed), _ptr(Wv_packed), _ptr(trig_mask), _ptr(kv), kv.numel(),
-                                   _ptr(workspace), workspace.numel(), _stream(stream)))
+    _check((_call_module or _call()).kv_project_a8(desc, ctx, Wk_packed, Wv_packed, trig_mask, kv, workspace, stream))
     return kv
 
 
@@ -367,7 +383,7 @@ def taq_cross_attention(desc: LayerDesc, q: torch.Tensor, q_scales: Optional[tor
                         trig_mask: torch.Tensor, o: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     if o is None:
         o = torch.empty((desc.batch, desc.n_query, desc.channels), dtype=torch.float16, device=kv.device)
-    _check(lib().taq_cross_attention(C.byref(desc), _ptr(q), _ptr(q_scales), _ptr(kv), _ptr(trig_mask), _ptr(o), _stream(stream)))
+    _check((_call_module or _call()).cross_attention(desc, q, q_scales, kv, trig_mask, o, stream))
     return o
 
 
@@ -382,8 +398,7 @@ def taq_layer_forward(desc: LayerDesc, x: torch.Tensor, Wq_packed: torch.Tensor,
         y = torch.empty((desc.batch, desc.n_query, desc.channels), dtype=torch.float16, device=x.device)
     if workspace is None:
         workspace = torch.empty(max(taq_workspace_bytes(desc, 1), 128), dtype=torch.uint8, device=x.device)
-    _check(lib().taq_layer_forward(C.byref(desc), _ptr(x), _ptr(Wq_packed), _ptr(Wout_packed), _ptr(kv), _ptr(trig_mask), _ptr(y),
-                                   _ptr(workspace), workspace.numel(), _stream(stream)))
+    _check((_call_module or _call()).layer_forward(desc, x, Wq_packed, Wout_packed, kv, trig_mask, y, workspace, stream))
     return y
 
 
@@ -394,8 +409,7 @@ def taq_query_attention(desc: LayerDesc, x: torch.Tensor, Wq_packed: torch.Tenso
         o = torch.empty((desc.batch, desc.n_query, desc.channels), dtype=torch.float16, device=x.device)
     if workspace is None:
         workspace = torch.empty(max(taq_workspace_bytes(desc, 1), 128), dtype=torch.uint8, device=x.device)
-    _check(lib().taq_query_attention(C.byref(desc), _ptr(x), _ptr(Wq_packed), _ptr(kv), _ptr(trig_mask), _ptr(o), _ptr(workspace),
-                                     workspace.numel(), _stream(stream)))
+    _check((_call_module or _call()).query_attention(desc, x, Wq_packed, kv, trig_mask, o, workspace, stream))
     return o
 
 
@@ -407,8 +421,7 @@ def taq_layer_forward_static(desc: LayerDesc, x: torch.Tensor, Wq_packed: torch.
                              kv: torch.Tensor, trig_mask: torch.Tensor, y: torch.Tensor, stream=None) -> torch.Tensor:
     """The layer pass on the library's built-in scratch array.  ``y`` must be supplied: this wrapper, like the
     entry point under it, allocates nothing."""
-    _check(lib().taq_layer_forward_static(C.byref(desc), _ptr(x), _ptr(Wq_packed), _ptr(Wout_packed), _ptr(kv), _ptr(trig_mask),
-                                          _ptr(y), _stream(stream)))
+    _check((_call_module or _call()).layer_forward_static(desc, x, Wq_packed, Wout_packed, kv, trig_mask, y, stream))
     return y
 
 
@@ -426,13 +439,12 @@ def taq_layer_forward_batched(desc: LayerDesc, reqs: torch.Tensor, n_requests: i
         y = torch.empty((n_requests, desc.n_query, desc.channels), dtype=torch.float16, device=x.device)
     if workspace is None:
         workspace = torch.empty(max(taq_workspace_bytes(desc, n_requests), 128), dtype=torch.uint8, device=x.device)
-    _check(lib().taq_layer_forward_batched(C.byref(desc), _ptr(reqs), n_requests, _ptr(x), _ptr(y), _ptr(workspace),
-                                           workspace.numel(), _stream(stream)))
+    _check((_call_module or _call()).layer_forward_batched(desc, reqs, n_requests, x, y, workspace, stream))
     return y
 
 
 def taq_kv_project_batched(desc: LayerDesc, reqs: torch.Tensor, n_requests: int, ctx: torch.Tensor, stream=None) -> None:
-    _check(lib().taq_kv_project_batched(C.byref(desc), _ptr(reqs), n_requests, _ptr(ctx), _stream(stream)))
+    _check((_call_module or _call()).kv_project_batched(desc, reqs, n_requests, ctx, stream))
 
 
 KERNEL_FAMILIES = ("linear_tensor", "linear_generic", "attention_tensor", "attention_generic", "query_attention_fused",
