@@ -175,9 +175,15 @@ cudaError_t launch_sensitivity_masks(uint8_t* masks, int batch, int n_ctx, cudaS
     return cudaGetLastError();
 }
 
-// One warp per (output channel, group).
+// TPG threads per (output channel, group): a warp for groups of up to 512 elements (the usual 128), half a block for longer ones
+// (a whole row of an 8-bit matrix).  Bound by reading W once (a 1280 x 1280 matrix is 6.6 MB, 1 us): a thread keeps its
+// elements in registers between the absmax and the codes, 16-byte loads, one word of codes per two lanes, codes by the
+// reciprocal where it decides (quant_code_127).  (With scalar loads, a division per element and a second pass over W that
+// eight lanes of strided words read, the four matrices of a 1280-channel layer took 32 us.)
+template <int TPG>
 __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restrict__ W, const float* __restrict__ bias, uint8_t* __restrict__ blob,
                                                            int n_out, int k_in, int bits, int group) {
+    constexpr int KEEP = 4, PER_BLOCK = 256 / TPG;              // float4 per thread in registers; items per block
     const WeightLayout L = weight_layout(n_out, k_in, bits, group);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         PackedHeader h;
@@ -186,44 +192,71 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restri
         h.off_codes = L.off_codes; h.off_scales = L.off_scales; h.off_bias = L.off_bias; h.total_bytes = L.total;
         *reinterpret_cast<PackedHeader*>(blob) = h;
     }
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, t = threadIdx.x % TPG, slot = threadIdx.x / TPG;
     const int qmax = bits == 8 ? 127 : 7;
     const long long items = (long long)n_out * L.n_groups;
-    const long long warps_total = (long long)gridDim.x * (blockDim.x >> 5);
     float* scales = reinterpret_cast<float*>(blob + L.off_scales);
     float* bias_out = reinterpret_cast<float*>(blob + L.off_bias);
-    uint8_t* codes = blob + L.off_codes;
-    for (long long it = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < items; it += warps_total) {
-        const int n = (int)(it / L.n_groups), g = (int)(it % L.n_groups);
-        const int lo = g * L.group_len, hi = min(k_in, lo + L.group_len);
-        const float* wr = W + (size_t)n * k_in;
+    __shared__ float part[8];
+    // (every thread of a block makes the same number of rounds: the longer groups meet at barriers)
+    for (long long it0 = (long long)blockIdx.x * PER_BLOCK; it0 < items; it0 += (long long)gridDim.x * PER_BLOCK) {
+        const bool real = it0 + slot < items;
+        const long long it = real ? it0 + slot : items - 1;
+        const int n = items < (1LL << 31) ? (int)((uint32_t)it / (uint32_t)L.n_groups) : (int)(it / L.n_groups), g = (int)(it - (long long)n * L.n_groups);
+        const int lo = g * L.group_len, n4 = (min(k_in, lo + L.group_len) - lo) / 4;      // (group lengths and fan-ins are multiples of 8)
+        const float4* w4 = reinterpret_cast<const float4*>(W + (size_t)n * k_in + lo);
+        float4 keep[KEEP];
         float a = 0.f;
-        for (int k = lo + lane; k < hi; k += 32) a = fmaxf(a, fabsf(wr[k]));
+        auto absmax4 = [&](const float4& v) { a = fmaxf(a, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
+#pragma unroll
+        for (int j = 0; j < KEEP; ++j) keep[j] = t + TPG * j < n4 ? w4[t + TPG * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < KEEP; ++j) absmax4(keep[j]);
+        for (int i = t + TPG * KEEP; i < n4; i += TPG) absmax4(w4[i]);
         a = warp_max(a);
+        if (TPG > 32) {
+            __syncthreads();
+            if (lane == 0) part[threadIdx.x >> 5] = a;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < TPG / 32; ++k) a = fmaxf(a, part[slot * (TPG / 32) + k]);
+        }
         const float s = quant_scale(a, (float)qmax);
-        if (lane == 0) {
+        const float rs = s > 0.f ? __frcp_rn(s) : 0.f;
+        const float r_lo = __uint_as_float(__float_as_uint(rs) - 2u), r_hi = __uint_as_float(__float_as_uint(rs) + 2u);
+        auto code = [&](float x) { return s > 0.f ? min(max(quant_code_127(x, s, r_lo, r_hi), -qmax), qmax) : 0; };
+        if (real && t == 0) {
             scales[(size_t)n * L.n_groups + g] = s;
             if (g == 0) bias_out[n] = bias ? bias[n] : 0.f;
         }
-        if (bits == 8) {
-            for (int k = lo + lane; k < hi; k += 32) ((int8_t*)codes)[(size_t)n * L.row_bytes + k] = (int8_t)quant_code(wr[k], s, qmax);
-        } else {
-            for (int k = lo + 8 * lane; k < hi; k += 256) {   // group bounds are multiples of 8: a word never straddles groups
+        uint8_t* row = blob + L.off_codes + (size_t)n * L.row_bytes;
+        auto encode = [&](const float4& v, int i, bool have) {               // elements 4 i .. 4 i + 3 of the group
+            const int c[4] = {code(v.x), code(v.y), code(v.z), code(v.w)};
+            if (bits == 8) {
+                if (real && have) reinterpret_cast<char4*>(row + lo)[i] = make_char4((signed char)c[0], (signed char)c[1], (signed char)c[2], (signed char)c[3]);
+            } else {                                             // a word is eight elements: two neighbouring lanes
                 uint32_t word = 0;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) word |= (uint32_t)(quant_code(wr[k + e], s, qmax) + 8) << (4 * w4_nibble_pos(e));
-                *reinterpret_cast<uint32_t*>(codes + (size_t)n * L.row_bytes + (k >> 1)) = word;
+                for (int e = 0; e < 4; ++e) word |= (uint32_t)(c[e] + 8) << (4 * w4_nibble_pos(e + 4 * (lane & 1)));
+                word |= __shfl_xor_sync(0xffffffffu, word, 1);
+                if (real && have && (lane & 1) == 0) reinterpret_cast<uint32_t*>(row + lo / 2)[i >> 1] = word;
             }
-        }
+        };
+#pragma unroll
+        for (int j = 0; j < KEEP; ++j)
+            if (TPG * j < n4) encode(keep[j], t + TPG * j, t + TPG * j < n4);
+        for (int i0 = TPG * KEEP; i0 < n4; i0 += TPG) encode(i0 + t < n4 ? w4[i0 + t] : make_float4(0.f, 0.f, 0.f, 0.f), i0 + t, i0 + t < n4);
     }
 }
 
 cudaError_t launch_pack_weights(const taq_weight_desc& d, const float* W, const float* bias, void* packed, cudaStream_t stream) {
     const WeightLayout L = weight_layout(d.n_out, d.k_in, d.bits, d.group);
-    long long items = (long long)d.n_out * L.n_groups;
-    long long blocks = (items + 7) / 8;
+    const bool wide = L.group_len > 512;
+    const long long items = (long long)d.n_out * L.n_groups, per_block = wide ? 2 : 8;
+    long long blocks = (items + per_block - 1) / per_block;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
-    pack_weights_kernel<<<(unsigned)blocks, 256, 0, stream>>>(W, bias, (uint8_t*)packed, d.n_out, d.k_in, d.bits, d.group);
+    if (wide) pack_weights_kernel<128><<<(unsigned)blocks, 256, 0, stream>>>(W, bias, (uint8_t*)packed, d.n_out, d.k_in, d.bits, d.group);
+    else pack_weights_kernel<32><<<(unsigned)blocks, 256, 0, stream>>>(W, bias, (uint8_t*)packed, d.n_out, d.k_in, d.bits, d.group);
     return cudaGetLastError();
 }
 
