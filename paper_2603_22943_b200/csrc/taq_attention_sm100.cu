@@ -609,10 +609,9 @@ int pick_heads_per_cta(const AttnArgs& a, int n_z) {
 template <int D, bool Q8, bool TAIL_ONLY>
 cudaError_t launch_k(const AttnArgs& a, int n_z, cudaStream_t stream) {
     using C = Cfg<D>;
-    {   // (the attribute belongs to the current device's copy of the function: set on every launch, it is cheap)
-        cudaError_t e = cudaFuncSetAttribute(attention_sm100_kernel<D, Q8, TAIL_ONLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::TOTAL);
-        if (e != cudaSuccess) return e;
-    }
+    static std::atomic<unsigned long long> limit_set;
+    cudaError_t e = allow_shared_memory((const void*)attention_sm100_kernel<D, Q8, TAIL_ONLY>, C::TOTAL, limit_set);
+    if (e != cudaSuccess) return e;
     const int hg = pick_heads_per_cta<D>(a, n_z);
     dim3 grid((a.n_query + ROWS - 1) / ROWS, a.heads / hg, n_z);
     CUtensorMap tmap_q, tmap_o;

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "taq.h"
 
 namespace taq {
@@ -155,6 +157,19 @@ struct AttnArgs {
     int early_kv;               // the previous kernel in the stream is known not to write the K~/V~ blocks
     int* status;
 };
+
+// Raises a kernel's dynamic shared-memory limit, once per device (`done` is a bit per device; the attribute belongs to the
+// device's copy of the function).
+inline cudaError_t allow_shared_memory(const void* kernel, int bytes, std::atomic<unsigned long long>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 // Launch with the programmatic-serialization attribute (see ptx::pdl_wait): the kernel's prologue may overlap the
 // tail of the previous kernel in the stream.

@@ -885,8 +885,8 @@ static cudaError_t launch_c320(const taq_layer_desc& d, const __half* x, const v
         q_in ? (tail == 72 ? layer_c320_kernel<72, false, true> : tail == 64 ? layer_c320_kernel<64, false, true> : layer_c320_kernel<0, false, true>) :
         fuse_out ? (tail == 72 ? layer_c320_kernel<72, true> : tail == 64 ? layer_c320_kernel<64, true> : layer_c320_kernel<0, true>)
                  : (tail == 72 ? layer_c320_kernel<72, false> : tail == 64 ? layer_c320_kernel<64, false> : layer_c320_kernel<0, false>);
-    // (the attribute belongs to the current device's copy of the function: set on every launch, it is cheap)
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TOTAL);
+    static std::atomic<unsigned long long> limit_set[9];
+    cudaError_t e = allow_shared_memory((const void*)kern, TOTAL, limit_set[(q_in ? 0 : fuse_out ? 3 : 6) + (tail == 72 ? 0 : tail == 64 ? 1 : 2)]);
     if (e != cudaSuccess) return e;
     if (fuse_out) return launch_pdl_cluster(kern, grid, dim3(1, 2, 1), dim3(NTHREADS), (size_t)TOTAL, stream, tmap, tmap_y, a);
     return launch_pdl(kern, grid, dim3(NTHREADS), (size_t)TOTAL, stream, tmap, tmap_y, a);

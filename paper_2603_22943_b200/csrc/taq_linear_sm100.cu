@@ -912,7 +912,7 @@ bool tile_carries(const LinearArgs& a, const Problem& p, int bn) {
 // The cheapest layout by a small model of a CTA's life in SM cycles: a fixed part (launch, barriers, first loads, epilogue), the K
 // loop at the pace of the tensor core, and the exchange of partial sums when the loop is split; a persistent CTA pays
 // the fixed part once and the K loop per tile.
-Choice choose(const LinearArgs& a, int n_z) {
+Choice choose_anew(const LinearArgs& a, int n_z) {
     const Problem p = problem_of(a);
     Choice best{};
     auto finish = [&](Choice& c, long long tiles, long long ctas) {
@@ -946,6 +946,22 @@ Choice choose(const LinearArgs& a, int n_z) {
     return best;
 }
 
+// The last few problems of the calling thread: a program runs the same layers again and again.
+Choice choose(const LinearArgs& a, int n_z) {
+    struct Key { long long rows; int n_out, k_in, bits, group, heads, epi, n_ctx, n_z, flags, pad; };
+    struct Known { Key key; Choice choice; };
+    constexpr int N = 16;
+    thread_local Known known[N] = {};
+    thread_local int next = 0;
+    const Key k = {a.rows, a.n_out, a.k_in, a.bits, a.group, a.heads, a.epi, a.n_ctx, n_z, 4 | (a.xq ? 1 : 0) | (a.reqs ? 2 : 0), 0};
+    for (const Known& e : known)
+        if (memcmp(&e.key, &k, sizeof(k)) == 0) return e.choice;
+    Known& e = known[next];
+    next = (next + 1) % N;
+    e.key = k;
+    return e.choice = choose_anew(a, n_z);
+}
+
 template <int BN>
 cudaError_t launch_bn(const CUtensorMap& tmap, EncodeTiledFn enc, const LinearArgs& a, int n_z, const Choice& ch, cudaStream_t stream) {
     using TL = Tile<BN>;
@@ -968,10 +984,9 @@ cudaError_t launch_bn(const CUtensorMap& tmap, EncodeTiledFn enc, const LinearAr
                          CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
-    {   // (the attribute belongs to the current device's copy of the function: set on every launch, it is cheap)
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
-        if (e != cudaSuccess) return e;
-    }
+    static std::atomic<unsigned long long> limit_set[8];
+    cudaError_t e = allow_shared_memory((const void*)kern, SMEM_LIMIT, limit_set[(a.epi == EPI_KV) * 4 + i8 * 2 + w8]);
+    if (e != cudaSuccess) return e;
     if (ch.lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(ch.grid), dim3(ch.lay.nsplit * (ch.lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
     return launch_pdl(kern, dim3(ch.grid), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
 }

@@ -914,8 +914,8 @@ static cudaError_t launch_c320(const taq_layer_desc& d, const __half* x, const v
     }
     (void)a8;                                         // only the integer-activation variant is built from this file
     void (*kern)(const CUtensorMap, const CUtensorMap, const QAttnArgs) = tail ? qattn_c320_kernel<true, true, true> : qattn_c320_kernel<false, true, true>;
-    // (the attribute belongs to the current device's copy of the function: set on every launch, it is cheap)
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TOTAL);
+    static std::atomic<unsigned long long> limit_set[2];
+    cudaError_t e = allow_shared_memory((const void*)kern, TOTAL, limit_set[tail ? 1 : 0]);
     if (e != cudaSuccess) return e;
     if (fuse_out) return launch_pdl_cluster(kern, grid, dim3(1, 2, 1), dim3(NTHREADS), (size_t)TOTAL, stream, tmap, tmap_y, a);
     return launch_pdl(kern, grid, dim3(NTHREADS), (size_t)TOTAL, stream, tmap, tmap_y, a);
