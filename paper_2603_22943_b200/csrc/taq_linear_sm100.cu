@@ -43,7 +43,7 @@ constexpr int BM = 128;
 constexpr int BK = 64;                     // fp16 elements per 128-byte operand row; the int8 variant has 2 BK
 constexpr int A_TILE_BYTES = BM * 128;     // 16 KB
 constexpr int MAX_STAGE = 6;               // ring depths, in pairs of k-blocks
-constexpr int MAX_SLOT = 4;                // accumulators in TMEM
+constexpr int MAX_SLOT = 8;                // accumulators in TMEM
 constexpr int SMEM_LIMIT = 227 * 1024;
 
 // Tile shapes: 160 columns (a multiple of every SD head width), 80 for launches with few rows, 128 and 64 for heads of 64 channels
@@ -62,8 +62,8 @@ struct Tile {
     static constexpr int W_PROD = 0, W_MMA = 1, W_AUX = 2, W_FOLD = 4, W_BUILD = W_FOLD + NF;
     static constexpr int R_FOLD = 128, R_BUILD = 48, R_REST = 56;
     static_assert(128 * (R_REST + NF / 4 * R_FOLD + NB / 4 * R_BUILD) == NTHREADS * 72, "register split");
-    static constexpr uint32_t TMEM_COLS = BN >= 128 ? 512 : 256;
-    static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 or 4
+    static constexpr uint32_t TMEM_COLS = 512;
+    static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 to 8
     static constexpr int B_TILE = BN * 128;                                   // one k-block
     static constexpr int NCH = BN * 16 / (NBUILD / 2);                        // 16-byte tile chunks per builder thread and pair of k-blocks
     static constexpr int PART_ROW = HC * 4 + 16;                              // a thread's partial sums in transit, padded against bank conflicts
@@ -82,28 +82,39 @@ struct Bars {
 constexpr int N_BARS = 4 * MAX_STAGE + 2 * MAX_SLOT + 4 + 2 + 8 + 4;        // the barriers above, one after the other
 static_assert(offsetof(Bars, tmem_base) == N_BARS * 8, "barriers are contiguous");
 
-// How a launch is laid out: CTAs that share the K loop of a tile, ring depths in pairs of k-blocks, bytes of an output staging area
-// of its own (several tiles per CTA), heads of 160 channels on two tiles, tiles.
-struct LinearLayout { int nsplit, nsa, nsb, staging, head_pair, row_tiles, n_tiles; };
-
 // Shared-memory plan of one launch (host and device agree through these numbers).
-struct Plan { int ring_bytes, off_scales, scale_bytes, off_bias, off_xchg, off_staging, off_bars, total; };
+struct Plan { int ring_bytes, off_scales, scale_bytes, off_bias, off_xchg, off_bars, total; };
 
-// nsa, nsb: pairs of k-blocks in the rings; staging: bytes of an output staging area of its own (0: the epilogue stages in the
-// rings, which are free by then unless the CTA walks several tiles).
+// nsa, nsb: pairs of k-blocks in the rings; persistent: a CTA walks several tiles.
 template <int BN>
-__host__ __device__ inline Plan make_plan(int n_groups, int nsa, int nsb, int staging) {
+inline Plan make_plan(int n_groups, int nsa, int nsb, bool persistent) {
     Plan p;
     p.ring_bytes = 2 * (nsa * A_TILE_BYTES + nsb * Tile<BN>::B_TILE);
-    p.off_staging = p.ring_bytes;
-    p.off_scales = p.off_staging + staging;                                   // two buffers of float [n_groups][BN], then bias [BN]
+    p.off_scales = p.ring_bytes;                                              // (two buffers of) float [n_groups][BN], then bias [BN]
     p.scale_bytes = (n_groups + 1) * BN * 4;
     p.off_bias = p.off_scales + n_groups * BN * 4;
-    p.off_xchg = p.off_scales + (staging ? 2 : 1) * p.scale_bytes;            // (one tile per CTA: one buffer) float [4][128]
+    p.off_xchg = p.off_scales + (persistent ? 2 : 1) * p.scale_bytes;         // float [4][128]
     p.off_bars = p.off_xchg + 4 * 128 * 4 + 128;           // (K~/V~: the slots and the bitmap use the second half)
     p.total = p.off_bars + 1024 + 1024;                                       // barriers + slack to align the base to 1024
     return p;
 }
+
+// How a launch is laid out: CTAs that share the K loop of a tile, ring depths in pairs of k-blocks, heads of 160 channels on two
+// tiles, tiles; and what every thread would otherwise work out for itself at the start (a third of a small launch's prologue):
+// the blob's layout, the shared-memory plan, multipliers for the divisions by n_cols and n_rows.
+struct LinearLayout {
+    int nsplit, nsa, nsb, head_pair, persistent;
+    int n_tiles, n_cols, n_rows;            // tiles of the launch: n_cols column tiles (K's and V's) per row tile, n_rows row tiles per z
+    uint32_t mul_cols, mul_rows;            // see quotient()
+    int n_groups, kb_per_group, n_kb;
+    uint32_t row_bytes;
+    unsigned long long off_scales, off_bias;
+    Plan plan;
+};
+
+// t / d by a multiplication (mul = 2^32 / d + 1, exact for t and d below 2^16; 0: divide).
+__device__ __forceinline__ int quotient(int t, int d, uint32_t mul) { return mul ? (int)__umulhi((uint32_t)t, mul) : d == 1 ? t : t / d; }
+uint32_t multiplier(int d, long long n) { return d > 1 && d < 65536 && n < 65536 ? (uint32_t)((1ull << 32) / (unsigned)d + 1) : 0u; }
 
 __device__ __forceinline__ void ffma2(unsigned long long& acc, uint32_t lo, uint32_t hi, unsigned long long s) {
     unsigned long long v;
@@ -137,25 +148,24 @@ __device__ __forceinline__ typename Code<I8, W8>::T zero_codes() {
 // through bulk copies between the shared memories, every CTA adding and storing its share of the tile's rows.
 template <int BN, bool I8, bool W8, bool KV>
 __global__ void __launch_bounds__(Tile<BN>::NTHREADS, 1)
-linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_y, const LinearArgs a, const LinearLayout lay) {
+linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ LinearArgs a, const __grid_constant__ LinearLayout lay) {
     using TL = Tile<BN>;
     using CodeT = typename Code<I8, W8>::T;
     constexpr int HC = TL::HC, NCG = TL::NCG, NSLOT = TL::NSLOT, NCH = TL::NCH;
     constexpr int BKE = I8 ? 2 * BK : BK;             // elements per K block
-    constexpr int FC = HC == 80 ? 16 : HC == 64 ? 32 : HC;      // columns in flight while a group is folded
+    constexpr int FC = HC >= 64 ? 16 : HC;            // columns of a group that are loaded at a time while it is folded
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* smem = smem_dyn + ((1024u - (ptx::smem_u32(smem_dyn) & 1023u)) & 1023u);   // 1024-byte aligned, still provably shared
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nsplit = lay.nsplit, nsa = lay.nsa, nsb = lay.nsb;
     const int rank = nsplit > 1 ? (int)(blockIdx.x % (unsigned)nsplit) : 0;
-    const WeightLayout L = weight_layout(a.n_out, a.k_in, a.bits, a.group);
-    const int n_groups = L.n_groups;
-    const Plan P = make_plan<BN>(n_groups, nsa, nsb, lay.staging);
+    const int n_groups = lay.n_groups;
+    const Plan& P = lay.plan;
     static_assert(sizeof(Bars) <= 1024, "barrier block");
     Bars* bars = reinterpret_cast<Bars*>(smem + P.off_bars);
-    const int n_kb_all = (a.k_in + BKE - 1) / BKE;      // (int8: the last block may be ragged; TMA and the expansion zero-fill)
-    const int kb_per_group = n_groups == 1 ? n_kb_all : L.group_len / BKE;   // k-blocks in a full group (the last group may be shorter)
+    const int n_kb_all = lay.n_kb;                      // (int8: the last block may be ragged; TMA and the expansion zero-fill)
+    const int kb_per_group = lay.kb_per_group;          // k-blocks in a full group (the last group may be shorter)
     // this CTA's share of the K loop: a run of whole scale groups, or (one scale per output channel) of k-blocks
     int g_begin = 0, g_end = n_groups, kb_begin = 0, kb_stop = n_kb_all;
     if (nsplit > 1) {
@@ -170,29 +180,28 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     const bool clustered = nsplit > 1;
     const bool with_bias = !KV && a.epi != EPI_Q8_HEAD && (I8 || rank == 0);   // (of CTAs that share a tile one starts from the bias)
     // Tiles: column tile fastest, so that the CTAs running at one time share rows of x; then row tile, then z.
-    const int n_col = a.n_out / BN, n_cols = KV ? 2 * n_col : n_col, n_rows = lay.row_tiles;
-    const int tile0 = (int)(blockIdx.x / (unsigned)nsplit), tile_step = (int)(gridDim.x / (unsigned)nsplit);
+    const int tile0 = (int)blockIdx.x / nsplit, tile_step = lay.persistent ? (int)gridDim.x : lay.n_tiles;      // (several tiles: never split)
     auto tile_of = [&](int t, int& z, int& row0, int& col0, int& kv_which) {
-        const int cz = t / n_cols;
-        int c = t - cz * n_cols;
-        z = cz / n_rows;
-        row0 = (cz - z * n_rows) * BM;
-        kv_which = KV && c >= n_col ? 1 : 0;
-        if (kv_which) c -= n_col;
+        const int cz = quotient(t, lay.n_cols, lay.mul_cols);
+        int c = t - cz * lay.n_cols;
+        z = quotient(cz, lay.n_rows, lay.mul_rows);
+        row0 = (cz - z * lay.n_rows) * BM;
+        kv_which = KV && 2 * c >= lay.n_cols ? 1 : 0;
+        if (kv_which) c -= lay.n_cols >> 1;
         col0 = c * BN;
     };
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(30); }
     if (warp == TL::W_PROD) {
-        // (one lane per barrier: fifty in a row by one thread took a fifth of a small launch's start)
+        // (one lane per barrier: sixty in a row by one thread took a fifth of a small launch's start)
         uint64_t* all = bars->full_a;
+        constexpr int FULL_B = 2 * MAX_STAGE, EMPTY_B = 3 * MAX_STAGE, ACC_FREE = 4 * MAX_STAGE + MAX_SLOT, SCALE_FULL = ACC_FREE + MAX_SLOT, SCALE_FREE = SCALE_FULL + 2;
+#pragma unroll
         for (int i = lane; i < N_BARS; i += 32) {
-            const uint64_t* bar = all + i;
-            const uint32_t count = bar >= bars->full_b && bar < bars->empty_b ? TL::NB / 2 : bar >= bars->acc_free && bar < bars->scale_full ? TL::NF :
-                                   bar >= bars->scale_full && bar < bars->scale_free ? 2 : bar >= bars->scale_free && bar < &bars->tmem_ready ? TL::NF :
-                                   bar == &bars->peer_ready && clustered ? nsplit - 1 : 1;
-            ptx::mbar_init(all + i, count);
+            const int count = i >= FULL_B && i < EMPTY_B ? TL::NB / 2 : i < ACC_FREE ? 1 : i < SCALE_FULL ? TL::NF : i < SCALE_FREE ? 2 : i < SCALE_FREE + 2 ? TL::NF :
+                              i == SCALE_FREE + 3 && clustered ? nsplit - 1 : 1;       // (the last: peer_ready)
+            ptx::mbar_init(all + i, (uint32_t)count);
         }
         ptx::mbar_fence_init();
         __syncwarp();
@@ -208,13 +217,14 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
     } else if (warp == TL::W_AUX && lane == 0) {
         ptx::tma_prefetch_desc(&tmap_x);
-        ptx::tma_prefetch_desc(&tmap_y);
     }
-    // Every role passes this barrier before it touches another role's state; the builders do so with their first codes under way.
-    auto start = [&]() {
-        __syncthreads();
+    // Every role passes this barrier before it touches another role's state; the builders do so with their first codes under way,
+    // and the producer, whose own barriers are all it needs, only announces itself and starts to load.
+    auto start = [&](bool wait) {
+        if (wait) asm volatile("bar.sync 14, %0;" ::"n"(TL::NTHREADS) : "memory");
+        else asm volatile("bar.arrive 14, %0;" ::"n"(TL::NTHREADS) : "memory");
         ptx::pdl_trigger();
-        if (clustered) ptx::cluster_arrive();                // waited for right before the first operation on another CTA
+        if (clustered) ptx::cluster_arrive_relaxed();        // waited for right before the first operation on another CTA
     };
     auto blob_of = [&](int z, int kv_which) { return (const uint8_t*)(a.reqs ? ((KV ? kv_which : a.which) == 0 ? a.reqs[z].Wq : a.reqs[z].Wout) : kv_which ? a.w2 : a.w); };
     auto give_up = [&]() { raise_status(a.status, TAQ_ERR_TIMEOUT); bars->abort_flag = 1; };
@@ -307,7 +317,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
     if (warp >= TL::W_FOLD && warp < TL::W_BUILD) {
         // ---------------- folders ----------------
-        start();
+        start(true);
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::R_FOLD));
         const int ft = tid - 32 * TL::W_FOLD;
         const int q = warp & 3;                              // TMEM lane quarter this warp may read
@@ -339,15 +349,21 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 ptx::tc_fence_after_sync();
                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + slot * BN + cb;
                 const float* sg = scales + g * BN;
+                // (the next columns are on their way from TMEM while these are multiplied and added: a group of 80 columns took
+                // 850 cycles one load after the other, and the folders, not the tensor core, set the pace of a large launch)
+                uint32_t v[2][FC / 8][8];
+#pragma unroll
+                for (int i = 0; i < FC / 8; ++i) ptx::tmem_ld8(taddr + i * 8, v[0][i]);
 #pragma unroll
                 for (int c0 = 0; c0 < HC; c0 += FC) {
-                    uint32_t v[FC / 8][8];
+                    const int k = (c0 / FC) & 1;
+                    ptx::tmem_ld_wait(v[k][0]);
 #pragma unroll
-                    for (int i = 0; i < FC / 8; ++i) ptx::tmem_ld8(taddr + c0 + i * 8, v[i]);
-                    ptx::tmem_ld_wait(v[0]);
+                    for (int i = 1; i < FC / 8; ++i) ptx::reg_fence8(v[k][i]);
+                    if (c0 + FC < HC) {
 #pragma unroll
-                    for (int i = 1; i < FC / 8; ++i) ptx::reg_fence8(v[i]);
-                    if (c0 + FC == HC) {                     // the accumulator is in registers: the tensor core may have it back
+                        for (int i = 0; i < FC / 8; ++i) ptx::tmem_ld8(taddr + c0 + FC + i * 8, v[k ^ 1][i]);
+                    } else {                                 // the accumulator is in registers: the tensor core may have it back
                         ptx::tc_fence_before_sync();
                         __syncwarp();
                         if (lane == 0) ptx::mbar_arrive(&bars->acc_free[slot]);
@@ -355,13 +371,14 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                     for (int i = 0; i < FC / 8; ++i) {
                         const ulonglong2 s0 = *reinterpret_cast<const ulonglong2*>(sg + c0 + i * 8), s1 = *reinterpret_cast<const ulonglong2*>(sg + c0 + i * 8 + 4);
+                        uint32_t (&w)[8] = v[k][i];
                         if (I8) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[i][e] = __float_as_uint(__int2float_rn((int)v[i][e]));
+                            for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(__int2float_rn((int)w[e]));
                         }
                         unsigned long long* yy = y2 + (c0 + i * 8) / 2;
-                        ffma2(yy[0], v[i][0], v[i][1], s0.x); ffma2(yy[1], v[i][2], v[i][3], s0.y);
-                        ffma2(yy[2], v[i][4], v[i][5], s1.x); ffma2(yy[3], v[i][6], v[i][7], s1.y);
+                        ffma2(yy[0], w[0], w[1], s0.x); ffma2(yy[1], w[2], w[3], s0.y);
+                        ffma2(yy[2], w[4], w[5], s1.x); ffma2(yy[3], w[6], w[7], s1.y);
                     }
                 }
                 if (++slot == NSLOT) { slot = 0; ph_acc ^= 1; }
@@ -433,7 +450,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (bars->abort_flag) break;
             }
             // ... but not over this CTA's outgoing pieces, which may still be in flight: the staging area begins behind them
-            unsigned char* staging = smem + (lay.staging ? P.off_staging : clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0);
+            unsigned char* staging = smem + (clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0);
 
             const long long row = (long long)row0 + r;
             const bool live = mine && row < a.rows;
@@ -449,47 +466,51 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             }
 
             // ---------------- epilogue on this thread's HC columns ----------------
-            // Dense outputs are staged per warp in shared memory as boxes of 32 rows and leave by TMA stores (the tensor map
-            // clips rows beyond the matrix).  A box row is 80 bytes (an odd number of 16-byte units) or swizzled, so that
-            // the row-per-lane writes are free of bank conflicts.
-            const bool store_rows = mine && (long long)row0 + q * 32 < a.rows;
-            if (!KV && a.epi != EPI_Q8_HEAD) {
-                auto dense = [&](auto f16_c) {
-                    constexpr bool F16 = decltype(f16_c)::value;
-                    constexpr bool B80 = HC % 40 == 0;
-                    constexpr int BOX = B80 ? (F16 ? 40 : 20) : 32;                  // columns
-                    constexpr int BOX_BYTES = B80 ? 2560 : F16 ? 2048 : 4096, NBOX = HC / BOX;
-                    // (several tiles per CTA: one box buffer per warp; else every box has a place of its own in the rings)
-                    unsigned char* st = staging + (size_t)fw * (lay.staging ? 1 : NBOX) * BOX_BYTES;
+            // Dense outputs.  A CTA with one tile stages each warp's rows in shared memory (its rings are free) and stores them with
+            // neighbouring lanes on neighbouring chunks of a row; a CTA that walks several tiles stores a row per lane straight from
+            // the registers, in pieces of 32 bytes.  (TMA stores cost a one-tile CTA 1 000 cycles of waiting until the box was
+            // read, and the folders of the others 2 600 per tile of fences and waits for the box before.)
+            auto put = [&](const uint32_t* w, auto bytes_c) {                        // the thread's columns, `bytes` in w
+                constexpr int ROW = decltype(bytes_c)::value, ESZ = ROW / HC, CHUNK = ROW % 16 == 0 ? 16 : 8, N = ROW / CHUNK;
+                using V = typename std::conditional<CHUNK == 16, uint4, uint2>::type;
+                uint8_t* dst = (uint8_t*)a.y + (((size_t)z * a.rows + row0 + q * 32) * a.n_out + col0 + cb) * ESZ;
+                const uint32_t pitch = (uint32_t)a.n_out * ESZ;
+                const long long left = mine ? a.rows - ((long long)row0 + q * 32) : 0;
+                if (lay.persistent) {
+                    if (lane >= left) return;
+                    dst += (size_t)lane * pitch;
+                    if (ROW % 32 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 31u) == 0) {
 #pragma unroll
-                    for (int b = 0; b < NBOX; ++b) {
-                        if (lay.staging) {                                           // the previous store has read the buffer
-                            if (lane == 0) ptx::bulk_store_wait_read();
-                            __syncwarp();
-                        }
+                        for (int i = 0; i < ROW / 32; ++i) ptx::store_32b(dst + i * 32, w + i * 8);
+                    } else {
 #pragma unroll
-                        for (int c = 0; c < BOX; c += F16 ? 8 : 4) {
-                            const int k = b * BOX + c;
-                            if (F16) {
-                                float f[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) f[e] = y[(k + e) % HC];
-                                *reinterpret_cast<uint4*>(B80 ? st + lane * 80 + c * 2 : st + ptx::sw64_offset(lane, c / 8)) = pack8(f);
-                            } else {
-                                *reinterpret_cast<float4*>(B80 ? st + lane * 80 + c * 4 : st + ptx::sw128_offset(lane, c / 4)) =
-                                    make_float4(y[k], y[(k + 1) % HC], y[(k + 2) % HC], y[(k + 3) % HC]);
-                            }
-                        }
-                        ptx::fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0 && store_rows) {
-                            ptx::tma_store_3d(&tmap_y, st, col0 + cb + b * BOX, row0 + q * 32, z);
-                            ptx::bulk_store_commit();
-                        }
-                        if (!lay.staging) st += BOX_BYTES;
+                        for (int i = 0; i < N; ++i) reinterpret_cast<V*>(dst)[i] = reinterpret_cast<const V*>(w)[i];
                     }
-                };
-                if (a.epi == EPI_F16) dense(std::true_type{}); else dense(std::false_type{});
+                } else {
+                    unsigned char* st = staging + (size_t)fw * 32 * ROW;
+#pragma unroll
+                    for (int i = 0; i < N; ++i) reinterpret_cast<V*>(st + lane * ROW)[i] = reinterpret_cast<const V*>(w)[i];
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < N; ++i) {
+                        const int j = lane + 32 * i, rr = j / N, part = j - rr * N;
+                        if (rr < left) *reinterpret_cast<V*>(dst + (size_t)rr * pitch + part * CHUNK) = *reinterpret_cast<const V*>(st + j * CHUNK);
+                    }
+                }
+            };
+            if (!KV && a.epi == EPI_F16) {
+                alignas(16) uint32_t w[HC / 2];
+#pragma unroll
+                for (int c = 0; c < HC; c += 2) {
+                    const __half2 h = __floats2half2_rn(y[c], y[c + 1]);
+                    w[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
+                }
+                put(w, std::integral_constant<int, HC * 2>{});
+            } else if (!KV && a.epi == EPI_F32) {
+                alignas(16) uint32_t w[HC];
+#pragma unroll
+                for (int c = 0; c < HC; ++c) w[c] = __float_as_uint(y[c]);
+                put(w, std::integral_constant<int, HC * 4>{});
             } else {
                 // Per-(row, head) symmetric int8.  A thread's columns are whole heads (two of 40, or one), or half of what the row
                 // has of a head in this tile.
@@ -529,24 +550,14 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const float s0 = quant_scale(am0, qmax), s1 = two ? quant_scale(am1, qmax) : s0;
                 const float r0 = s0 > 0.f ? __frcp_rn(s0) : 0.f, r1 = s1 > 0.f ? __frcp_rn(s1) : 0.f;
                 if constexpr (!KV) {
-                    // Q~ = Q_a(Q), Eq. 2 third line.  Boxes of 80 columns (one warp's, or 40 of each of the row's two threads),
-                    // 64 or 32.
-                    constexpr bool SHARED_BOX = HC == 40;
-                    unsigned char* st = staging + (SHARED_BOX ? (size_t)q * 2560 : (size_t)fw * 32 * HC);
-                    if (tile != tile0) {                     // the previous tile's store has read the box
-                        if (lane == 0) ptx::bulk_store_wait_read();
-                        if (SHARED_BOX) asm volatile("bar.sync %0, 64;" ::"r"(6 + q) : "memory"); else __syncwarp();
-                    }
+                    // Q~ = Q_a(Q), Eq. 2 third line
+                    alignas(16) uint32_t w[HC / 4];
 #pragma unroll
-                    for (int c = 0; c < HC; c += 8)
-                        *reinterpret_cast<uint2*>(HC == 80 ? st + lane * 80 + c : HC == 40 ? st + lane * 80 + cg * 40 + c :
-                                                  HC == 64 ? st + ptx::sw64_offset(lane, c / 16) + (c & 8) : st + ptx::sw32_offset(lane, c / 16) + (c & 8)) = quant8(y + c, c < SPLIT_AT ? r0 : r1);
-                    ptx::fence_proxy_async_smem();
-                    if (SHARED_BOX) asm volatile("bar.sync %0, 64;" ::"r"(6 + q) : "memory"); else __syncwarp();
-                    if (lane == 0 && store_rows && (!SHARED_BOX || cg == 0)) {
-                        ptx::tma_store_3d(&tmap_y, st, SHARED_BOX ? col0 : colg, row0 + q * 32, z);
-                        ptx::bulk_store_commit();
+                    for (int c = 0; c < HC; c += 8) {
+                        const uint2 code = quant8(y + c, c < SPLIT_AT ? r0 : r1);
+                        w[c / 4] = code.x; w[c / 4 + 1] = code.y;
                     }
+                    put(w, std::integral_constant<int, HC>{});
                     if (live) {
                         float* sc = a.scales + ((size_t)z * a.rows + row) * a.heads;
                         if (colg == h0 * d) sc[h0] = s0;
@@ -594,7 +605,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             sbuf ^= 1;
             if (sbuf == 0) ph_scale ^= 1;
         }
-        if (lane == 0) ptx::bulk_store_wait_read();          // shared memory is given back only after the stores have read it
         __syncwarp();
         if constexpr (KV) kv_together(true, ft);
         if (clustered && !joined) ptx::cluster_wait();
@@ -608,7 +618,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // of a tile row hit all banks.
         constexpr int CB = (int)sizeof(CodeT);
         const int c16 = bt & 15, n0 = bt >> 4;
-        const uint32_t row_step = (uint32_t)(TL::NBUILD / 2 / 16) * (uint32_t)L.row_bytes;
+        const uint32_t row_step = (uint32_t)(TL::NBUILD / 2 / 16) * lay.row_bytes;
         const int n_pair = (n_kb + 1) / 2;
         // Codes are fetched one turn ahead, across tile boundaries: all of a pair's chunks where they take at most ten registers
         // (more would spill), else half of them, the rest when they are needed.
@@ -629,13 +639,13 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             if (new_tile) {
                 int z, row0, col0, kv_which;
                 tile_of(tile, z, row0, col0, kv_which);
-                src = blob_of(z, kv_which) + L.off_codes + (size_t)(col0 + n0) * L.row_bytes + (size_t)(kb_begin + 2 * pair) * (8 * CB) + c16 * CB;
+                src = blob_of(z, kv_which) + 128 + (size_t)(col0 + n0) * lay.row_bytes + (size_t)(kb_begin + 2 * pair) * (8 * CB) + c16 * CB;
             }
 #pragma unroll
             for (int j = 0; j < NPRE; ++j) pw[j] = load(j);
         };
         fetch(true);
-        start();
+        start(true);
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_BUILD));
         int s = group;
         uint32_t ph = 1;
@@ -667,7 +677,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         if constexpr (KV) kv_together(false, TL::NFOLD + tid - 32 * TL::W_BUILD);
         if (clustered) ptx::cluster_wait();
     } else {
-        start();
+        start(warp != TL::W_PROD);
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_REST));
         if (warp == TL::W_PROD) {
             // ---------------- producer: activation tiles ----------------
@@ -711,6 +721,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 uint32_t pha = 0, phb = 0, ph_free = 1, a_lo = a_lo0, b_lo = b_lo0;
                 bool ok = true, recycled = false;            // recycled: every accumulator has been used once
                 bool next_a = false, next_b = false;         // the next pair was seen complete already
+                int todo = ((n_kb + 1) / 2) * ((lay.n_tiles - tile0 + tile_step - 1) / tile_step);      // pairs left
                 for (int tile = tile0; tile < lay.n_tiles && ok; tile += tile_step) {
                     int left = 0;                            // k-blocks left in the current group
                     uint32_t d_tmem = 0;
@@ -743,8 +754,10 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                             }
                         }
                         if (!ok) break;
-                        ptx::mma_commit(&bars->empty_a[sa]); // these free the stages once the MMAs have read them
-                        ptx::mma_commit(&bars->empty_b[sb]);
+                        // these free the stages once the MMAs have read them (a commit costs 60 cycles: none where nothing follows)
+                        if (todo > nsa) ptx::mma_commit(&bars->empty_a[sa]);
+                        if (todo > nsb) ptx::mma_commit(&bars->empty_b[sb]);
+                        --todo;
                         a_lo += 2 * A_TILE_BYTES >> 4;
                         b_lo += 2 * TL::B_TILE >> 4;
                         if (++sa == nsa) { sa = 0; pha ^= 1; a_lo = a_lo0; }
@@ -764,8 +777,8 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 int z, row0, col0, kv_which;
                 tile_of(tile, z, row0, col0, kv_which);
                 const uint8_t* blob = blob_of(z, kv_which);
-                const float* gs = reinterpret_cast<const float*>(blob + L.off_scales) + (size_t)col0 * n_groups;
-                const float* gb = reinterpret_cast<const float*>(blob + L.off_bias) + col0;
+                const float* gs = reinterpret_cast<const float*>(blob + lay.off_scales) + (size_t)col0 * n_groups;
+                const float* gb = reinterpret_cast<const float*>(blob + lay.off_bias) + col0;
                 if (it >= 2 && !ptx::mbar_wait(&bars->scale_free[sbuf], ph)) { give_up(); break; }
                 float* sc = reinterpret_cast<float*>(smem + P.off_scales + sbuf * P.scale_bytes);
                 // [BN][n_groups] -> [n_groups][BN], so that a group's scales of consecutive columns are contiguous
@@ -774,7 +787,8 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     for (int g = g_begin; g < g_end; ++g) sc[g * BN + n] = __ldg(gs + (size_t)n * n_groups + g);
                     sc[n_groups * BN + n] = with_bias ? __ldg(gb + n) : 0.f;
                 }
-                if (KV && warp == TL::W_AUX) {               // slot of every token of the sequence among its trigger tokens, and their bitmap
+                if (KV && warp == TL::W_AUX) {               // (the mask may come from the previous kernel) slot of every token of the sequence among its trigger tokens, and their bitmap
+                    ptx::pdl_wait();
                     const uint8_t* mask = a.reqs ? a.reqs[z].trig_mask : a.mask + (size_t)z * a.n_ctx;
                     int* slots = reinterpret_cast<int*>(smem + P.off_xchg) + 256;
                     int before = 0;
@@ -804,7 +818,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     ptx::tc_fence_before_sync();
     // (No CTA of a cluster may leave while a copy out of its shared memory is in flight: by this barrier every copy has
     // been received.  Every thread arrives, whatever happened to its waits.)
-    if (clustered) { ptx::cluster_arrive(); ptx::cluster_wait(); }
+    if (clustered) { ptx::cluster_arrive_relaxed(); ptx::cluster_wait(); }
     __syncthreads();
     if (tid == 0) { TAQ_PROF(9); TAQ_GPROF(29); }
     if (warp == TL::W_MMA) {
@@ -836,6 +850,7 @@ struct Problem {                       // what the choice depends on
     int n_groups, group_len, bke, n_kb, d, ncols_factor;
     bool i8;
     long long row_tiles;
+    WeightLayout L;
 };
 Problem problem_of(const LinearArgs& a) {
     const WeightLayout L = weight_layout(a.n_out, a.k_in, a.bits, a.group);
@@ -847,6 +862,7 @@ Problem problem_of(const LinearArgs& a) {
     p.d = a.epi == EPI_Q8_HEAD || a.epi == EPI_KV ? a.n_out / a.heads : 0;
     p.ncols_factor = a.epi == EPI_KV ? 2 : 1;
     p.row_tiles = (a.rows + BM - 1) / BM;
+    p.L = L;
     return p;
 }
 // k-blocks of the longest share when the K loop is split
@@ -863,10 +879,10 @@ template <int BN>
 bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, bool persistent, Choice& c) {
     using TL = Tile<BN>;
     const int n_pair = (share_of(p, nsplit) + 1) / 2;
-    int staging = 0, staged = 0;
+    int staged = 0;
     const int tile_bytes = a.epi == EPI_F16 ? BM * BN * 2 : a.epi == EPI_F32 ? BM * BN * 4 : a.epi == EPI_Q8_HEAD ? BM * BN : 128 * (BN + 1) * 4 + BN / p.d * 1024;      // (K~/V~: the fp32 tile and the rows' scales)
     if (persistent) {
-        staging = TL::NF * (TL::HC % 40 == 0 ? 2560 : a.epi == EPI_F32 ? 4096 : 2048);
+        // (stored from the registers)
     } else if (nsplit == 1) {
         staged = tile_bytes;
     } else {
@@ -874,14 +890,18 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
         staged = 2 * send > send + tile_bytes ? 2 * send : send + tile_bytes;
     }
     int nsa = n_pair < 2 ? 1 : 2, nsb = n_pair < 2 ? 1 : 2;
-    while (make_plan<BN>(p.n_groups, nsa, nsb, staging).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
-    auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, staging).total <= SMEM_LIMIT; };
+    while (make_plan<BN>(p.n_groups, nsa, nsb, persistent).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
+    auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, persistent).total <= SMEM_LIMIT; };
     while (nsb < (persistent ? MAX_STAGE : n_pair) && nsb < MAX_STAGE && fits(nsa, nsb + 1)) ++nsb;
     while (nsa < 3 && nsa < n_pair && fits(nsa + 1, nsb)) ++nsa;
-    const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, staging);
+    const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, persistent);
     if (P.total > SMEM_LIMIT || P.ring_bytes < staged) return false;
     c.bn = BN;
-    c.lay.nsplit = nsplit; c.lay.nsa = nsa; c.lay.nsb = nsb; c.lay.staging = staging; c.lay.head_pair = head_pair;
+    c.lay.nsplit = nsplit; c.lay.nsa = nsa; c.lay.nsb = nsb; c.lay.head_pair = head_pair; c.lay.persistent = persistent;
+    c.lay.plan = P;
+    c.lay.n_groups = p.n_groups; c.lay.n_kb = p.n_kb;
+    c.lay.kb_per_group = p.n_groups == 1 ? p.n_kb : p.group_len / p.bke;
+    c.lay.row_bytes = (uint32_t)p.L.row_bytes; c.lay.off_scales = p.L.off_scales; c.lay.off_bias = p.L.off_bias;
     c.total = P.total; c.ring = P.ring_bytes; c.staged = staged;
     return true;
 }
@@ -916,7 +936,9 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
     const Problem p = problem_of(a);
     Choice best{};
     auto finish = [&](Choice& c, long long tiles, long long ctas) {
-        c.lay.row_tiles = (int)p.row_tiles; c.lay.n_tiles = (int)tiles;
+        c.lay.n_tiles = (int)tiles;
+        c.lay.n_cols = a.n_out / c.bn * p.ncols_factor; c.lay.n_rows = (int)p.row_tiles;
+        c.lay.mul_cols = multiplier(c.lay.n_cols, tiles); c.lay.mul_rows = multiplier(c.lay.n_rows, tiles);
         c.grid = (int)ctas;
         return c;
     };
@@ -963,32 +985,19 @@ Choice choose(const LinearArgs& a, int n_z) {
 }
 
 template <int BN>
-cudaError_t launch_bn(const CUtensorMap& tmap, EncodeTiledFn enc, const LinearArgs& a, int n_z, const Choice& ch, cudaStream_t stream) {
+cudaError_t launch_bn(const CUtensorMap& tmap, const LinearArgs& a, const Choice& ch, cudaStream_t stream) {
     using TL = Tile<BN>;
     const bool i8 = a.xq != nullptr, w8 = a.bits == 8;
-    void (*kern)(const CUtensorMap, const CUtensorMap, const LinearArgs, const LinearLayout) =
+    void (*kern)(const CUtensorMap, const LinearArgs, const LinearLayout) =
         a.epi == EPI_KV ? (i8 ? (w8 ? linear_sm100_kernel<BN, true, true, true> : linear_sm100_kernel<BN, true, false, true>)
                               : (w8 ? linear_sm100_kernel<BN, false, true, true> : linear_sm100_kernel<BN, false, false, true>))
                         : (i8 ? (w8 ? linear_sm100_kernel<BN, true, true, false> : linear_sm100_kernel<BN, true, false, false>)
                               : (w8 ? linear_sm100_kernel<BN, false, true, false> : linear_sm100_kernel<BN, false, false, false>));
-    CUtensorMap tmap_y = tmap;                        // (unused by the K~/V~ epilogue, which scatters into the cache block)
-    if (a.epi != EPI_KV) {                            // the output matrix [n_z][rows][n_out] in the epilogue's boxes of 32 rows
-        const cuuint64_t esz = a.epi == EPI_F16 ? 2 : a.epi == EPI_F32 ? 4 : 1;
-        const cuuint64_t dims[3] = {(cuuint64_t)a.n_out, (cuuint64_t)a.rows, (cuuint64_t)n_z};
-        const cuuint64_t strides[2] = {(cuuint64_t)a.n_out * esz, (cuuint64_t)a.n_out * esz * (cuuint64_t)a.rows};
-        const bool b80 = TL::HC % 40 == 0;            // boxes of 80 bytes per row, or 32 (int8: HC) columns in the swizzle of that row length
-        const cuuint32_t box[3] = {(cuuint32_t)(b80 ? 80 / esz : esz == 1 ? TL::HC : 32), 32, 1}, estr[3] = {1, 1, 1};
-        CUresult r = enc(&tmap_y, a.epi == EPI_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : a.epi == EPI_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT8,
-                         3, a.y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         b80 ? CU_TENSOR_MAP_SWIZZLE_NONE : esz == 4 ? CU_TENSOR_MAP_SWIZZLE_128B : esz == 1 && TL::HC == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
-                         CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    }
     static std::atomic<unsigned long long> limit_set[8];
     cudaError_t e = allow_shared_memory((const void*)kern, SMEM_LIMIT, limit_set[(a.epi == EPI_KV) * 4 + i8 * 2 + w8]);
     if (e != cudaSuccess) return e;
-    if (ch.lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(ch.grid), dim3(ch.lay.nsplit * (ch.lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
-    return launch_pdl(kern, dim3(ch.grid), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, tmap_y, a, ch.lay);
+    if (ch.lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(ch.grid), dim3(ch.lay.nsplit * (ch.lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, a, ch.lay);
+    return launch_pdl(kern, dim3(ch.grid), dim3(TL::NTHREADS), (size_t)ch.total, stream, tmap, a, ch.lay);
 }
 
 // Shapes the tensor-core kernel takes at all (before looking for a layout).
@@ -1008,7 +1017,7 @@ bool takes_shape(const LinearArgs& a) {
 bool sm100_linear_supported(const LinearArgs& a) {
     if (!takes_shape(a)) return false;
     if ((a.xq ? reinterpret_cast<uintptr_t>(a.xq) : reinterpret_cast<uintptr_t>(a.x)) & 15u) return false;
-    if (a.epi != EPI_KV && (reinterpret_cast<uintptr_t>(a.y) & 15u)) return false;   // the output leaves by TMA stores
+    if (a.epi != EPI_KV && (reinterpret_cast<uintptr_t>(a.y) & 15u)) return false;   // the output leaves in pieces of 16 bytes
     return choose(a, 1).bn != 0 && encode_tiled_fn() != nullptr;
 }
 
@@ -1022,16 +1031,9 @@ void linear_plan_of(const LinearArgs& a, int out[10]) {
     if (!takes_shape(a)) return;
     const Choice c = choose(a, 1);
     if (c.bn == 0) return;
-    const int n_groups = weight_layout(a.n_out, a.k_in, a.bits, a.group).n_groups;
-    Plan P{};
-    switch (c.bn) {
-        case 64: P = make_plan<64>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
-        case 80: P = make_plan<80>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
-        case 128: P = make_plan<128>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
-        default: P = make_plan<160>(n_groups, c.lay.nsa, c.lay.nsb, c.lay.staging); break;
-    }
+    const Plan& P = c.lay.plan;
     out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = 0; out[3] = P.ring_bytes; out[4] = c.staged;
-    out[5] = P.off_staging; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
+    out[5] = P.off_scales; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
 }
 
 cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t stream) {
@@ -1051,10 +1053,10 @@ cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t strea
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     const Choice c = choose(a, n_z);
     switch (c.bn) {
-        case 64: return launch_bn<64>(tmap, enc, a, n_z, c, stream);
-        case 80: return launch_bn<80>(tmap, enc, a, n_z, c, stream);
-        case 128: return launch_bn<128>(tmap, enc, a, n_z, c, stream);
-        case 160: return launch_bn<160>(tmap, enc, a, n_z, c, stream);
+        case 64: return launch_bn<64>(tmap, a, c, stream);
+        case 80: return launch_bn<80>(tmap, a, c, stream);
+        case 128: return launch_bn<128>(tmap, a, c, stream);
+        case 160: return launch_bn<160>(tmap, a, c, stream);
     }
     return cudaErrorNotSupported;
 }
