@@ -52,16 +52,23 @@ constexpr int SMEM_LIMIT = 227 * 1024;
 template <int BN_>
 struct Tile {
     static constexpr int BN = BN_;
-    static constexpr int NCG = 2;                                             // column groups: folder threads per row
-    static constexpr int HC = BN / NCG;                                       // columns per folder thread
+    // Folder warps and builder warps: the wide tiles have sixteen and eight (a thread of eight folder warps would hold 80 sums, which
+    // spills, and two warps per scheduler hide neither TMEM nor shared-memory latency: a group took them 950 cycles), the
+    // narrow ones, which live for one tile, eight and sixteen (their weight tiles are all built before the activations arrive).
+    static constexpr bool BIG = BN >= 128;
+    static constexpr int NCG = BIG ? 4 : 2;                                   // column groups: folder threads per row
+    static constexpr int HC = BN / NCG;                                       // columns per folder thread: 40 or 32
     static constexpr int NF = 4 * NCG, NFOLD = 32 * NF;                       // folder warps, threads
-    static constexpr int NB = 16, NBUILD = 32 * NB;                           // builder warps, threads
+    static constexpr int NB = 24 - NF, NBUILD = 32 * NB;                      // builder warps, threads
     // Warpgroups keep one role each, and registers go where they are needed.  What the block is launched with covers it:
-    //   896 threads x 72 = 128 x (56 + 2 x 128 + 4 x 48)
+    //   896 threads x 72 = 128 x (56 + 4 x 88 + 2 x 48) = 128 x (56 + 2 x 128 + 4 x 48)
     static constexpr int NTHREADS = 128 + NFOLD + NBUILD;
     static constexpr int W_PROD = 0, W_MMA = 1, W_AUX = 2, W_FOLD = 4, W_BUILD = W_FOLD + NF;
-    static constexpr int R_FOLD = 128, R_BUILD = 48, R_REST = 56;
+    static constexpr int R_FOLD = BIG ? 88 : 128, R_BUILD = 48, R_REST = 56;
     static_assert(128 * (R_REST + NF / 4 * R_FOLD + NB / 4 * R_BUILD) == NTHREADS * 72, "register split");
+    // ... and of the K~/V~ epilogue's second half, see kv_together: 896 x 72 >= 128 x (56 + 4 x 80 + 2 x 64) = 128 x (56 + 2 x 80 + 4 x 72)
+    static constexpr int R_KV_FOLD = 80, R_KV_BUILD = BIG ? 64 : 72;
+    static_assert(NF * R_KV_FOLD + NB * R_KV_BUILD <= NF * R_FOLD + NB * R_BUILD, "register split");
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 to 8
     static constexpr int B_TILE = BN * 128;                                   // one k-block
@@ -75,11 +82,11 @@ struct Bars {
     uint64_t full_a[MAX_STAGE], empty_a[MAX_STAGE], full_b[MAX_STAGE], empty_b[MAX_STAGE];
     uint64_t acc_full[MAX_SLOT], acc_free[MAX_SLOT];
     uint64_t scale_full[2], scale_free[2];
-    uint64_t tmem_ready, peer_ready, part_full[8], pair_full[4];
+    uint64_t tmem_ready, peer_ready, part_full[16], pair_full[4];
     uint32_t tmem_base;
     volatile int abort_flag;
 };
-constexpr int N_BARS = 4 * MAX_STAGE + 2 * MAX_SLOT + 4 + 2 + 8 + 4;        // the barriers above, one after the other
+constexpr int N_BARS = 4 * MAX_STAGE + 2 * MAX_SLOT + 4 + 2 + 16 + 4;       // the barriers above, one after the other
 static_assert(offsetof(Bars, tmem_base) == N_BARS * 8, "barriers are contiguous");
 
 // Shared-memory plan of one launch (host and device agree through these numbers).
@@ -93,8 +100,8 @@ inline Plan make_plan(int n_groups, int nsa, int nsb, bool persistent) {
     p.off_scales = p.ring_bytes;                                              // (two buffers of) float [n_groups][BN], then bias [BN]
     p.scale_bytes = (n_groups + 1) * BN * 4;
     p.off_bias = p.off_scales + n_groups * BN * 4;
-    p.off_xchg = p.off_scales + (persistent ? 2 : 1) * p.scale_bytes;         // float [4][128]
-    p.off_bars = p.off_xchg + 4 * 128 * 4 + 128;           // (K~/V~: the slots and the bitmap use the second half)
+    p.off_xchg = p.off_scales + (persistent ? 2 : 1) * p.scale_bytes;         // float [4][128], then (K~/V~) the slots [128] and the bitmap [4]
+    p.off_bars = p.off_xchg + 5 * 128 * 4 + 128;
     p.total = p.off_bars + 1024 + 1024;                                       // barriers + slack to align the base to 1024
     return p;
 }
@@ -153,7 +160,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     using CodeT = typename Code<I8, W8>::T;
     constexpr int HC = TL::HC, NCG = TL::NCG, NSLOT = TL::NSLOT, NCH = TL::NCH;
     constexpr int BKE = I8 ? 2 * BK : BK;             // elements per K block
-    constexpr int FC = HC >= 64 ? 16 : HC;            // columns of a group that are loaded at a time while it is folded
+    constexpr int FC = TL::BIG ? 8 : HC;            // columns of a group that are loaded at a time while it is folded
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* smem = smem_dyn + ((1024u - (ptx::smem_u32(smem_dyn) & 1023u)) & 1023u);   // 1024-byte aligned, still provably shared
 
@@ -245,7 +252,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         OperandGeom G;
         const bool images = operand_geom(d, T, &G);
         uint8_t* img0 = blk + KL.off_operands + (size_t)head0 * G.head_bytes;
-        const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 256;
+        const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;
         const float* ys = reinterpret_cast<const float*>(smem + kv_staging_off);
         const float2* hs = reinterpret_cast<const float2*>(smem + kv_staging_off + 128 * KV_STRIDE * 4);
         const int own_shift = nsplit == 1 ? 7 : nsplit == 2 ? 6 : 5;         // (CTAs that share the tile finish the rows of some lane quarters each)
@@ -305,13 +312,13 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             }
         }
     };
-    // The folders hand registers to the builders on the way, 128 x (56 + 2 x 80 + 4 x 72) = 896 x 72: they give theirs back before
+    // The folders hand registers to the builders on the way: they give theirs back before
     // the barrier, the builders ask behind it.  (A builder that asked as soon as it ran out of work could be given what the
     // folders' first request was still waiting for, and neither would ever go on.)
     auto kv_together = [&](bool folder, int w) {
-        if (folder) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        if (folder) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_KV_FOLD));
         asm volatile("bar.sync 15, %0;" ::"n"(TL::NFOLD + TL::NBUILD) : "memory");
-        if (!folder) asm volatile("setmaxnreg.inc.sync.aligned.u32 72;");
+        if (!folder) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::R_KV_BUILD));
         if (!bars->abort_flag) kv_store(w);
     };
 
@@ -328,6 +335,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         int slot = 0, sbuf = 0;
         uint32_t ph_acc = 0, ph_scale = 0;
         bool joined = false;                                 // has waited for the cluster's first barrier
+        bool alive = true;                                   // no wait has run out (a warp skips work then, never a barrier)
         uint32_t tmem_base = 0;
         if (ptx::mbar_wait(&bars->tmem_ready, 0)) tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base); else give_up();
         for (int tile = tile0; tile < lay.n_tiles; tile += tile_step) {
@@ -336,7 +344,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             const float* scales = reinterpret_cast<const float*>(smem + P.off_scales + sbuf * P.scale_bytes) + cb;
             const float* bias = scales + n_groups * BN;
             unsigned long long y2[HC / 2];
-            bool ok = ptx::mbar_wait(&bars->scale_full[sbuf], ph_scale);
+            bool ok = alive && ptx::mbar_wait(&bars->scale_full[sbuf], ph_scale);
 #pragma unroll
             for (int c = 0; c < HC; c += 4) {                // the sums start from the bias (zero where there is none; int8: added last)
                 const ulonglong2 b4 = *reinterpret_cast<const ulonglong2*>(bias + c);
@@ -383,18 +391,16 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 if (++slot == NSLOT) { slot = 0; ph_acc ^= 1; }
             }
-            if (!ok) give_up();
+            if (!ok && alive) { give_up(); alive = false; }
             if (tile == tile0) ptx::pdl_wait();              // (already satisfied: the activations have arrived) orders the stores below
             if (ft == 0) TAQ_PROF(7);
-            asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");         // every folder gets here; the decision below is uniform
-            if (bars->abort_flag) break;
             if (!I8 && lane == 0) ptx::mbar_arrive(&bars->scale_free[sbuf]);     // scales and biases of this tile have been read
 
             float y[HC];
 #pragma unroll
             for (int c = 0; c < HC / 2; ++c) asm("mov.b64 {%0, %1}, %2;" : "=f"(y[2 * c]), "=f"(y[2 * c + 1]) : "l"(y2[c]));
 
-            bool mine = true;                                // this CTA finishes the warp's rows
+            bool mine = alive;                               // this CTA finishes the warp's rows
             if (clustered) {
                 // All of this CTA's MMAs are complete (every group was folded), so its rings are free: they hold the partial
                 // sums in transit.  CTA `owner` of the cluster finishes the rows of 4 / nsplit lane quarters: a folder warp
@@ -402,12 +408,12 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 // every other CTA and adds them in rank order, so that every output is the same sum whoever computes it.
                 const int per_cta = 4 / nsplit, owner = q / per_cta;
                 const uint32_t base = ptx::cluster_ctarank() - (uint32_t)rank;        // ranks along x are consecutive
-                mine = owner == rank;
+                mine = alive && owner == rank;
                 ptx::cluster_wait();                         // the other CTAs' barriers exist
                 joined = true;
                 if (ft < nsplit && ft != rank) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), base + (uint32_t)ft));
                 const int n_send = NCG * (4 - per_cta);
-                if (!mine) {
+                if (owner != rank) {
                     unsigned char* piece = smem + (cg * (4 - per_cta) + (q < rank * per_cta ? q : q - per_cta)) * TL::PIECE;
                     float* out = reinterpret_cast<float*>(piece + lane * TL::PART_ROW);
 #pragma unroll
@@ -447,7 +453,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");     // pieces read: the epilogue stages output where they were ...
                 if (ft == 0) TAQ_PROF(10);
-                if (bars->abort_flag) break;
+                mine = mine && !bars->abort_flag;
             }
             // ... but not over this CTA's outgoing pieces, which may still be in flight: the staging area begins behind them
             unsigned char* staging = smem + (clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0);
@@ -479,9 +485,26 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (lay.persistent) {
                     if (lane >= left) return;
                     dst += (size_t)lane * pitch;
-                    if (ROW % 32 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 31u) == 0) {
+                    const uint32_t odd = (uint32_t)reinterpret_cast<uintptr_t>(dst) & 31u;
+                    if constexpr (ROW == 40) {               // 8 + 16 + 16 or 16 + 16 + 8 bytes
+                        const uint2 *w2 = reinterpret_cast<const uint2*>(w);
+                        if (odd & 8u) {
+                            *reinterpret_cast<uint2*>(dst) = w2[0];
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) reinterpret_cast<uint4*>(dst + 8)[i] = make_uint4(w[2 + 4 * i], w[3 + 4 * i], w[4 + 4 * i], w[5 + 4 * i]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) reinterpret_cast<uint4*>(dst)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+                            *reinterpret_cast<uint2*>(dst + 32) = w2[4];
+                        }
+                    } else if (odd == 0) {
 #pragma unroll
                         for (int i = 0; i < ROW / 32; ++i) ptx::store_32b(dst + i * 32, w + i * 8);
+                        if constexpr (ROW % 32 == 16) *reinterpret_cast<uint4*>(dst + ROW - 16) = *reinterpret_cast<const uint4*>(w + ROW / 4 - 4);
+                    } else if (odd == 16 && ROW % 32 == 16) {
+                        *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(w);
+#pragma unroll
+                        for (int i = 0; i < ROW / 32; ++i) ptx::store_32b(dst + 16 + i * 32, w + 4 + i * 8);
                     } else {
 #pragma unroll
                         for (int i = 0; i < N; ++i) reinterpret_cast<V*>(dst)[i] = reinterpret_cast<const V*>(w)[i];
@@ -512,57 +535,51 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int c = 0; c < HC; ++c) w[c] = __float_as_uint(y[c]);
                 put(w, std::integral_constant<int, HC * 4>{});
             } else {
-                // Per-(row, head) symmetric int8.  A thread's columns are whole heads (two of 40, or one), or half of what the row
-                // has of a head in this tile.
+                // Per-(row, head) symmetric int8.  A thread's columns are one head or a half or a quarter of one.
                 const int d = a.n_out / a.heads;
                 const int colg = col0 + cb;
                 const int h0 = colg / d;
-                constexpr int SPLIT_AT = HC == 80 ? 40 : HC;  // two heads of 40: columns 0..39 are head h0, the rest h0 + 1
-                const bool two = HC == 80 && d == 40;
-                float am0 = 0.f, am1 = 0.f;
+                float am = 0.f;
 #pragma unroll
-                for (int c = 0; c < HC; ++c) { if (c < SPLIT_AT) am0 = fmaxf(am0, fabsf(y[c])); else am1 = fmaxf(am1, fabsf(y[c])); }
-                if (!two) { am0 = fmaxf(am0, am1); am1 = am0; }
-                if (d > HC) {
-                    float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [2][128]
-                    xc[cg * 128 + r] = am0;
-                    asm volatile("bar.sync %0, 64;" ::"r"(2 + q) : "memory");
-                    am0 = fmaxf(am0, xc[(cg ^ 1) * 128 + r]);
+                for (int c = 0; c < HC; ++c) am = fmaxf(am, fabsf(y[c]));
+                if (d > HC) {                                // the row's threads with columns of the same head combine their absmax
+                    float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [NCG][128], and of a head pair [128] out, [128] in
+                    const int per_head = min(NCG, d / HC), first = cg / per_head * per_head;
+                    xc[cg * 128 + r] = am;
+                    asm volatile("bar.sync %0, %1;" ::"r"(2 + q), "n"(NCG * 32) : "memory");
+#pragma unroll
+                    for (int k = 0; k < NCG; ++k) if (k < per_head) am = fmaxf(am, xc[(first + k) * 128 + r]);
+                    if (lay.persistent) asm volatile("bar.sync %0, %1;" ::"r"(6 + q), "n"(NCG * 32) : "memory");      // (read before the next tile's are written)
                     if (!KV && lay.head_pair && mine) {
                         // The head's other columns belong to a CTA of the same cluster (same rows, same share of the K loop):
                         // each sends its rows' absmax over, one 128-byte copy between the shared memories per 32 rows.
                         const uint32_t me = ptx::cluster_ctarank();
                         const uint32_t other = me < (uint32_t)nsplit ? me + nsplit : me - nsplit;
                         if (cg == 0) {
-                            xc[256 + r] = am0;
+                            xc[256 + r] = am;
                             ptx::fence_proxy_async_smem();
                             __syncwarp();
                             if (lane == 0)
                                 ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(xc + 384 + q * 32), other), xc + 256 + q * 32, 128u, ptx::map_to_cta(ptx::smem_u32(&bars->pair_full[q]), other));
                         }
-                        if (ptx::mbar_wait(&bars->pair_full[q], 0)) am0 = fmaxf(am0, xc[384 + r]);
+                        if (ptx::mbar_wait(&bars->pair_full[q], 0)) am = fmaxf(am, xc[384 + r]);
                         else give_up();
                         __syncwarp();
                     }
-                    am1 = am0;
                 }
                 const float qmax = KV && a.kv_qmax ? (float)a.kv_qmax : 127.f;
-                const float s0 = quant_scale(am0, qmax), s1 = two ? quant_scale(am1, qmax) : s0;
-                const float r0 = s0 > 0.f ? __frcp_rn(s0) : 0.f, r1 = s1 > 0.f ? __frcp_rn(s1) : 0.f;
+                const float s = quant_scale(am, qmax), rs = s > 0.f ? __frcp_rn(s) : 0.f;
+                const bool owner = colg == h0 * d;           // holds the head's first column: writes its scale
                 if constexpr (!KV) {
                     // Q~ = Q_a(Q), Eq. 2 third line
                     alignas(16) uint32_t w[HC / 4];
 #pragma unroll
                     for (int c = 0; c < HC; c += 8) {
-                        const uint2 code = quant8(y + c, c < SPLIT_AT ? r0 : r1);
+                        const uint2 code = quant8(y + c, rs);
                         w[c / 4] = code.x; w[c / 4 + 1] = code.y;
                     }
                     put(w, std::integral_constant<int, HC>{});
-                    if (live) {
-                        float* sc = a.scales + ((size_t)z * a.rows + row) * a.heads;
-                        if (colg == h0 * d) sc[h0] = s0;
-                        if (two) sc[h0 + 1] = s1;
-                    }
+                    if (live && owner) a.scales[((size_t)z * a.rows + row) * a.heads + h0] = s;
                 } else {
                     // Eq. 2 for K or V of one sequence (a row tile is one sequence; rows beyond its T tokens are the padding keys of
                     // the images): rows of ordinary tokens -> int8 codes + scale, rows of trigger tokens -> fp16; and the same
@@ -570,7 +587,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     // that were not written here): K~ as a row of fp16 integers, V~ as a column of fp16(code * scale).  The
                     // fp32 tile goes through shared memory to kv_store below.
                     const int T = a.n_ctx;
-                    const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 256;      // [128] and the bitmap [4], by the scales' warps
+                    const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;      // [128] and the bitmap [4], by the scales' warps
                     const taq_kv_layout KL = kv_layout(a.heads, T, d, a.max_trigger);
                     uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * KL.block_bytes;
                     OperandGeom G;
@@ -584,18 +601,14 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                         for (int c = 0; c < HC; ++c) ys[r * KV_STRIDE + cb + c] = y[c];
                         const float logit_unit = 1.4426950408889634f / sqrtf((float)d);
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            if (k == 1 && !two) break;
-                            const int h = h0 + k;
-                            const float s = plain ? (k ? s1 : s0) : 0.f;
-                            if (k == 0 && colg != h * d) continue;           // the head's first column is another thread's (or CTA's)
-                            hs[(h - head0) * 128 + r] = make_float2(s, plain ? (k ? r1 : r0) : 0.f);
-                            if (r < T) reinterpret_cast<float*>(blk + (kv_which ? KL.off_v_scales : KL.off_k_scales))[(size_t)h * T + r] = s;
-                            if (!kv_which && h == 0) reinterpret_cast<int32_t*>(blk + KL.off_trig_slot)[r] = slot >= 0 ? slot : -1;
+                        if (owner) {
+                            const float sk = plain ? s : 0.f;
+                            hs[(h0 - head0) * 128 + r] = make_float2(sk, plain ? rs : 0.f);
+                            if (r < T) reinterpret_cast<float*>(blk + (kv_which ? KL.off_v_scales : KL.off_k_scales))[(size_t)h0 * T + r] = sk;
+                            if (!kv_which && h0 == 0) reinterpret_cast<int32_t*>(blk + KL.off_trig_slot)[r] = slot >= 0 ? slot : -1;
                             if (!kv_which && images && r < kOperandKeys) {
-                                OperandConsts* cst = reinterpret_cast<OperandConsts*>(blk + KL.off_operands + (size_t)h * G.head_bytes + G.k_bytes + G.vt_bytes);
-                                cst->logit_factor[r] = (slot >= 0 ? 1.0f : s) * logit_unit;
+                                OperandConsts* cst = reinterpret_cast<OperandConsts*>(blk + KL.off_operands + (size_t)h0 * G.head_bytes + G.k_bytes + G.vt_bytes);
+                                cst->logit_factor[r] = (slot >= 0 ? 1.0f : sk) * logit_unit;
                                 if (r < 4) cst->trig_bits[r] = (uint32_t)slots[128 + r];
                             }
                         }
@@ -618,11 +631,12 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // of a tile row hit all banks.
         constexpr int CB = (int)sizeof(CodeT);
         const int c16 = bt & 15, n0 = bt >> 4;
-        const uint32_t row_step = (uint32_t)(TL::NBUILD / 2 / 16) * lay.row_bytes;
+        const uint32_t row_step = (uint32_t)(TL::NBUILD / 32) * lay.row_bytes;
         const int n_pair = (n_kb + 1) / 2;
-        // Codes are fetched one turn ahead, across tile boundaries: all of a pair's chunks where they take at most ten registers
-        // (more would spill), else half of them, the rest when they are needed.
-        constexpr int NPRE = NCH * (CB / 4) <= 10 ? NCH : (NCH + 1) / 2;
+        // Codes are fetched one turn ahead, across tile boundaries: as many of a pair's chunks as twenty registers hold (more would
+        // spill), the rest when they are needed.
+        constexpr int NPRE = NCH * (CB / 4) <= 20 ? NCH : NCH * (CB / 4) <= 40 ? NCH / 2 : NCH / 4;
+        static_assert(NCH % NPRE == 0, "rounds");
         CodeT pw[NPRE];
         const uint8_t* src = nullptr;                        // codes of the fetched pair
         int tile = tile0, pair = group;                      // the fetched pair
@@ -657,11 +671,12 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             if (c16 < 8 || 2 * pair + 1 < n_kb) {
 #pragma unroll
                 for (int j = 0; j < NPRE; ++j) *reinterpret_cast<uint4*>(tile_b + ptx::sw128_offset(n0 + j * (TL::NBUILD / 32), c16 & 7)) = expand_chunk<I8, W8>(pw[j]);
-                if constexpr (NPRE < NCH) {
 #pragma unroll
-                    for (int j = NPRE; j < NCH; ++j) pw[j - NPRE] = load(j);
+                for (int j0 = NPRE; j0 < NCH; j0 += NPRE) {
 #pragma unroll
-                    for (int j = NPRE; j < NCH; ++j) *reinterpret_cast<uint4*>(tile_b + ptx::sw128_offset(n0 + j * (TL::NBUILD / 32), c16 & 7)) = expand_chunk<I8, W8>(pw[j - NPRE]);
+                    for (int j = 0; j < NPRE; ++j) pw[j] = load(j0 + j);
+#pragma unroll
+                    for (int j = 0; j < NPRE; ++j) *reinterpret_cast<uint4*>(tile_b + ptx::sw128_offset(n0 + (j0 + j) * (TL::NBUILD / 32), c16 & 7)) = expand_chunk<I8, W8>(pw[j]);
                 }
             }
             if (bt == 0 && pair < 10) TAQ_PROF(60 + 2 * pair);
@@ -790,7 +805,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (KV && warp == TL::W_AUX) {               // (the mask may come from the previous kernel) slot of every token of the sequence among its trigger tokens, and their bitmap
                     ptx::pdl_wait();
                     const uint8_t* mask = a.reqs ? a.reqs[z].trig_mask : a.mask + (size_t)z * a.n_ctx;
-                    int* slots = reinterpret_cast<int*>(smem + P.off_xchg) + 256;
+                    int* slots = reinterpret_cast<int*>(smem + P.off_xchg) + 512;
                     int before = 0;
                     for (int k = 0; k < 4; ++k) {
                         const int t = 32 * k + lane;
