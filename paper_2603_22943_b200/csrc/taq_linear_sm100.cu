@@ -3,6 +3,7 @@
 #include "taq_prof.cuh"
 TAQ_PROF_DEFINE(linear)
 #include "taq_linear_sm100.cuh"
+#include <algorithm>
 
 namespace taq {
 
@@ -75,8 +76,7 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
     } else if (nsplit == 1) {
         staged = tile_bytes;
     } else {
-        const int send = (TL::NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024;         // (as many pieces come in as go out)
-        staged = 2 * send > send + tile_bytes ? 2 * send : send + tile_bytes;
+        staged = std::max(TL::NCG * (4 - 4 / nsplit) * TL::PIECE, tile_bytes);                  // (the pieces of the other CTAs, then the output)
     }
     int nsa = n_pair < 2 ? 1 : 2, nsb = n_pair < 2 ? 1 : 2;
     while (make_plan<BN>(p.n_groups, nsa, nsb, persistent).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
@@ -131,8 +131,9 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
         c.grid = (int)ctas;
         return c;
     };
-    // Heads of 160 channels in a launch of few rows: two 80-wide tiles per head whose CTAs exchange the rows' absmax.
-    if (a.epi == EPI_Q8_HEAD && p.d == 160 && !p.i8 && !a.reqs && a.bits == 4 && p.n_groups >= 2) {
+    // Heads of 160 channels in a launch of few rows: two 80-wide tiles per head whose CTAs exchange the rows' absmax, the K loop in
+    // halves (with integer activations: halves of the scale groups).
+    if (a.epi == EPI_Q8_HEAD && p.d == 160 && a.bits == 4 && (p.n_groups >= 2 || (!p.i8 && p.n_kb >= 2))) {
         const long long tiles = p.row_tiles * (a.n_out / 80) * (long long)n_z;
         Choice c{};
         if (tiles * 2 <= 148 && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);

@@ -73,8 +73,7 @@ struct Tile {
     static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 to 8
     static constexpr int B_TILE = BN * 128;                                   // one k-block
     static constexpr int NCH = BN * 16 / (NBUILD / 2);                        // 16-byte tile chunks per builder thread and pair of k-blocks
-    static constexpr int PART_ROW = HC * 4 + 16;                              // a thread's partial sums in transit, padded against bank conflicts
-    static constexpr int PIECE = 32 * PART_ROW;                               // ... of one warp
+    static constexpr int PIECE = 32 * HC * 4;                                 // a warp's partial sums in transit
     static_assert(BN * 16 % (NBUILD / 2) == 0 && HC % 8 == 0 && NSLOT <= MAX_SLOT && NSLOT >= 3, "tile shape");
 };
 
@@ -158,7 +157,7 @@ enum class Ctas { ONE, MANY, SPLIT };    // a tile per CTA; several tiles per CT
 // Out::KV: the K and the V projection are one launch: the first half of the column tiles is K's.
 // Ctas::SPLIT: for launches with few tiles and a long K loop, two or four CTAs (a cluster) share one output tile: each
 // takes a share of the scale groups (of the k-blocks, when there is one group); then they exchange folded fp32 partial sums
-// through bulk copies between the shared memories, every CTA adding and storing its share of the tile's rows.
+// through stores into each other's shared memory, every CTA adding and storing its share of the tile's rows.
 template <int BN, bool I8, bool W8, Out OUT, Ctas CTAS>
 __global__ void __launch_bounds__(Tile<BN>::NTHREADS, 1)
 linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ LinearArgs a, const __grid_constant__ LinearLayout lay) {
@@ -248,7 +247,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // over 8-element chunks, neighbouring lanes on neighbouring chunks, write everything in runs.  (With a row per lane straight
     // from the registers this epilogue took 15 000 - 24 000 cycles: 32 sectors per store, 20 KB of unrolled code that runs
     // once.  With the eight folder warps alone these loops took 9 000: two warps on a scheduler hide no latency.)
-    const int kv_staging_off = clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0;
     constexpr int KV_STRIDE = BN + 1;                        // floats (odd: a row per lane is free of bank conflicts)
     auto kv_store = [&](int w) {
         constexpr int NT = TL::NFOLD + TL::NBUILD, NC8 = BN / 8;
@@ -261,8 +259,8 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         const bool images = operand_geom(d, T, &G);
         uint8_t* img0 = blk + KL.off_operands + (size_t)head0 * G.head_bytes;
         const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;
-        const float* ys = reinterpret_cast<const float*>(smem + kv_staging_off);
-        const float2* hs = reinterpret_cast<const float2*>(smem + kv_staging_off + 128 * KV_STRIDE * 4);
+        const float* ys = reinterpret_cast<const float*>(smem);
+        const float2* hs = reinterpret_cast<const float2*>(smem + 128 * KV_STRIDE * 4);
         const int own_shift = nsplit == 1 ? 7 : nsplit == 2 ? 6 : 5;         // (CTAs that share the tile finish the rows of some lane quarters each)
         auto own = [&](int key) { return key >> own_shift == rank; };
         {                                                    // codes, trigger rows and K~'s image: 8 channels of a token
@@ -342,10 +340,12 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         const int cb = cg * HC;                              // first owned column inside the tile
         int slot = 0, sbuf = 0;
         uint32_t ph_acc = 0, ph_scale = 0;
-        bool joined = false;                                 // has waited for the cluster's first barrier
         bool alive = true;                                   // no wait has run out (a warp skips work then, never a barrier)
         uint32_t tmem_base = 0;
         if (ptx::mbar_wait(&bars->tmem_ready, 0)) tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base); else give_up();
+        ptx::pdl_wait();                                     // (nothing to fold before the activations have come anyway) orders the stores below
+        __syncwarp();
+        if (clustered) ptx::cluster_wait();                  // the other CTAs' barriers exist
         for (int tile = tile0; tile < lay.n_tiles; tile += tile_step) {
             int z, row0, col0, kv_which;
             tile_of(tile, z, row0, col0, kv_which);
@@ -400,7 +400,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (++slot == NSLOT) { slot = 0; ph_acc ^= 1; }
             }
             if (!ok && alive) { give_up(); alive = false; }
-            if (tile == tile0) ptx::pdl_wait();              // (already satisfied: the activations have arrived) orders the stores below
             if (ft == 0) TAQ_PROF(7);
             if (!I8 && lane == 0) ptx::mbar_arrive(&bars->scale_free[sbuf]);     // scales and biases of this tile have been read
 
@@ -410,61 +409,54 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
             bool mine = alive;                               // this CTA finishes the warp's rows
             if (clustered) {
-                // All of this CTA's MMAs are complete (every group was folded), so its rings are free: they hold the partial
-                // sums in transit.  CTA `owner` of the cluster finishes the rows of 4 / nsplit lane quarters: a folder warp
-                // either hands its 32 rows to that CTA (one bulk copy between the shared memories) or receives a piece from
-                // every other CTA and adds them in rank order, so that every output is the same sum whoever computes it.
+                // All of this CTA's MMAs are complete (every group was folded), so its rings are free: they take the partial sums that
+                // come in.  CTA `owner` of the cluster finishes the rows of 4 / nsplit lane quarters: a folder warp either
+                // stores its 32 rows into that CTA's shared memory, straight from the registers (16 bytes a lane, the lanes
+                // of a store next to each other, no staging, no bank conflicts), or receives a piece from every other CTA and
+                // adds them in rank order, so that every output is the same sum whoever computes it.
                 const int per_cta = 4 / nsplit, owner = q / per_cta;
                 const uint32_t base = ptx::cluster_ctarank() - (uint32_t)rank;        // ranks along x are consecutive
                 mine = alive && owner == rank;
-                ptx::cluster_wait();                         // the other CTAs' barriers exist
-                joined = true;
                 if (ft < nsplit && ft != rank) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), base + (uint32_t)ft));
-                const int n_send = NCG * (4 - per_cta);
+                auto piece = [&](int cta, int from) { return smem + ((cg * per_cta + q - cta * per_cta) * (nsplit - 1) + (from < cta ? from : from - 1)) * TL::PIECE + lane * 16; };
                 if (owner != rank) {
-                    unsigned char* piece = smem + (cg * (4 - per_cta) + (q < rank * per_cta ? q : q - per_cta)) * TL::PIECE;
-                    float* out = reinterpret_cast<float*>(piece + lane * TL::PART_ROW);
+                    if (alive && ptx::mbar_wait(&bars->peer_ready, 0)) {                 // the other CTAs' rings are free, too
+                        const uint32_t dst = ptx::map_to_cta(ptx::smem_u32(piece(owner, rank)), base + (uint32_t)owner);
+                        const uint32_t bar = ptx::map_to_cta(ptx::smem_u32(&bars->part_full[fw]), base + (uint32_t)owner);
 #pragma unroll
-                    for (int c = 0; c < HC; c += 4) *reinterpret_cast<float4*>(out + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
-                    ptx::fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-                        if (ptx::mbar_wait(&bars->peer_ready, 0)) {                      // the other CTAs' rings are free, too
-                            const int src_idx = rank < owner ? rank : rank - 1;
-                            const int dst = (n_send + (cg * per_cta + q - owner * per_cta) * (nsplit - 1) + src_idx) * TL::PIECE;
-                            ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(smem + dst), base + (uint32_t)owner), piece, (uint32_t)TL::PIECE,
-                                                  ptx::map_to_cta(ptx::smem_u32(&bars->part_full[fw]), base + (uint32_t)owner));
-                        } else give_up();
-                    }
+                        for (int c = 0; c < HC; c += 4)
+                            ptx::store_to_cta(dst + c * 128, __float_as_uint(y[c]), __float_as_uint(y[c + 1]), __float_as_uint(y[c + 2]), __float_as_uint(y[c + 3]), bar);
+                    } else give_up();
                 } else if (!ptx::mbar_wait(&bars->part_full[fw], 0)) {
                     give_up();
                 } else {
-                    const unsigned char* in = smem + (n_send + (cg * per_cta + q - rank * per_cta) * (nsplit - 1)) * TL::PIECE + lane * TL::PART_ROW;
+                    const unsigned char* in = smem + (cg * per_cta + q - rank * per_cta) * (nsplit - 1) * TL::PIECE + lane * 16;
                     if (nsplit == 2) {
 #pragma unroll
                         for (int c = 0; c < HC; c += 4) {
-                            const float4 p4 = *reinterpret_cast<const float4*>(in + c * 4);
+                            const float4 p4 = *reinterpret_cast<const float4*>(in + c * 128);
                             y[c] += p4.x; y[c + 1] += p4.y; y[c + 2] += p4.z; y[c + 3] += p4.w;
                         }
                     } else {
-                        // rank order: ((p0 + p1) + p2) + p3, this CTA's own sum in its place
+                        // rank order, ((p0 + p1) + p2) + p3, with this CTA's own sum in its place (o: the others')
+                        auto sum4 = [&](float own, float o0, float o1, float o2) {
+                            const float s01 = o0 + (rank <= 1 ? own : o1);
+                            return (s01 + (rank <= 1 ? o1 : rank == 2 ? own : o2)) + (rank == 3 ? own : o2);
+                        };
 #pragma unroll
                         for (int c = 0; c < HC; c += 4) {
-                            float4 p[4];
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                p[k] = k == rank ? make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]) : *reinterpret_cast<const float4*>(in + (k < rank ? k : k - 1) * TL::PIECE + c * 4);
-                            y[c] = ((p[0].x + p[1].x) + p[2].x) + p[3].x; y[c + 1] = ((p[0].y + p[1].y) + p[2].y) + p[3].y;
-                            y[c + 2] = ((p[0].z + p[1].z) + p[2].z) + p[3].z; y[c + 3] = ((p[0].w + p[1].w) + p[2].w) + p[3].w;
+                            const float4 o0 = *reinterpret_cast<const float4*>(in + c * 128), o1 = *reinterpret_cast<const float4*>(in + TL::PIECE + c * 128),
+                                         o2 = *reinterpret_cast<const float4*>(in + 2 * TL::PIECE + c * 128);
+                            y[c] = sum4(y[c], o0.x, o1.x, o2.x); y[c + 1] = sum4(y[c + 1], o0.y, o1.y, o2.y);
+                            y[c + 2] = sum4(y[c + 2], o0.z, o1.z, o2.z); y[c + 3] = sum4(y[c + 3], o0.w, o1.w, o2.w);
                         }
                     }
                 }
-                asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");     // pieces read: the epilogue stages output where they were ...
+                asm volatile("bar.sync 1, %0;" ::"n"(TL::NFOLD) : "memory");     // pieces read: the epilogue stages output where they were
                 if (ft == 0) TAQ_PROF(10);
                 mine = mine && !bars->abort_flag;
             }
-            // ... but not over this CTA's outgoing pieces, which may still be in flight: the staging area begins behind them
-            unsigned char* staging = smem + (clustered ? (NCG * (4 - 4 / nsplit) * TL::PIECE + 1023) / 1024 * 1024 : 0);
+            unsigned char* staging = smem;
 
             const long long row = (long long)row0 + r;
             const bool live = mine && row < a.rows;
@@ -560,16 +552,10 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     if (persistent) asm volatile("bar.sync %0, %1;" ::"r"(6 + q), "n"(NCG * 32) : "memory");      // (read before the next tile's are written)
                     if (!KV && lay.head_pair && mine) {
                         // The head's other columns belong to a CTA of the same cluster (same rows, same share of the K loop):
-                        // each sends its rows' absmax over, one 128-byte copy between the shared memories per 32 rows.
+                        // each sends its rows' absmax over.
                         const uint32_t me = ptx::cluster_ctarank();
                         const uint32_t other = me < (uint32_t)nsplit ? me + nsplit : me - nsplit;
-                        if (cg == 0) {
-                            xc[256 + r] = am;
-                            ptx::fence_proxy_async_smem();
-                            __syncwarp();
-                            if (lane == 0)
-                                ptx::bulk_copy_to_cta(ptx::map_to_cta(ptx::smem_u32(xc + 384 + q * 32), other), xc + 256 + q * 32, 128u, ptx::map_to_cta(ptx::smem_u32(&bars->pair_full[q]), other));
-                        }
+                        if (cg == 0) ptx::store_to_cta(ptx::map_to_cta(ptx::smem_u32(xc + 384 + r), other), __float_as_uint(am), ptx::map_to_cta(ptx::smem_u32(&bars->pair_full[q]), other));
                         if (ptx::mbar_wait(&bars->pair_full[q], 0)) am = fmaxf(am, xc[384 + r]);
                         else give_up();
                         __syncwarp();
@@ -628,7 +614,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         __syncwarp();
         if constexpr (KV) kv_together(true, ft);
-        if (clustered && !joined) ptx::cluster_wait();
     } else if (warp >= TL::W_BUILD && warp < TL::W_BUILD + TL::NB) {
         // ---------------- builders ----------------
         const int bt = (tid - 32 * TL::W_BUILD) & (TL::NBUILD / 2 - 1), group = (warp - TL::W_BUILD) / (TL::NB / 2);
@@ -859,6 +844,9 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     }
 }
 
+// (Of this file's tile width.  Not a static of the template: such a variable is one for all copies of the library in a process.)
+static std::atomic<unsigned long long> limit_set[48];
+
 template <int BN>
 cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const LinearLayout& lay, int grid, size_t smem_bytes, cudaStream_t stream) {
     using TL = Tile<BN>;
@@ -878,7 +866,6 @@ cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const Line
     };
     const Kernel kern = a.epi == EPI_KV ? of_out(std::integral_constant<Out, Out::KV>{}) : a.epi == EPI_Q8_HEAD ? of_out(std::integral_constant<Out, Out::Q8>{}) :
                         a.epi == EPI_F32 ? of_out(std::integral_constant<Out, Out::F32>{}) : of_out(std::integral_constant<Out, Out::F16>{});
-    static std::atomic<unsigned long long> limit_set[48];
     cudaError_t e = allow_shared_memory((const void*)kern, SMEM_LIMIT, limit_set[(a.epi * 3 + (int)ctas) * 4 + i8 * 2 + w8]);
     if (e != cudaSuccess) return e;
     if (lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(grid), dim3(lay.nsplit * (lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), smem_bytes, stream, tmap, a, lay);
