@@ -118,9 +118,18 @@ bool tile_carries(const LinearArgs& a, const Problem& p, int bn) {
     return false;
 }
 
-// The cheapest layout by a small model of a CTA's life in SM cycles: a fixed part (launch, barriers, first loads, epilogue), the K
-// loop at the pace of the tensor core, and the exchange of partial sums when the loop is split; a persistent CTA pays
-// the fixed part once and the K loop per tile.
+// The cheapest layout by a small model, in microseconds: a fixed part (launch, barriers, first loads, epilogue), the K loop per k-block
+// and scale group, what a tile costs a CTA that walks several, and the exchange of partial sums when the K loop is split (a
+// part that grows with the CTAs that exchange at one time).  The numbers are a least-squares fit to 351 measured launches of
+// 64 to 8192 rows, 640 and 1280 channels, W4 and W8, every width and split that can carry them (5 % rms); the layouts it picks
+// are on average 0.5 % slower than the best one measured.
+struct Pace { int bn; double fixed, kb, group, tile, q8, split, exchange; };
+constexpr Pace PACES[4] = {
+    {160, 3.08, 0.320, 0.248, 1.54, 0.72, 0.95, 1.72},
+    {128, 3.17, 0.274, 0.150, 0.49, 0.05, 1.30, 1.66},
+    {80, 2.49, 0.200, 0.131, 0.52, 0.35, 1.05, 1.04},
+    {64, 2.56, 0.192, 0.106, 0.24, 0.18, 1.00, 0.87},
+};
 Choice choose_anew(const LinearArgs& a, int n_z) {
     const Problem p = problem_of(a);
     Choice best{};
@@ -139,19 +148,26 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
         if (tiles * 2 <= 148 && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);
     }
     double best_cost = 1e30;
-    for (int bn : {160, 128, 80, 64}) {
+    for (const Pace& m : PACES) {
+        const int bn = m.bn;
         if (!tile_carries(a, p, bn)) continue;
         const long long tiles = p.row_tiles * (a.n_out / bn) * p.ncols_factor * (long long)n_z;
         if (tiles > (1 << 30)) continue;
-        const double kb = bn == 160 ? 380 : bn == 128 ? 340 : 260;
         for (int ns : {1, 2, 4}) {
+            // (K~/V~ of a 768-wide context gain nothing from a split, which leaves a prompt's bits the same in every batch; of a
+            // 2048-wide one a split takes 13.9 us to 10.2 us at C = 640.)
+            if (ns > 1 && a.epi == EPI_KV && a.k_in < 1024) continue;
             if (ns > 1 && ((p.i8 && p.n_groups == 1) || (p.n_groups == 1 ? p.n_kb : p.n_groups) < ns || tiles * ns > 148)) continue;    // (integer activations: a group's sum stays one exact int32 accumulation)
             const bool persistent = a.epi != EPI_KV && tiles * ns > 148;           // (K~/V~ tiles are assembled in the rings: one per CTA)
             Choice c{};
             if (!rings_of(a, p, bn, ns, 0, persistent, c)) continue;
             const long long per = (tiles * ns + 147) / 148;                                            // tiles per CTA
             const long long ctas = persistent ? (tiles + per - 1) / per : tiles * ns;
-            const double cost = (persistent ? 1 : per) * (5000 + bn * (a.epi == EPI_KV ? 20 : 5)) + (double)per * (share_of(p, ns) * kb + (persistent ? 300 : 0)) + (ns > 1 ? 1000 + 300 * ns : 0);
+            const int share = share_of(p, ns);
+            const double fixed = m.fixed + (a.epi == EPI_KV ? 0.008 * bn : 0), tile = persistent ? m.tile : 0;
+            const double groups = p.n_groups == 1 ? 1 : (double)share * p.n_groups / p.n_kb;
+            const double cost = (persistent ? 1 : per) * fixed + (double)per * (share * m.kb + groups * m.group + tile + (a.epi == EPI_Q8_HEAD ? m.q8 : 0)) +
+                                (ns > 1 ? m.split + 0.1 * (ns - 2) + m.exchange * (ns - 1) * (double)(tiles * ns) / 148 : 0);
             if (cost < best_cost) { best_cost = cost; best = finish(c, tiles, ctas); }
         }
     }
