@@ -1,0 +1,63 @@
+"""The kernels' branches at the sizes where they can go wrong: every tile width of the dequant-GEMM with one tile per CTA, several
+tiles per CTA and a cluster per tile, first and last rows of a tile, heads over two tiles; the merged K/V projection at its
+smallest and largest contexts; the packing kernel's group lengths."""
+from dataclasses import replace
+
+import pytest
+
+import test_gpu_layer as layer
+import test_gpu_quantizers as quantizers
+import test_gpu_int8_activations as int8_activations
+from paper_2603_22943_b200 import binding as tb
+from paper_2603_22943_b200 import synth
+import taq_testlib as tl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads", [
+    (1, 640, 640, 4, 128, 8),          # one row, 80-wide tiles
+    (129, 640, 640, 8, 0, 10),         # a second row tile of one row, 64-wide tiles
+    (2047, 640, 640, 4, 128, 10),      # 128-wide tiles, one per CTA
+    (5616, 640, 640, 4, 128, 10),      # ... and several per CTA
+    (5505, 640, 640, 8, 0, 8),         # 80-wide tiles, several per CTA, a last row tile of one row
+    (4225, 640, 640, 4, 128, 8),       # 160-wide tiles, several per CTA
+    (64, 1280, 1280, 4, 128, 20),      # a cluster per 64-wide tile, shares of whole groups
+    (300, 1280, 1280, 8, 0, 20),       # ... and of k-blocks
+    (129, 1280, 1280, 4, 0, 8),        # heads over two tiles, shares of k-blocks
+    (129, 1280, 1280, 8, 0, 8),        # a cluster per 160-wide tile
+    (1100, 1280, 1280, 8, 0, 8),       # 160-wide tiles, one per CTA
+    (97, 320, 192, 4, 128, 8),         # an odd number of k-blocks, a short last group
+    (200, 320, 64, 8, 0, 8),           # one k-block
+])
+def test_linear_tiles(rows, n_out, k_in, bits, group, heads):
+    for kind in (tb.TAQ_OUT_F16, tb.TAQ_OUT_F32, tb.TAQ_OUT_INT8_HEAD_ROWS):
+        assert tb.taq_linear_plan(tb.weight_desc(n_out, k_in, bits, group), rows, kind, heads=heads)["bn"] > 0
+    layer.test_quantized_linear(rows, n_out, k_in, bits, group, heads)
+
+
+@pytest.mark.parametrize("rows,k_in,n_out,bits,group", [
+    (1, 320, 320, 4, 128), (257, 1280, 1280, 4, 128), (4225, 640, 640, 4, 128), (300, 656, 640, 8, 0),
+])
+def test_integer_linear_tiles(rows, k_in, n_out, bits, group):
+    int8_activations.test_integer_gemm_equals_the_integer_definition(rows, k_in, n_out, bits, group)
+
+
+@pytest.mark.parametrize("channels,heads,ctx_dim,n_ctx,batch,w_bits", [
+    (320, 8, 768, 9, 1, 4), (320, 8, 768, 80, 3, 8), (640, 8, 768, 77, 2, 4), (640, 10, 2048, 20, 1, 4),
+    (1280, 20, 2048, 77, 1, 8), (1280, 8, 768, 64, 2, 8), (640, 10, 2048, 77, 9, 4),
+])
+def test_kv_projection(channels, heads, ctx_dim, n_ctx, batch, w_bits):
+    shape = replace(synth.config1(), batch=batch, channels=channels, heads=heads, ctx_dim=ctx_dim, n_ctx=n_ctx, w_bits=w_bits, w_group=128 if w_bits == 4 else 0,
+                    trigger=(1, n_ctx - 1), n_query=130, name=f"edge_{channels}_{heads}_{ctx_dim}_{n_ctx}")
+    layer.test_kv_project(shape)
+    data = synth.make_layer(shape)
+    y, parts = tl.gpu_layer(shape, data, return_parts=True)          # reads the operand images that the projection left
+    tl.check_layer(shape, data, y, parts)
+
+
+@pytest.mark.parametrize("n_out,k_in,bits,group", [
+    (40, 512, 4, 256), (24, 1024, 4, 512), (16, 2560, 8, 0), (9, 136, 8, 0), (33, 352, 4, 32), (7, 1000, 4, 128), (5, 2560, 4, 0),
+])
+def test_pack_group_lengths(n_out, k_in, bits, group):
+    quantizers.test_pack_weights_codes_bit_exact(n_out, k_in, bits, group)
