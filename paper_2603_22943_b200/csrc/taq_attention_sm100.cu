@@ -17,6 +17,7 @@
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
 #include "taq_sm100_parts.cuh"
+#include <algorithm>
 #include <cstddef>
 #include <cstring>
 
@@ -120,7 +121,7 @@ struct QRegs {
 };
 
 template <int D, bool Q8, bool TAIL_ONLY>
-__global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a, const int heads_per_cta) {
+__global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a) {
     using C = Cfg<D>;
     constexpr int DP = C::DP;
     extern __shared__ unsigned char smem_dyn[];
@@ -132,8 +133,8 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
     const int zb = blockIdx.z;
     const int b = a.reqs ? 0 : zb;
     const int row0 = blockIdx.x * ROWS;
-    const int h_begin = blockIdx.y * heads_per_cta;
-    const int HG = heads_per_cta;
+    const int h_begin = H * (int)blockIdx.y / (int)gridDim.y;         // the heads dealt out as evenly as they go
+    const int HG = H * ((int)blockIdx.y + 1) / (int)gridDim.y - h_begin;
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(126); }
@@ -585,23 +586,21 @@ EncodeTiledFn encode_tiled_fn3() {
     return fn;
 }
 
+// CTAs per row tile, among which the heads are dealt out: the number with the shortest estimated time, in units of a head: a CTA's
+// heads and its start and end (two heads' time; where two CTAs share an SM the second one hides most of it), times the waves.
+// A partial last wave of two CTAs per SM costs less than a full one.  (Measured, 64 row tiles x 10 heads of 64: five CTAs of
+// two heads each, 320 in two waves, 17.4 us; four of two or three heads, one wave, 14.9.  45 tiles x 8 heads of 80: two CTAs
+// of four heads 11.5 us, three of two or three 9.4.)
 template <int D>
-int pick_heads_per_cta(const AttnArgs& a, int n_z) {
-    // One CTA per SM: the head group with the shortest estimated time, a CTA's start and end counted as two heads and a last wave in
-    // full (180 CTAs of two heads take longer than 90 of four).  Two CTAs per SM: the largest group that still fills the
-    // places to about three quarters (there the second CTA of an SM hides the first one's gaps, and fewer, longer CTAs lose).
+int pick_head_groups(const AttnArgs& a, int n_z) {
     const long long tiles = (long long)((a.n_query + ROWS - 1) / ROWS) * n_z;
     int best = 1;
     double best_cost = 1e30;
-    for (int hg = 1; hg <= a.heads; ++hg) {
-        if (a.heads % hg) continue;
-        const long long ctas = tiles * (a.heads / hg);
-        if (Cfg<D>::CTAS_PER_SM == 2) {
-            if (ctas >= 222) best = hg;
-            continue;
-        }
-        const double cost = (double)((ctas + 147) / 148) * (2.0 + hg);
-        if (cost <= best_cost) { best_cost = cost; best = hg; }
+    for (int groups = 1; groups <= a.heads; ++groups) {
+        const long long ctas = tiles * groups, places = 148 * Cfg<D>::CTAS_PER_SM, waves = (ctas + places - 1) / places;
+        const int most = (a.heads + groups - 1) / groups;
+        const double cost = Cfg<D>::CTAS_PER_SM == 2 ? (0.75 * (double)waves + 0.25 * std::max(1.0, (double)ctas / (double)places)) * (0.4 + most) : (double)waves * (2.0 + most);
+        if (cost <= best_cost) { best_cost = cost; best = groups; }
     }
     return best;
 }
@@ -612,8 +611,7 @@ cudaError_t launch_k(const AttnArgs& a, int n_z, cudaStream_t stream) {
     static std::atomic<unsigned long long> limit_set;
     cudaError_t e = allow_shared_memory((const void*)attention_sm100_kernel<D, Q8, TAIL_ONLY>, C::TOTAL, limit_set);
     if (e != cudaSuccess) return e;
-    const int hg = pick_heads_per_cta<D>(a, n_z);
-    dim3 grid((a.n_query + ROWS - 1) / ROWS, a.heads / hg, n_z);
+    dim3 grid((a.n_query + ROWS - 1) / ROWS, pick_head_groups<D>(a, n_z), n_z);
     CUtensorMap tmap_q, tmap_o;
     memset(&tmap_q, 0, sizeof(tmap_q));
     memset(&tmap_o, 0, sizeof(tmap_o));
@@ -630,7 +628,7 @@ cudaError_t launch_k(const AttnArgs& a, int n_z, cudaStream_t stream) {
         if (enc(&tmap_o, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, (void*)a.o, dims, ostr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
-    return launch_pdl(attention_sm100_kernel<D, Q8, TAIL_ONLY>, grid, dim3(ATT_THREADS), (size_t)C::TOTAL, stream, tmap_q, tmap_o, a, hg);
+    return launch_pdl(attention_sm100_kernel<D, Q8, TAIL_ONLY>, grid, dim3(ATT_THREADS), (size_t)C::TOTAL, stream, tmap_q, tmap_o, a);
 }
 
 template <int D>
