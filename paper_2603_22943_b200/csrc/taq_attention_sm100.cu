@@ -12,7 +12,11 @@
 //              by bulk copies, one head ahead: the whole image into the second buffer (head widths up to 64), or,
 //              with a single buffer, K~ as soon as this head's S is complete and V~^T as soon as its PV is.
 // Head widths up to 64: two CTAs share an SM, and the row threads read Q~ and write O themselves.  Head widths 80 and
-// 160: one CTA per SM; Q~ tiles arrive and O tiles leave by TMA through a staging buffer.
+// 160: one CTA per SM; Q~ tiles arrive and O tiles leave by TMA, and from the second head on warps of their own do that work:
+//   warps 12-15  expand the next head's codes (fp16 Q~: load it straight into the operand tile);
+//   warps 16-19  bring the previous head's O from TMEM to global memory.
+// (With the row warps doing everything in turn a head of 160 channels took 5 700 cycles: softmax 1 650, codes 1 100, O 2 250,
+// probabilities 600.)
 #include "taq_prof.cuh"
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
@@ -34,8 +38,11 @@ constexpr int ROW_WARPS = 8;         // two threads per query row
 constexpr int MMA_WARP = 8, COPY_WARP = 9;
 // Three warpgroups: two of row warps, and one of the MMA and copy warps with two idle ones, which gives registers to the rows where
 // two CTAs share an SM (384 threads launched with 80 each = 128 x (2 x 104 + 32); with 96 for everybody the softmax spilled).
-constexpr int ATT_THREADS = 384;
 constexpr int R_ROWS = 104, R_REST = 32;
+// Wide heads: five warpgroups, 640 threads launched with 96 registers each >= 128 x (2 x 128 + 40 + 72 + 104).
+constexpr int Q_WARP = 12, O_WARP = 16;
+constexpr int R_WIDE_ROWS = 128, R_WIDE_REST = 40, R_WIDE_Q = 72, R_WIDE_O = 104;
+static_assert(2 * R_WIDE_ROWS + R_WIDE_REST + R_WIDE_Q + R_WIDE_O <= 5 * 96, "register split");
 
 template <int D>
 struct Cfg {
@@ -48,7 +55,7 @@ struct Cfg {
     static constexpr int VT_BYTES = 2 * VT_BLOCK;
     static constexpr int HEAD_BYTES = K_BYTES + VT_BYTES + kOperandConstBytes;
     static constexpr int KVBUF = D <= 64 ? 2 : 1;            // K~/V~ images in flight
-    static constexpr int OBUF = D == 40 ? 2 : 1;             // O accumulators in TMEM
+    static constexpr int OBUF = D == 64 ? 1 : 2;             // O accumulators in TMEM
     static constexpr int OFF_KV = 0;
     static constexpr int OFF_Q = OFF_KV + KVBUF * HEAD_BYTES;
     static constexpr int OFF_P = OFF_Q + KBQ * A_BLOCK;
@@ -58,15 +65,15 @@ struct Cfg {
     static constexpr bool SPLIT_KV = KVBUF == 1;
     static constexpr int CST_SLOT = 384;
     static constexpr int OFF_CST = OFF_P + 2 * A_BLOCK;
-    // Wide heads move Q~ and O by TMA through one staging buffer (a row's codes or outputs of one head are 80 to 320
+    // Wide heads move Q~ and O by TMA (a row's codes or outputs of one head are 80 to 320
     // bytes at a stride of the whole channel width: per-thread global accesses of that shape keep the load/store
-    // unit busy for longer than the arithmetic takes).  The buffer holds the next head's raw Q~ tile until it has been
-    // expanded into the operand tile, then the previous head's O tile until the store has read it; int8 codes get a
-    // second, smaller buffer, so that their load never waits for the store.
+    // unit busy for longer than the arithmetic takes): O through one staging buffer, int8 codes through a second one, fp16 Q~
+    // straight into the operand tile.
     static constexpr bool TMA_IO = D >= 80;
+    static constexpr int THREADS = TMA_IO ? 640 : 384;
     static constexpr int OFF_U = OFF_CST + (SPLIT_KV ? 3 * CST_SLOT : 0);
-    static constexpr int UO_BYTES = ROWS * D * 2;                  // an O tile, or a raw fp16 Q tile
-    static constexpr int U_BYTES = TMA_IO ? UO_BYTES + ROWS * D : 0; // + a raw int8 Q~ tile, which then has a buffer of its own
+    static constexpr int UO_BYTES = ROWS * D * 2;                  // an O tile
+    static constexpr int U_BYTES = TMA_IO ? UO_BYTES + ROWS * D : 0; // + a raw int8 Q~ tile
     static constexpr int OFF_MISC = OFF_U + U_BYTES;
     static constexpr int TOTAL = OFF_MISC + 4096 + 128 + 1024;   // misc block + slack for 1024-byte alignment
     static constexpr uint32_t TMEM_S = 0, TMEM_O = 2 * TP;
@@ -77,7 +84,7 @@ struct Cfg {
 };
 
 struct Misc {
-    uint64_t kv_full[2], kv_free[2], q_full, s_full[2], p_full, o_full[2], drain, qraw_full;
+    uint64_t kv_full[2], kv_free[2], q_full, s_full[2], p_full, o_full[2], drain, qraw_full, o_free[2], u_free;
     uint32_t tmem_base;
     volatile int abort_flag;
     float2 xchg[2][2][ROWS];     // [head parity][half][row]: (max, sum) of a thread's half of the softmax
@@ -121,7 +128,7 @@ struct QRegs {
 };
 
 template <int D, bool Q8, bool TAIL_ONLY>
-__global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a) {
+__global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a) {
     using C = Cfg<D>;
     constexpr int DP = C::DP;
     extern __shared__ unsigned char smem_dyn[];
@@ -140,7 +147,10 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(126); }
     if (warp == COPY_WARP) {                          // one lane per barrier
         uint64_t* all = misc->kv_full;
-        if (lane < N_BARS) ptx::mbar_init(all + lane, all + lane == &misc->q_full || all + lane == &misc->p_full ? ROW_WARPS : 1);     // (one arrival per row warp)
+        // one arrival per row warp; q_full of an fp16 tile that TMA loads: one; o_free: one per warp of the O warps
+        const uint64_t* bar = all + lane;
+        const int count = bar == &misc->p_full ? ROW_WARPS : bar == &misc->q_full ? (C::TMA_IO && !Q8 ? 1 : ROW_WARPS) : bar == &misc->o_free[0] || bar == &misc->o_free[1] ? 4 : 1;
+        if (lane < N_BARS) ptx::mbar_init(all + lane, (uint32_t)count);
         if (lane == 0) misc->abort_flag = 0;
         ptx::mbar_fence_init();
         if (C::TMA_IO && lane == 0) { ptx::tma_prefetch_desc(&tmap_q); ptx::tma_prefetch_desc(&tmap_o); }
@@ -154,8 +164,114 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
 
     const taq_kv_layout KL = kv_layout(H, T, D, a.max_trigger);
 
+    // Raw tiles of even and odd heads complete barriers of their own: who waits for the second head only must not take the phase
+    // before the first one for it.  (Wide heads have one image buffer, the second kv_free is theirs to use.)
+    auto qraw_full = [&](int hi) { return hi & 1 ? &misc->kv_free[1] : &misc->qraw_full; };
+
     constexpr bool REG_SPLIT = C::CTAS_PER_SM == 2;
-    if (warp >= MMA_WARP) {
+    if (C::TMA_IO && warp >= Q_WARP) {
+        if constexpr (C::TMA_IO) {
+        if (warp < O_WARP) {
+            // ---------------- Q~ of the second head and on ----------------
+            asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_WIDE_Q));
+            bool alive = true;
+            if constexpr (Q8) {
+                // the chunks of the raw tile, dealt out as in stage_q_u below; they are read before S of the head before is
+                // complete (its operand tile is free then), and the raw tile of the head after next lands under all that
+                constexpr int CPR = D / 8, N = ROWS * CPR / 128;
+                const unsigned char* UQ = smem + C::OFF_U + C::UO_BYTES;
+                const int t = tid - 32 * Q_WARP;
+                for (int hi = 1; hi < HG; ++hi) {
+                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(hi), (hi >> 1) & 1));
+                    uint2 raw[N];
+#pragma unroll
+                    for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint2*>(UQ + (size_t)(t + 128 * i) * 8);
+                    asm volatile("bar.sync 6, 128;" ::: "memory");           // the raw tile has been read
+                    if (t == 0 && alive && hi + 1 < HG) {
+                        ptx::mbar_arrive_expect_tx(qraw_full(hi + 1), (uint32_t)(ROWS * D));
+                        ptx::tma_load_3d(smem + C::OFF_U + C::UO_BYTES, &tmap_q, qraw_full(hi + 1), (h_begin + hi + 1) * D, row0, zb);
+                    }
+                    __syncwarp();
+                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[(hi - 1) & 1], ((hi - 1) >> 1) & 1));
+                    if (alive) {
+#pragma unroll
+                        for (int i = 0; i < N; ++i) {
+                            const int j = t + 128 * i, row = j / CPR, cc = j - row * CPR;
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(row, cc & 7)) = codes_w8_to_half(raw[i]);
+                        }
+                        ptx::fence_proxy_async_smem();
+                    }
+                    __syncwarp();
+                    if (alive && lane < ROW_WARPS / 4) ptx::mbar_arrive(&misc->q_full);      // (two lanes of each of four warps: as many as row warps)
+                }
+            } else if (warp == Q_WARP && lane == 0) {
+                // (channels behind the head's last in its last 64-wide block are never multiplied)
+                ptx::pdl_wait();
+                for (int hi = 0; hi < HG && alive; ++hi) {
+                    if (hi > 0) alive = ptx::mbar_wait(&misc->s_full[(hi - 1) & 1], ((hi - 1) >> 1) & 1);
+                    if (!alive) break;
+                    ptx::mbar_arrive_expect_tx(&misc->q_full, (uint32_t)(C::KBQ * C::A_BLOCK));
+                    for (int kb = 0; kb < C::KBQ; ++kb) ptx::tma_load_3d(smem + C::OFF_Q + kb * C::A_BLOCK, &tmap_q, &misc->q_full, (h_begin + hi) * D + kb * 64, row0, zb);
+                }
+            }
+            if (!alive) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
+        } else {
+            // ---------------- O of all heads but the last ----------------
+            asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_WIDE_O));
+            unsigned char* U = smem + C::OFF_U;
+            const int q4 = warp & 3, r = q4 * 32 + lane, t = tid - 32 * O_WARP;
+            const float inv255 = 1.0f / (a.p_log ? 256.0f : a.p_bits == 4 ? 15.0f : 255.0f);
+            bool alive = true;
+            ptx::pdl_wait();
+            for (int hi = 0; hi + 1 < HG; ++hi) {
+                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[hi & 1], (hi >> 1) & 1));
+                if (t == 0) ptx::bulk_store_wait_read();     // (the tile of the head before)
+                __syncwarp();
+                asm volatile("bar.sync 7, 128;" ::: "memory");
+                if (alive) {
+                    ptx::tc_fence_after_sync();
+                    const uint32_t t_o = tmem_base + C::TMEM_O + (hi & 1) * DP + ((uint32_t)(q4 * 32) << 16);
+#pragma unroll
+                    for (int c0 = 0; c0 < D; c0 += 40) {
+                        uint32_t v[5][8];
+#pragma unroll
+                        for (int i = 0; i < 5; ++i) ptx::tmem_ld8(t_o + c0 + i * 8, v[i]);
+                        ptx::tmem_ld_wait(v[0]);
+#pragma unroll
+                        for (int i = 1; i < 5; ++i) ptx::reg_fence8(v[i]);
+                        if (c0 + 40 == D) {
+                            ptx::tc_fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) ptx::mbar_arrive(&misc->o_free[hi & 1]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 5; ++i) {
+                            uint32_t pk[4];
+#pragma unroll
+                            for (int e2 = 0; e2 < 4; ++e2) {
+                                __half2 hv = __floats2half2_rn(__uint_as_float(v[i][2 * e2]) * inv255, __uint_as_float(v[i][2 * e2 + 1]) * inv255);
+                                pk[e2] = *reinterpret_cast<uint32_t*>(&hv);
+                            }
+                            *reinterpret_cast<uint4*>(U + ((size_t)r * D + c0 + i * 8) * 2) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        }
+                    }
+                    ptx::fence_proxy_async_smem();
+                }
+                asm volatile("bar.sync 7, 128;" ::: "memory");
+                if (t == 0 && alive) {
+                    ptx::tma_store_3d(&tmap_o, U, (h_begin + hi) * D, row0, zb);
+                    ptx::bulk_store_commit();
+                }
+            }
+            if (t == 0) {
+                ptx::bulk_store_wait_read();
+                ptx::mbar_arrive(&misc->u_free);
+            }
+            if (!alive) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
+        }
+        }
+    } else if (warp >= MMA_WARP) {
+    if constexpr (C::TMA_IO) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_WIDE_REST));
     if constexpr (REG_SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_REST));
     if (warp == COPY_WARP) {
         // ---------------- K~/V~ operand images, one head ahead ----------------
@@ -227,6 +343,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
             const int buf = hi % C::KVBUF;
             if (C::SPLIT_KV && !wait(&misc->kv_full[1], hi & 1)) return false;
             if (!wait(&misc->p_full, hi & 1)) return false;
+            if (C::TMA_IO && hi >= 2 && !wait(&misc->o_free[hi & 1], ((hi >> 1) - 1) & 1)) return false;     // (the O warps have read the head before last)
             ptx::tc_fence_after_sync();
             {
                 if (hi < 8) TAQ_PROF(96 + hi);
@@ -268,6 +385,7 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
         __syncwarp();
     }
     } else {
+        if constexpr (C::TMA_IO) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_WIDE_ROWS));
         if constexpr (REG_SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R_ROWS));
         // ---------------- row threads: two per query row (TMEM lane), each with half of the keys ----------------
         const int q4 = warp & 3, half = warp >> 2;
@@ -287,44 +405,37 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
         if (tid == 0) TAQ_PROF(1);
 
         if constexpr (C::TMA_IO) {
-            // ---- Q~ in and O out by TMA through the staging buffer U ----
+            // ---- the first head's Q~ in and the last head's O out; the heads between are others' work ----
             // Every warp walks every barrier of the loop, whatever happened to its waits: a warp whose wait ran out
             // skips the work, never a barrier.
             unsigned char* U = smem + C::OFF_U;
-            constexpr bool SEPQ = Q8;                        // the raw Q~ tile has its own buffer
-            unsigned char* UQ = SEPQ ? U + C::UO_BYTES : U;
-            constexpr int QESZ = Q8 ? 1 : 2;
-            constexpr uint32_t QRAW_BYTES = (uint32_t)(ROWS * D * QESZ);
             auto all256 = [&]() { asm volatile("bar.sync 5, 256;" ::: "memory"); };
-            auto load_q = [&](int hi) {          // one thread: raw Q~ tile of head hi (rows beyond n_query read as zero)
-                ptx::mbar_arrive_expect_tx(&misc->qraw_full, QRAW_BYTES);
-                ptx::tma_load_3d(UQ, &tmap_q, &misc->qraw_full, (h_begin + hi) * D, row0, zb);
-            };
-            // raw tile of head hi -> fp16 operand tile.  The 16-byte chunks of the tile are dealt out in linear order (thread t
+            // raw tile of the first head -> fp16 operand tile.  The 16-byte chunks of the tile are dealt out in linear order (thread t
             // takes chunks t, t + 256, ...): consecutive lanes read consecutive words of the raw tile and write the eight
             // chunk slots of a swizzled operand row, both free of bank conflicts.
-            auto stage_q_u = [&](int hi) {
+            auto stage_q_u = [&]() {
                 static_assert(D % 8 == 0 && (ROWS * (D / 8)) % 256 == 0, "chunks per thread");
                 constexpr int CPR = D / 8;                   // chunks per row
-                alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->qraw_full, hi & 1));
+                unsigned char* UQ = U + C::UO_BYTES;
+                auto load_q = [&](int hi) {                  // one thread: raw Q~ tile of head hi (rows beyond n_query read as zero)
+                    ptx::mbar_arrive_expect_tx(qraw_full(hi), (uint32_t)(ROWS * D));
+                    ptx::tma_load_3d(UQ, &tmap_q, qraw_full(hi), (h_begin + hi) * D, row0, zb);
+                };
+                if (tid == 0) load_q(0);
+                alive = __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(0), 0));
                 if (alive) {
-                    uint4 t16[ROWS * CPR / 256];
-#pragma unroll
-                    for (int i = 0; i < ROWS * CPR / 256; ++i) {
-                        const int j = tid + 256 * i;
-                        if (Q8) t16[i] = codes_w8_to_half(*reinterpret_cast<const uint2*>(UQ + (size_t)j * 8));
-                        else t16[i] = *reinterpret_cast<const uint4*>(UQ + (size_t)j * 16);
-                    }
 #pragma unroll
                     for (int i = 0; i < ROWS * CPR / 256; ++i) {
                         const int j = tid + 256 * i;
                         const int row = j / CPR, cc = j - row * CPR;
-                        *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(row, cc & 7)) = t16[i];
+                        *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(row, cc & 7)) = codes_w8_to_half(*reinterpret_cast<const uint2*>(UQ + (size_t)j * 8));
                     }
                     ptx::fence_proxy_async_smem();
                 }
                 __syncwarp();
                 if (alive && lane == 0) ptx::mbar_arrive(&misc->q_full);
+                all256();                                    // the raw tile has been read by everybody
+                if (tid == 0 && HG > 1 && alive) load_q(1);
             };
             // this thread's half of O of head hi: acc / 255 -> fp16 into U (the dense [128][D] tile)
             auto stage_o_u = [&](int hi) {
@@ -355,12 +466,11 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 ptx::bulk_store_commit();
             };
 
-            if (tid == 0) load_q(0);
             float sq = 1.0f, sq_next = 1.0f;
-            if (Q8) sq = valid ? __ldg(a.q_scales + grow * H + h_begin) : 0.f;
-            stage_q_u(0);
-            all256();                                        // U has been read by everybody
-            if (tid == 0 && HG > 1) load_q(1);
+            if (Q8) {
+                sq = valid ? __ldg(a.q_scales + grow * H + h_begin) : 0.f;
+                stage_q_u();
+            }
 
             for (int hi = 0; hi < HG; ++hi) {
                 const uint32_t ph = hi & 1;
@@ -399,23 +509,11 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 } else {
                     asm volatile("bar.sync %0, 64;" ::"r"(1 + q4) : "memory");
                 }
-                // S of this head is complete, so the Q~ operand tile is free: expand the next head's codes, which have had
-                // the softmax to arrive
-                if (tid == 128 && hi < 8) TAQ_PROF(104 + hi);
-                if (more) stage_q_u(hi + 1);
                 if (tid == 0 && hi < 8) TAQ_PROF(32 + hi);
-                if (tid == 128 && hi < 8) TAQ_PROF(112 + hi);
-                if (SEPQ && tid == 0) ptx::bulk_store_wait_read();      // (the store of the head before last: long done)
-                all256();                                    // the raw tile has been read by everybody, U by the store
-                if (SEPQ && tid == 0 && hi + 2 < HG && alive) load_q(hi + 2);
-                if (hi > 0) {                                // O of the previous head: TMEM -> U -> global (TMA store)
-                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) % C::OBUF], ((hi - 1) / C::OBUF) & 1));
-                    if (alive) {
-                        ptx::tc_fence_after_sync();
-                        stage_o_u(hi - 1);
-                    }
-                    all256();
-                    if (tid == 0 && alive) send_o(hi - 1);
+                // the P tile is free once the previous head's PV has completed
+                if (hi > 0) {
+                    alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(hi - 1) & 1], ((hi - 1) >> 1) & 1));
+                    ptx::tc_fence_after_sync();
                 }
                 if (tid == 0 && hi < 8) TAQ_PROF(48 + hi);
                 if (alive) {
@@ -427,17 +525,10 @@ __global__ void __launch_bounds__(ATT_THREADS, Cfg<D>::CTAS_PER_SM) attention_sm
                 __syncwarp();
                 if (alive && lane == 0) ptx::mbar_arrive(&misc->p_full);
                 if (tid == 0 && hi < 8) TAQ_PROF(64 + hi);
-                if (!SEPQ && tid == 0) {                     // shared buffer: once the store has read it, the raw tile of the head after next may land
-                    ptx::bulk_store_wait_read();
-                    if (hi + 2 < HG && alive) load_q(hi + 2);
-                }
                 sq = sq_next;
             }
             alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->o_full[(HG - 1) % C::OBUF], ((HG - 1) / C::OBUF) & 1));
-            if (SEPQ) {                                      // the store of the head before must have read U
-                if (tid == 0) ptx::bulk_store_wait_read();
-                all256();
-            }
+            alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->u_free, 0));      // the store of the head before has read U
             if (alive) {
                 ptx::tc_fence_after_sync();
                 stage_o_u(HG - 1);
@@ -615,20 +706,20 @@ cudaError_t launch_k(const AttnArgs& a, int n_z, cudaStream_t stream) {
     CUtensorMap tmap_q, tmap_o;
     memset(&tmap_q, 0, sizeof(tmap_q));
     memset(&tmap_o, 0, sizeof(tmap_o));
-    if (C::TMA_IO) {      // Q~ and O as [n_z][n_query][channels] in boxes of 128 rows x one head
+    if (C::TMA_IO) {      // Q~ and O as [n_z][n_query][channels] in boxes of 128 rows x one head (fp16 Q~: x 64 channels, as the operand tile has them)
         EncodeTiledFn enc = encode_tiled_fn3();
         if (!enc) return cudaErrorNotSupported;
         const cuuint64_t qesz = Q8 ? 1 : 2;
         const cuuint64_t dims[3] = {(cuuint64_t)a.channels, (cuuint64_t)a.n_query, (cuuint64_t)n_z};
         const cuuint64_t qstr[2] = {(cuuint64_t)a.channels * qesz, (cuuint64_t)a.channels * qesz * (cuuint64_t)a.n_query};
         const cuuint64_t ostr[2] = {(cuuint64_t)a.channels * 2, (cuuint64_t)a.channels * 2 * (cuuint64_t)a.n_query};
-        const cuuint32_t box[3] = {(cuuint32_t)D, ROWS, 1}, estr[3] = {1, 1, 1};
-        if (enc(&tmap_q, Q8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(a.q), dims, qstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        const cuuint32_t box[3] = {(cuuint32_t)D, ROWS, 1}, qbox[3] = {(cuuint32_t)(Q8 ? D : 64), ROWS, 1}, estr[3] = {1, 1, 1};
+        if (enc(&tmap_q, Q8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(a.q), dims, qstr, qbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                Q8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return cudaErrorInvalidValue;
         if (enc(&tmap_o, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, (void*)a.o, dims, ostr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }
-    return launch_pdl(attention_sm100_kernel<D, Q8, TAIL_ONLY>, grid, dim3(ATT_THREADS), (size_t)C::TOTAL, stream, tmap_q, tmap_o, a);
+    return launch_pdl(attention_sm100_kernel<D, Q8, TAIL_ONLY>, grid, dim3(C::THREADS), (size_t)C::TOTAL, stream, tmap_q, tmap_o, a);
 }
 
 template <int D>
