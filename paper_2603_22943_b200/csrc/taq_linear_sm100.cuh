@@ -543,7 +543,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                 for (int c = 0; c < HC; ++c) am = fmaxf(am, fabsf(y[c]));
                 if (d > HC) {                                // the row's threads with columns of the same head combine their absmax
-                    float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [NCG][128], and of a head pair [128] out, [128] in
+                    float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [NCG][128], and at 384 the absmax of a head pair's other half
                     const int per_head = min(NCG, d / HC), first = cg / per_head * per_head;
                     xc[cg * 128 + r] = am;
                     asm volatile("bar.sync %0, %1;" ::"r"(2 + q), "n"(NCG * 32) : "memory");
@@ -833,7 +833,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
     // ---------------- teardown ----------------
     ptx::tc_fence_before_sync();
-    // (No CTA of a cluster may leave while a copy out of its shared memory is in flight: by this barrier every copy has
+    // (No CTA of a cluster may leave while another one may still store into its shared memory: by this barrier everything has
     // been received.  Every thread arrives, whatever happened to its waits.)
     if (clustered) { ptx::cluster_arrive_relaxed(); ptx::cluster_wait(); }
     __syncthreads();

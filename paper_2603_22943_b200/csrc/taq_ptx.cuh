@@ -136,12 +136,6 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* gmem_src, 
                  : "memory");
 }
 
-// Untiled bulk copy shared -> global (the executing thread's earlier shared-memory writes must have been fenced
-// with fence_proxy_async_smem).  Both addresses 16-byte aligned, size a multiple of 16 bytes.
-__device__ __forceinline__ void bulk_store(void* gmem_dst, const void* smem_src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 ::"l"(reinterpret_cast<uint64_t>(gmem_dst)), "r"(smem_u32(smem_src)), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ void bulk_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Waits until the bulk stores of this thread have finished reading shared memory.
 __device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -161,7 +155,7 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* smem_slot, uint32_t ncols) 
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// 32 lanes x 8 / 16 consecutive 32-bit columns: thread l of the warp receives lane (lane_base + l).
+// 32 lanes x 8 consecutive 32-bit columns: thread l of the warp receives lane (lane_base + l).
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -173,30 +167,12 @@ __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
     return r;
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(taddr));
-}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // Registers written by tcgen05.ld hold their values only after tcgen05.wait::ld.  These two tie the registers to
 // the wait (or to a point after it) so that no use of them can be scheduled earlier.
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-                 :: "memory");
-}
 __device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
-                 :: "memory");
-}
-__device__ __forceinline__ void reg_fence(uint32_t (&r)[16]) {
-    asm volatile(""
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                  :: "memory");
 }
 
@@ -205,35 +181,15 @@ __device__ __forceinline__ void reg_fence8(uint32_t (&r)[8]) {
 }
 
 // ---- tcgen05.mma ------------------------------------------------------------------------------------
-// Shared-memory matrix descriptor of a K-major operand tile stored with the 128-byte swizzle: rows of 128 bytes
-// (64 fp16), groups of 8 rows 1024 bytes apart, 16-byte chunks XOR-ed with the row index inside the group.  The
-// tile base must be 1024-byte aligned; `byte_off` selects the 16-element K slice inside the 128-byte row.
-__device__ __forceinline__ uint64_t desc_k_sw128(uint32_t smem_addr_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr_bytes >> 4) & 0x3FFF);          // start address
-    d |= (uint64_t)1 << 16;                                     // leading byte offset (unused with swizzle)
-    d |= (uint64_t)(1024 >> 4) << 32;                           // stride byte offset: next group of 8 rows
-    d |= (uint64_t)1 << 46;                                     // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                                     // 128-byte swizzle
-    return d;
-}
-// The same for the 64-byte swizzle: rows of 64 bytes (32 fp16), groups of 8 rows 512 bytes apart, the 16-byte chunk
-// index XOR-ed with bits 1..2 of the row index (address bits 4..5 with bits 7..8).
-__device__ __forceinline__ uint64_t desc_k_sw64(uint32_t smem_addr_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((smem_addr_bytes >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;                                     // 64-byte swizzle
-    return d;
-}
-// The two halves of those descriptors, for issue loops that advance the start address only: the low word of a tile
-// at shared-memory address `a` is desc_lo(a); 16 bytes further is +1 (shared-memory addresses stay below 2^18, so
-// the 14-bit field never wraps), the high word is a constant of the layout.
+// Shared-memory matrix descriptors of K-major operand tiles, in two halves, for issue loops that advance the start address only.
+// 128-byte swizzle: rows of 128 bytes (64 fp16), groups of 8 rows 1024 bytes apart, 16-byte chunks XOR-ed with the row index
+// inside the group, tile base 1024-byte aligned.  The low word holds the start address (16 bytes further is +1: shared-memory
+// addresses stay below 2^18, so the 14-bit field never wraps) and the leading byte offset, which the swizzle does not
+// use; the high word, a constant of the layout, the distance to the next group of 8 rows, the descriptor version of this
+// architecture and the swizzle.
 __device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr_bytes) { return ((smem_addr_bytes >> 4) & 0x3FFFu) | (1u << 16); }
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);
-constexpr uint32_t kDescHiSw64 = (512u >> 4) | (1u << 14) | (4u << 29);
+constexpr uint32_t kDescHiSw64 = (512u >> 4) | (1u << 14) | (4u << 29);      // rows of 64 bytes, groups of 8 rows 512 bytes apart
 constexpr uint32_t kDescHiSw32 = (256u >> 4) | (1u << 14) | (6u << 29);      // rows of 32 bytes, groups of 8 rows 256 bytes apart
 __device__ __forceinline__ uint64_t desc_join(uint32_t hi, uint32_t lo) { return ((uint64_t)hi << 32) | lo; }
 // Instruction descriptor: fp16 x fp16 -> fp32, both operands K-major, M = 128, N = n.
