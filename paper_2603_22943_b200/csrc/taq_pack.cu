@@ -65,10 +65,33 @@ __device__ __forceinline__ int quant_code_127(float x, float s, float r_lo, floa
     if (a != c) return code_127_by_division(x, s);     // (fp16 data: about 4 values in 10000, e.g. exactly half of the row maximum)
     return (int)(a << 24) >> 24;                       // the low byte, sign-extended
 }
+// The same for eight fp16 values with one test for all of them: with a branch per value 8192 x 640 values took 9.5 us, now 4.9;
+// 64 x 1280, a launch of one wave, 2.9 -> 2.4.
+__device__ __noinline__ uint2 codes8_by_division(uint4 v, float s) {
+    const __half* h = reinterpret_cast<const __half*>(&v);
+    uint32_t w[2] = {0, 0};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e >> 2] |= (uint32_t)((int)fminf(fmaxf(rintf(__fdiv_rn(__half2float(h[e]), s)), -127.f), 127.f) & 0xFF) << (8 * (e & 3));
+    return make_uint2(w[0], w[1]);
+}
+__device__ __forceinline__ uint2 codes8(const uint4& v, float s, float r_lo, float r_hi) {
+    const __half2* h = reinterpret_cast<const __half2*>(&v);
+    uint32_t lo[8], bad = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 f = __half22float2(h[e]);
+        lo[2 * e] = __float_as_uint(fmaf(f.x, r_lo, 12582912.0f));
+        lo[2 * e + 1] = __float_as_uint(fmaf(f.y, r_lo, 12582912.0f));
+        bad |= (lo[2 * e] ^ __float_as_uint(fmaf(f.x, r_hi, 12582912.0f))) | (lo[2 * e + 1] ^ __float_as_uint(fmaf(f.y, r_hi, 12582912.0f)));
+    }
+    if (bad) return codes8_by_division(v, s);
+    auto low4 = [&](int i) { return __byte_perm(__byte_perm(lo[i], lo[i + 1], 0x0040), __byte_perm(lo[i + 2], lo[i + 3], 0x0040), 0x5410); };
+    return make_uint2(low4(0), low4(4));
+}
 
 // Per-token quantizer of fp16 activations (the inputs of the integer-activation projections): one warp per row of
 // `cols` fp16 values (a multiple of 8), which it keeps in registers between the absmax pass and the code pass when the
-// row is short enough (KEEP x 256 columns), so that the row is read once.  Same results as quantize_rows_kernel.
+// row is short enough (KEEP x 256 columns), so that the row is read once; KEEP as small as the row allows.  Same results as quantize_rows_kernel.
 template <int KEEP>
 __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __restrict__ x, long long rows, int cols,
                                                                 int8_t* __restrict__ codes, float* __restrict__ scales) {
@@ -82,11 +105,11 @@ __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __
     for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += warps_total) {
         const uint4* xr = reinterpret_cast<const uint4*>(x + r * cols);
         uint4 keep[KEEP];
-        float a = 0.f;
+        __half2 a2 = __float2half2_rn(0.f);                      // (maxima of fp16 magnitudes are exact)
         auto absmax8 = [&](const uint4& v) {
             const __half2* h = reinterpret_cast<const __half2*>(&v);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) { const float2 f = __half22float2(h[e]); a = fmaxf(a, fmaxf(fabsf(f.x), fabsf(f.y))); }
+            for (int e = 0; e < 4; ++e) a2 = __hmax2(a2, __habs2(h[e]));
         };
 #pragma unroll
         for (int j = 0; j < KEEP; ++j) {
@@ -97,30 +120,18 @@ __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __
 #pragma unroll
         for (int j = 0; j < KEEP; ++j) absmax8(keep[j]);
         for (int i = lane + 32 * KEEP; i < chunks; i += 32) absmax8(xr[i]);
-        a = warp_max(a);
+        const float a = warp_max(fmaxf(__low2float(a2), __high2float(a2)));
         const float s = quant_scale(a, 127.f);
-        const float rs = s > 0.f ? __frcp_rn(s) : 0.f;
-        const float r_lo = __uint_as_float(__float_as_uint(rs) - 2u), r_hi = __uint_as_float(__float_as_uint(rs) + 2u);
+        const float rs = __frcp_rn(s);
+        const float r_lo = s > 0.f ? __uint_as_float(__float_as_uint(rs) - 2u) : 0.f, r_hi = s > 0.f ? __uint_as_float(__float_as_uint(rs) + 2u) : 0.f;
         if (lane == 0) scales[r] = s;
         uint2* cr = reinterpret_cast<uint2*>(codes + r * cols);
-        auto encode = [&](const uint4& v) {
-            const __half2* h = reinterpret_cast<const __half2*>(&v);
-            uint32_t w[2] = {0, 0};
-            if (s > 0.f) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 f = __half22float2(h[e]);
-                    w[e >> 1] |= ((uint32_t)(quant_code_127(f.x, s, r_lo, r_hi) & 0xFF) | ((uint32_t)(quant_code_127(f.y, s, r_lo, r_hi) & 0xFF) << 8)) << (16 * (e & 1));
-                }
-            }
-            return make_uint2(w[0], w[1]);
-        };
 #pragma unroll
         for (int j = 0; j < KEEP; ++j) {
             const int i = lane + 32 * j;
-            if (i < chunks) cr[i] = encode(keep[j]);
+            if (i < chunks) cr[i] = codes8(keep[j], s, r_lo, r_hi);
         }
-        for (int i = lane + 32 * KEEP; i < chunks; i += 32) cr[i] = encode(xr[i]);
+        for (int i = lane + 32 * KEEP; i < chunks; i += 32) cr[i] = codes8(xr[i], s, r_lo, r_hi);
     }
 }
 
@@ -128,8 +139,8 @@ cudaError_t launch_quantize_rows_f16(const __half* x, long long rows, int cols, 
     if (rows == 0) return cudaSuccess;
     long long blocks = (rows + 7) / 8;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
-    if (cols <= 512) return launch_pdl(quantize_rows_f16_kernel<2>, dim3((unsigned)blocks), dim3(256), 0, stream, x, rows, cols, codes, scales);
-    return launch_pdl(quantize_rows_f16_kernel<8>, dim3((unsigned)blocks), dim3(256), 0, stream, x, rows, cols, codes, scales);
+    auto* kern = cols <= 512 ? quantize_rows_f16_kernel<2> : cols <= 768 ? quantize_rows_f16_kernel<3> : cols <= 1280 ? quantize_rows_f16_kernel<5> : quantize_rows_f16_kernel<8>;
+    return launch_pdl(kern, dim3((unsigned)blocks), dim3(256), 0, stream, x, rows, cols, codes, scales);
 }
 
 // ---- helpers of the token-sensitivity sweep (Eq. 1) -------------------------------------------------------------
