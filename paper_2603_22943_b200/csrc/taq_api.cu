@@ -403,6 +403,7 @@ static taq_status layer_forward_impl(const taq_layer_desc* d, const taq_request*
     o.y = y;
     o.rows = (long long)d->batch * d->n_query; o.n_out = d->channels; o.k_in = d->channels; o.bits = d->w_bits; o.group = d->w_group;
     o.heads = 1; o.epi = EPI_F16; o.status = status;
+    o.early_weights = 1;        // the kernel before it in the stream is the attention above, which writes O only
     return run_linear(o, n_req, st);
 }
 
@@ -532,6 +533,7 @@ taq_status taq_layer_forward_a8(const taq_layer_desc* d, const void* x_f16_dev, 
     q.heads = d->q_bits == 8 ? d->heads : 1;
     q.epi = d->q_bits == 8 ? EPI_Q8_HEAD : EPI_F16;
     q.status = status;
+    q.early_weights = 1;        // the kernel before it in the stream is the quantizer above, which writes xq / xs only
     s = run_linear_i8(q, st);
     if (s != TAQ_OK) return s;
     AttnArgs at = attn_args(d, status);
@@ -547,6 +549,7 @@ taq_status taq_layer_forward_a8(const taq_layer_desc* d, const void* x_f16_dev, 
     o.y = y_f16_dev;
     o.rows = rows; o.n_out = d->channels; o.k_in = d->channels; o.bits = d->w_bits; o.group = d->w_group;
     o.heads = 1; o.epi = EPI_F16; o.status = status;
+    o.early_weights = 1;
     return run_linear_i8(o, st);
 }
 
@@ -591,6 +594,7 @@ taq_status taq_kv_project_a8(const taq_layer_desc* d, const void* ctx_f16_dev, c
     a.heads = d->heads; a.n_ctx = d->n_ctx; a.max_trigger = d->max_trigger;
     a.epi = EPI_KV; a.kv_qmax = d->kv_bits == 4 ? 7 : 127;
     a.status = status;
+    a.early_weights = 1;        // the quantizer above writes cq / cs only
     return run_kv_projection(*d, a, Wk_packed_dev, Wv_packed_dev, d->batch, 1, st);
 }
 

@@ -139,6 +139,7 @@ struct LinearArgs {
     int heads;                  // EPI_Q8_HEAD / EPI_KV
     int n_ctx, max_trigger;     // EPI_KV: rows = batch * n_ctx
     int kv_which;               // EPI_KV on CUDA cores: 0 = K, 1 = V
+    int early_weights;          // the previous kernel in the stream is known not to write the weights: they may be read before it has finished
     int kv_qmax;                // EPI_KV: 127 (int8 rows) or 7 (4-bit rows); 0 is read as 127
     int epi;
     int* status;

@@ -237,7 +237,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     auto start = [&](bool wait) {
         if (wait) asm volatile("bar.sync 14, %0;" ::"n"(TL::NTHREADS) : "memory");
         else asm volatile("bar.arrive 14, %0;" ::"n"(TL::NTHREADS) : "memory");
-        ptx::pdl_trigger();
         if (clustered) ptx::cluster_arrive_relaxed();        // waited for right before the first operation on another CTA
     };
     auto blob_of = [&](int z, int kv_which) { return (const uint8_t*)(a.reqs ? ((KV ? kv_which : a.which) == 0 ? a.reqs[z].Wq : a.reqs[z].Wout) : kv_which ? a.w2 : a.w); };
@@ -413,13 +412,17 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 // come in.  CTA `owner` of the cluster finishes the rows of 4 / nsplit lane quarters: a folder warp either
                 // stores its 32 rows into that CTA's shared memory, straight from the registers (16 bytes a lane, the lanes
                 // of a store next to each other, no staging, no bank conflicts), or receives a piece from every other CTA and
-                // adds them in rank order, so that every output is the same sum whoever computes it.
+                // adds them in rank order, so that every output is the same sum whoever computes it.  Rows beyond the last one
+                // stay where they are (the exchange goes at about 25 bytes a cycle, and a launch of 64 rows is half padding).
+                const bool padding = !KV && (long long)row0 + q * 32 >= a.rows;          // (K~/V~: rows beyond the last are keys of the images)
                 const int per_cta = 4 / nsplit, owner = q / per_cta;
                 const uint32_t base = ptx::cluster_ctarank() - (uint32_t)rank;        // ranks along x are consecutive
-                mine = alive && owner == rank;
+                mine = alive && owner == rank && !padding;
                 if (ft < nsplit && ft != rank) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), base + (uint32_t)ft));
                 auto piece = [&](int cta, int from) { return smem + ((cg * per_cta + q - cta * per_cta) * (nsplit - 1) + (from < cta ? from : from - 1)) * TL::PIECE + lane * 16; };
-                if (owner != rank) {
+                if (padding) {
+                    // nothing to send, nothing comes
+                } else if (owner != rank) {
                     if (alive && ptx::mbar_wait(&bars->peer_ready, 0)) {                 // the other CTAs' rings are free, too
                         const uint32_t dst = ptx::map_to_cta(ptx::smem_u32(piece(owner, rank)), base + (uint32_t)owner);
                         const uint32_t bar = ptx::map_to_cta(ptx::smem_u32(&bars->part_full[fw]), base + (uint32_t)owner);
@@ -427,7 +430,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         for (int c = 0; c < HC; c += 4)
                             ptx::store_to_cta(dst + c * 128, __float_as_uint(y[c]), __float_as_uint(y[c + 1]), __float_as_uint(y[c + 2]), __float_as_uint(y[c + 3]), bar);
                     } else give_up();
-                } else if (!ptx::mbar_wait(&bars->part_full[fw], 0)) {
+                } else if (!ptx::mbar_wait(&bars->part_full[fw], 0) || !ptx::mbar_wait(&bars->peer_ready, 0)) {      // (peer_ready: no arrival may come in after the CTA has left)
                     give_up();
                 } else {
                     const unsigned char* in = smem + (cg * per_cta + q - rank * per_cta) * (nsplit - 1) * TL::PIECE + lane * 16;
@@ -633,8 +636,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         CodeT pw[NPRE];
         const uint8_t* src = nullptr;                        // codes of the fetched pair
         int tile = tile0, pair = group;                      // the fetched pair
-        // (Packed weights are written by taq_pack_weights, which never lets its successor start early: they are complete
-        // before this kernel can run at all and are fetched and expanded under the previous kernel's tail.)
+        // (Weights that the previous kernel in the stream is known not to write are fetched and expanded under its tail.)
         auto load = [&](int j) {
             const int i = 2 * pair + (c16 >> 3);
             const bool have = i < n_kb && (!I8 || (kb_begin + 2 * pair) * BKE + c16 * 16 < a.k_in);
@@ -651,9 +653,10 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
             for (int j = 0; j < NPRE; ++j) pw[j] = load(j);
         };
-        fetch(true);
+        if (a.early_weights) fetch(true);
         start(true);
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_BUILD));
+        if (!a.early_weights) { ptx::pdl_wait(); fetch(true); }
         int s = group;
         uint32_t ph = 1;
         bool passed = false, ok = true;                      // passed: the ring has been passed once
@@ -691,6 +694,9 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             // ---------------- producer: activation tiles ----------------
             if (lane == 0) {
                 ptx::pdl_wait();                             // the activations may come from the previous kernel
+                // (Not before the wait: the successor's early reads, K~/V~ images and weights, may be of data that whatever ran before
+                // this kernel wrote.)
+                ptx::pdl_trigger();
                 TAQ_PROF(1); TAQ_GPROF(28);
                 int s = 0, issued = 0;
                 uint32_t ph = 1;
@@ -779,6 +785,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         else if (warp < TL::W_AUX + 2) {
             // ---------------- scales and biases, one tile ahead ----------------
+            if (!a.early_weights) ptx::pdl_wait();
             int sbuf = 0, it = 0;
             uint32_t ph = 1;
             for (int tile = tile0; tile < lay.n_tiles; tile += tile_step, ++it) {

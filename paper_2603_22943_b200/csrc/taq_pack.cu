@@ -95,10 +95,11 @@ __device__ __forceinline__ uint2 codes8(const uint4& v, float s, float r_lo, flo
 template <int KEEP>
 __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __restrict__ x, long long rows, int cols,
                                                                 int8_t* __restrict__ codes, float* __restrict__ scales) {
-    // Launched with the programmatic-serialization attribute: the successor (the integer GEMM) may start its prologue
-    // now; this kernel's input may come from the predecessor, so it is read only after the wait.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Launched with the programmatic-serialization attribute: the input may come from the predecessor, so it is read only after the
+    // wait.  Only then may the successor (the integer GEMM) start its prologue: it reads its weights at once, which whatever
+    // ran before this kernel may have written.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const long long warps_total = (long long)gridDim.x * (blockDim.x >> 5);
     const int chunks = cols / 8;                                 // 16-byte chunks of a row
@@ -276,6 +277,7 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restri
             for (int i0 = TPG * KEEP; i0 < n4[u]; i0 += TPG) encode(i0 + t < n4[u] ? w4[u][i0 + t] : make_float4(0.f, 0.f, 0.f, 0.f), i0 + t, i0 + t < n4[u]);
         }
     }
+    __threadfence();      // (a successor may read the blob as soon as the last block has gone, see the layer kernel)
 }
 
 cudaError_t launch_pack_weights(const taq_weight_desc& d, const float* W, const float* bias, void* packed, cudaStream_t stream) {
