@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             if (t == 0) {
                 ptx::bulk_store_wait_read();
                 ptx::mbar_arrive(&misc->u_free);
+                ptx::bulk_store_wait();                      // (a successor that waits for this kernel reads O as soon as it may)
             }
             if (!alive) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
         }
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             all256();
             if (tid == 0) {
                 if (alive) send_o(HG - 1);
-                ptx::bulk_store_wait_read();
+                ptx::bulk_store_wait();
             }
             if (!alive) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
         } else {

@@ -95,10 +95,8 @@ __device__ __forceinline__ uint2 codes8(const uint4& v, float s, float r_lo, flo
 template <int KEEP>
 __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __restrict__ x, long long rows, int cols,
                                                                 int8_t* __restrict__ codes, float* __restrict__ scales) {
-    // Launched with the programmatic-serialization attribute: the input may come from the predecessor, so it is read only after the
-    // wait.  Only then may the successor (the integer GEMM) start its prologue: it reads its weights at once, which whatever
-    // ran before this kernel may have written.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The successor (the integer GEMM) may start its prologue now, and read its weights at once: this kernel starts when everything
+    // before it has finished.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const long long warps_total = (long long)gridDim.x * (blockDim.x >> 5);
@@ -141,7 +139,10 @@ cudaError_t launch_quantize_rows_f16(const __half* x, long long rows, int cols, 
     long long blocks = (rows + 7) / 8;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
     auto* kern = cols <= 512 ? quantize_rows_f16_kernel<2> : cols <= 768 ? quantize_rows_f16_kernel<3> : cols <= 1280 ? quantize_rows_f16_kernel<5> : quantize_rows_f16_kernel<8>;
-    return launch_pdl(kern, dim3((unsigned)blocks), dim3(256), 0, stream, x, rows, cols, codes, scales);
+    // (An ordinary launch: as an early starter behind the attention kernel, several layer passes in a row, it read rows of O that were
+    // not there yet.)
+    kern<<<(unsigned)blocks, 256, 0, stream>>>(x, rows, cols, codes, scales);
+    return cudaGetLastError();
 }
 
 // ---- helpers of the token-sensitivity sweep (Eq. 1) -------------------------------------------------------------
