@@ -469,14 +469,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
 
             float sq = 1.0f, sq_next = 1.0f;
             if (Q8) {
-                sq = valid ? __ldg(a.q_scales + grow * H + h_begin) : 0.f;
+                sq = valid ? a.q_scales[grow * H + h_begin] : 0.f;
                 stage_q_u();
             }
 
             for (int hi = 0; hi < HG; ++hi) {
                 const uint32_t ph = hi & 1;
                 const bool more = hi + 1 < HG;
-                if (Q8 && more) sq_next = valid ? __ldg(a.q_scales + grow * H + h_begin + hi + 1) : 0.f;
+                if (Q8 && more) sq_next = valid ? a.q_scales[grow * H + h_begin + hi + 1] : 0.f;
                 alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[ph], (hi >> 1) & 1));
                 if (tid == 0 && hi < 8) TAQ_PROF(16 + hi);
                 float e[HK];

@@ -620,24 +620,24 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             unsigned char* q_tile = smem + OFF_R0 + hi * A_TILE;
             const size_t grow = (size_t)zb * a.n_query + (valid ? n : 0);
             const size_t elem = grow * (size_t)(H * D) + (size_t)(h_begin + hi) * D;
-            // all loads first (read-only path), then the conversions and the stores: one round trip to L2, not five
+            // all loads first, then the conversions and the stores: one round trip to L2, not five
             uint4 t16[D / 8];
             if (a.q_bits == 8) {
                 uint2 c8[D / 8];
 #pragma unroll
                 for (int cc = 0; cc < D / 8; ++cc)
-                    c8[cc] = valid ? __ldg(reinterpret_cast<const uint2*>((const int8_t*)a.q + elem + cc * 8)) : make_uint2(0, 0);
+                    c8[cc] = valid ? *reinterpret_cast<const uint2*>((const int8_t*)a.q + elem + cc * 8) : make_uint2(0, 0);
 #pragma unroll
                 for (int cc = 0; cc < D / 8; ++cc) t16[cc] = codes_w8_to_half(c8[cc]);
             } else {
 #pragma unroll
                 for (int cc = 0; cc < D / 8; ++cc)
-                    t16[cc] = valid ? __ldg(reinterpret_cast<const uint4*>((const __half*)a.q + elem + cc * 8)) : make_uint4(0, 0, 0, 0);
+                    t16[cc] = valid ? *reinterpret_cast<const uint4*>((const __half*)a.q + elem + cc * 8) : make_uint4(0, 0, 0, 0);
             }
 #pragma unroll
             for (int cc = 0; cc < D / 8; ++cc) *reinterpret_cast<uint4*>(q_tile + ptx::sw128_offset(r, cc)) = t16[cc];
             *reinterpret_cast<uint4*>(q_tile + ptx::sw128_offset(r, D / 8)) = make_uint4(0, 0, 0, 0);   // channels 40..47
-            sq = a.q_bits == 8 ? (valid ? __ldg(a.q_scales + grow * H + h_begin + hi) : 0.f) : 1.0f;
+            sq = a.q_bits == 8 ? (valid ? a.q_scales[grow * H + h_begin + hi] : 0.f) : 1.0f;
         } else {
             float amax = 0.f;
 #pragma unroll

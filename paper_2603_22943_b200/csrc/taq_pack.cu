@@ -93,8 +93,7 @@ __device__ __forceinline__ uint2 codes8(const uint4& v, float s, float r_lo, flo
 // `cols` fp16 values (a multiple of 8), which it keeps in registers between the absmax pass and the code pass when the
 // row is short enough (KEEP x 256 columns), so that the row is read once; KEEP as small as the row allows.  Same results as quantize_rows_kernel.
 template <int KEEP>
-__global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* __restrict__ x, long long rows, int cols,
-                                                                int8_t* __restrict__ codes, float* __restrict__ scales) {
+__global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* x, long long rows, int cols, int8_t* codes, float* scales) {
     // The successor (the integer GEMM) may start its prologue now, and read its weights at once: this kernel starts when everything
     // before it has finished.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -1,0 +1,111 @@
+"""Layer passes enqueued one behind the other, as a denoising loop does: every kernel may start while its predecessor is still
+running, so each one's reads of what the predecessor writes, and its writes over what the predecessor reads, are put to the test
+only here.  The passes of a sequence have inputs of their own and take turns on workspaces of their own and on one that all
+share; each pass must give, bit for bit, what it gives alone on an idle GPU."""
+import pytest
+import torch
+
+from paper_2603_22943_b200 import binding as tb
+
+pytestmark = pytest.mark.gpu
+
+ROUNDS = 8
+
+
+def _sections(desc, a_bits):
+    """(name, offset, bytes per row) of a pass's workspace; every section starts on a multiple of 128 bytes."""
+    rows, c, h = desc.batch * desc.n_query, desc.channels, desc.heads
+    out, off = [], 0
+    for name, per_row in ([("activation codes", c), ("activation scales", 4)] if a_bits == 8 else []) + [("Q~", c), ("Q~ scales", 4 * h), ("O", 2 * c)]:
+        out.append((name, off, per_row))
+        off += (rows * per_row + 127) // 128 * 128
+    return out
+
+
+def _where(desc, a_bits, got, want):
+    """Which sections of two workspaces differ, in which rows and heads."""
+    text, rows, h = [], desc.batch * desc.n_query, desc.heads
+    for name, off, per_row in _sections(desc, a_bits):
+        d = (got[off: off + rows * per_row] != want[off: off + rows * per_row]).view(rows, per_row)
+        if bool(d.any()):
+            r = d.any(1).nonzero().flatten().tolist()
+            heads = d.view(rows, h, per_row // h).any(2).any(0).nonzero().flatten().tolist() if per_row % h == 0 else "-"
+            text.append(f"{name}: {len(r)} rows {r[:12]}, heads {heads}")
+    return "; ".join(text) or "same"
+
+
+def _state(batch, n_query, channels, heads, w_bits, a_bits, seed):
+    gen = torch.Generator("cuda").manual_seed(seed)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    group, dc, t = (128 if w_bits == 4 else 0), 768, 77
+    desc = tb.layer_desc(batch, n_query, channels, heads, t, dc, w_bits, group, max_trigger=2)
+    pack = lambda n_out, k_in, bias=None: tb.taq_pack_weights(tb.weight_desc(n_out, k_in, w_bits, group), normal(n_out, k_in) / k_in ** 0.5, bias)
+    mask = torch.zeros((batch, t), dtype=torch.uint8, device="cuda")
+    mask[:, 4:6] = 1
+    ctx = normal(batch, t, dc).half()
+    wk, wv, wq, wout = pack(channels, dc), pack(channels, dc), pack(channels, channels), pack(channels, channels, 0.1 * normal(channels))
+    kv = (tb.taq_kv_project_a8 if a_bits == 8 else tb.taq_kv_project)(desc, ctx, wk, wv, mask)
+    x = normal(batch, n_query, channels)
+    x[..., seed % channels] *= 20
+    forward = tb.taq_layer_forward_a8 if a_bits == 8 else tb.taq_layer_forward
+    size = tb.taq_workspace_bytes_a8(desc) if a_bits == 8 else tb.taq_workspace_bytes(desc)
+    x = x.half()
+    return desc, size, lambda y, ws: forward(desc, x, wq, wout, kv, mask, y, ws)
+
+
+@pytest.mark.parametrize("batch,n_query,channels,heads,w_bits,a_bits", [
+    (3, 2700, 1280, 8, 4, 8),           # heads of 160: four per CTA of the attention, ragged row tiles
+    (3, 2700, 1280, 8, 8, 8),
+    (3, 2700, 1280, 8, 4, 16),
+    (2, 256, 1280, 8, 4, 8),            # one head per CTA, projections over clusters
+    (2, 1024, 640, 8, 8, 8),            # heads of 80
+    (3, 2500, 640, 8, 4, 8),
+    (3, 2500, 640, 8, 8, 16),
+    (2, 1500, 640, 10, 4, 8),           # heads of 64
+    (2, 700, 320, 8, 8, 8),             # heads of 40 outside the one-kernel layer: all four heads of a CTA at once
+    (2, 700, 320, 8, 8, 16),
+    (2, 700, 320, 8, 4, 16),            # the one-kernel layers
+    (2, 700, 320, 8, 4, 8),
+])
+def test_passes_in_a_row_equal_passes_alone(batch, n_query, channels, heads, w_bits, a_bits):
+    states = [_state(batch, n_query, channels, heads, w_bits, a_bits, seed) for seed in (1, 2)]
+    size = max(s[1] for s in states)
+    new_y = lambda: torch.full((batch, n_query, channels), float("nan"), dtype=torch.float16, device="cuda")
+    new_ws = lambda: torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda")
+    want = []
+    for desc, _, forward in states:
+        y, ws = new_y(), new_ws()
+        torch.cuda.synchronize()
+        forward(y, ws)
+        torch.cuda.synchronize()
+        want.append((y, ws))
+    ys = [(which, new_y()) for which in list(range(len(states))) * (2 * ROUNDS)]
+
+    def sequence(shared, own):                           # A B A B .. on one workspace, then each on its own
+        for i, (which, y) in enumerate(ys):
+            states[which][2](y, shared if i < len(ys) // 2 else own[which])
+
+    def check(how, shared, own):
+        torch.cuda.synchronize()
+        tb.taq_poll_device_status()
+        wrong = []
+        for i, (which, y) in enumerate(ys):
+            d = (y.view(torch.int16) != want[which][0].view(torch.int16)).view(-1, channels).any(1).nonzero().flatten().tolist()
+            if d:
+                wrong.append(f"pass {i}: Y rows {len(d)} {d[:8]}")
+            y.fill_(float("nan"))
+        if wrong:
+            desc = states[0][0]
+            pytest.fail(how + ": " + "; ".join(wrong[:6]) + " | last pass on the shared workspace: " + _where(desc, a_bits, shared, want[-1][1]) +
+                        "".join(f" | own workspace {i}: " + _where(desc, a_bits, own[i], want[i][1]) for i in range(len(states))))
+
+    shared, own = new_ws(), [new_ws() for _ in states]
+    torch.cuda.synchronize()
+    sequence(shared, own)
+    check("enqueued call by call", shared, own)
+    graph = torch.cuda.CUDAGraph()                       # (small passes are enqueued more slowly than they run; a graph leaves no gaps)
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        sequence(shared, own)
+    for _ in range(3):
+        graph.replay()
+        check("from a graph", shared, own)
