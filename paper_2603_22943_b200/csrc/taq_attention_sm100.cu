@@ -181,11 +181,14 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                 constexpr int CPR = D / 8, N = ROWS * CPR / 128;
                 const unsigned char* UQ = smem + C::OFF_U + C::UO_BYTES;
                 const int t = tid - 32 * Q_WARP;
+                if (t == 0) ptx::pdl_wait();                             // (this thread loads Q~ of the third head and on)
+                __syncwarp();
                 for (int hi = 1; hi < HG; ++hi) {
                     alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(hi), (hi >> 1) & 1));
                     uint2 raw[N];
 #pragma unroll
                     for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint2*>(UQ + (size_t)(t + 128 * i) * 8);
+                    ptx::fence_proxy_async_smem();                           // (generic reads before the TMA load that overwrites them)
                     asm volatile("bar.sync 6, 128;" ::: "memory");           // the raw tile has been read
                     if (t == 0 && alive && hi + 1 < HG) {
                         ptx::mbar_arrive_expect_tx(qraw_full(hi + 1), (uint32_t)(ROWS * D));

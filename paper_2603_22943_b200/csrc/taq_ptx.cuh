@@ -55,8 +55,9 @@ __device__ __forceinline__ bool elect_one() {
 // ---- programmatic dependent launch ---------------------------------------------------------------------
 // A kernel launched with the programmatic-serialization attribute may start while its predecessor in the stream
 // is still draining.  pdl_wait() returns once the predecessor has completed and its writes are visible; nothing
-// that the predecessor may have written (or may still read) is touched before it.  pdl_trigger() lets the
-// successor's CTAs be scheduled as soon as resources allow.  Both are no-ops for an ordinary launch.
+// that the predecessor may have written (or may still read) is touched before it, and every thread that reads such data
+// itself, by TMA too, passes a pdl_wait() of its own.  pdl_trigger() lets the successor's CTAs be scheduled as soon as
+// resources allow.  Both are no-ops for an ordinary launch.
 // Such data never goes through the read-only path (__ldg, or a const __restrict__ parameter): that path is for memory nobody
 // writes as long as the kernel lives, a kernel that starts early is alive while its predecessor writes, and the compiler
 // may move a read-only load across the wait.
