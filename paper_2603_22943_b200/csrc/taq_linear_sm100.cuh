@@ -640,7 +640,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         auto load = [&](int j) {
             const int i = 2 * pair + (c16 >> 3);
             const bool have = i < n_kb && (!I8 || (kb_begin + 2 * pair) * BKE + c16 * 16 < a.k_in);
-            return have ? __ldg(reinterpret_cast<const CodeT*>(src + (uint32_t)j * row_step)) : zero_codes<I8, W8>();
+            return have ? ptx::load_global(reinterpret_cast<const CodeT*>(src + (uint32_t)j * row_step)) : zero_codes<I8, W8>();
         };
         auto fetch = [&](bool new_tile) {
             while (pair >= n_pair) { pair -= n_pair; tile += tile_step; new_tile = true; }
@@ -799,12 +799,12 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 // [BN][n_groups] -> [n_groups][BN], so that a group's scales of consecutive columns are contiguous; eight loads at a time
                 // are on their way
                 const int t = (warp - TL::W_AUX) * 32 + lane, n_all = BN * n_groups;
-                for (int n = t; n < BN; n += 64) sc[n_all + n] = with_bias ? __ldg(gb + n) : 0.f;
+                for (int n = t; n < BN; n += 64) sc[n_all + n] = with_bias ? ptx::load_global(gb + n) : 0.f;
 #pragma unroll 1
                 for (int base = t; base < n_all; base += 64 * 8) {
                     float v[8];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = base + 64 * j < n_all ? __ldg(gs + base + 64 * j) : 0.f;
+                    for (int j = 0; j < 8; ++j) v[j] = base + 64 * j < n_all ? ptx::load_global(gs + base + 64 * j) : 0.f;
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         const int i = base + 64 * j, n = quotient(i, n_groups, lay.mul_groups);

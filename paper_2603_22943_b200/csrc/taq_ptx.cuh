@@ -63,6 +63,16 @@ __device__ __forceinline__ bool elect_one() {
 // may move a read-only load across the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// An ordinary load from a global address that the compiler may not recognise as one; stays behind a pdl_wait() before it.
+template <typename T>
+__device__ __forceinline__ T load_global(const T* p) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one load");
+    union { T v; uint32_t w[sizeof(T) / 4]; } u;
+    if constexpr (sizeof(T) == 4) asm volatile("ld.global.b32 %0, [%1];" : "=r"(u.w[0]) : "l"(p));
+    else if constexpr (sizeof(T) == 8) asm volatile("ld.global.v2.b32 {%0, %1}, [%2];" : "=r"(u.w[0]), "=r"(u.w[1]) : "l"(p));
+    else asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(u.w[0]), "=r"(u.w[1]), "=r"(u.w[2]), "=r"(u.w[3]) : "l"(p));
+    return u.v;
+}
 
 // ---- thread-block clusters: the peer CTA's shared memory and barriers ---------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {

@@ -49,8 +49,8 @@ def _state(batch, n_query, channels, heads, w_bits, a_bits, seed):
     x[..., seed % channels] *= 20
     forward = tb.taq_layer_forward_a8 if a_bits == 8 else tb.taq_layer_forward
     size = tb.taq_workspace_bytes_a8(desc) if a_bits == 8 else tb.taq_workspace_bytes(desc)
-    x = x.half()
-    return desc, size, lambda y, ws: forward(desc, x, wq, wout, kv, mask, y, ws)
+    x, blobs = x.half(), (wq, wout, kv)
+    return desc, size, lambda y, ws, b=blobs: forward(desc, x, b[0], b[1], b[2], mask, y, ws), blobs
 
 
 @pytest.mark.parametrize("batch,n_query,channels,heads,w_bits,a_bits", [
@@ -73,7 +73,7 @@ def test_passes_in_a_row_equal_passes_alone(batch, n_query, channels, heads, w_b
     new_y = lambda: torch.full((batch, n_query, channels), float("nan"), dtype=torch.float16, device="cuda")
     new_ws = lambda: torch.full((size,), 0xFF, dtype=torch.uint8, device="cuda")
     want = []
-    for desc, _, forward in states:
+    for desc, _, forward, _ in states:
         y, ws = new_y(), new_ws()
         torch.cuda.synchronize()
         forward(y, ws)
@@ -109,3 +109,51 @@ def test_passes_in_a_row_equal_passes_alone(batch, n_query, channels, heads, w_b
     for _ in range(3):
         graph.replay()
         check("from a graph", shared, own)
+
+
+@pytest.mark.parametrize("batch,n_query,channels,heads,w_bits,a_bits", [
+    (2, 256, 1280, 8, 4, 16),
+    (1, 64, 1280, 8, 8, 16),
+    (2, 256, 1280, 8, 4, 8),
+    (2, 1024, 640, 8, 4, 16),
+    (2, 1024, 640, 10, 8, 8),
+    (2, 700, 320, 8, 8, 16),
+])
+def test_weights_and_keys_written_right_before_a_pass_are_the_ones_it_uses(batch, n_query, channels, heads, w_bits, a_bits):
+    """As when a checkpoint is swapped in: two checkpoints' blobs are written in turn over the same memory (by an elementwise
+    kernel from their complements), each time right before the pass that uses them."""
+    states = [_state(batch, n_query, channels, heads, w_bits, a_bits, seed) for seed in (3, 4)]
+    complements = [[~b.view(torch.uint8) for b in s[3]] for s in states]
+    place = [torch.zeros_like(c) for c in complements[0]]
+    ws = torch.zeros(states[0][1], dtype=torch.uint8, device="cuda")
+    new_y = lambda: torch.full((batch, n_query, channels), float("nan"), dtype=torch.float16, device="cuda")
+    want = []
+    for s in states:
+        y = new_y()
+        s[2](y, ws)
+        torch.cuda.synchronize()
+        want.append(y)
+    ys = [new_y() for _ in range(2 * ROUNDS)]
+
+    def sequence(last):                                  # the blob written last, with nothing between it and the pass
+        for i, y in enumerate(ys):
+            for k in [k for k in range(3) if k != last] + [last]:
+                torch.bitwise_not(complements[i % 2][k], out=place[k])
+            states[i % 2][2](y, ws, place)
+
+    def check(how):
+        torch.cuda.synchronize()
+        tb.taq_poll_device_status()
+        for i, y in enumerate(ys):
+            assert torch.equal(y.view(torch.int16), want[i % 2].view(torch.int16)), (how, i)
+            y.fill_(float("nan"))
+
+    for last in range(3):
+        sequence(last)
+        check(f"call by call, {last} written last")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+            sequence(last)
+        for _ in range(2):
+            graph.replay()
+            check(f"from a graph, {last} written last")
