@@ -292,10 +292,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(30); }
+    const uint8_t* wq_blob = (const uint8_t*)a.wq;
     if (warp == 0) {
-        // One lane per barrier (45 in a row by one thread take a while); then, still in front of the CTA's first barrier, the packed
-        // weights: they are written by taq_pack_weights, which never lets its successor start early, so they are complete
-        // before this kernel can run at all and are fetched (and expanded) under the previous kernel's tail.
+        // (A launch over requests is mostly one of several waves, in which this wait is over at once: the address is on its way
+        // while the barriers are set up.)
+        if (!Q_IN && a.reqs) { ptx::pdl_wait(); wq_blob = (const uint8_t*)a.reqs[zb].Wq; }
+        // One lane per barrier (45 in a row by one thread take a while).
         uint64_t* all = misc->a_full;
         for (int i = lane; i < N_BARS; i += 32) {
             const uint64_t* bar = all + i;
@@ -315,22 +317,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         if (lane == 0) {
             misc->abort_flag = 0;
             if (FUSE_OUT) ptx::mbar_arrive_expect_tx(&misc->o_all, (N_OTILE / 2) * O_TILE);     // the partner's five tiles
-            if (!Q_IN) {
-                const uint32_t scale_bytes = (uint32_t)(NQ * n_groups * 4);
-                const uint8_t* blob = (const uint8_t*)(a.reqs ? a.reqs[zb].Wq : a.wq);
-                ptx::mbar_arrive_expect_tx(&misc->w_full, RAW_BYTES + scale_bytes);
-                ptx::bulk_load(smem + OFF_RAW, blob + L.off_codes + (size_t)col0 * L.row_bytes, RAW_BYTES, &misc->w_full);
-                ptx::bulk_load(smem + OFF_SC, blob + L.off_scales + (size_t)col0 * n_groups * 4, scale_bytes, &misc->w_full);
-            }
             ptx::tma_prefetch_desc(&tmap_x);
             ptx::tma_prefetch_desc(&tmap_y);
         }
     }
     if (warp == 1) ptx::tmem_alloc(&misc->tmem_base, TMEM_COLS);
     ptx::tc_fence_before_sync();
-    __syncthreads();
+    // The producer, whose own barriers are all it needs, only announces itself and starts to load.  (A barrier of its own, used
+    // once: a warp that does not wait here may be at the CTA's last barrier, number 0, before the others have left this one.)
+    if (warp == 0) asm volatile("bar.arrive 6, %0;" ::"n"(NTHREADS) : "memory");
+    else asm volatile("bar.sync 6, %0;" ::"n"(NTHREADS) : "memory");
     ptx::tc_fence_after_sync();
-    const uint32_t tmem_base = misc->tmem_base;
+    const uint32_t tmem_base = misc->tmem_base;              // (not the producer's to read)
     ptx::pdl_trigger();
     // The partner's barriers must exist before anything arrives on them.  Every thread arrives at the cluster barrier
     // here and waits on it much later, right before its warp's first operation on the partner's shared memory (or at
@@ -347,8 +345,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
         // ---------------- producer ----------------
         if (lane == 0) {
             const uint32_t scale_bytes = (uint32_t)(NQ * n_groups * 4);
-            ptx::pdl_wait();                              // X and the K~/V~ block may come from the previous kernel
+            // Weights, X, the K~/V~ block and the request table may all come from the previous kernel.  (While Wq was asked for in front
+            // of the wait a launch of one row tile behind another one took 11.5 us, now 12.5; 8192 rows 14.2, now 14.1.)
+            ptx::pdl_wait();
             TAQ_PROF(1); TAQ_GPROF(28);
+            if (!Q_IN) {
+                ptx::mbar_arrive_expect_tx(&misc->w_full, RAW_BYTES + scale_bytes);
+                ptx::bulk_load(smem + OFF_RAW, wq_blob + L.off_codes + (size_t)col0 * L.row_bytes, RAW_BYTES, &misc->w_full);
+                ptx::bulk_load(smem + OFF_SC, wq_blob + L.off_scales + (size_t)col0 * n_groups * 4, scale_bytes, &misc->w_full);
+            }
             for (int kb = 0; kb < NKB && !Q_IN; ++kb) {   // the whole X tile at once: every K block has its own buffer
                 ptx::mbar_arrive_expect_tx(&misc->a_full[kb], A_TILE);
                 ptx::tma_load_3d(smem + OFF_R0 + kb * A_TILE, &tmap_x, &misc->a_full[kb], kb * BK, row0, zb);

@@ -277,7 +277,6 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restri
             for (int i0 = TPG * KEEP; i0 < n4[u]; i0 += TPG) encode(i0 + t < n4[u] ? w4[u][i0 + t] : make_float4(0.f, 0.f, 0.f, 0.f), i0 + t, i0 + t < n4[u]);
         }
     }
-    __threadfence();      // (a successor may read the blob as soon as the last block has gone, see the layer kernel)
 }
 
 cudaError_t launch_pack_weights(const taq_weight_desc& d, const float* W, const float* bias, void* packed, cudaStream_t stream) {

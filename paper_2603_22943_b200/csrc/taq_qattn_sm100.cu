@@ -348,15 +348,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) qattn_c320_kernel(const __grid_co
     if (warp == 0) {
         // ---------------- producer ----------------
         if (lane == 0) {
-            // Packed weights are written by taq_pack_weights, which never lets its successor start early: they are complete
-            // before this kernel can run at all and are fetched (and expanded) under the previous kernel's tail.
+            ptx::pdl_wait();                              // the weights, X and the K~/V~ block may all come from the previous kernel
+            TAQ_PROF(1); TAQ_GPROF(28);
             const uint8_t* blob = (const uint8_t*)(a.reqs ? a.reqs[zb].Wq : a.wq);
             const uint32_t scale_bytes = (uint32_t)(NQ * n_groups * 4);
             ptx::mbar_arrive_expect_tx(&misc->w_full, RAW_BYTES + scale_bytes);
             ptx::bulk_load(smem + OFF_RAW, blob + L.off_codes + (size_t)col0 * L.row_bytes, RAW_BYTES, &misc->w_full);
             ptx::bulk_load(smem + OFF_SC, blob + L.off_scales + (size_t)col0 * n_groups * 4, scale_bytes, &misc->w_full);
-            ptx::pdl_wait();                              // X (and in general the K~/V~ block) may come from the previous kernel
-            TAQ_PROF(1); TAQ_GPROF(28);
             for (int kb = 0; kb < NKB; ++kb) {            // the whole X tile at once: every K block has its own buffer
                 ptx::mbar_arrive_expect_tx(&misc->a_full[kb], A_TILE);
                 ptx::tma_load_3d(smem + OFF_A + kb * A_TILE, &tmap_x, &misc->a_full[kb], kb * BK, row0, zb);

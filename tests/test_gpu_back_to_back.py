@@ -118,6 +118,8 @@ def test_passes_in_a_row_equal_passes_alone(batch, n_query, channels, heads, w_b
     (2, 1024, 640, 8, 4, 16),
     (2, 1024, 640, 10, 8, 8),
     (2, 700, 320, 8, 8, 16),
+    (2, 700, 320, 8, 4, 16),
+    (2, 700, 320, 8, 4, 8),
 ])
 def test_weights_and_keys_written_right_before_a_pass_are_the_ones_it_uses(batch, n_query, channels, heads, w_bits, a_bits):
     """As when a checkpoint is swapped in: two checkpoints' blobs are written in turn over the same memory (by an elementwise
