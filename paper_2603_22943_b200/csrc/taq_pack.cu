@@ -2,6 +2,7 @@
 // Integer codes are compared bit for bit with the CPU definition, so every floating-point step here is an
 // explicit IEEE binary32 operation (__fdiv_rn, rintf); nothing may be contracted or approximated.
 #include "taq_common.cuh"
+#include "taq_ptx.cuh"
 
 namespace taq {
 
@@ -94,9 +95,11 @@ __device__ __forceinline__ uint2 codes8(const uint4& v, float s, float r_lo, flo
 // row is short enough (KEEP x 256 columns), so that the row is read once; KEEP as small as the row allows.  Same results as quantize_rows_kernel.
 template <int KEEP>
 __global__ void __launch_bounds__(256) quantize_rows_f16_kernel(const __half* x, long long rows, int cols, int8_t* codes, float* scales) {
-    // The successor (the integer GEMM) may start its prologue now, and read its weights at once: this kernel starts when everything
-    // before it has finished.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Starts early; its rows may come from the predecessor, and its codes go where the predecessor's predecessor may still read.
+    // Only behind the wait may the successor (the integer GEMM) start: it reads its weights at once, which whatever ran before
+    // this kernel may have written.
+    ptx::pdl_wait();
+    ptx::pdl_trigger();
     const int lane = threadIdx.x & 31;
     const long long warps_total = (long long)gridDim.x * (blockDim.x >> 5);
     const int chunks = cols / 8;                                 // 16-byte chunks of a row
@@ -138,10 +141,7 @@ cudaError_t launch_quantize_rows_f16(const __half* x, long long rows, int cols, 
     long long blocks = (rows + 7) / 8;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
     auto* kern = cols <= 512 ? quantize_rows_f16_kernel<2> : cols <= 768 ? quantize_rows_f16_kernel<3> : cols <= 1280 ? quantize_rows_f16_kernel<5> : quantize_rows_f16_kernel<8>;
-    // (An ordinary launch: as an early starter behind the attention kernel, several layer passes in a row, it read rows of O that were
-    // not there yet.)
-    kern<<<(unsigned)blocks, 256, 0, stream>>>(x, rows, cols, codes, scales);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)blocks), dim3(256), 0, stream, x, rows, cols, codes, scales);
 }
 
 // ---- helpers of the token-sensitivity sweep (Eq. 1) -------------------------------------------------------------
