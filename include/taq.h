@@ -341,8 +341,10 @@ taq_status taq_poll_device_status(void* stream, int32_t* block_id_out);
  *
  * Which kernel family served the calls so far.  The library prefers its tensor-core kernels and keeps generic
  * CUDA-core kernels for shapes they do not cover; the generic ones are 10-40x slower, so a caller (or a test) that
- * cares can check that none ran.  Counters are per process, counted on the host at launch time, and are not
- * synchronised with the GPU.  counts_out: int64 [n]; entries beyond TAQ_N_KERNEL_FAMILIES read 0. */
+ * cares can check that none ran.  A family's counter goes up by one per product, attention or layer pass that it serves:
+ * the launches of that family, except that one tensor-core launch may serve the K and the V projection together and counts
+ * two.  Quantizers, packing and operand images have no family.  Counters are per process, counted on the host at launch
+ * time, and are not synchronised with the GPU.  counts_out: int64 [n]; entries beyond TAQ_N_KERNEL_FAMILIES read 0. */
 enum {
     TAQ_KERNEL_LINEAR_TENSOR = 0,          /* dequant-GEMM on tcgen05 (also the integer-activation variant) */
     TAQ_KERNEL_LINEAR_GENERIC = 1,         /* dequant-GEMM on CUDA cores */

@@ -452,7 +452,7 @@ KERNEL_FAMILIES = ("linear_tensor", "linear_generic", "attention_tensor", "atten
 
 
 def taq_dispatch_counts() -> dict:
-    """Launches per kernel family since the last taq_dispatch_reset()."""
+    """Products, attentions and layer passes per kernel family since the last taq_dispatch_reset() (a merged K/V launch counts two)."""
     arr = (C.c_int64 * len(KERNEL_FAMILIES))()
     _check(lib().taq_dispatch_counts(arr, len(KERNEL_FAMILIES)))
     return {k: int(arr[i]) for i, k in enumerate(KERNEL_FAMILIES)}

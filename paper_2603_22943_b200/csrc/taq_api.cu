@@ -92,9 +92,9 @@ static Workspace workspace_layout(const taq_layer_desc* d, int n_requests) {
     return w;
 }
 
-// Launches per kernel family since the last taq_dispatch_reset (host-side counters; see taq_dispatch_counts in taq.h).
+// What each kernel family has served since the last taq_dispatch_reset (host-side counters; see taq_dispatch_counts in taq.h).
 static std::atomic<long long> g_dispatch[TAQ_N_KERNEL_FAMILIES];
-static void count_launch(int family) { g_dispatch[family].fetch_add(1, std::memory_order_relaxed); }
+static void count_launch(int family, int served = 1) { g_dispatch[family].fetch_add(served, std::memory_order_relaxed); }
 
 static taq_status run_linear(const LinearArgs& a, int n_z, cudaStream_t st) {
     cudaError_t e;
@@ -112,15 +112,13 @@ static taq_status run_linear_i8(const LinearArgs& a, cudaStream_t st) {
 }
 
 // K/V projection with Eq. 2.  On the tensor cores one launch computes both and writes the operand images as well; the generic
-// kernel takes a launch for each, and the images are built from its rows afterwards.  (The dispatch counter counts
-// projections, so that a merged launch reads 2.)
+// kernel takes a launch for each, and the images are built from its rows afterwards.
 static taq_status run_kv_projection(const taq_layer_desc& d, LinearArgs a, const void* Wk, const void* Wv, int n_blocks, int n_z, cudaStream_t st) {
     a.w = Wk; a.w2 = Wv;
     LinearArgs t = a;                      // there a row tile is one sequence: z = sequence or request
     t.rows = d.n_ctx;
     if (sm100_linear_supported(t)) {
-        count_launch(TAQ_KERNEL_LINEAR_TENSOR);
-        count_launch(TAQ_KERNEL_LINEAR_TENSOR);
+        count_launch(TAQ_KERNEL_LINEAR_TENSOR, 2);
         cudaError_t e = launch_linear_sm100(t, n_blocks, st);
         return e == cudaSuccess ? TAQ_OK : cuda_fail(e, "K/V projection launch");
     }
