@@ -498,8 +498,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                         for (int i = 1; i < HK / 8; ++i) ptx::reg_fence8(u8[i]);
                     }
                     ptx::tc_fence_before_sync();
-                    const OperandConsts* cst = C::SPLIT_KV ? reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % 3) * C::CST_SLOT)
-                                                           : reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
+                    const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % 3) * C::CST_SLOT);
                     float m_loc, l_loc;
                     softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, sq, T, key0, e, m_loc, l_loc);
                     trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
@@ -608,8 +607,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             ptx::tc_fence_before_sync();
 
             // ---- this thread's half of the softmax; the row's two threads then exchange (max, sum) ----
-            const OperandConsts* cst = C::SPLIT_KV ? reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % 3) * C::CST_SLOT)
-                                                   : reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
+            const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
             float e[HK];
             float m_loc, l_loc;
             softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, sq, T, key0, e, m_loc, l_loc);

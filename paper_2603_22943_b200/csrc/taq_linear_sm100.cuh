@@ -863,8 +863,12 @@ cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const Line
     auto of_types = [&](auto out, auto ctas_c) -> Kernel {
         constexpr Out O = decltype(out)::value;
         constexpr Ctas C = decltype(ctas_c)::value;
-        return i8 ? (w8 ? linear_sm100_kernel<BN, true, true, O, C> : linear_sm100_kernel<BN, true, false, O, C>)
-                  : (w8 ? linear_sm100_kernel<BN, false, true, O, C> : linear_sm100_kernel<BN, false, false, O, C>);
+        if constexpr (C == Ctas::SPLIT) {      // (8-bit weights have one scale group, which integer activations keep in one accumulation)
+            if (i8 && w8) return nullptr;
+        } else {
+            if (i8 && w8) return linear_sm100_kernel<BN, true, true, O, C>;
+        }
+        return i8 ? linear_sm100_kernel<BN, true, false, O, C> : w8 ? linear_sm100_kernel<BN, false, true, O, C> : linear_sm100_kernel<BN, false, false, O, C>;
     };
     auto of_out = [&](auto out) -> Kernel {
         constexpr Ctas MANY = decltype(out)::value == Out::KV ? Ctas::ONE : Ctas::MANY;          // (K~/V~ tiles: one per CTA)
@@ -873,6 +877,7 @@ cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const Line
     };
     const Kernel kern = a.epi == EPI_KV ? of_out(std::integral_constant<Out, Out::KV>{}) : a.epi == EPI_Q8_HEAD ? of_out(std::integral_constant<Out, Out::Q8>{}) :
                         a.epi == EPI_F32 ? of_out(std::integral_constant<Out, Out::F32>{}) : of_out(std::integral_constant<Out, Out::F16>{});
+    if (!kern) return cudaErrorNotSupported;
     cudaError_t e = allow_shared_memory((const void*)kern, SMEM_LIMIT, limit_set[(a.epi * 3 + (int)ctas) * 4 + i8 * 2 + w8]);
     if (e != cudaSuccess) return e;
     if (lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(grid), dim3(lay.nsplit * (lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), smem_bytes, stream, tmap, a, lay);
