@@ -360,8 +360,8 @@ void taq_dispatch_reset(void);
 
 /* The launch plan the tensor-core dequant-GEMM would take for a problem (host arithmetic only; nothing is launched
  * and no GPU is needed).  plan_out: int32 [10] = {tile width BN (0: the tensor-core kernel does not take the
- * problem), ring stages, weight mode (0 codes staged once, 1 codes are the operand, 2 codes sliced per K block), bytes
- * of the ring, bytes of the ring the epilogue reuses as its staging area, offset of the staged codes, offset of the
+ * problem), ring stages in k-blocks, CTAs that share the K loop of a tile (1, 2 or 4), bytes of the ring, bytes of the
+ * ring the epilogue reuses as its staging area, offset of the scales (the first section behind the ring), offset of the
  * bias, offset of the barriers, total shared memory, shared-memory limit}.  Every region must lie inside `total`, the
  * staging area inside the ring.  int8_activations / batched select the variant as taq_quantized_linear_i8 and the
  * per-request calls do. */

@@ -462,7 +462,7 @@ def taq_dispatch_reset() -> None:
     lib().taq_dispatch_reset()
 
 
-LINEAR_PLAN_FIELDS = ("bn", "nstage", "mode", "ring_bytes", "staging_bytes", "off_raw", "off_bias", "off_bars", "total", "limit")
+LINEAR_PLAN_FIELDS = ("bn", "nstage", "split", "ring_bytes", "staging_bytes", "off_raw", "off_bias", "off_bars", "total", "limit")
 
 
 def taq_linear_plan(desc: "WeightDesc", rows: int, out_kind: int, heads: int = 1, int8_activations: bool = False, batched: bool = False) -> dict:

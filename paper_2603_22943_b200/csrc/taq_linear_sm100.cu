@@ -211,9 +211,9 @@ bool sm100_linear_supported(const LinearArgs& a) {
     return choose(a, 1).bn != 0 && encode_tiled_fn() != nullptr;
 }
 
-// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed): tile width, ring depth in k-blocks, how the
-// codes reach the CTA (0: from global memory through registers), and the byte ranges of shared memory that the rings,
-// the epilogue's staging area in them and the fixed sections occupy.  out: {bn, nstage, mode, ring_bytes, staging_bytes,
+// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed): tile width, ring depth in k-blocks, CTAs that
+// share a tile's K loop, and the byte ranges of shared memory that the rings,
+// the epilogue's staging area in them and the fixed sections occupy.  out: {bn, nstage, split, ring_bytes, staging_bytes,
 // off_raw (the first fixed section), off_bias, off_bars, total, limit}.  bn = 0: the tensor-core kernel does not take it.
 void linear_plan_of(const LinearArgs& a, int out[10]) {
     for (int i = 0; i < 10; ++i) out[i] = 0;
@@ -222,7 +222,7 @@ void linear_plan_of(const LinearArgs& a, int out[10]) {
     const Choice c = choose(a, 1);
     if (c.bn == 0) return;
     const Plan& P = c.lay.plan;
-    out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = 0; out[3] = P.ring_bytes; out[4] = c.staged;
+    out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = c.lay.nsplit; out[3] = P.ring_bytes; out[4] = c.staged;
     out[5] = P.off_scales; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
 }
 

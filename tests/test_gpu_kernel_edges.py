@@ -15,31 +15,47 @@ import taq_testlib as tl
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads", [
-    (1, 640, 640, 4, 128, 8),          # one row, 80-wide tiles
-    (129, 640, 640, 8, 0, 10),         # a second row tile of one row, 64-wide tiles
-    (2047, 640, 640, 4, 128, 10),      # 128-wide tiles, one per CTA
-    (5616, 640, 640, 4, 128, 10),      # ... and several per CTA
-    (5505, 640, 640, 8, 0, 8),         # 80-wide tiles, several per CTA, a last row tile of one row
-    (4225, 640, 640, 4, 128, 8),       # 160-wide tiles, several per CTA
-    (64, 1280, 1280, 4, 128, 20),      # a cluster per 64-wide tile, shares of whole groups
-    (300, 1280, 1280, 8, 0, 20),       # ... and of k-blocks
-    (129, 1280, 1280, 4, 0, 8),        # heads over two tiles, shares of k-blocks
-    (129, 1280, 1280, 8, 0, 8),        # a cluster per 160-wide tile
-    (1100, 1280, 1280, 8, 0, 8),       # 160-wide tiles, one per CTA
-    (97, 320, 192, 4, 128, 8),         # an odd number of k-blocks, a short last group
-    (200, 320, 64, 8, 0, 8),           # one k-block
+def layout(rows, n_out, k_in, bits, group, kind, heads=1, int8_activations=False):
+    """Tile width of a launch, "x2" or "x4" where so many CTAs share a tile, "+" where a CTA walks several tiles (148 SMs)."""
+    plan = tb.taq_linear_plan(tb.weight_desc(n_out, k_in, bits, group), rows, kind, heads=heads, int8_activations=int8_activations)
+    ctas = (rows + 127) // 128 * (n_out // plan["bn"]) * plan["split"] if plan["bn"] else 0
+    return f"{plan['bn']}" + (f"x{plan['split']}" if plan["split"] > 1 else "") + ("+" if ctas > 148 else "")
+
+
+# (the layouts of the fp16 and fp32 outputs and of the per-head int8 output: a change of the rule that chooses them says here which
+# of them is no longer run)
+@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
+    (1, 640, 640, 4, 128, 8, "64", "80"),              # one row
+    (129, 640, 640, 8, 0, 10, "64", "64"),             # a second row tile of one row
+    (2047, 640, 640, 4, 128, 10, "80", "128"),
+    (5616, 640, 640, 4, 128, 10, "64+", "64+"),
+    (5505, 640, 640, 8, 0, 8, "64+", "80+"),           # a last row tile of one row
+    (4225, 640, 640, 4, 128, 8, "160", "160"),
+    (64, 1280, 1280, 4, 128, 20, "64x2", "64x2"),      # shares of whole groups
+    (300, 1280, 1280, 8, 0, 20, "64x2", "64x2"),       # ... and of k-blocks
+    (129, 1280, 1280, 4, 0, 8, "64x2", "80x2"),        # heads over two tiles
+    (129, 1280, 1280, 8, 0, 8, "64x2", "160x2"),
+    (1100, 1280, 1280, 8, 0, 8, "80", "160x2"),
+    (97, 320, 192, 4, 128, 8, "64", "80"),             # an odd number of k-blocks, a short last group
+    (200, 320, 64, 8, 0, 8, "80", "80"),               # one k-block
+    (64, 1280, 1280, 8, 0, 8, "64x2", "160x4"),
+    (3000, 1280, 320, 4, 128, 20, "128+", "128+"),
+    (4300, 1280, 1280, 4, 128, 8, "160+", "160+"),
+    (1, 640, 768, 4, 128, 8, "64x2", "80x2"),
 ])
-def test_linear_tiles(rows, n_out, k_in, bits, group, heads):
-    for kind in (tb.TAQ_OUT_F16, tb.TAQ_OUT_F32, tb.TAQ_OUT_INT8_HEAD_ROWS):
-        assert tb.taq_linear_plan(tb.weight_desc(n_out, k_in, bits, group), rows, kind, heads=heads)["bn"] > 0
+def test_linear_tiles(rows, n_out, k_in, bits, group, heads, dense, per_head):
+    for kind in (tb.TAQ_OUT_F16, tb.TAQ_OUT_F32):
+        assert layout(rows, n_out, k_in, bits, group, kind) == dense
+    assert layout(rows, n_out, k_in, bits, group, tb.TAQ_OUT_INT8_HEAD_ROWS, heads) == per_head
     layer.test_quantized_linear(rows, n_out, k_in, bits, group, heads)
 
 
-@pytest.mark.parametrize("rows,k_in,n_out,bits,group", [
-    (1, 320, 320, 4, 128), (257, 1280, 1280, 4, 128), (4225, 640, 640, 4, 128), (300, 656, 640, 8, 0),
+@pytest.mark.parametrize("rows,k_in,n_out,bits,group,dense", [
+    (1, 320, 320, 4, 128, "64"), (257, 1280, 1280, 4, 128, "64"), (4225, 640, 640, 4, 128, "160"), (300, 656, 640, 8, 0, "64"),
+    (1, 1280, 1280, 4, 128, "64x2"), (5505, 64, 320, 4, 128, "64+"), (3000, 320, 1280, 4, 128, "128+"),
 ])
-def test_integer_linear_tiles(rows, k_in, n_out, bits, group):
+def test_integer_linear_tiles(rows, k_in, n_out, bits, group, dense):
+    assert layout(rows, n_out, k_in, bits, group, tb.TAQ_OUT_F32, int8_activations=True) == dense
     int8_activations.test_integer_gemm_equals_the_integer_definition(rows, k_in, n_out, bits, group)
 
 
