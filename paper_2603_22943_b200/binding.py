@@ -202,8 +202,8 @@ def taq_packed_weight_bytes(desc: WeightDesc) -> int:
 def taq_pack_weights(desc: WeightDesc, W: torch.Tensor, bias: Optional[torch.Tensor] = None,
                      packed: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """W fp32 [n_out,k_in] -> packed blob (uint8 tensor)."""
-    nbytes = taq_packed_weight_bytes(desc)
     if packed is None:
+        nbytes = taq_packed_weight_bytes(desc)
         if nbytes == 0:
             _check(lib().taq_pack_weights(C.byref(desc), _ptr(W), _ptr(bias), None, 0, _stream(stream)))
         packed = torch.zeros(nbytes, dtype=torch.uint8, device=W.device)
