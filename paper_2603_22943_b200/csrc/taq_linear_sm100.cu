@@ -122,7 +122,12 @@ bool tile_carries(const LinearArgs& a, const Problem& p, int bn) {
 // and scale group, what a tile costs a CTA that walks several, and the exchange of partial sums when the K loop is split (a
 // part that grows with the CTAs that exchange at one time).  The numbers are a least-squares fit to 351 measured launches of
 // 64 to 8192 rows, 640 and 1280 channels, W4 and W8, every width and split that can carry them (5 % rms); the layouts it picks
-// are on average 0.5 % slower than the best one measured.
+// are on average 0.5 % slower than the best one measured.  It decides beyond that, too.  320 channels, 32 to 8192 rows, W4 and W8,
+// fp16 and per-head int8 rows: of 20 launches 17 are within 2 % of the best layout, two within 4 %, and 8192 W8 rows per head
+// take 7.6 us where 80-wide tiles take 6.9.  Two terms are set by hand: 0.2 us more for four CTAs than for two, and for K~/V~ an
+// epilogue that grows with the tile's width (0.008 us a column).  Of 30 projections of 1, 2 and 8 prompts, 320 to 1280 channels,
+// contexts of 768 and 2048, W4 and W8, 28 are within 2 % of the best layout; the other two (1280 channels, W4, 1 and 2
+// prompts) the rule on narrow contexts below keeps from it.
 struct Pace { int bn; double fixed, kb, group, tile, q8, split, exchange; };
 constexpr Pace PACES[4] = {
     {160, 3.08, 0.320, 0.248, 1.54, 0.72, 0.95, 1.72},
@@ -154,8 +159,10 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
         const long long tiles = p.row_tiles * (a.n_out / bn) * p.ncols_factor * (long long)n_z;
         if (tiles > (1 << 30)) continue;
         for (int ns : {1, 2, 4}) {
-            // (K~/V~ of a 768-wide context gain nothing from a split, which leaves a prompt's bits the same in every batch; of a
-            // 2048-wide one a split takes 13.9 us to 10.2 us at C = 640.)
+            // (K~/V~: the line lies between the two widths of text contexts in use.  From a 768-wide context a split gains 0 to 2 % at
+            // 320 and 640 channels (one prompt, W4: 9.8 us, in halves 9.7) and at 1280 10 % with W4, nothing with W8 (14.7
+            // and 13.3 us, 13.2 and 13.1); unsplit, a prompt's bits are the same in every batch.  Of a 2048-wide one four CTAs take
+            // 14.6 us to 11.2 at 640 channels.)
             if (ns > 1 && a.epi == EPI_KV && a.k_in < 1024) continue;
             if (ns > 1 && ((p.i8 && p.n_groups == 1) || (p.n_groups == 1 ? p.n_kb : p.n_groups) < ns || tiles * ns > 148)) continue;    // (integer activations: a group's sum stays one exact int32 accumulation)
             const bool persistent = a.epi != EPI_KV && tiles * ns > 148;           // (K~/V~ tiles are assembled in the rings: one per CTA)

@@ -147,7 +147,8 @@ __device__ __forceinline__ typename Code<I8, W8>::T zero_codes() {
 
 // The output and the CTAs' share of the work are compiled in, not looked up: most launches last 6 to 9 us, and a kernel without
 // the other outputs' code took 0.3 to 0.6 us less of them than one kernel for all (2048 x 640 x 640: Q~ 6.8 -> 6.1 us, fp16
-// 6.25 -> 5.8 us; 8192 rows, Q~: 16.2 -> 15.6 us).
+// 6.25 -> 5.8 us; 8192 rows, Q~: 16.2 -> 15.6 us.  Since a launch that does not know its predecessor waits for its weights, and over
+// buffers larger than L2, the three take 6.7, 6.2 and 17.4 us.)
 enum class Out { F16, F32, Q8, KV };     // fp16 or fp32 rows; int8 rows with a scale per head; K~/V~
 enum class Ctas { ONE, MANY, SPLIT };    // a tile per CTA; several tiles per CTA; a cluster of two or four CTAs per tile
 
