@@ -159,3 +159,69 @@ def test_weights_and_keys_written_right_before_a_pass_are_the_ones_it_uses(batch
         for _ in range(2):
             graph.replay()
             check(f"from a graph, {last} written last")
+
+
+@pytest.mark.parametrize("n_requests,n_query,channels", [(3, 700, 320), (1, 64, 320), (2, 300, 640)])
+def test_request_table_written_right_before_a_batched_pass_is_the_one_it_uses(n_requests, n_query, channels):
+    """Two sets of requests' tables are written in turn over the same memory, right before the pass that reads them."""
+    gen = torch.Generator("cuda").manual_seed(5)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    desc = tb.layer_desc(1, n_query, channels, 8, 77, 768, 4, 128, max_trigger=2)
+    pack = lambda n_out, k_in: tb.taq_pack_weights(tb.weight_desc(n_out, k_in, 4, 128), normal(n_out, k_in) / k_in ** 0.5)
+    mask = torch.zeros((n_requests, 77), dtype=torch.uint8, device="cuda")
+    mask[:, 4:6] = 1
+    x, ws = normal(n_requests, n_query, channels).half(), torch.zeros(tb.taq_workspace_bytes(desc, n_requests), dtype=torch.uint8, device="cuda")
+    keep, tables, want = [], [], []
+    for _ in range(2):
+        kv = torch.zeros((n_requests, tb.taq_kv_bytes(desc)), dtype=torch.uint8, device="cuda")
+        wkv = [(pack(channels, 768), pack(channels, 768), kv[r], mask[r]) for r in range(n_requests)]
+        tb.taq_kv_project_batched(desc, tb.make_request_table(wkv, "cuda"), n_requests, normal(n_requests, 77, 768).half())
+        use = [(pack(channels, channels), pack(channels, channels), kv[r], mask[r]) for r in range(n_requests)]
+        keep.append((wkv, use))
+        tables.append(tb.make_request_table(use, "cuda"))
+        y = torch.full((n_requests, n_query, channels), float("nan"), dtype=torch.float16, device="cuda")
+        tb.taq_layer_forward_batched(desc, tables[-1], n_requests, x, y, ws)
+        torch.cuda.synchronize()
+        want.append(y)
+    place, complements = tables[0].clone(), [~t for t in tables]         # (a valid table from the start)
+    ys = [torch.full_like(want[0], float("nan")) for _ in range(2 * ROUNDS)]
+    torch.cuda.synchronize()
+    for i, y in enumerate(ys):
+        torch.bitwise_not(complements[i % 2], out=place)
+        tb.taq_layer_forward_batched(desc, place, n_requests, x, y, ws)
+    torch.cuda.synchronize()
+    tb.taq_poll_device_status()
+    for i, y in enumerate(ys):
+        assert torch.equal(y.view(torch.int16), want[i % 2].view(torch.int16)), i
+
+
+@pytest.mark.parametrize("channels,heads,ctx_dim,w_bits,a_bits", [(320, 8, 768, 4, 16), (1280, 8, 768, 8, 8), (640, 10, 2048, 4, 8), (640, 10, 2048, 4, 16)])
+def test_projection_weights_written_right_before_the_call_are_the_ones_it_uses(channels, heads, ctx_dim, w_bits, a_bits):
+    gen = torch.Generator("cuda").manual_seed(6)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    group = 128 if w_bits == 4 else 0
+    desc = tb.layer_desc(2, 64, channels, heads, 77, ctx_dim, w_bits, group, max_trigger=2)
+    project = tb.taq_kv_project_a8 if a_bits == 8 else tb.taq_kv_project
+    mask = torch.zeros((2, 77), dtype=torch.uint8, device="cuda")
+    mask[:, 4:6] = 1
+    ctx = normal(2, 77, ctx_dim).half()
+    weights = [[tb.taq_pack_weights(tb.weight_desc(channels, ctx_dim, w_bits, group), normal(channels, ctx_dim) / ctx_dim ** 0.5) for _ in range(2)] for _ in range(2)]
+    new_kv = lambda: torch.zeros(tb.taq_kv_bytes(desc), dtype=torch.uint8, device="cuda")
+    want = []
+    for wk, wv in weights:
+        want.append(new_kv())
+        project(desc, ctx, wk, wv, mask, want[-1])
+        torch.cuda.synchronize()
+    complements = [[~w for w in pair] for pair in weights]
+    place = [torch.zeros_like(w) for w in weights[0]]
+    for order in ((0, 1), (1, 0)):
+        kvs = [new_kv() for _ in range(2 * ROUNDS)]
+        torch.cuda.synchronize()
+        for i, kv in enumerate(kvs):
+            for k in order:
+                torch.bitwise_not(complements[i % 2][k], out=place[k])
+            project(desc, ctx, place[0], place[1], mask, kv)
+        torch.cuda.synchronize()
+        tb.taq_poll_device_status()
+        for i, kv in enumerate(kvs):
+            assert torch.equal(kv, want[i % 2]), (order, i)
