@@ -777,8 +777,11 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         b_lo += 2 * TL::B_TILE >> 4;
                         if (++sa == nsa) { sa = 0; pha ^= 1; a_lo = a_lo0; }
                         if (++sb == nsb) { sb = 0; phb ^= 1; b_lo = b_lo0; }
-                        next_b = ptx::mbar_try_wait(&bars->full_b[sb], phb);
-                        next_a = ptx::mbar_try_wait(&bars->full_a[sa], pha);
+                        // (a try_wait suspends the thread for some time: none for a pair that does not come)
+                        if (todo > 0) {
+                            next_b = ptx::mbar_try_wait(&bars->full_b[sb], phb);
+                            next_a = ptx::mbar_try_wait(&bars->full_a[sa], pha);
+                        }
                     }
                 }
                 if (!ok) give_up();
