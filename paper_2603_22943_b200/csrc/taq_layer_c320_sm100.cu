@@ -19,7 +19,7 @@
 //            finished lie; every tile is sent to the partner CTA as soon as it is complete.  The K steps over the CTA's
 //            own tiles run while the partner's are in flight (each CTA begins with its own channels; every scale group
 //            still has its own accumulator).  The Wout tiles are expanded during phase 3 into the dead K~ buffers, later
-//            into the dead V~^T buffers.  Y leaves as one TMA tensor store per head group of 40 channels.
+//            into the dead V~^T buffers.  Y leaves through shared memory in runs of 320 bytes.
 // Shared memory is reused: X tile -> Q~ / P tiles -> O tiles -> Y staging; weight tiles -> K~ and V~^T tiles -> weight ring.
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
@@ -55,7 +55,7 @@ constexpr int O_TILE = ROWS * 64;               // 8 KB: 32 channels of O (64-by
 constexpr int N_OTILE = KIN / 32;
 constexpr int K_BYTES = TP * 128;               // 10 KB: one head's K~ image
 constexpr int VT_BLOCK = DP * 128, VT_BYTES = 2 * VT_BLOCK;     // 12 KB: one head's V~^T image (keys 0..63, 64..79)
-constexpr int Y_STAGE = ROWS * D * 2;           // 10 KB: 40 channels of Y, dense rows of 80 bytes
+constexpr int Y_PITCH = NQ * 2 + 16;            // staged rows of Y
 constexpr int RAW_BYTES = NQ * (KIN / 2);       // 25600: packed codes of the CTA's 160 channels
 constexpr int SCALE_BYTES = 2048;               // >= NQ * MAX_GROUPS * 4
 
@@ -73,7 +73,7 @@ static_assert(OFF_PB + HG * PB_TILE <= OFF_R1, "P tiles fit into the X tile");
 static_assert(N_OTILE * O_TILE <= NKB * A_TILE, "O tiles fit into the X tile");
 static_assert(HG * VT_BYTES <= 3 * B_TILE && 2 * B_TILE <= 3 * B_TILE, "V~^T tiles fit into the phase-1 ring");
 static_assert(HG * K_BYTES == 2 * B_TILE, "the K~ tiles are exactly two ring stages");
-static_assert(HG * Y_STAGE <= NKB * A_TILE, "Y staging fits into the X tile");
+static_assert(ROWS * Y_PITCH <= NKB * A_TILE, "Y staging fits into the X tile");
 static_assert(NQ * MAX_GROUPS * 4 <= SCALE_BYTES, "scale table");
 
 constexpr int NS4 = 4;                          // ring stages of phase 4
@@ -112,6 +112,7 @@ struct LayerArgs {
     const void* kv;             // blocks [B] (single problem)
     const taq_request* reqs;    // nullable; then one sequence per request
     __half* o;                  // [z][N][C]  (query-attention variant)
+    __half* y;                  // [z][N][C]  (layer variant)
     const void* q;              // attention-only variant: Q~ codes (int8) or Q (fp16) [z][N][C] ...
     const float* q_scales;      // ... and the row scales [z][N][H] (q_bits = 8)
     int n_query, heads, n_ctx, max_trigger, group, q_bits, p_bits;
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             misc->abort_flag = 0;
             if (FUSE_OUT) ptx::mbar_arrive_expect_tx(&misc->o_all, (N_OTILE / 2) * O_TILE);     // the partner's five tiles
             ptx::tma_prefetch_desc(&tmap_x);
-            ptx::tma_prefetch_desc(&tmap_y);
+            if (!FUSE_OUT) ptx::tma_prefetch_desc(&tmap_y);
         }
     }
     if (warp == 1) ptx::tmem_alloc(&misc->tmem_base, TMEM_COLS);
@@ -784,11 +785,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             fold_groups(1, rank != 0);
             if (wt == 0) TAQ_PROF(36);
             // Every MMA of phase 4 is complete, and the partner has received this CTA's O tiles (peer_got): region 0 is
-            // free.  The head group's 128 x 40 block of Y is staged there as dense rows of 80 bytes (conflict-free for
-            // row-per-lane 16-byte writes) and leaves as one TMA tensor store; rows beyond n_query are clipped.
+            // free.  The four warps of a lane quarter (one per head) put their 40 channels of 32 rows side by side (rows padded so
+            // that a row per lane is free of bank conflicts), then store them with neighbouring lanes on neighbouring chunks, 320
+            // bytes of a row in a run.  (With a TMA tensor store per head, rows of 80 bytes, 2 700 cycles went by between
+            // the last fold and the end of the read that the CTA has to wait for, now 2 000, most of them 40 KB on their way out at 32 bytes a
+            // cycle: 8192 rows 14.08 -> 13.62 us, 64 requests of 4096 rows 411 -> 401.)
             ok = ok && ptx::mbar_wait(&misc->peer_got, 0, WL) && !misc->abort_flag;
             if (!ok) give_up();
-            unsigned char* stage = smem + OFF_R0 + hi * Y_STAGE;
+            unsigned char* stage = smem + OFF_R0 + q4 * 32 * Y_PITCH;
             if (ok) {
                 const float* bias = reinterpret_cast<const float*>(smem + OFF_BIAS) + cb;
 #pragma unroll
@@ -796,15 +800,19 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
                     float f[8];
 #pragma unroll
                     for (int e2 = 0; e2 < 8; ++e2) f[e2] = y[c + e2] + bias[c + e2];
-                    *reinterpret_cast<uint4*>(stage + r * (D * 2) + c * 2) = pack8(f);
+                    *reinterpret_cast<uint4*>(stage + lane * Y_PITCH + (cb + c) * 2) = pack8(f);
                 }
             }
-            ptx::fence_proxy_async_smem();
-            asm volatile("bar.sync %0, 128;" ::"r"(2 + hi) : "memory");
-            if (q4 == 0 && lane == 0 && !misc->abort_flag) {
-                ptx::tma_store_3d(&tmap_y, stage, col0 + cb, row0, zb);
-                ptx::bulk_store_commit();
-                ptx::bulk_store_wait_read();                     // shared memory is given back only after the store has read it
+            asm volatile("bar.sync %0, 128;" ::"r"(2 + q4) : "memory");
+            {
+                constexpr int N = NQ / 8;                        // 16-byte chunks of a row
+                __half* out = a.y + ((size_t)zb * a.n_query + row0 + q4 * 32) * KIN + col0;
+                const int left = ok ? a.n_query - (row0 + q4 * 32) : 0;
+#pragma unroll
+                for (int i = 0; i < N / 4; ++i) {
+                    const int j = hi * 32 + lane + 128 * i, rr = j / N, part = j - rr * N;
+                    if (rr < left) *reinterpret_cast<uint4*>(out + (size_t)rr * KIN + part * 8) = *reinterpret_cast<const uint4*>(stage + rr * Y_PITCH + part * 16);
+                }
             }
             if (wt == 0) { TAQ_PROF(37); TAQ_GPROF(27); }
             ptx::cluster_wait();
@@ -867,22 +875,21 @@ static cudaError_t launch_c320(const taq_layer_desc& d, const __half* x, const v
     const cuuint32_t box[3] = {BK, ROWS, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     const bool fuse_out = y != nullptr, q_in = q != nullptr;
-    __half* out = fuse_out ? y : o;
     // (the attention-only variant loads no X: its map is built on the output so that the argument is a valid map)
-    CUresult r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, q_in ? (void*)out : (void*)const_cast<__half*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    CUresult r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, q_in ? (void*)o : (void*)const_cast<__half*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     LayerArgs a{};
-    a.wq = wq; a.kv = kv; a.reqs = reqs; a.o = o; a.wout = wout; a.q = q; a.q_scales = q_scales;
+    a.wq = wq; a.kv = kv; a.reqs = reqs; a.o = o; a.y = y; a.wout = wout; a.q = q; a.q_scales = q_scales;
     a.n_query = d.n_query; a.heads = d.heads; a.n_ctx = d.n_ctx; a.max_trigger = d.max_trigger; a.group = d.w_group; a.q_bits = d.q_bits; a.p_bits = d.p_bits;
     a.wait_cycles = g_wait_cycles;
     a.status = status;
     dim3 grid((d.n_query + ROWS - 1) / ROWS, d.heads / HG, n_z);
     const int tail = d.n_ctx > 72 ? 72 : d.n_ctx > 64 ? 64 : 0;     // first key that can lie beyond the context (the kernel masks from there on)
-    CUtensorMap tmap_y;                               // the output (Y, or O of the variants without to_out), stored per head group
-    {
+    CUtensorMap tmap_y = tmap;                        // the output of the variants without to_out, stored per head group
+    if (!fuse_out) {
         const cuuint32_t ybox[3] = {D, ROWS, 1};      // one head group: 40 channels = 80 bytes per row, dense in shared memory
-        r = enc(&tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, out, dims, strides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        r = enc(&tmap_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, o, dims, strides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     }

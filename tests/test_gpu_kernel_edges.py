@@ -4,6 +4,7 @@ smallest and largest contexts; the packing kernel's group lengths."""
 from dataclasses import replace
 
 import pytest
+import torch
 
 import test_gpu_layer as layer
 import test_gpu_quantizers as quantizers
@@ -77,3 +78,19 @@ def test_kv_projection(channels, heads, ctx_dim, n_ctx, batch, w_bits):
 ])
 def test_pack_group_lengths(n_out, k_in, bits, group):
     quantizers.test_pack_weights_codes_bit_exact(n_out, k_in, bits, group)
+
+
+@pytest.mark.parametrize("n_query", [1, 31, 33, 127, 129, 160, 257])
+def test_one_kernel_layer_writes_its_rows_only(n_query):
+    """C = 320: the rows of Y leave in quarters of a tile; rows of two sequences side by side, nothing beyond the last."""
+    shape = synth.shrink(synth.config2(), n_query)
+    data = synth.make_layer(shape)
+    _, parts = tl.gpu_layer(shape, data, return_parts=True)
+    n = shape.rows * shape.channels
+    buf = torch.full((n + 2048,), -7.0, dtype=torch.float16, device="cuda")
+    P = parts["packed"]
+    tb.taq_layer_forward(parts["desc"], tl.dev(data["X"]), P["Wq"], P["Wout"], parts["kv"], parts["mask"], buf[1024: 1024 + n])
+    tb.taq_poll_device_status()
+    assert bool((buf[:1024] == -7.0).all()) and bool((buf[1024 + n:] == -7.0).all())
+    y = buf[1024: 1024 + n].reshape(shape.batch, n_query, shape.channels).cpu().numpy()
+    tl.check_layer(shape, data, y, parts)
