@@ -187,17 +187,27 @@ cudaError_t launch_sensitivity_masks(uint8_t* masks, int batch, int n_ctx, cudaS
     return cudaGetLastError();
 }
 
-// TPG threads per (output channel, group): a warp for groups of up to 512 elements (the usual 128: four of them at a time, so
-// that a warp has 2 KB on the way), half a block for longer ones (a whole row of an 8-bit matrix).  Bound by reading W once (a
-// 1280 x 1280 matrix is 6.6 MB, 1 us): a thread keeps its elements in registers between the absmax and the codes, 16-byte
-// loads, one word of codes per two lanes, codes by the reciprocal where it decides (quant_code_127).  (With scalar loads, a
-// division per element and a second pass over W that eight lanes of strided words read, the four matrices of a 1280-channel
-// layer took 32 us; one group per warp at a time left 24 us of kernels.)
-template <int TPG, int ITEMS>
-__global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restrict__ W, const float* __restrict__ bias, uint8_t* __restrict__ blob,
-                                                           int n_out, int k_in, int bits, int group) {
-    constexpr int KEEP = 4 / ITEMS, PER_BLOCK = 256 / TPG * ITEMS;      // float4 per thread and item in registers; items per block
+// TPG threads per (output channel, group): eight for groups of up to 128 elements (the usual W4), a warp for those of up to 512, half a
+// block for longer ones (a whole row of an 8-bit matrix).  A thread keeps up to sixteen elements in registers between the absmax and
+// the codes: 16-byte loads, neighbouring threads on neighbouring ones, one word of codes per two threads, codes by the
+// reciprocal where it decides, with one test for four of them.  What bounds it is the chain of one group (load, absmax, an IEEE division,
+// codes, store) and the launch, not the 6.6 MB of a 1280 x 1280 matrix (1 us): with a warp per group and four groups in a
+// row the chain had four divisions and twenty shuffles instead of one and three (launches in a graph: 320 x 320 4.2 -> 2.5 us, 1280 x 1280
+// 5.5 -> 4.0, 2560 x 2560 19.2 -> 10.4; whole rows of 8-bit codes 5.5 -> 4.5).  The kernel starts under its predecessor's tail: without
+// that the four matrices of a 1280-channel layer, call by call, took 3 us more.
+template <int TPG>
+__global__ void __launch_bounds__(256) pack_weights_kernel(const float* W, const float* bias, uint8_t* blob, int n_out, int k_in, int bits, int group) {
+    constexpr int KEEP = 4, PER_BLOCK = 256 / TPG;                      // float4 per thread in registers; groups per block
     const WeightLayout L = weight_layout(n_out, k_in, bits, group);
+    const int lane = threadIdx.x & 31, t = threadIdx.x % TPG, slot = threadIdx.x / TPG;
+    const int qmax = bits == 8 ? 127 : 7;
+    const long long items = (long long)n_out * L.n_groups;
+    float* scales = reinterpret_cast<float*>(blob + L.off_scales);
+    float* bias_out = reinterpret_cast<float*>(blob + L.off_bias);
+    __shared__ float part[8];
+    // (W may come from the previous kernel, and the one before it may still read the blob.)
+    ptx::pdl_wait();
+    ptx::pdl_trigger();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         PackedHeader h;
         h.magic = kWeightMagic; h.version = 1; h.n_out = n_out; h.k_in = k_in; h.bits = bits; h.group = group;
@@ -205,77 +215,73 @@ __global__ void __launch_bounds__(256) pack_weights_kernel(const float* __restri
         h.off_codes = L.off_codes; h.off_scales = L.off_scales; h.off_bias = L.off_bias; h.total_bytes = L.total;
         *reinterpret_cast<PackedHeader*>(blob) = h;
     }
-    const int lane = threadIdx.x & 31, t = threadIdx.x % TPG, slot = threadIdx.x / TPG;
-    const int qmax = bits == 8 ? 127 : 7;
-    const long long items = (long long)n_out * L.n_groups;
-    float* scales = reinterpret_cast<float*>(blob + L.off_scales);
-    float* bias_out = reinterpret_cast<float*>(blob + L.off_bias);
-    __shared__ float part[8];
-    // (every thread of a block makes the same number of rounds: the longer groups meet at barriers)
+    // (every thread of a block makes the same number of rounds: the longer groups meet at barriers, the others at shuffles)
     for (long long it0 = (long long)blockIdx.x * PER_BLOCK; it0 < items; it0 += (long long)gridDim.x * PER_BLOCK) {
-        float4 keep[ITEMS][KEEP];
-        float a[ITEMS];
-        int n[ITEMS], g[ITEMS], n4[ITEMS];
-        const float4* w4[ITEMS];
-        bool real[ITEMS];
-        auto absmax4 = [&](float& m, const float4& v) { m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
+        const bool real = it0 + slot < items;
+        const long long it = real ? it0 + slot : items - 1;
+        const int n = items < (1LL << 31) ? (int)((uint32_t)it / (uint32_t)L.n_groups) : (int)(it / L.n_groups), g = (int)(it - (long long)n * L.n_groups);
+        const int lo = g * L.group_len, n4 = (min(k_in, lo + L.group_len) - lo) / 4;              // (group lengths and fan-ins are multiples of 8)
+        const float4* w4 = reinterpret_cast<const float4*>(W + (size_t)n * k_in + lo);
+        float4 keep[KEEP];
+        float a = 0.f;
+        auto absmax4 = [&](const float4& v) { a = fmaxf(a, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const long long id = it0 + slot * ITEMS + u;
-            real[u] = id < items;
-            const long long it = real[u] ? id : items - 1;
-            n[u] = items < (1LL << 31) ? (int)((uint32_t)it / (uint32_t)L.n_groups) : (int)(it / L.n_groups);
-            g[u] = (int)(it - (long long)n[u] * L.n_groups);
-            const int lo = g[u] * L.group_len;
-            n4[u] = (min(k_in, lo + L.group_len) - lo) / 4;              // (group lengths and fan-ins are multiples of 8)
-            w4[u] = reinterpret_cast<const float4*>(W + (size_t)n[u] * k_in + lo);
+        for (int j = 0; j < KEEP; ++j) keep[j] = t + TPG * j < n4 ? ptx::load_global(w4 + t + TPG * j) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < KEEP; ++j) keep[u][j] = t + TPG * j < n4[u] ? w4[u][t + TPG * j] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        for (int j = 0; j < KEEP; ++j) absmax4(keep[j]);
+        for (int i = t + TPG * KEEP; i < n4; i += TPG) absmax4(ptx::load_global(w4 + i));
+        __syncwarp();
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            a[u] = 0.f;
-#pragma unroll
-            for (int j = 0; j < KEEP; ++j) absmax4(a[u], keep[u][j]);
-            for (int i = t + TPG * KEEP; i < n4[u]; i += TPG) absmax4(a[u], w4[u][i]);
-            a[u] = warp_max(a[u]);
-        }
+        for (int o = TPG < 32 ? TPG / 2 : 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
         if (TPG > 32) {
             __syncthreads();
-            if (lane == 0) part[threadIdx.x >> 5] = a[0];
+            if (lane == 0) part[threadIdx.x >> 5] = a;
             __syncthreads();
 #pragma unroll
-            for (int k = 0; k < TPG / 32; ++k) a[0] = fmaxf(a[0], part[slot * (TPG / 32) + k]);
+            for (int k = 0; k < TPG / 32; ++k) a = fmaxf(a, part[slot * (TPG / 32) + k]);
         }
+        const float s = quant_scale(a, (float)qmax);
+        const float rs = s > 0.f ? __frcp_rn(s) : 0.f;
+        const float r_lo = __uint_as_float(__float_as_uint(rs) - 2u), r_hi = __uint_as_float(__float_as_uint(rs) + 2u);
+        if (real && t == 0) {
+            scales[(size_t)n * L.n_groups + g] = s;
+            if (g == 0) bias_out[n] = bias ? ptx::load_global(bias + n) : 0.f;
+        }
+        uint8_t* row = blob + L.off_codes + (size_t)n * L.row_bytes;
+        auto encode = [&](const float4& v, int i, bool have) {           // elements 4 i .. 4 i + 3 of the group
+            const float x[4] = {v.x, v.y, v.z, v.w};
+            int c[4] = {0, 0, 0, 0};
+            if (s > 0.f) {                                               // (see quant_code_127)
+                uint32_t bad = 0;
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const float s = quant_scale(a[u], (float)qmax);
-            const float rs = s > 0.f ? __frcp_rn(s) : 0.f;
-            const float r_lo = __uint_as_float(__float_as_uint(rs) - 2u), r_hi = __uint_as_float(__float_as_uint(rs) + 2u);
-            auto code = [&](float x) { return s > 0.f ? min(max(quant_code_127(x, s, r_lo, r_hi), -qmax), qmax) : 0; };
-            if (real[u] && t == 0) {
-                scales[(size_t)n[u] * L.n_groups + g[u]] = s;
-                if (g[u] == 0) bias_out[n[u]] = bias ? bias[n[u]] : 0.f;
-            }
-            const int lo = g[u] * L.group_len;
-            uint8_t* row = blob + L.off_codes + (size_t)n[u] * L.row_bytes;
-            auto encode = [&](const float4& v, int i, bool have) {           // elements 4 i .. 4 i + 3 of the group
-                const int c[4] = {code(v.x), code(v.y), code(v.z), code(v.w)};
-                if (bits == 8) {
-                    if (real[u] && have) reinterpret_cast<char4*>(row + lo)[i] = make_char4((signed char)c[0], (signed char)c[1], (signed char)c[2], (signed char)c[3]);
-                } else {                                         // a word is eight elements: two neighbouring lanes
-                    uint32_t word = 0;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) word |= (uint32_t)(c[e] + 8) << (4 * w4_nibble_pos(e + 4 * (lane & 1)));
-                    word |= __shfl_xor_sync(0xffffffffu, word, 1);
-                    if (real[u] && have && (lane & 1) == 0) reinterpret_cast<uint32_t*>(row + lo / 2)[i >> 1] = word;
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t u = __float_as_uint(fmaf(x[e], r_lo, 12582912.0f));
+                    bad |= u ^ __float_as_uint(fmaf(x[e], r_hi, 12582912.0f));
+                    c[e] = (int)(u << 24) >> 24;                         // the low byte, sign-extended
                 }
-            };
+                if (bad) {
 #pragma unroll
-            for (int j = 0; j < KEEP; ++j)
-                if (TPG * j < n4[u]) encode(keep[u][j], t + TPG * j, t + TPG * j < n4[u]);
-            for (int i0 = TPG * KEEP; i0 < n4[u]; i0 += TPG) encode(i0 + t < n4[u] ? w4[u][i0 + t] : make_float4(0.f, 0.f, 0.f, 0.f), i0 + t, i0 + t < n4[u]);
-        }
+                    for (int e = 0; e < 4; ++e) c[e] = quant_code_127(x[e], s, r_lo, r_hi);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) c[e] = min(max(c[e], -qmax), qmax);
+            }
+            if (bits == 8) {
+                if (real && have) reinterpret_cast<char4*>(row + lo)[i] = make_char4((signed char)c[0], (signed char)c[1], (signed char)c[2], (signed char)c[3]);
+            } else {                                                     // a word is eight elements: two neighbouring threads
+                // (w4_nibble_pos: elements 0..3 in nibbles 0, 4, 1, 5, elements 4..7 in 2, 6, 3, 7)
+                uint32_t word = (uint32_t)(c[0] + 8) | (uint32_t)(c[1] + 8) << 16 | (uint32_t)(c[2] + 8) << 4 | (uint32_t)(c[3] + 8) << 20;
+                word <<= 8 * (lane & 1);
+                __syncwarp();
+                word |= __shfl_xor_sync(0xffffffffu, word, 1);
+                if (real && have && (lane & 1) == 0) reinterpret_cast<uint32_t*>(row + lo / 2)[i >> 1] = word;
+            }
+        };
+#pragma unroll
+        for (int j = 0; j < KEEP; ++j)
+            if (TPG < 32 || TPG * j < n4) encode(keep[j], t + TPG * j, t + TPG * j < n4);          // (several groups in a warp: all of its threads shuffle)
+        if (TPG >= 32)
+            for (int i0 = TPG * KEEP; i0 < n4; i0 += TPG) encode(i0 + t < n4 ? ptx::load_global(w4 + i0 + t) : make_float4(0.f, 0.f, 0.f, 0.f), i0 + t, i0 + t < n4);
     }
 }
 
@@ -284,10 +290,8 @@ cudaError_t launch_pack_weights(const taq_weight_desc& d, const float* W, const 
     const long long items = (long long)d.n_out * L.n_groups, per_block = L.group_len > 512 ? 2 : L.group_len > 128 ? 8 : 32;
     long long blocks = (items + per_block - 1) / per_block;
     if (blocks > 148LL * 32) blocks = 148LL * 32;
-    void (*kern)(const float*, const float*, uint8_t*, int, int, int, int) =
-        L.group_len > 512 ? pack_weights_kernel<128, 1> : L.group_len > 128 ? pack_weights_kernel<32, 1> : pack_weights_kernel<32, 4>;
-    kern<<<(unsigned)blocks, 256, 0, stream>>>(W, bias, (uint8_t*)packed, d.n_out, d.k_in, d.bits, d.group);
-    return cudaGetLastError();
+    auto* kern = L.group_len > 512 ? pack_weights_kernel<128> : L.group_len > 128 ? pack_weights_kernel<32> : pack_weights_kernel<8>;
+    return launch_pdl(kern, dim3((unsigned)blocks), dim3(256), 0, stream, W, bias, (uint8_t*)packed, d.n_out, d.k_in, d.bits, d.group);
 }
 
 __global__ void __launch_bounds__(256) unpack_weights_kernel(const uint8_t* __restrict__ blob, int8_t* __restrict__ codes_out,
