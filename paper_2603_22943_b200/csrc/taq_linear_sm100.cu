@@ -4,6 +4,7 @@
 TAQ_PROF_DEFINE(linear)
 #include "taq_linear_sm100.cuh"
 #include <algorithm>
+#include <cmath>
 
 namespace taq {
 
@@ -91,6 +92,24 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
     c.lay.n_groups = p.n_groups; c.lay.n_kb = p.n_kb; c.lay.mul_groups = multiplier(p.n_groups, (long long)BN * p.n_groups);
     c.lay.kb_per_group = p.n_groups == 1 ? p.n_kb : p.group_len / p.bke;
     c.lay.row_bytes = (uint32_t)p.L.row_bytes; c.lay.off_scales = p.L.off_scales; c.lay.off_bias = p.L.off_bias;
+    if (p.d) {
+        c.lay.d = p.d; c.lay.mul_d = multiplier(p.d, a.n_out);
+        c.lay.per_head = std::max(1, std::min(TL::NCG, p.d / TL::HC));
+    }
+    if (a.epi == EPI_KV) {
+        const taq_kv_layout KL = kv_layout(a.heads, a.n_ctx, p.d, a.max_trigger);
+        if (KL.block_bytes >= (1ull << 31)) return false;
+        auto& G = c.lay.kv;
+        G.off_v_codes = (uint32_t)KL.off_v_codes; G.off_k_scales = (uint32_t)KL.off_k_scales; G.off_v_scales = (uint32_t)KL.off_v_scales;
+        G.off_k_trigger = (uint32_t)KL.off_k_trigger; G.off_v_trigger = (uint32_t)KL.off_v_trigger; G.off_trig_slot = (uint32_t)KL.off_trig_slot;
+        G.off_operands = (uint32_t)KL.off_operands; G.block_bytes = KL.block_bytes;
+        OperandGeom g{};
+        G.images = operand_geom(p.d, a.n_ctx, &g);
+        G.head_bytes = (uint32_t)g.head_bytes; G.k_bytes = (uint32_t)g.k_bytes; G.vt_bytes = (uint32_t)g.vt_bytes;
+        G.dp = g.dp; G.kbq = g.kbq; G.n_heads = BN / p.d;
+        G.mul_dp = g.dp ? multiplier(g.dp, BN / p.d * g.dp) : 0;
+        G.logit_unit = 1.4426950408889634f / sqrtf((float)p.d);
+    }
     c.total = P.total; c.ring = P.ring_bytes; c.staged = staged;
     return true;
 }
@@ -183,12 +202,12 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
 
 // The last few problems of the calling thread: a program runs the same layers again and again.
 Choice choose(const LinearArgs& a, int n_z) {
-    struct Key { long long rows; int n_out, k_in, bits, group, heads, epi, n_ctx, n_z, flags, pad; };
+    struct Key { long long rows; int n_out, k_in, bits, group, heads, epi, n_ctx, n_z, flags, max_trigger; };
     struct Known { Key key; Choice choice; };
     constexpr int N = 16;
     thread_local Known known[N] = {};
     thread_local int next = 0;
-    const Key k = {a.rows, a.n_out, a.k_in, a.bits, a.group, a.heads, a.epi, a.n_ctx, n_z, 4 | (a.xq ? 1 : 0) | (a.reqs ? 2 : 0), 0};
+    const Key k = {a.rows, a.n_out, a.k_in, a.bits, a.group, a.heads, a.epi, a.n_ctx, n_z, 4 | (a.xq ? 1 : 0) | (a.reqs ? 2 : 0), a.max_trigger};
     for (const Known& e : known)
         if (memcmp(&e.key, &k, sizeof(k)) == 0) return e.choice;
     Known& e = known[next];

@@ -110,12 +110,23 @@ inline Plan make_plan(int n_groups, int nsa, int nsb, bool persistent) {
 // the blob's layout, the shared-memory plan, multipliers for the divisions by n_cols and n_rows.
 struct LinearLayout {
     int nsplit, nsa, nsb, head_pair, persistent;
+    int d, per_head;                        // per-head outputs: head width, folder threads per (row, head) (four divisions less per thread:
+    uint32_t mul_d;                         // 2048 x 1280 x 1280 14.7 -> 13.8 us, 8192 x 320 x 320 8.1 -> 7.3)
     int n_tiles, n_cols, n_rows;            // tiles of the launch: n_cols column tiles (K's and V's) per row tile, n_rows row tiles per z
     uint32_t mul_cols, mul_rows, mul_groups;            // see quotient()
     int n_groups, kb_per_group, n_kb;
     uint32_t row_bytes;
     unsigned long long off_scales, off_bias;
     Plan plan;
+    // K~/V~: the block of a sequence (kv_layout) and its images (operand_geom), offsets below 2^31.  (At the end: in the middle of what
+    // every launch reads it cost a small launch 0.3 us.)
+    struct {
+        uint32_t off_v_codes, off_k_scales, off_v_scales, off_k_trigger, off_v_trigger, off_trig_slot, off_operands, head_bytes, k_bytes, vt_bytes;
+        unsigned long long block_bytes;
+        int images, dp, kbq, n_heads;       // n_heads: of a tile
+        uint32_t mul_dp;
+        float logit_unit;                   // log2(e) / sqrt(d)
+    } kv;
 };
 
 // t / d by a multiplication (mul = 2^32 / d + 1, exact for t and d below 2^16; 0: divide).
@@ -246,28 +257,28 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // K~/V~, second half: all folders and builders, once the fp32 tile and the scales of its rows are in shared memory.  Short loops
     // over 8-element chunks, neighbouring lanes on neighbouring chunks, write everything in runs.  (With a row per lane straight
     // from the registers this epilogue took 15 000 - 24 000 cycles: 32 sectors per store, 20 KB of unrolled code that runs
-    // once.  With the eight folder warps alone these loops took 9 000: two warps on a scheduler hide no latency.)
+    // once.  With the eight folder warps alone these loops took 9 000: two warps on a scheduler hide no latency.
+    // With the block's layout worked out here, 2 300 cycles went by before the first load; it comes from the host now: two
+    // prompts of 77 x 768, W4, 320 channels 10.0 -> 8.6 us, 1280 channels 15.3 -> 14.0.)
     constexpr int KV_STRIDE = BN + 1;                        // floats (odd: a row per lane is free of bank conflicts)
     auto kv_store = [&](int w) {
         constexpr int NT = TL::NFOLD + TL::NBUILD, NC8 = BN / 8;
         int z, row0, col0, kv_which;
         tile_of(tile0, z, row0, col0, kv_which);
-        const int T = a.n_ctx, d = a.n_out / a.heads, nh = BN / d, head0 = col0 / d;
-        const taq_kv_layout KL = kv_layout(a.heads, T, d, a.max_trigger);
-        uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * KL.block_bytes;
-        OperandGeom G;
-        const bool images = operand_geom(d, T, &G);
-        uint8_t* img0 = blk + KL.off_operands + (size_t)head0 * G.head_bytes;
+        const auto& G = lay.kv;
+        const int T = a.n_ctx, d = lay.d, head0 = quotient(col0, d, lay.mul_d);
+        uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * G.block_bytes;
+        uint8_t* img0 = blk + G.off_operands + (uint32_t)head0 * G.head_bytes;
         const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;
         const float* ys = reinterpret_cast<const float*>(smem);
         const float2* hs = reinterpret_cast<const float2*>(smem + 128 * KV_STRIDE * 4);
         const int own_shift = nsplit == 1 ? 7 : nsplit == 2 ? 6 : 5;         // (CTAs that share the tile finish the rows of some lane quarters each)
         auto own = [&](int key) { return key >> own_shift == rank; };
         {                                                    // codes, trigger rows and K~'s image: 8 channels of a token
-            const int c = (w % NC8) * 8, hl = c / d, ch = c - hl * d, h = head0 + hl;
-            uint8_t* codes = blk + (kv_which ? KL.off_v_codes : KL.off_k_codes) + (size_t)h * T * d + ch;
-            uint8_t* trigs = blk + (kv_which ? KL.off_v_trigger : KL.off_k_trigger) + ((size_t)h * d + ch) * 2;
-            uint8_t* k_img = img0 + (size_t)hl * G.head_bytes + (ch >> 6) * (kOperandKeys * 128);
+            const int c = (w % NC8) * 8, hl = quotient(c, d, lay.mul_d), ch = c - hl * d, h = head0 + hl;
+            uint8_t* codes = blk + (kv_which ? G.off_v_codes : 0u) + (uint32_t)(h * T * d + ch);
+            uint8_t* trigs = blk + (kv_which ? G.off_v_trigger : G.off_k_trigger) + (uint32_t)(h * d + ch) * 2;
+            uint8_t* k_img = img0 + (uint32_t)hl * G.head_bytes + (ch >> 6) * (kOperandKeys * 128);
             for (int t = w / NC8; t < T && w < NT / NC8 * NC8; t += NT / NC8) {
                 if (!own(t)) continue;
                 const int slot = slots[t];
@@ -282,39 +293,43 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     k8 = pack8(f);
                     *reinterpret_cast<uint4*>(trigs + (size_t)slot * a.n_out * 2) = k8;
                 }
-                if (images && !kv_which) *reinterpret_cast<uint4*>(k_img + ptx::sw128_offset(t, (ch >> 3) & 7)) = k8;
+                if (G.images && !kv_which) *reinterpret_cast<uint4*>(k_img + ptx::sw128_offset(t, (ch >> 3) & 7)) = k8;
             }
         }
-        if (!images) return;
+        if (!G.images) return;
         if (!kv_which) {                                     // K~'s padding: keys T..79, and the channels behind the head's last
             const int ncc = G.kbq * 8;
-            for (int line = w >> 3; line < nh * kOperandKeys; line += NT / 8) {
+            for (int line = w >> 3; line < G.n_heads * kOperandKeys; line += NT / 8) {
                 const int hl = line / kOperandKeys, t = line - hl * kOperandKeys;
                 if (!own(t)) continue;
                 for (int cc = (w & 7) + (t >= T || d >= 64 ? 0 : d / 8 & ~7); cc < ncc; cc += 8)
-                    if (t >= T || cc * 8 >= d) *reinterpret_cast<uint4*>(img0 + (size_t)hl * G.head_bytes + (cc >> 3) * (kOperandKeys * 128) + ptx::sw128_offset(t, cc & 7)) = make_uint4(0, 0, 0, 0);
+                    if (t >= T || cc * 8 >= d) *reinterpret_cast<uint4*>(img0 + (uint32_t)hl * G.head_bytes + (cc >> 3) * (kOperandKeys * 128) + ptx::sw128_offset(t, cc & 7)) = make_uint4(0, 0, 0, 0);
             }
         } else {
             // V~^T: 8 keys of a channel per lane; a warp takes 8 channels x 4 chunks of keys (reads of the fp32 tile without bank
-            // conflicts, stores of 64 contiguous bytes).
+            // conflicts, stores of 64 contiguous bytes).  Everything is read first (rows and columns beyond the last token and
+            // channel, too: something of the tile, not used), so that a chunk costs one round trip to shared memory.
             const int wl = w & 31;
-            for (int u = w >> 5; u < nh * (G.dp >> 3) * 4; u += NT / 32) {
-                const int jc = (u & 3) * 4 + (wl >> 3), line = (u >> 2) * 8 + (wl & 7), hl = line / G.dp, ch = line - hl * G.dp;
+            for (int u = w >> 5; u < G.n_heads * (G.dp >> 3) * 4; u += NT / 32) {
+                const int jc = (u & 3) * 4 + (wl >> 3), line = (u >> 2) * 8 + (wl & 7), hl = quotient(line, G.dp, G.mul_dp), ch = line - hl * G.dp;
                 if (!own(jc * 8)) continue;
-                const float* col = ys + jc * 8 * KV_STRIDE + hl * d + ch;
-                const int n_real = ch < d ? min(8, T - jc * 8) : 0;
+                const float* col = ys + jc * 8 * KV_STRIDE + hl * d + min(ch, d - 1);
+                const float4* sc4 = reinterpret_cast<const float4*>(hs + hl * 128 + jc * 8);
+                const int n_real = ch < d ? T - jc * 8 : 0;
+                float x[8];
+                float4 sc[4];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[e] = col[e * KV_STRIDE];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[e] = sc4[e];
                 __half v[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    float x = 0.f;
-                    if (e < n_real) {
-                        x = col[e * KV_STRIDE];
-                        const float2 sc = hs[hl * 128 + jc * 8 + e];
-                        if (slots[jc * 8 + e] < 0) x = __fmul_rn(fmaf(x, sc.y, 12582912.0f) - 12582912.0f, sc.x);
-                    }
-                    v[e] = __float2half_rn(x);
+                    const float s1 = e & 1 ? sc[e / 2].z : sc[e / 2].x, rs = e & 1 ? sc[e / 2].w : sc[e / 2].y;
+                    const float quantized = __fmul_rn(fmaf(x[e], rs, 12582912.0f) - 12582912.0f, s1);
+                    v[e] = __float2half_rn(e >= n_real ? 0.f : rs < 0.f ? x[e] : quantized);      // (rs < 0: a trigger row)
                 }
-                *reinterpret_cast<uint4*>(img0 + (size_t)hl * G.head_bytes + G.k_bytes + (jc >> 3) * (G.dp * 128) + ptx::sw128_offset(ch, jc & 7)) = *reinterpret_cast<const uint4*>(v);
+                *reinterpret_cast<uint4*>(img0 + (uint32_t)hl * G.head_bytes + G.k_bytes + (jc >> 3) * (G.dp * 128) + ptx::sw128_offset(ch, jc & 7)) = *reinterpret_cast<const uint4*>(v);
             }
         }
     };
@@ -540,15 +555,15 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 put(w, std::integral_constant<int, HC * 4>{});
             } else {
                 // Per-(row, head) symmetric int8.  A thread's columns are one head or a half or a quarter of one.
-                const int d = a.n_out / a.heads;
+                const int d = lay.d;
                 const int colg = col0 + cb;
-                const int h0 = colg / d;
+                const int h0 = quotient(colg, d, lay.mul_d);
                 float am = 0.f;
 #pragma unroll
                 for (int c = 0; c < HC; ++c) am = fmaxf(am, fabsf(y[c]));
                 if (d > HC) {                                // the row's threads with columns of the same head combine their absmax
                     float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [NCG][128], and at 384 the absmax of a head pair's other half
-                    const int per_head = min(NCG, d / HC), first = cg / per_head * per_head;
+                    const int per_head = lay.per_head, first = cg & ~(per_head - 1);
                     xc[cg * 128 + r] = am;
                     asm volatile("bar.sync %0, %1;" ::"r"(2 + q), "n"(NCG * 32) : "memory");
 #pragma unroll
@@ -586,27 +601,24 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     // fp32 tile goes through shared memory to kv_store below.
                     const int T = a.n_ctx;
                     const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;      // [128] and the bitmap [4], by the scales' warps
-                    const taq_kv_layout KL = kv_layout(a.heads, T, d, a.max_trigger);
-                    uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * KL.block_bytes;
-                    OperandGeom G;
-                    const bool images = operand_geom(d, T, &G);
-                    const int head0 = col0 / d;
+                    const auto& G = lay.kv;
+                    uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * G.block_bytes;
+                    const int head0 = quotient(col0, d, lay.mul_d);
                     float* ys = reinterpret_cast<float*>(staging);                   // [128][KV_STRIDE]
-                    float2* hs = reinterpret_cast<float2*>(staging + 128 * KV_STRIDE * 4);   // [nh][128] scale and its reciprocal
+                    float2* hs = reinterpret_cast<float2*>(staging + 128 * KV_STRIDE * 4);   // [heads][128] scale and its reciprocal (trigger rows: 0 and -1)
                     if (mine) {
                         const int slot = slots[r];           // >= 0: trigger row, -1: ordinary (or padding), -2: a trigger row beyond the capacity
                         const bool plain = r < T && slot == -1;
 #pragma unroll
                         for (int c = 0; c < HC; ++c) ys[r * KV_STRIDE + cb + c] = y[c];
-                        const float logit_unit = 1.4426950408889634f / sqrtf((float)d);
                         if (owner) {
                             const float sk = plain ? s : 0.f;
-                            hs[(h0 - head0) * 128 + r] = make_float2(sk, plain ? rs : 0.f);
-                            if (r < T) reinterpret_cast<float*>(blk + (kv_which ? KL.off_v_scales : KL.off_k_scales))[(size_t)h0 * T + r] = sk;
-                            if (!kv_which && h0 == 0) reinterpret_cast<int32_t*>(blk + KL.off_trig_slot)[r] = slot >= 0 ? slot : -1;
-                            if (!kv_which && images && r < kOperandKeys) {
-                                OperandConsts* cst = reinterpret_cast<OperandConsts*>(blk + KL.off_operands + (size_t)h0 * G.head_bytes + G.k_bytes + G.vt_bytes);
-                                cst->logit_factor[r] = (slot >= 0 ? 1.0f : sk) * logit_unit;
+                            hs[(h0 - head0) * 128 + r] = make_float2(sk, plain ? rs : slot >= 0 ? -1.f : 0.f);
+                            if (r < T) reinterpret_cast<float*>(blk + (kv_which ? G.off_v_scales : G.off_k_scales))[(uint32_t)(h0 * T + r)] = sk;
+                            if (!kv_which && h0 == 0) reinterpret_cast<int32_t*>(blk + G.off_trig_slot)[r] = slot >= 0 ? slot : -1;
+                            if (!kv_which && G.images && r < kOperandKeys) {
+                                OperandConsts* cst = reinterpret_cast<OperandConsts*>(blk + G.off_operands + (uint32_t)h0 * G.head_bytes + G.k_bytes + G.vt_bytes);
+                                cst->logit_factor[r] = (slot >= 0 ? 1.0f : sk) * G.logit_unit;
                                 if (r < 4) cst->trig_bits[r] = (uint32_t)slots[128 + r];
                             }
                         }

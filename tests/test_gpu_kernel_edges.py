@@ -94,3 +94,23 @@ def test_one_kernel_layer_writes_its_rows_only(n_query):
     assert bool((buf[:1024] == -7.0).all()) and bool((buf[1024 + n:] == -7.0).all())
     y = buf[1024: 1024 + n].reshape(shape.batch, n_query, shape.channels).cpu().numpy()
     tl.check_layer(shape, data, y, parts)
+
+
+def test_kv_projections_of_one_shape_and_two_trigger_capacities():
+    """The capacity moves everything behind the trigger rows in a K~/V~ block; nothing of one call's layout is kept for the other."""
+    shape = synth.shrink(synth.config2(), 8)
+    data = synth.make_layer(shape)
+    P = tl.pack_layer_weights(shape, data)
+    blocks = {}
+    for capacity in (2, 5, 2):
+        desc = tl.gpu_desc(shape, max_trigger=capacity)
+        kv = torch.zeros(tb.taq_kv_bytes(desc), dtype=torch.uint8, device="cuda")
+        tb.taq_kv_project(desc, tl.dev(data["ctx"]), P["Wk"], P["Wv"], tl.dev(data["mask"]), kv)
+        blocks[capacity] = tl.parse_kv_block(desc, kv)
+        L = tb.taq_kv_layout_of(desc)
+        blocks[capacity]["images"] = kv.view(shape.batch, -1)[:, L.off_operands:].cpu().numpy()
+    tb.taq_poll_device_status()
+    for name in ("K_codes", "V_codes", "K_scales", "V_scales", "slot", "images"):
+        assert (blocks[2][name] == blocks[5][name]).all(), name
+    for name in ("K_trigger", "V_trigger"):
+        assert (blocks[2][name] == blocks[5][name][:, :2]).all(), name
