@@ -66,9 +66,9 @@ struct Tile {
     static constexpr int W_PROD = 0, W_MMA = 1, W_AUX = 2, W_FOLD = 4, W_BUILD = W_FOLD + NF;
     static constexpr int R_FOLD = BIG ? 88 : 128, R_BUILD = 48, R_REST = 56;
     static_assert(128 * (R_REST + NF / 4 * R_FOLD + NB / 4 * R_BUILD) == NTHREADS * 72, "register split");
-    // ... and of the K~/V~ epilogue's second half, see kv_together: 896 x 72 >= 128 x (56 + 4 x 80 + 2 x 64) = 128 x (56 + 2 x 80 + 4 x 72)
-    static constexpr int R_KV_FOLD = 80, R_KV_BUILD = BIG ? 64 : 72;
-    static_assert(NF * R_KV_FOLD + NB * R_KV_BUILD <= NF * R_FOLD + NB * R_BUILD, "register split");
+    // ... and of the K~/V~ epilogue's second half, one for both roles (they run the same code): the 72 of the launch.
+    static constexpr int R_KV = 72;
+    static_assert((NF + NB) * R_KV <= NF * R_FOLD + NB * R_BUILD, "register split");
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr int NSLOT = TMEM_COLS / BN;                              // accumulators in TMEM: 3 to 8
     static constexpr int B_TILE = BN * 128;                                   // one k-block
@@ -333,16 +333,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             }
         }
     };
-    // The folders hand registers to the builders on the way: they give theirs back before
-    // the barrier, the builders ask behind it.  (A builder that asked as soon as it ran out of work could be given what the
-    // folders' first request was still waiting for, and neither would ever go on.)
-    auto kv_together = [&](bool folder, int w) {
-        if (folder) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_KV_FOLD));
-        asm volatile("bar.sync 15, %0;" ::"n"(TL::NFOLD + TL::NBUILD) : "memory");
-        if (!folder) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::R_KV_BUILD));
-        if (!bars->abort_flag) kv_store(w);
-    };
-
     if (warp >= TL::W_FOLD && warp < TL::W_BUILD) {
         // ---------------- folders ----------------
         start(true);
@@ -629,7 +619,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             if (sbuf == 0) ph_scale ^= 1;
         }
         __syncwarp();
-        if constexpr (KV) kv_together(true, ft);
     } else if (warp >= TL::W_BUILD && warp < TL::W_BUILD + TL::NB) {
         // ---------------- builders ----------------
         const int bt = (tid - 32 * TL::W_BUILD) & (TL::NBUILD / 2 - 1), group = (warp - TL::W_BUILD) / (TL::NB / 2);
@@ -698,8 +687,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         if (!ok) give_up();
         __syncwarp();
-        if constexpr (KV) kv_together(false, TL::NFOLD + tid - 32 * TL::W_BUILD);
-        if (clustered) ptx::cluster_wait();
+        if (!KV && clustered) ptx::cluster_wait();
     } else {
         start(warp != TL::W_PROD);
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_REST));
@@ -852,6 +840,19 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         __syncwarp();
         if (clustered) ptx::cluster_wait();
+    }
+
+    if (KV && warp >= TL::W_FOLD) {
+        // The folders hand registers to the builders on the way: they give theirs back before the barrier, the builders ask behind
+        // it.  (A builder that asked as soon as it ran out of work could be given what the folders' first request was still
+        // waiting for, and neither would ever go on.)  One copy of what follows for both: it runs once, and what it costs
+        // is to fetch it.
+        if (warp < TL::W_BUILD) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TL::R_KV));
+        asm volatile("bar.sync 15, %0;" ::"n"(TL::NFOLD + TL::NBUILD) : "memory");
+        if (warp >= TL::W_BUILD) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(TL::R_KV));
+        if (!bars->abort_flag) kv_store(tid - 32 * TL::W_FOLD);
+        __syncwarp();
+        if (clustered && warp >= TL::W_BUILD) ptx::cluster_wait();
     }
 
     // ---------------- teardown ----------------
