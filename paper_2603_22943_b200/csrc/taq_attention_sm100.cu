@@ -10,13 +10,14 @@
 //   warp 8     one thread issues the MMAs: S of head h+1 is in flight while the rows are in the softmax of head h;
 //   warp 9     one thread fetches each head's K~/V~ operand image (written once per prompt by the K/V projection)
 //              by bulk copies, one head ahead: the whole image into the second buffer (head widths up to 64), or,
-//              with a single buffer, K~ as soon as this head's S is complete and V~^T as soon as its PV is.
+//              with a single buffer, K~ as soon as this head's S is complete and V~^T as soon as its PV is (wide heads with
+//              int8 Q~: K~ into a second buffer, V~^T by a thread of warp 10).
 // Head widths up to 64: two CTAs share an SM, and the row threads read Q~ and write O themselves.  Head widths 80 and
 // 160: one CTA per SM; Q~ tiles arrive and O tiles leave by TMA, and from the second head on warps of their own do that work:
 //   warps 12-15  expand the next head's codes (fp16 Q~: load it straight into the operand tile);
 //   warps 16-19  bring the previous head's O from TMEM to global memory.
 // (With the row warps doing everything in turn a head of 160 channels took 5 700 cycles: softmax 1 650, codes 1 100, O 2 250,
-// probabilities 600; now 4 300.)
+// probabilities 600; now 4 000.)
 #include "taq_prof.cuh"
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
@@ -35,7 +36,7 @@ using namespace parts;
 
 constexpr int ROWS = 128;
 constexpr int ROW_WARPS = 8;         // two threads per query row
-constexpr int MMA_WARP = 8, COPY_WARP = 9;
+constexpr int MMA_WARP = 8, COPY_WARP = 9, V_WARP = 10;
 // Three warpgroups: two of row warps, and one of the MMA and copy warps with two idle ones, which gives registers to the rows where
 // two CTAs share an SM (384 threads launched with 80 each = 128 x (2 x 104 + 32); with 96 for everybody the softmax spilled).
 constexpr int R_ROWS = 104, R_REST = 32;
@@ -44,7 +45,12 @@ constexpr int Q_WARP = 12, O_WARP = 16;
 constexpr int R_WIDE_ROWS = 128, R_WIDE_REST = 40, R_WIDE_Q = 72, R_WIDE_O = 104;
 static_assert(2 * R_WIDE_ROWS + R_WIDE_REST + R_WIDE_Q + R_WIDE_O <= 5 * 96, "register split");
 
-template <int D>
+// Head widths 80 and 160 with int8 Q~ (K2) have two K~ buffers, so that a head's K~ is there long before its S may start: with one it
+// was asked for when the S before it was complete, and S came 400 - 800 cycles after the rows were ready for it (16 x 1024 rows, 8 heads of
+// 80: 18.7 -> 17.2 us, 3 x 1872 9.4 -> 9.0, 64 x 256, 8 heads of 160 25.6 -> 25.2).  What makes room for
+// the second one at 160 channels: the last 32 (16) channels of Q~ and the last 16 keys of P are tiles of 64- and 32-byte rows of
+// their own instead of half-empty 128-byte ones.
+template <int D, bool Q8>
 struct Cfg {
     static constexpr int DP = (D + 15) / 16 * 16;            // head width padded to the MMA K / N granule
     static constexpr int KBQ = (DP + 63) / 64;               // 64-wide k-blocks of the Q~ and K~ tiles
@@ -56,48 +62,63 @@ struct Cfg {
     static constexpr int HEAD_BYTES = K_BYTES + VT_BYTES + kOperandConstBytes;
     static constexpr int KVBUF = D <= 64 ? 2 : 1;            // K~/V~ images in flight
     static constexpr int OBUF = D == 64 ? 1 : 2;             // O accumulators in TMEM
-    static constexpr int OFF_KV = 0;
-    static constexpr int OFF_Q = OFF_KV + KVBUF * HEAD_BYTES;
-    static constexpr int OFF_P = OFF_Q + KBQ * A_BLOCK;
+    static constexpr bool K2 = D >= 80 && Q8;
+    static constexpr int QFULL = K2 ? DP / 64 : KBQ, QTAIL = K2 ? DP % 64 : 0;     // 64-wide blocks of the Q~ tile, channels of its narrow one
+    static constexpr int OFF_KV = 0;                         // images; wide heads: K~ (twice if K2), V~^T
+    static constexpr int OFF_V = OFF_KV + (K2 ? 2 : 1) * K_BYTES;
+    static constexpr int OFF_Q = D <= 64 ? OFF_KV + KVBUF * HEAD_BYTES : OFF_V + VT_BYTES;
+    static constexpr int OFF_P = OFF_Q + QFULL * A_BLOCK + ROWS * QTAIL * 2;
+    static constexpr int P_BYTES = D >= 80 ? A_BLOCK + ROWS * 32 : 2 * A_BLOCK;
     // One image buffer (wide heads): the next head's K~ loads as soon as this head's S is complete and its V~^T as soon
     // as this head's PV is, each with a barrier of its own; the constants of a head then live in a rotating slot of their
-    // own (three slots: the softmax of head h - 1 may still read its slot when the constants of head h + 1 arrive).
+    // own (three slots: the softmax of head h - 1 may still read its slot when the constants of head h + 1 arrive; with two K~
+    // buffers they arrive a head earlier, hence four).
     static constexpr bool SPLIT_KV = KVBUF == 1;
-    static constexpr int CST_SLOT = 384;
-    static constexpr int OFF_CST = OFF_P + 2 * A_BLOCK;
+    static constexpr int CST_SLOT = 384, CST_SLOTS = K2 ? 4 : 3;
+    static constexpr int OFF_CST = OFF_P + P_BYTES;
     // Wide heads move Q~ and O by TMA (a row's codes or outputs of one head are 80 to 320
     // bytes at a stride of the whole channel width: per-thread global accesses of that shape keep the load/store
     // unit busy for longer than the arithmetic takes): O through one staging buffer, int8 codes through a second one, fp16 Q~
     // straight into the operand tile.
     static constexpr bool TMA_IO = D >= 80;
     static constexpr int THREADS = TMA_IO ? 640 : 384;
-    static constexpr int OFF_U = OFF_CST + (SPLIT_KV ? 3 * CST_SLOT : 0);
+    static constexpr int OFF_U = OFF_CST + (SPLIT_KV ? CST_SLOTS * CST_SLOT : 0);
     static constexpr int UO_BYTES = ROWS * D * 2;                  // an O tile
     static constexpr int U_BYTES = TMA_IO ? UO_BYTES + ROWS * D : 0; // + a raw int8 Q~ tile
     static constexpr int OFF_MISC = OFF_U + U_BYTES;
-    static constexpr int TOTAL = OFF_MISC + 4096 + 128 + 1024;   // misc block + slack for 1024-byte alignment
+    static constexpr int TOTAL = OFF_MISC + 4096 + 192 + 1024;   // misc block + slack for 1024-byte alignment
     static constexpr uint32_t TMEM_S = 0, TMEM_O = 2 * TP;
     static constexpr uint32_t TMEM_COLS = (2 * TP + OBUF * DP) <= 256 ? 256 : 512;
     static constexpr int CTAS_PER_SM = (2 * (TOTAL + 1024) <= 232448 && TMEM_COLS == 256) ? 2 : 1;
     static_assert(HEAD_BYTES % 1024 == 0 && K_BYTES % 1024 == 0 && VT_BLOCK % 1024 == 0, "operand tiles must keep 1024-byte alignment");
     static_assert(TOTAL <= 232448, "shared memory budget");
+    static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0 && OFF_U % 128 == 0, "tile alignment");
+    // 16-byte chunk cc (8 channels) of a row of the Q~ tile; chunk of a row of P (8 keys)
+    static __device__ __forceinline__ uint32_t q_offset(int row, int cc) {
+        if (QTAIL == 0 || cc < 8 * QFULL) return (cc >> 3) * A_BLOCK + ptx::sw128_offset(row, cc & 7);
+        return QFULL * A_BLOCK + (QTAIL == 16 ? ptx::sw32_offset(row, cc - 8 * QFULL) : ptx::sw64_offset(row, cc - 8 * QFULL));
+    }
+    static __device__ __forceinline__ uint32_t p_offset(int row, int chunk) {
+        if (D < 80) return (chunk >> 3) * A_BLOCK + ptx::sw128_offset(row, chunk & 7);
+        return chunk < 8 ? ptx::sw128_offset(row, chunk) : A_BLOCK + ptx::sw32_offset(row, chunk - 8);
+    }
 };
 
 struct Misc {
-    uint64_t kv_full[2], kv_free[2], q_full, s_full[2], p_full, o_full[2], drain, qraw_full, o_free[2], u_free;
+    uint64_t kv_full[2], kv_free[2], q_full, s_full[2], p_full, o_full[2], drain, qraw_full, o_free[2], u_free, k_odd;
     uint32_t tmem_base;
     volatile int abort_flag;
     float2 xchg[2][2][ROWS];     // [head parity][half][row]: (max, sum) of a thread's half of the softmax
 };
 constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
-static_assert(sizeof(Misc) <= 4096 + 128 && N_BARS <= 32, "misc block");
+static_assert(sizeof(Misc) <= 4096 + 192 && N_BARS <= 32, "misc block");
 static_assert(sizeof(OperandConsts) % 16 == 0 && sizeof(OperandConsts) <= 384, "constants slot");
 
 // Half of the query codes (or fp16 values) of one row and head, held in registers between the global load and
 // the store into the operand tile: the row's two threads take the lower and the upper half of the 16-byte chunks.
 template <int D, bool Q8>
 struct QRegs {
-    static constexpr int CH2 = (Cfg<D>::DP / 8 + 1) / 2;      // chunks (8 channels) per thread
+    static constexpr int CH2 = (Cfg<D, Q8>::DP / 8 + 1) / 2;      // chunks (8 channels) per thread
     uint4 v[Q8 ? (CH2 + 1) / 2 : CH2];
     __device__ __forceinline__ void load(const void* q, size_t elem_off, bool valid, int half) {
         const int c0 = half * CH2;
@@ -128,8 +149,8 @@ struct QRegs {
 };
 
 template <int D, bool Q8, bool TAIL_ONLY>
-__global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a) {
-    using C = Cfg<D>;
+__global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) attention_sm100_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_o, const AttnArgs a) {
+    using C = Cfg<D, Q8>;
     constexpr int DP = C::DP;
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* smem = smem_dyn + ((1024u - (ptx::smem_u32(smem_dyn) & 1023u)) & 1023u);   // 1024-byte aligned, still provably shared
@@ -167,6 +188,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
     // Raw tiles of even and odd heads complete barriers of their own: who waits for the second head only must not take the phase
     // before the first one for it.  (Wide heads have one image buffer, the second kv_free is theirs to use.)
     auto qraw_full = [&](int hi) { return hi & 1 ? &misc->kv_free[1] : &misc->qraw_full; };
+    auto k_full = [&](int hi) { return C::K2 && (hi & 1) ? &misc->k_odd : &misc->kv_full[0]; };      // (K~ of wide heads)
+    auto k_parity = [&](int hi) { return (uint32_t)(C::K2 ? hi >> 1 : hi) & 1u; };
 
     constexpr bool REG_SPLIT = C::CTAS_PER_SM == 2;
     if (C::TMA_IO && warp >= Q_WARP) {
@@ -176,18 +199,20 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_WIDE_Q));
             bool alive = true;
             if constexpr (Q8) {
-                // the chunks of the raw tile, dealt out as in stage_q_u below; they are read before S of the head before is
-                // complete (its operand tile is free then), and the raw tile of the head after next lands under all that
-                constexpr int CPR = D / 8, N = ROWS * CPR / 128;
+                // A thread is a row: sixteen codes per load (rows of 80 or 160 bytes: no or two-way bank conflicts), and every place in the
+                // operand tile is a constant beside the row's.  They are read before S of the head before is complete (its operand
+                // tile is free then), and the raw tile of the head after next lands under all that.  (With the chunks dealt out in
+                // linear order, row and place worked out for each, S of a head of 160 channels was 2 500 cycles later.)
+                constexpr int N = D / 16;
                 const unsigned char* UQ = smem + C::OFF_U + C::UO_BYTES;
                 const int t = tid - 32 * Q_WARP;
                 if (t == 0) ptx::pdl_wait();                             // (this thread loads Q~ of the third head and on)
                 __syncwarp();
                 for (int hi = 1; hi < HG; ++hi) {
                     alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(hi), (hi >> 1) & 1));
-                    uint2 raw[N];
+                    uint4 raw[N];
 #pragma unroll
-                    for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint2*>(UQ + (size_t)(t + 128 * i) * 8);
+                    for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint4*>(UQ + t * D + i * 16);
                     ptx::fence_proxy_async_smem();                           // (generic reads before the TMA load that overwrites them)
                     asm volatile("bar.sync 6, 128;" ::: "memory");           // the raw tile has been read
                     if (t == 0 && alive && hi + 1 < HG) {
@@ -199,8 +224,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                     if (alive) {
 #pragma unroll
                         for (int i = 0; i < N; ++i) {
-                            const int j = t + 128 * i, row = j / CPR, cc = j - row * CPR;
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(row, cc & 7)) = codes_w8_to_half(raw[i]);
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i)) = codes_w8_to_half(make_uint2(raw[i].x, raw[i].y));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i + 1)) = codes_w8_to_half(make_uint2(raw[i].z, raw[i].w));
                         }
                         ptx::fence_proxy_async_smem();
                     }
@@ -234,21 +259,17 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                 if (alive) {
                     ptx::tc_fence_after_sync();
                     const uint32_t t_o = tmem_base + C::TMEM_O + (hi & 1) * DP + ((uint32_t)(q4 * 32) << 16);
-#pragma unroll
-                    for (int c0 = 0; c0 < D; c0 += 40) {
-                        uint32_t v[5][8];
-#pragma unroll
-                        for (int i = 0; i < 5; ++i) ptx::tmem_ld8(t_o + c0 + i * 8, v[i]);
+                    // (a loop of 40 instructions: beside the softmax the instructions of all roles do not fit the cache near the schedulers,
+                    // and unrolled, 400 of them a head, this took 100 - 200 cycles from every softmax)
+#pragma unroll 1
+                    for (int c0 = 0; c0 < D; c0 += 16) {
+                        uint32_t v[2][8];
+                        ptx::tmem_ld8(t_o + c0, v[0]);
+                        ptx::tmem_ld8(t_o + c0 + 8, v[1]);
                         ptx::tmem_ld_wait(v[0]);
+                        ptx::reg_fence8(v[1]);
 #pragma unroll
-                        for (int i = 1; i < 5; ++i) ptx::reg_fence8(v[i]);
-                        if (c0 + 40 == D) {
-                            ptx::tc_fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) ptx::mbar_arrive(&misc->o_free[hi & 1]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 5; ++i) {
+                        for (int i = 0; i < 2; ++i) {
                             uint32_t pk[4];
 #pragma unroll
                             for (int e2 = 0; e2 < 4; ++e2) {
@@ -258,6 +279,9 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                             *reinterpret_cast<uint4*>(U + ((size_t)r * D + c0 + i * 8) * 2) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                         }
                     }
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&misc->o_free[hi & 1]);
                     ptx::fence_proxy_async_smem();
                 }
                 asm volatile("bar.sync 7, 128;" ::: "memory");
@@ -284,6 +308,19 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             const uint8_t* blk = a.reqs ? (const uint8_t*)a.reqs[zb].kv : (const uint8_t*)a.kv + (size_t)b * KL.block_bytes;
             const uint8_t* img = blk + KL.off_operands + (size_t)h_begin * KL.operand_head_bytes;
             int issued = 0;
+            if (C::K2) {
+                for (int hi = 0; hi < HG; ++hi) {            // a buffer is free when the S before last is complete
+                    if (hi >= 2 && !ptx::mbar_wait(&misc->s_full[hi & 1], ((hi - 2) >> 1) & 1)) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
+                    if (misc->abort_flag) break;
+                    const uint8_t* src = img + (size_t)hi * KL.operand_head_bytes;
+                    ptx::mbar_arrive_expect_tx(k_full(hi), C::K_BYTES + (uint32_t)sizeof(OperandConsts));
+                    ptx::bulk_load(smem + C::OFF_KV + (hi & 1) * C::K_BYTES, src, C::K_BYTES, k_full(hi));
+                    ptx::bulk_load(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT, src + C::K_BYTES + C::VT_BYTES, (uint32_t)sizeof(OperandConsts), k_full(hi));
+                    issued = hi + 1;
+                }
+                if (misc->abort_flag)     // let copies that were issued land before the CTA goes away
+                    for (int hi = issued > 2 ? issued - 2 : 0; hi < issued; ++hi) (void)ptx::mbar_wait(k_full(hi), k_parity(hi));
+            } else
             if (C::SPLIT_KV) {
                 // kv_full[0]: K~ and the constants of a head; kv_full[1]: its V~^T
                 int issued_v = 0;
@@ -293,12 +330,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                     const uint8_t* src = img + (size_t)hi * KL.operand_head_bytes;
                     ptx::mbar_arrive_expect_tx(&misc->kv_full[0], C::K_BYTES + (uint32_t)sizeof(OperandConsts));
                     ptx::bulk_load(smem + C::OFF_KV, src, C::K_BYTES, &misc->kv_full[0]);
-                    ptx::bulk_load(smem + C::OFF_CST + (hi % 3) * C::CST_SLOT, src + C::K_BYTES + C::VT_BYTES, (uint32_t)sizeof(OperandConsts), &misc->kv_full[0]);
+                    ptx::bulk_load(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT, src + C::K_BYTES + C::VT_BYTES, (uint32_t)sizeof(OperandConsts), &misc->kv_full[0]);
                     issued = hi + 1;
                     if (hi >= 1 && !ptx::mbar_wait(&misc->kv_free[0], (hi - 1) & 1)) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
                     if (misc->abort_flag) break;
                     ptx::mbar_arrive_expect_tx(&misc->kv_full[1], C::VT_BYTES);
-                    ptx::bulk_load(smem + C::OFF_KV + C::K_BYTES, src + C::K_BYTES, C::VT_BYTES, &misc->kv_full[1]);
+                    ptx::bulk_load(smem + C::OFF_V, src + C::K_BYTES, C::VT_BYTES, &misc->kv_full[1]);
                     issued_v = hi + 1;
                 }
                 if (misc->abort_flag) {   // let copies that were issued land before the CTA goes away
@@ -319,6 +356,22 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             }
             }
         }
+    } else if (C::K2 && warp == V_WARP) {
+        // ---------------- V~^T of wide heads with two K~ buffers: as soon as the PV before it is complete ----------------
+        if (lane == 0) {
+            if (!a.early_kv) ptx::pdl_wait();
+            const uint8_t* blk = a.reqs ? (const uint8_t*)a.reqs[zb].kv : (const uint8_t*)a.kv + (size_t)b * KL.block_bytes;
+            const uint8_t* img = blk + KL.off_operands + (size_t)h_begin * KL.operand_head_bytes + C::K_BYTES;
+            int issued = 0;
+            for (int hi = 0; hi < HG; ++hi) {
+                if (hi >= 1 && !ptx::mbar_wait(&misc->kv_free[0], (hi - 1) & 1)) { raise_status(a.status, TAQ_ERR_TIMEOUT); misc->abort_flag = 1; }
+                if (misc->abort_flag) break;
+                ptx::mbar_arrive_expect_tx(&misc->kv_full[1], C::VT_BYTES);
+                ptx::bulk_load(smem + C::OFF_V, img + (size_t)hi * KL.operand_head_bytes, C::VT_BYTES, &misc->kv_full[1]);
+                issued = hi + 1;
+            }
+            if (misc->abort_flag && issued) (void)ptx::mbar_wait(&misc->kv_full[1], (issued - 1) & 1);
+        }
     } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer ----------------
         // One elected thread walks it alone (a wait on a complete barrier costs it 60 cycles; a vote of the whole warp and a poll
@@ -330,15 +383,18 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
         const uint32_t kv_lo0 = ptx::desc_lo(ptx::smem_u32(smem + C::OFF_KV));
         auto issue_s = [&](int hi) -> bool {
             const int buf = hi % C::KVBUF;
-            if (!wait(&misc->kv_full[buf], C::SPLIT_KV ? (hi & 1) : (hi / C::KVBUF) & 1) || !wait(&misc->q_full, hi & 1)) return false;
+            if (C::SPLIT_KV ? !wait(k_full(hi), k_parity(hi)) : !wait(&misc->kv_full[buf], (hi / C::KVBUF) & 1)) return false;
+            if (!wait(&misc->q_full, hi & 1)) return false;
             ptx::tc_fence_after_sync();
             {
                 if (hi < 8) TAQ_PROF(80 + hi);
-                const uint32_t k_lo = kv_lo0 + buf * (C::HEAD_BYTES >> 4);
+                const uint32_t k_lo = kv_lo0 + (C::SPLIT_KV ? (C::K2 ? (hi & 1) * (C::K_BYTES >> 4) : 0) : buf * (C::HEAD_BYTES >> 4));
 #pragma unroll
-                for (int ks = 0; ks < DP / 16; ++ks)
-                    ptx::mma_f16_ss(tmem_base + C::TMEM_S + (hi & 1) * TP, ptx::desc_join(HI, q_lo0 + (ks / 4) * (C::A_BLOCK >> 4) + (ks % 4) * 2),
-                                    ptx::desc_join(HI, k_lo + (ks / 4) * (C::K_BLOCK >> 4) + (ks % 4) * 2), ptx::idesc_f16_m128(TP), ks != 0);
+                for (int ks = 0; ks < DP / 16; ++ks) {
+                    const uint64_t qd = ks < 4 * C::QFULL ? ptx::desc_join(HI, q_lo0 + (ks / 4) * (C::A_BLOCK >> 4) + (ks % 4) * 2)
+                                                          : ptx::desc_join(C::QTAIL == 16 ? ptx::kDescHiSw32 : ptx::kDescHiSw64, q_lo0 + C::QFULL * (C::A_BLOCK >> 4) + (ks - 4 * C::QFULL) * 2);
+                    ptx::mma_f16_ss(tmem_base + C::TMEM_S + (hi & 1) * TP, qd, ptx::desc_join(HI, k_lo + (ks / 4) * (C::K_BLOCK >> 4) + (ks % 4) * 2), ptx::idesc_f16_m128(TP), ks != 0);
+                }
                 ptx::mma_commit(&misc->s_full[hi & 1]);
             }
             return true;
@@ -351,11 +407,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             ptx::tc_fence_after_sync();
             {
                 if (hi < 8) TAQ_PROF(96 + hi);
-                const uint32_t vt_lo = kv_lo0 + ((buf * C::HEAD_BYTES + C::K_BYTES) >> 4);
+                const uint32_t vt_lo = C::SPLIT_KV ? kv_lo0 + ((C::OFF_V - C::OFF_KV) >> 4) : kv_lo0 + ((buf * C::HEAD_BYTES + C::K_BYTES) >> 4);
 #pragma unroll
-                for (int ks = 0; ks < TP / 16; ++ks)
-                    ptx::mma_f16_ss(tmem_base + C::TMEM_O + (hi % C::OBUF) * DP, ptx::desc_join(HI, p_lo0 + (ks / 4) * (C::A_BLOCK >> 4) + (ks % 4) * 2),
-                                    ptx::desc_join(HI, vt_lo + (ks / 4) * (C::VT_BLOCK >> 4) + (ks % 4) * 2), ptx::idesc_f16_m128(DP), ks != 0);
+                for (int ks = 0; ks < TP / 16; ++ks) {
+                    const uint64_t pd = C::TMA_IO && ks >= 4 ? ptx::desc_join(ptx::kDescHiSw32, p_lo0 + (C::A_BLOCK >> 4)) : ptx::desc_join(HI, p_lo0 + (ks / 4) * (C::A_BLOCK >> 4) + (ks % 4) * 2);
+                    ptx::mma_f16_ss(tmem_base + C::TMEM_O + (hi % C::OBUF) * DP, pd, ptx::desc_join(HI, vt_lo + (ks / 4) * (C::VT_BLOCK >> 4) + (ks % 4) * 2), ptx::idesc_f16_m128(DP), ks != 0);
+                }
                 ptx::mma_commit(&misc->o_full[hi % C::OBUF]);
                 ptx::mma_commit(&misc->kv_free[buf]);
             }
@@ -363,7 +420,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
         };
         bool ok = issue_s(0);
         for (int hi = 0; hi < HG && ok; ++hi) {
-            if (C::KVBUF == 2) {          // S of the next head first: it runs under this head's softmax
+            if (C::KVBUF == 2 || C::K2) { // S of the next head first: it runs under this head's softmax
                 if (hi + 1 < HG) ok = issue_s(hi + 1);
                 if (ok) ok = issue_pv(hi);
             } else {
@@ -402,6 +459,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
         const float cmax = a.p_bits == 4 ? 15.0f : 255.0f;     // last code
         const float pmax = a.p_log ? 256.0f : cmax;            // probabilities are held in units of 1 / pmax (linear codes: 1 / last code)
         const float inv255 = 1.0f / pmax;
+        auto p_place = [&](int chunk) { return smem + C::OFF_P + C::p_offset(r, chunk); };
         constexpr int CH2 = QRegs<D, Q8>::CH2;
         constexpr int OC = DP / 2;                       // O columns per thread
         bool alive = true;
@@ -414,12 +472,9 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
             // skips the work, never a barrier.
             unsigned char* U = smem + C::OFF_U;
             auto all256 = [&]() { asm volatile("bar.sync 5, 256;" ::: "memory"); };
-            // raw tile of the first head -> fp16 operand tile.  The 16-byte chunks of the tile are dealt out in linear order (thread t
-            // takes chunks t, t + 256, ...): consecutive lanes read consecutive words of the raw tile and write the eight
-            // chunk slots of a swizzled operand row, both free of bank conflicts.
+            // raw tile of the first head -> fp16 operand tile: half a row per thread
             auto stage_q_u = [&]() {
-                static_assert(D % 8 == 0 && (ROWS * (D / 8)) % 256 == 0, "chunks per thread");
-                constexpr int CPR = D / 8;                   // chunks per row
+                constexpr int N = D / 16, N2 = (N + 1) / 2;  // sixteen codes at a time
                 unsigned char* UQ = U + C::UO_BYTES;
                 auto load_q = [&](int hi) {                  // one thread: raw Q~ tile of head hi (rows beyond n_query read as zero)
                     ptx::mbar_arrive_expect_tx(qraw_full(hi), (uint32_t)(ROWS * D));
@@ -429,10 +484,12 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                 alive = __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(0), 0));
                 if (alive) {
 #pragma unroll
-                    for (int i = 0; i < ROWS * CPR / 256; ++i) {
-                        const int j = tid + 256 * i;
-                        const int row = j / CPR, cc = j - row * CPR;
-                        *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(row, cc & 7)) = codes_w8_to_half(*reinterpret_cast<const uint2*>(UQ + (size_t)j * 8));
+                    for (int i = 0; i < N2; ++i) {
+                        if (half * N2 + i < N) {
+                            const uint4 raw = *reinterpret_cast<const uint4*>(UQ + r * D + (half * N2 + i) * 16);
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i))) = codes_w8_to_half(make_uint2(raw.x, raw.y));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i) + 1)) = codes_w8_to_half(make_uint2(raw.z, raw.w));
+                        }
                     }
                     ptx::fence_proxy_async_smem();
                 }
@@ -498,7 +555,7 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                         for (int i = 1; i < HK / 8; ++i) ptx::reg_fence8(u8[i]);
                     }
                     ptx::tc_fence_before_sync();
-                    const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % 3) * C::CST_SLOT);
+                    const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT);
                     float m_loc, l_loc;
                     softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, sq, T, key0, e, m_loc, l_loc);
                     trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
@@ -520,8 +577,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                 }
                 if (tid == 0 && hi < 8) TAQ_PROF(48 + hi);
                 if (alive) {
-                    if (a.p_log) write_p_half_log(e, k255, cmax, trig, smem + C::OFF_P, C::A_BLOCK, r, half * (HK / 8));
-                    else write_p_half(e, k255, trig, smem + C::OFF_P, C::A_BLOCK, r, half * (HK / 8));
+                    if (a.p_log) write_p_half_log(e, k255, cmax, trig, half * (HK / 8), p_place);
+                    else write_p_half(e, k255, trig, half * (HK / 8), p_place);
                     ptx::fence_proxy_async_smem();
                     ptx::tc_fence_before_sync();
                 }
@@ -632,8 +689,8 @@ __global__ void __launch_bounds__(Cfg<D>::THREADS, Cfg<D>::CTAS_PER_SM) attentio
                 if (C::OBUF == 1) store_o(hi - 1);   // one O accumulator: empty it before the next PV may start
             }
             if (tid == 0 && hi < 8) TAQ_PROF(48 + hi);
-            if (a.p_log) write_p_half_log(e, k255, cmax, trig, smem + C::OFF_P, C::A_BLOCK, r, half * (HK / 8));
-            else write_p_half(e, k255, trig, smem + C::OFF_P, C::A_BLOCK, r, half * (HK / 8));
+            if (a.p_log) write_p_half_log(e, k255, cmax, trig, half * (HK / 8), p_place);
+            else write_p_half(e, k255, trig, half * (HK / 8), p_place);
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before_sync();
             __syncwarp();
@@ -684,15 +741,15 @@ EncodeTiledFn encode_tiled_fn3() {
 // A partial last wave of two CTAs per SM costs less than a full one.  (Measured, 64 row tiles x 10 heads of 64: five CTAs of
 // two heads each, 320 in two waves, 17.4 us; four of two or three heads, one wave, 14.9.  45 tiles x 8 heads of 80: two CTAs
 // of four heads 11.5 us, three of two or three 9.4.)
-template <int D>
+template <typename C>
 int pick_head_groups(const AttnArgs& a, int n_z) {
     const long long tiles = (long long)((a.n_query + ROWS - 1) / ROWS) * n_z;
     int best = 1;
     double best_cost = 1e30;
     for (int groups = 1; groups <= a.heads; ++groups) {
-        const long long ctas = tiles * groups, places = 148 * Cfg<D>::CTAS_PER_SM, waves = (ctas + places - 1) / places;
+        const long long ctas = tiles * groups, places = 148 * C::CTAS_PER_SM, waves = (ctas + places - 1) / places;
         const int most = (a.heads + groups - 1) / groups;
-        const double cost = Cfg<D>::CTAS_PER_SM == 2 ? (0.75 * (double)waves + 0.25 * std::max(1.0, (double)ctas / (double)places)) * (0.4 + most) : (double)waves * (2.0 + most);
+        const double cost = C::CTAS_PER_SM == 2 ? (0.75 * (double)waves + 0.25 * std::max(1.0, (double)ctas / (double)places)) * (0.4 + most) : (double)waves * (2.0 + most);
         if (cost <= best_cost) { best_cost = cost; best = groups; }
     }
     return best;
@@ -700,11 +757,11 @@ int pick_head_groups(const AttnArgs& a, int n_z) {
 
 template <int D, bool Q8, bool TAIL_ONLY>
 cudaError_t launch_k(const AttnArgs& a, int n_z, cudaStream_t stream) {
-    using C = Cfg<D>;
+    using C = Cfg<D, Q8>;
     static std::atomic<unsigned long long> limit_set;
     cudaError_t e = allow_shared_memory((const void*)attention_sm100_kernel<D, Q8, TAIL_ONLY>, C::TOTAL, limit_set);
     if (e != cudaSuccess) return e;
-    dim3 grid((a.n_query + ROWS - 1) / ROWS, pick_head_groups<D>(a, n_z), n_z);
+    dim3 grid((a.n_query + ROWS - 1) / ROWS, pick_head_groups<C>(a, n_z), n_z);
     CUtensorMap tmap_q, tmap_o;
     memset(&tmap_q, 0, sizeof(tmap_q));
     memset(&tmap_o, 0, sizeof(tmap_o));

@@ -109,8 +109,9 @@ __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const floa
 
 // Eq. 3 on the thread's HK probabilities e_j * k255 (units of 1/255): ordinary columns -> rint (exact, ties to even),
 // trigger columns -> fp16.  fma(e, k, 1.5 * 2^23 + 0x6400) leaves the integer code in the low byte and 0x64 above it,
-// which read as fp16 is 1024 + code.  `trig` holds the thread's HK trigger bits.  Writes chunks chunk0.. of row `r`.
-__device__ __forceinline__ void write_p_half(const float (&e)[HK], float k255, unsigned long long trig, unsigned char* p_tile, int a_block, int r, int chunk0) {
+// which read as fp16 is 1024 + code.  `trig` holds the thread's HK trigger bits.  Writes the row's chunks from chunk0 on, each where place(chunk) says.
+template <typename Place>
+__device__ __forceinline__ void write_p_half(const float (&e)[HK], float k255, unsigned long long trig, int chunk0, const Place& place) {
     const __half2 h1024 = __floats2half2_rn(1024.f, 1024.f);
 #pragma unroll
     for (int g = 0; g < HK / 8; ++g) {
@@ -134,8 +135,7 @@ __device__ __forceinline__ void write_p_half(const float (&e)[HK], float k255, u
                 pk[i] = __byte_perm(pk[i], *reinterpret_cast<uint32_t*>(&raw), sel);
             }
         }
-        const int chunk = chunk0 + g;
-        *reinterpret_cast<uint4*>(p_tile + (chunk >> 3) * a_block + ptx::sw128_offset(r, chunk & 7)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(place(chunk0 + g)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
 
@@ -147,7 +147,8 @@ __device__ __forceinline__ uint32_t log_code_to_half_bits(float t, float cmax) {
     const int c = (int)fminf(fmaxf(rintf(x), 0.f), cmax);
     return c <= 22 ? (uint32_t)(23 - c) << 10 : (c <= 32 ? 1u << (32 - c) : 0u);
 }
-__device__ __forceinline__ void write_p_half_log(const float (&e)[HK], float k256, float cmax, unsigned long long trig, unsigned char* p_tile, int a_block, int r, int chunk0) {
+template <typename Place>
+__device__ __forceinline__ void write_p_half_log(const float (&e)[HK], float k256, float cmax, unsigned long long trig, int chunk0, const Place& place) {
 #pragma unroll
     for (int g = 0; g < HK / 8; ++g) {
         const uint32_t bits = (uint32_t)(trig >> (8 * g)) & 0xFFu;
@@ -161,8 +162,7 @@ __device__ __forceinline__ void write_p_half_log(const float (&e)[HK], float k25
             if ((bits >> (2 * i + 1)) & 1u) h1 = __half_as_ushort(__float2half_rn(t1));
             pk[i] = h0 | (h1 << 16);
         }
-        const int chunk = chunk0 + g;
-        *reinterpret_cast<uint4*>(p_tile + (chunk >> 3) * a_block + ptx::sw128_offset(r, chunk & 7)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(place(chunk0 + g)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     }
 }
 
