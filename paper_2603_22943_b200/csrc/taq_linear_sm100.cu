@@ -163,9 +163,8 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
         c.lay.mul_cols = multiplier(c.lay.n_cols, tiles); c.lay.mul_rows = multiplier(c.lay.n_rows, tiles);
         c.grid = (int)ctas;
         // Packed weights asked for ahead of time, a share by each of up to 16 CTAs: where all CTAs of the launch find room beside its
-        // predecessor's (at most half the SMs: 2048 rows x 1280 x 1280, W4, on 128 of them lost up to 1.6 us) and the blob is large
-        // (two prompts, 320 channels, 132 KB: 8.91 us without, 8.97 with).  Weights of requests are known behind the wait only.
-        if (!a.reqs && ctas <= 74 && p.L.total >= (1u << 18) && p.L.total < (1u << 31)) {
+        // predecessor's, at most half the SMs.  Weights of requests are known behind the wait only.
+        if (!a.reqs && ctas <= 74 && p.L.total < (1u << 31)) {
             const uint32_t n = (uint32_t)std::min(ctas, 16LL), bytes = (uint32_t)align_up((p.L.total + n - 1) / n, 128);
             c.lay.blob_bytes = (uint32_t)p.L.total; c.lay.prefetch_bytes = bytes;
             c.lay.prefetch_ctas = (uint32_t)((p.L.total + bytes - 1) / bytes);

@@ -244,15 +244,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
     } else if (warp == TL::W_AUX && lane == 0) {
         ptx::tma_prefetch_desc(&tmap_x);
-    } else if (warp == TL::W_AUX + 1 && lane == 0) {
-        // Packed weights, on their way to L2 while the previous kernel runs (the builders may read only behind the wait).  Sixteen
-        // projections of a prompt 175.5 -> 173.2 us, the three launches of 64 x 1280 x 1280 W8 23.1 -> 22.7.  (Wide tiles of the other
-        // outputs have no register to spare for it: 116 bytes of spills, 2048 x 1280 x 1280 1.6 us more.)
-        if ((KV || !TL::BIG) && !persistent && blockIdx.x < lay.prefetch_ctas) {
-            const uint32_t from = blockIdx.x * lay.prefetch_bytes, n = min(lay.prefetch_bytes, lay.blob_bytes - from);
-            ptx::prefetch_l2((const uint8_t*)a.w + from, n);
-            if (KV) ptx::prefetch_l2((const uint8_t*)a.w2 + from, n);
-        }
     }
     // Every role passes this barrier before it touches another role's state; the builders do so with their first codes under way,
     // and the producer, whose own barriers are all it needs, only announces itself and starts to load.
@@ -799,6 +790,16 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         else if (warp < TL::W_AUX + 2) {
             // ---------------- scales and biases, one tile ahead ----------------
+            // Packed weights, on their way to L2 while the previous kernel runs (the builders may read only behind the wait).  Sixteen
+            // projections of a prompt 175.5 -> 171.5 us, sixteen layers of a denoising step 317.3 -> 315.4 (in front of the barrier above, which
+            // it kept everybody from, 172.1 and 316.5, and 8.99 instead of 8.91 for two prompts at 320 channels).  Not in the other
+            // tiles: the wide ones have no register to spare (116 bytes of spills, 2048 x 1280 x 1280 1.6 us more), and a layer of
+            // 1294 rows x 640, 64-wide tiles on 120 CTAs, which none of them asks for, lost 0.2 us of 20.9 to the code alone.
+            if ((KV || BN == 80) && !persistent && warp == TL::W_AUX + 1 && lane == 0 && blockIdx.x < lay.prefetch_ctas) {
+                const uint32_t from = blockIdx.x * lay.prefetch_bytes, n = min(lay.prefetch_bytes, lay.blob_bytes - from);
+                ptx::prefetch_l2((const uint8_t*)a.w + from, n);
+                if (KV) ptx::prefetch_l2((const uint8_t*)a.w2 + from, n);
+            }
             if (!a.early_weights) ptx::pdl_wait();
             int sbuf = 0, it = 0;
             uint32_t ph = 1;
