@@ -807,7 +807,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             {
                 constexpr int N = NQ / 8;                        // 16-byte chunks of a row
                 __half* out = a.y + ((size_t)zb * a.n_query + row0 + q4 * 32) * KIN + col0;
-                const int left = ok ? a.n_query - (row0 + q4 * 32) : 0;
+                const int left = ok && !misc->abort_flag ? a.n_query - (row0 + q4 * 32) : 0;     // (a warp that gave up has staged nothing, and raised the flag before the barrier)
 #pragma unroll
                 for (int i = 0; i < N / 4; ++i) {
                     const int j = hi * 32 + lane + 128 * i, rr = j / N, part = j - rr * N;

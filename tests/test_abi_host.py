@@ -176,3 +176,17 @@ def test_dispatch_counters_start_at_zero_and_reset(L):
 def test_wait_expiry_selftest_rejects_bad_limits(L):
     for bad in (0, -5, (1 << 31) + 1):                 # (refused on the host: nothing is launched)
         assert L.taq_selftest_wait_expiry(bad, None) == tb.TAQ_ERR_INVALID_ARG
+
+
+def test_rows_that_several_warps_staged_are_stored_only_if_none_of_them_gave_up():
+    """The layer kernels stage an output tile by several warps, meet at a barrier and store it.  A warp whose bounded wait ran out
+    stages nothing and raises the abort flag before it arrives there, so the flag is looked at behind the barrier: a pass that
+    timed out leaves Y as it was or writes right rows.  (Read from the source: a wait that runs out in one warp of a cluster
+    is not made to happen on a GPU, where the partner CTA's copies would still be on their way.)"""
+    for name, barrier, store in (("taq_layer_c320_sm100.cu", '"bar.sync %0, 128;" ::"r"(2 + q4)', "reinterpret_cast<uint4*>(out +"),
+                                 ("taq_layer_c320_sm100.cu", '"bar.sync %0, 128;" ::"r"(2 + hi)', "tma_store_3d(&tmap_y"),
+                                 ("taq_qattn_sm100.cu", '"bar.sync 1, 512;"', "tma_store_3d(&tmap_y, stage +")):
+        src = open(os.path.join(tbuild.CSRC, name)).read()
+        at = src.index(store)
+        between = src[src.rindex(barrier, 0, at): at]
+        assert "!misc->abort_flag" in between, (name, barrier)
