@@ -778,11 +778,10 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         b_lo += 2 * TL::B_TILE >> 4;
                         if (++sa == nsa) { sa = 0; pha ^= 1; a_lo = a_lo0; }
                         if (++sb == nsb) { sb = 0; phb ^= 1; b_lo = b_lo0; }
-                        // (a try_wait suspends the thread for some time: none for a pair that does not come)
-                        if (todo > 0) {
-                            next_b = ptx::mbar_try_wait(&bars->full_b[sb], phb);
-                            next_a = ptx::mbar_try_wait(&bars->full_a[sa], pha);
-                        }
+                        // (also behind the last pair, for one that does not come: with a test of `todo` in front launches of one wave took
+                        // 0.04 - 0.1 us more, 2048 x 640 x 640 6.04 -> 5.96 us without it, 64 x 320 x 320, per head, 4.59 -> 4.51)
+                        next_b = ptx::mbar_try_wait(&bars->full_b[sb], phb);
+                        next_a = ptx::mbar_try_wait(&bars->full_a[sa], pha);
                     }
                 }
                 if (!ok) give_up();
