@@ -545,20 +545,27 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 for (int c = 0; c < HC; ++c) w[c] = __float_as_uint(y[c]);
                 put(w, std::integral_constant<int, HC * 4>{});
             } else {
-                // Per-(row, head) symmetric int8.  A thread's columns are one head or a half or a quarter of one.
-                const int d = lay.d;
+                // Per-(row, head) symmetric int8.  A thread's columns are one head or a half or a quarter of one.  On 32-column threads
+                // heads are 64 wide, which is compiled in where it shortens the code (8192 x 1280 x 1280 of int8 rows and W8, heads of
+                // 64: 25.1 -> 23.2 us; with fp16 rows and W4 the persistent kernel would spill: 8192 x 640 x 640 15.8 -> 16.6; int8
+                // rows and W8, a tile per CTA: 1294 x 1280 x 1280 7.67 -> 7.77).
+                constexpr bool D64 = !KV && HC == 32 && (I8 != W8 || (I8 && persistent));
+                const int d = D64 ? 64 : lay.d;
                 const int colg = col0 + cb;
-                const int h0 = quotient(colg, d, lay.mul_d);
+                const int h0 = D64 ? colg / 64 : quotient(colg, d, lay.mul_d);
                 float am = 0.f;
 #pragma unroll
                 for (int c = 0; c < HC; ++c) am = fmaxf(am, fabsf(y[c]));
                 if (d > HC) {                                // the row's threads with columns of the same head combine their absmax
                     float* xc = reinterpret_cast<float*>(smem + P.off_xchg);     // [NCG][128], and at 384 the absmax of a head pair's other half
-                    const int per_head = lay.per_head, first = cg & ~(per_head - 1);
+                    // (the partners by exclusive or in the persistent kernels of int8 rows, which spill less: 8192 x 1280 x 1280, W8,
+                    // heads of 160, 27.0 -> 26.3 us; the others spill more that way)
+                    constexpr bool PARTNERS = I8 && persistent;
+                    const int per_head = D64 ? 2 : lay.per_head, first = cg & ~(per_head - 1);
                     xc[cg * 128 + r] = am;
                     asm volatile("bar.sync %0, %1;" ::"r"(2 + q), "n"(NCG * 32) : "memory");
 #pragma unroll
-                    for (int k = 0; k < NCG; ++k) if (k < per_head) am = fmaxf(am, xc[(first + k) * 128 + r]);
+                    for (int k = PARTNERS ? 1 : 0; k < NCG; ++k) if (k < per_head) am = fmaxf(am, xc[(PARTNERS ? cg ^ k : first + k) * 128 + r]);
                     if (persistent) asm volatile("bar.sync %0, %1;" ::"r"(6 + q), "n"(NCG * 32) : "memory");      // (read before the next tile's are written)
                     if (!KV && lay.head_pair && mine) {
                         // The head's other columns belong to a CTA of the same cluster (same rows, same share of the K loop):
