@@ -112,12 +112,12 @@ struct LayerArgs {
     const void* kv;             // blocks [B] (single problem)
     const taq_request* reqs;    // nullable; then one sequence per request
     __half* o;                  // [z][N][C]  (query-attention variant)
-    __half* y;                  // [z][N][C]  (layer variant)
     const void* q;              // attention-only variant: Q~ codes (int8) or Q (fp16) [z][N][C] ...
     const float* q_scales;      // ... and the row scales [z][N][H] (q_bits = 8)
     int n_query, heads, n_ctx, max_trigger, group, q_bits, p_bits;
     long long wait_cycles;      // limit of every device-side wait
     int* status;
+    __half* y;                  // [z][N][C]  (layer variant; in front of q it cost the attention-only variant 0.1 us of 8.3)
 };
 
 // The same by the first NT worker threads only (phase 4: the warps of the last head, whose probabilities are the last to
