@@ -781,7 +781,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) qattn_c320_kernel(const __grid_co
                 store_o(hi - 2);
             }
             if (lane == 0 && q4 == 0 && half == 0) TAQ_PROF(12 + 8 * grp + 4 * it);       // exchange (and previous O) done
-            write_p_half(e, k255, trig, half * (HK / 8), [&](int chunk) { return smem + OFF_P + (grp * 2 + (chunk >> 3)) * A_TILE + ptx::sw128_offset(r, chunk & 7); });
+            write_p_half(e, k255, trig, smem + OFF_P + grp * 2 * A_TILE, A_TILE, r, half * (HK / 8));
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before_sync();
             __syncwarp();
