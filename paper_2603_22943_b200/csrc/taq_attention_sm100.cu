@@ -10,7 +10,7 @@
 //   warp 8     one thread issues the MMAs: S of head h+1 is in flight while the rows are in the softmax of head h;
 //   warp 9     one thread fetches each head's K~/V~ operand image (written once per prompt by the K/V projection)
 //              by bulk copies, one head ahead: the whole image into the second buffer (head widths up to 64), or,
-//              with a single buffer, K~ as soon as this head's S is complete and V~^T as soon as its PV is (wide heads with
+//              with a single buffer, K~ as soon as this head's S is complete and V~^T as soon as its PV is (heads of 80 with
 //              int8 Q~: K~ into a second buffer, V~^T by a thread of warp 10).
 // Head widths up to 64: two CTAs share an SM, and the row threads read Q~ and write O themselves.  Head widths 80 and
 // 160: one CTA per SM; Q~ tiles arrive and O tiles leave by TMA, and from the second head on warps of their own do that work:
@@ -45,11 +45,13 @@ constexpr int Q_WARP = 12, O_WARP = 16;
 constexpr int R_WIDE_ROWS = 128, R_WIDE_REST = 40, R_WIDE_Q = 72, R_WIDE_O = 104;
 static_assert(2 * R_WIDE_ROWS + R_WIDE_REST + R_WIDE_Q + R_WIDE_O <= 5 * 96, "register split");
 
-// Head widths 80 and 160 with int8 Q~ (K2) have two K~ buffers, so that a head's K~ is there long before its S may start: with one it
+// Heads of 80 channels with int8 Q~ (K2) have two K~ buffers, so that a head's K~ is there long before its S may start: with one it
 // was asked for when the S before it was complete, and S came 400 - 800 cycles after the rows were ready for it (16 x 1024 rows, 8 heads of
-// 80: 18.7 -> 17.2 us, 3 x 1872 9.4 -> 9.0, 64 x 256, 8 heads of 160 25.6 -> 25.2).  What makes room for
-// the second one at 160 channels: the last 32 (16) channels of Q~ and the last 16 keys of P are tiles of 64- and 32-byte rows of
-// their own instead of half-empty 128-byte ones.
+// 80, inputs in L2: 17.4 -> 16.1 us, 3 x 1872 8.65 -> 8.22).  The last 16 channels of their Q~ and the last 16 keys of everybody's P are tiles
+// of 32-byte rows of their own instead of half-empty 128-byte ones.
+// At 160 channels a K~ asked for that early is in the way of the V~^T that is needed first (30 and 40 KB at some 20 bytes a cycle): one
+// buffer, and K~ behind V~^T in the order of one thread, takes 21.6 us for 16 x 1024 rows, 8 heads of 160, 12.5 for 2 x 4096 and 10.6 for 3 x
+// 1872, two buffers 22.9, 13.3 and 10.95.  (64 x 256 rows, where two row tiles and no more share an image, 24.4 and 24.2.)
 template <int D, bool Q8>
 struct Cfg {
     static constexpr int DP = (D + 15) / 16 * 16;            // head width padded to the MMA K / N granule
@@ -62,8 +64,8 @@ struct Cfg {
     static constexpr int HEAD_BYTES = K_BYTES + VT_BYTES + kOperandConstBytes;
     static constexpr int KVBUF = D <= 64 ? 2 : 1;            // K~/V~ images in flight
     static constexpr int OBUF = D == 64 ? 1 : 2;             // O accumulators in TMEM
-    static constexpr bool K2 = D >= 80 && Q8;
-    static constexpr int QFULL = K2 ? DP / 64 : KBQ, QTAIL = K2 ? DP % 64 : 0;     // 64-wide blocks of the Q~ tile, channels of its narrow one
+    static constexpr bool K2 = D == 80 && Q8;
+    static constexpr int QFULL = K2 ? DP / 64 : KBQ, QTAIL = K2 ? DP % 64 : 0;     // 64-wide blocks of the Q~ tile, channels of its narrow one (16)
     static constexpr int OFF_KV = 0;                         // images; wide heads: K~ (twice if K2), V~^T
     static constexpr int OFF_V = OFF_KV + (K2 ? 2 : 1) * K_BYTES;
     static constexpr int OFF_Q = D <= 64 ? OFF_KV + KVBUF * HEAD_BYTES : OFF_V + VT_BYTES;
@@ -92,11 +94,12 @@ struct Cfg {
     static constexpr int CTAS_PER_SM = (2 * (TOTAL + 1024) <= 232448 && TMEM_COLS == 256) ? 2 : 1;
     static_assert(HEAD_BYTES % 1024 == 0 && K_BYTES % 1024 == 0 && VT_BLOCK % 1024 == 0, "operand tiles must keep 1024-byte alignment");
     static_assert(TOTAL <= 232448, "shared memory budget");
+    static_assert(QTAIL == 0 || QTAIL == 16, "narrow tile of Q~: 32-byte rows");
     static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0 && OFF_U % 128 == 0, "tile alignment");
     // 16-byte chunk cc (8 channels) of a row of the Q~ tile; chunk of a row of P (8 keys)
     static __device__ __forceinline__ uint32_t q_offset(int row, int cc) {
         if (QTAIL == 0 || cc < 8 * QFULL) return (cc >> 3) * A_BLOCK + ptx::sw128_offset(row, cc & 7);
-        return QFULL * A_BLOCK + (QTAIL == 16 ? ptx::sw32_offset(row, cc - 8 * QFULL) : ptx::sw64_offset(row, cc - 8 * QFULL));
+        return QFULL * A_BLOCK + ptx::sw32_offset(row, cc - 8 * QFULL);
     }
     static __device__ __forceinline__ uint32_t p_offset(int row, int chunk) {
         if (D < 80) return (chunk >> 3) * A_BLOCK + ptx::sw128_offset(row, chunk & 7);
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             }
         }
     } else if (C::K2 && warp == V_WARP) {
-        // ---------------- V~^T of wide heads with two K~ buffers: as soon as the PV before it is complete ----------------
+        // ---------------- V~^T of heads with two K~ buffers: as soon as the PV before it is complete ----------------
         if (lane == 0) {
             if (!a.early_kv) ptx::pdl_wait();
             const uint8_t* blk = a.reqs ? (const uint8_t*)a.reqs[zb].kv : (const uint8_t*)a.kv + (size_t)b * KL.block_bytes;
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
 #pragma unroll
                 for (int ks = 0; ks < DP / 16; ++ks) {
                     const uint64_t qd = ks < 4 * C::QFULL ? ptx::desc_join(HI, q_lo0 + (ks / 4) * (C::A_BLOCK >> 4) + (ks % 4) * 2)
-                                                          : ptx::desc_join(C::QTAIL == 16 ? ptx::kDescHiSw32 : ptx::kDescHiSw64, q_lo0 + C::QFULL * (C::A_BLOCK >> 4) + (ks - 4 * C::QFULL) * 2);
+                                                          : ptx::desc_join(ptx::kDescHiSw32, q_lo0 + C::QFULL * (C::A_BLOCK >> 4) + (ks - 4 * C::QFULL) * 2);
                     ptx::mma_f16_ss(tmem_base + C::TMEM_S + (hi & 1) * TP, qd, ptx::desc_join(HI, k_lo + (ks / 4) * (C::K_BLOCK >> 4) + (ks % 4) * 2), ptx::idesc_f16_m128(TP), ks != 0);
                 }
                 ptx::mma_commit(&misc->s_full[hi & 1]);
@@ -425,10 +428,12 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                 if (ok) ok = issue_pv(hi);
             } else {
                 // one image buffer: the next head's K~ arrives some time after this head's S; its S goes as soon as K~ and Q~
-                // are there (it then runs under this head's softmax), at the latest after this head's PV
+                // are there (it then runs under this head's softmax), at the latest after this head's PV.  Nothing to look out for once it
+                // is under way, nor behind the last head (while this loop waited for the probabilities there, too, a CTA of one
+                // head took 0.1 us longer).
                 bool s_next = hi + 1 >= HG;
-                for (const long long t0 = clock64(); ok;) {
-                    if (!s_next && ptx::mbar_try_wait(&misc->kv_full[0], (hi + 1) & 1) && ptx::mbar_try_wait(&misc->q_full, (hi + 1) & 1)) ok = s_next = issue_s(hi + 1);
+                for (const long long t0 = clock64(); ok && !s_next;) {
+                    if (ptx::mbar_try_wait(&misc->kv_full[0], (hi + 1) & 1) && ptx::mbar_try_wait(&misc->q_full, (hi + 1) & 1)) ok = s_next = issue_s(hi + 1);
                     if (ptx::mbar_try_wait(&misc->p_full, hi & 1)) break;
                     if (clock64() - t0 > ptx::kWaitCycles) ok = false;
                 }
