@@ -96,9 +96,9 @@ struct Cfg {
     static_assert(TOTAL <= 232448, "shared memory budget");
     static_assert(QTAIL == 0 || QTAIL == 16, "narrow tile of Q~: 32-byte rows");
     static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0 && OFF_U % 128 == 0, "tile alignment");
-    // 16-byte chunk cc (8 channels) of a row of the Q~ tile; chunk of a row of P (8 keys)
-    static __device__ __forceinline__ uint32_t q_offset(int row, int cc) {
-        if (QTAIL == 0 || cc < 8 * QFULL) return (cc >> 3) * A_BLOCK + ptx::sw128_offset(row, cc & 7);
+    // 16-byte chunk cc ^ flip (8 channels; flip 0 or 2) of a row of the Q~ tile; chunk of a row of P (8 keys)
+    static __device__ __forceinline__ uint32_t q_offset(int row, int cc, int flip = 0) {
+        if (QTAIL == 0 || cc < 8 * QFULL) return (cc >> 3) * A_BLOCK + (ptx::sw128_offset(row, cc & 7) ^ (flip << 4));
         return QFULL * A_BLOCK + ptx::sw32_offset(row, cc - 8 * QFULL);
     }
     static __device__ __forceinline__ uint32_t p_offset(int row, int chunk) {
@@ -202,20 +202,23 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R_WIDE_Q));
             bool alive = true;
             if constexpr (Q8) {
-                // A thread is a row: sixteen codes per load (rows of 80 or 160 bytes: no or two-way bank conflicts), and every place in the
-                // operand tile is a constant beside the row's.  They are read before S of the head before is complete (its operand
+                // A thread is a row: sixteen codes per load, and every place in the operand tile is a constant beside the row's.  Rows of 80
+                // bytes are free of bank conflicts; of rows of 160 bytes four start 32 bytes apart and the next four at the same
+                // banks, so these take their chunks in pairs the other way round (`swap`: 16 x 1024 rows, 8 heads of 160, 21.5 -> 21.3 us, 64
+                // x 256 24.1 -> 23.8).  They are read before S of the head before is complete (its operand
                 // tile is free then), and the raw tile of the head after next lands under all that.  (With the chunks dealt out in
                 // linear order, row and place worked out for each, S of a head of 160 channels was 2 500 cycles later.)
                 constexpr int N = D / 16;
                 const unsigned char* UQ = smem + C::OFF_U + C::UO_BYTES;
-                const int t = tid - 32 * Q_WARP;
+                const int t = tid - 32 * Q_WARP, swap = D == 160 ? (t >> 2) & 1 : 0;
+                static_assert(D != 160 || (N % 2 == 0 && C::QTAIL == 0), "pairs of chunks");
                 if (t == 0) ptx::pdl_wait();                             // (this thread loads Q~ of the third head and on)
                 __syncwarp();
                 for (int hi = 1; hi < HG; ++hi) {
                     alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(hi), (hi >> 1) & 1));
                     uint4 raw[N];
 #pragma unroll
-                    for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint4*>(UQ + t * D + i * 16);
+                    for (int i = 0; i < N; ++i) raw[i] = *reinterpret_cast<const uint4*>(UQ + t * D + (i ^ swap) * 16);
                     ptx::fence_proxy_async_smem();                           // (generic reads before the TMA load that overwrites them)
                     asm volatile("bar.sync 6, 128;" ::: "memory");           // the raw tile has been read
                     if (t == 0 && alive && hi + 1 < HG) {
@@ -227,8 +230,8 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                     if (alive) {
 #pragma unroll
                         for (int i = 0; i < N; ++i) {
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i)) = codes_w8_to_half(make_uint2(raw[i].x, raw[i].y));
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i + 1)) = codes_w8_to_half(make_uint2(raw[i].z, raw[i].w));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].x, raw[i].y));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i + 1, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].z, raw[i].w));
                         }
                         ptx::fence_proxy_async_smem();
                     }
