@@ -225,3 +225,99 @@ def test_projection_weights_written_right_before_the_call_are_the_ones_it_uses(c
         tb.taq_poll_device_status()
         for i, kv in enumerate(kvs):
             assert torch.equal(kv, want[i % 2]), (order, i)
+
+
+@pytest.mark.parametrize("batch,n_query,channels,heads,w_bits,a_bits", [
+    (1, 64, 1280, 8, 8, 16),
+    (2, 256, 1280, 8, 4, 8),
+    (2, 1024, 640, 8, 4, 16),
+    (2, 700, 320, 8, 8, 8),
+    (2, 700, 320, 8, 4, 16),
+    (2, 700, 320, 8, 4, 8),
+])
+def test_checkpoints_packed_in_place_between_passes(batch, n_query, channels, heads, w_bits, a_bits):
+    """Two checkpoints take turns on the same four blobs: their matrices are written by an elementwise kernel, packed over the blobs
+    that the previous pass has just read, and used at once by a K/V projection and a layer pass."""
+    gen = torch.Generator("cuda").manual_seed(7)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    group, dc, t = (128 if w_bits == 4 else 0), 768, 77
+    desc = tb.layer_desc(batch, n_query, channels, heads, t, dc, w_bits, group, max_trigger=2)
+    mask = torch.zeros((batch, t), dtype=torch.uint8, device="cuda")
+    mask[:, 4:6] = 1
+    ctx, x, bias = normal(batch, t, dc).half(), normal(batch, n_query, channels).half(), 0.1 * normal(channels)
+    shapes = [(channels, dc), (channels, dc), (channels, channels), (channels, channels)]          # Wk, Wv, Wq, Wout
+    wds = [tb.weight_desc(n_out, k_in, w_bits, group) for n_out, k_in in shapes]
+    negatives = [[normal(n_out, k_in) / k_in ** 0.5 for n_out, k_in in shapes] for _ in range(2)]
+    w = [torch.zeros_like(m) for m in negatives[0]]
+    blobs = [torch.zeros(tb.taq_packed_weight_bytes(d), dtype=torch.uint8, device="cuda") for d in wds]
+    kv = torch.zeros(tb.taq_kv_bytes(desc), dtype=torch.uint8, device="cuda")
+    size = tb.taq_workspace_bytes_a8(desc) + tb.lib().taq_kv_project_a8_workspace_bytes(desc)
+    ws = torch.zeros(size, dtype=torch.uint8, device="cuda")
+
+    def swap_in(which, k):
+        torch.neg(negatives[which][k], out=w[k])
+        tb.taq_pack_weights(wds[k], w[k], bias if k == 3 else None, blobs[k])
+
+    def one(which, y, wait=lambda: None):
+        for k in (0, 1):
+            swap_in(which, k)
+            wait()
+        if a_bits == 8:
+            tb.taq_kv_project_a8(desc, ctx, blobs[0], blobs[1], mask, kv, ws)
+        else:
+            tb.taq_kv_project(desc, ctx, blobs[0], blobs[1], mask, kv)
+        wait()
+        for k in (3, 2):
+            swap_in(which, k)
+            wait()
+        (tb.taq_layer_forward_a8 if a_bits == 8 else tb.taq_layer_forward)(desc, x, blobs[2], blobs[3], kv, mask, y, ws)
+        wait()
+
+    new_y = lambda: torch.full((batch, n_query, channels), float("nan"), dtype=torch.float16, device="cuda")
+    want = [new_y(), new_y()]
+    for which in range(2):
+        one(which, want[which], torch.cuda.synchronize)
+    assert not torch.equal(want[0], want[1]) and not bool(want[0].isnan().any())
+    ys = [new_y() for _ in range(2 * ROUNDS)]
+
+    def check(how):
+        torch.cuda.synchronize()
+        tb.taq_poll_device_status()
+        for i, y in enumerate(ys):
+            assert torch.equal(y.view(torch.int16), want[i % 2].view(torch.int16)), (how, i)
+            y.fill_(float("nan"))
+
+    def sequence():
+        for i, y in enumerate(ys):
+            one(i % 2, y)
+
+    sequence()
+    check("call by call")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        sequence()
+    for _ in range(2):
+        graph.replay()
+        check("from a graph")
+
+
+def test_matrices_packed_back_to_back_into_one_blob():
+    """Packing calls in a row, into two blobs in turn and from one W that an elementwise kernel rewrites in between: no call starts to
+    write a blob, or reads W, before what was launched in front of it is through."""
+    gen = torch.Generator("cuda").manual_seed(8)
+    normal = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    for n_out, k_in, bits, group in ((1280, 1280, 4, 128), (640, 2048, 8, 0), (320, 768, 4, 0)):
+        wd = tb.weight_desc(n_out, k_in, bits, group)
+        negatives = [normal(n_out, k_in) for _ in range(3)]
+        want = [tb.taq_pack_weights(wd, -m) for m in negatives]
+        torch.cuda.synchronize()
+        w, place = torch.zeros_like(negatives[0]), [torch.zeros_like(want[0]) for _ in range(2)]
+        got = [torch.zeros_like(want[0]) for _ in range(12)]
+        for i, g in enumerate(got):
+            torch.neg(negatives[i % 3], out=w)
+            tb.taq_pack_weights(wd, w, None, place[i % 2])
+            tb.taq_pack_weights(wd, w, None, place[1 - i % 2])
+            g.copy_(place[i % 2])
+        torch.cuda.synchronize()
+        for i, g in enumerate(got):
+            assert torch.equal(g, want[i % 3]) and torch.equal(place[i % 2], want[(len(got) - 1) % 3]), i

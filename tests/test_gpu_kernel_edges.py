@@ -75,6 +75,7 @@ def test_kv_projection(channels, heads, ctx_dim, n_ctx, batch, w_bits):
 
 @pytest.mark.parametrize("n_out,k_in,bits,group", [
     (40, 512, 4, 256), (24, 1024, 4, 512), (16, 2560, 8, 0), (9, 136, 8, 0), (33, 352, 4, 32), (7, 1000, 4, 128), (5, 2560, 4, 0),
+    (1200, 4160, 4, 32), (19000, 512, 4, 256), (9600, 520, 8, 0),        # more groups than 4736 blocks take at once, for 8, 32 and 128 threads per group
 ])
 def test_pack_group_lengths(n_out, k_in, bits, group):
     quantizers.test_pack_weights_codes_bit_exact(n_out, k_in, bits, group)
