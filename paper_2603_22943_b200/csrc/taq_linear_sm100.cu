@@ -123,6 +123,8 @@ bool rings_of(const LinearArgs& a, const Problem& p, int bn, int nsplit, int hea
     return false;
 }
 
+constexpr int SMS = 148;                                 // of a B200
+
 // Whether a tile of bn columns can carry the epilogue: per-head outputs want a thread's 80 or 64 columns to be whole heads, or a
 // head of 160 channels on the two threads of a row.
 bool tile_carries(const LinearArgs& a, const Problem& p, int bn) {
@@ -164,7 +166,7 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
         c.grid = (int)ctas;
         // Packed weights asked for ahead of time, a share by each of up to 16 CTAs: where all CTAs of the launch find room beside its
         // predecessor's, at most half the SMs.  Weights of requests are known behind the wait only.
-        if (!a.reqs && ctas <= 74 && p.L.total < (1u << 31)) {
+        if (!a.reqs && ctas <= SMS / 2 && p.L.total < (1u << 31)) {
             const uint32_t n = (uint32_t)std::min(ctas, 16LL), bytes = (uint32_t)align_up((p.L.total + n - 1) / n, 128);
             c.lay.blob_bytes = (uint32_t)p.L.total; c.lay.prefetch_bytes = bytes;
             c.lay.prefetch_ctas = (uint32_t)((p.L.total + bytes - 1) / bytes);
@@ -176,7 +178,7 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
     if (a.epi == EPI_Q8_HEAD && p.d == 160 && a.bits == 4 && (p.n_groups >= 2 || (!p.i8 && p.n_kb >= 2))) {
         const long long tiles = p.row_tiles * (a.n_out / 80) * (long long)n_z;
         Choice c{};
-        if (tiles * 2 <= 148 && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);
+        if (tiles * 2 <= SMS && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);
     }
     double best_cost = 1e30;
     for (const Pace& m : PACES) {
@@ -190,17 +192,17 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
             // and 13.3 us, 13.2 and 13.1); unsplit, a prompt's bits are the same in every batch.  Of a 2048-wide one four CTAs take
             // 14.6 us to 11.2 at 640 channels.)
             if (ns > 1 && a.epi == EPI_KV && a.k_in < 1024) continue;
-            if (ns > 1 && ((p.i8 && p.n_groups == 1) || (p.n_groups == 1 ? p.n_kb : p.n_groups) < ns || tiles * ns > 148)) continue;    // (integer activations: a group's sum stays one exact int32 accumulation)
-            const bool persistent = a.epi != EPI_KV && tiles * ns > 148;           // (K~/V~ tiles are assembled in the rings: one per CTA)
+            if (ns > 1 && ((p.i8 && p.n_groups == 1) || (p.n_groups == 1 ? p.n_kb : p.n_groups) < ns || tiles * ns > SMS)) continue;    // (integer activations: a group's sum stays one exact int32 accumulation)
+            const bool persistent = a.epi != EPI_KV && tiles * ns > SMS;           // (K~/V~ tiles are assembled in the rings: one per CTA)
             Choice c{};
             if (!rings_of(a, p, bn, ns, 0, persistent, c)) continue;
-            const long long per = (tiles * ns + 147) / 148;                                            // tiles per CTA
+            const long long per = (tiles * ns + SMS - 1) / SMS;                                            // tiles per CTA
             const long long ctas = persistent ? (tiles + per - 1) / per : tiles * ns;
             const int share = share_of(p, ns);
             const double fixed = m.fixed + (a.epi == EPI_KV ? 0.008 * bn : 0), tile = persistent ? m.tile : 0;
             const double groups = p.n_groups == 1 ? 1 : (double)share * p.n_groups / p.n_kb;
             const double cost = (persistent ? 1 : per) * fixed + (double)per * (share * m.kb + groups * m.group + tile + (a.epi == EPI_Q8_HEAD ? m.q8 : 0)) +
-                                (ns > 1 ? m.split + 0.1 * (ns - 2) + m.exchange * (ns - 1) * (double)(tiles * ns) / 148 : 0);
+                                (ns > 1 ? m.split + 0.1 * (ns - 2) + m.exchange * (ns - 1) * (double)(tiles * ns) / SMS : 0);
             if (cost < best_cost) { best_cost = cost; best = finish(c, tiles, ctas); }
         }
     }
