@@ -17,7 +17,7 @@
 //   warps 12-15  expand the next head's codes (fp16 Q~: load it straight into the operand tile);
 //   warps 16-19  bring the previous head's O from TMEM to global memory.
 // (With the row warps doing everything in turn a head of 160 channels took 5 700 cycles: softmax 1 650, codes 1 100, O 2 250,
-// probabilities 600; now 4 000.)
+// probabilities 600.)
 #include "taq_prof.cuh"
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"

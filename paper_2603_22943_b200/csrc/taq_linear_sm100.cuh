@@ -22,8 +22,11 @@
 //
 // What bounds it.  A 64-wide K block of a 160-column tile is 320 cycles of tensor time; the MMA thread needs 60 cycles per wait
 // on a complete barrier, 60 per commit and 45 per MMA (measured), hence barriers per pair of blocks, looked at one pair ahead.
-// Nothing in the loops may spill: beside 200 KB of shared memory there is next to no L1, and a spilled register is a
-// round trip to L2 (a first version with 120 bytes of spills ran at half the speed), hence the register split.
+// A register spilled in a loop is a round trip to L2, since beside 200 KB of shared memory there is next to no L1 (a first version
+// with 120 bytes of spills ran at half the speed), hence the register split.  What `-Xptxas -v` still reports at 72
+// registers: 4 to 64 bytes stored and up to 108 loaded in most 160-wide kernels and some of the others, none in the rest.  Whether such a
+// kernel pays for them is told by its time only: the unsplit 160-wide K/V kernels went from 8 / 8 bytes to 36 / 84 when their epilogue was
+// shortened, and two prompts at 1280 channels from 15.3 to 14.0 us.
 #pragma once
 #include "taq_ptx.cuh"
 #include "taq_sm100.cuh"
@@ -798,9 +801,11 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             // ---------------- scales and biases, one tile ahead ----------------
             // Packed weights, on their way to L2 while the previous kernel runs (the builders may read only behind the wait).  Sixteen
             // projections of a prompt 175.5 -> 171.5 us, sixteen layers of a denoising step 317.3 -> 315.4 (in front of the barrier above, which
-            // it kept everybody from, 172.1 and 316.5, and 8.99 instead of 8.91 for two prompts at 320 channels).  Not in the other
-            // tiles: the wide ones have no register to spare (116 bytes of spills, 2048 x 1280 x 1280 1.6 us more), and a layer of
-            // 1294 rows x 640, 64-wide tiles on 120 CTAs, which none of them asks for, lost 0.2 us of 20.9 to the code alone.
+            // it kept everybody from, 172.1 and 316.5, and 8.99 instead of 8.91 for two prompts at 320 channels).  In the K/V kernels of
+            // every width (the wide ones spill as much without it: 36 bytes stored, 84 loaded in 160-wide tiles, none in the 128- and 64-wide
+            // ones) and in the 80-wide ones.  Not in the others that are no K/V kernels: the wide ones have no register to spare there (116 bytes of
+            // spills, 2048 x 1280 x 1280 1.6 us more), and a layer of 1294 rows x 640, 64-wide tiles on 120 CTAs, which none of
+            // them asks for, lost 0.2 us of 20.9 to the code alone.
             if ((KV || BN == 80) && !persistent && warp == TL::W_AUX + 1 && lane == 0 && blockIdx.x < lay.prefetch_ctas) {
                 const uint32_t from = blockIdx.x * lay.prefetch_bytes, n = min(lay.prefetch_bytes, lay.blob_bytes - from);
                 ptx::prefetch_l2((const uint8_t*)a.w + from, n);
