@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                 // A thread is a row: sixteen codes per load, and every place in the operand tile is a constant beside the row's.  Rows of 80
                 // bytes are free of bank conflicts; of rows of 160 bytes four start 32 bytes apart and the next four at the same
                 // banks, so these take their chunks in pairs the other way round (`swap`: 16 x 1024 rows, 8 heads of 160, 21.5 -> 21.3 us, 64
-                // x 256 24.1 -> 23.8).  They are read before S of the head before is complete (its operand
+                // x 256 24.4 -> 24.1).  They are read before S of the head before is complete (its operand
                 // tile is free then), and the raw tile of the head after next lands under all that.  (With the chunks dealt out in
                 // linear order, row and place worked out for each, S of a head of 160 channels was 2 500 cycles later.)
                 constexpr int N = D / 16;
