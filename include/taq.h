@@ -358,7 +358,7 @@ enum {
 taq_status taq_dispatch_counts(int64_t* counts_out, int32_t n);
 void taq_dispatch_reset(void);
 
-/* The launch plan the tensor-core dequant-GEMM would take for a problem (host arithmetic only; nothing is launched
+/* The launch plan the tensor-core dequant-GEMM with one CTA, or a cluster, per tile would take for a problem (host arithmetic only; nothing is launched
  * and no GPU is needed).  plan_out: int32 [10] = {tile width BN (0: the tensor-core kernel does not take the
  * problem), ring stages in k-blocks, CTAs that share the K loop of a tile (1, 2 or 4), bytes of the ring, bytes of the
  * ring the epilogue reuses as its staging area, offset of the scales (the first section behind the ring), offset of the
@@ -367,6 +367,12 @@ void taq_dispatch_reset(void);
  * per-request calls do. */
 taq_status taq_linear_plan(const taq_weight_desc* desc, int64_t rows, int32_t out_kind, int32_t heads,
                            int32_t int8_activations, int32_t batched, int32_t* plan_out);
+
+/* Launches of many rows of fp16 activations with fp16 or per-head int8 outputs run on pairs of CTAs instead, which compute
+ * tiles of 256 rows together.  The same plan for those (tile width 0: the problem runs as taq_linear_plan says); the staging area lies
+ * inside the bytes counted as the ring.  n_requests: requests of a batched call, 0 for a single problem. */
+taq_status taq_linear_pair_plan(const taq_weight_desc* desc, int64_t rows, int32_t out_kind, int32_t heads,
+                                int32_t n_requests, int32_t* plan_out);
 
 /* Failure-detection self-test.  Every wait inside the kernels is bounded (about one second of SM clock); when one
  * runs out the block records TAQ_ERR_TIMEOUT in the device status word and returns.  This call launches one block

@@ -33,7 +33,7 @@ EXPORTS = [
     "taq_kv_project_a8_workspace_bytes", "taq_kv_project_a8", "taq_token_sensitivity_workspace_bytes",
     "taq_token_sensitivity", "taq_kv_set_prob_mask", "taq_hash_prompt", "taq_kv_cache_create", "taq_kv_cache_destroy",
     "taq_kv_cache_acquire", "taq_kv_cache_release", "taq_kv_cache_drop_checkpoint", "taq_kv_cache_get_stats",
-    "taq_dispatch_counts", "taq_dispatch_reset", "taq_linear_plan", "taq_selftest_wait_expiry",
+    "taq_dispatch_counts", "taq_dispatch_reset", "taq_linear_plan", "taq_linear_pair_plan", "taq_selftest_wait_expiry",
 ]
 
 
@@ -126,6 +126,7 @@ def lib() -> C.CDLL:
         L.taq_dispatch_reset.restype = None
         L.taq_dispatch_reset.argtypes = []
         L.taq_linear_plan.argtypes = [C.POINTER(WeightDesc), i64, i32, i32, i32, i32, C.POINTER(i32)]
+        L.taq_linear_pair_plan.argtypes = [C.POINTER(WeightDesc), i64, i32, i32, i32, C.POINTER(i32)]
         L.taq_selftest_wait_expiry.argtypes = [i64, vp]
         L.taq_static_workspace_capacity.restype = sz
         L.taq_static_workspace_capacity.argtypes = []
@@ -469,6 +470,13 @@ def taq_linear_plan(desc: "WeightDesc", rows: int, out_kind: int, heads: int = 1
     """Shared-memory plan of the tensor-core dequant-GEMM for a problem (host arithmetic; needs no GPU)."""
     arr = (C.c_int32 * 10)()
     _check(lib().taq_linear_plan(C.byref(desc), rows, out_kind, heads, int(int8_activations), int(batched), arr))
+    return {k: int(arr[i]) for i, k in enumerate(LINEAR_PLAN_FIELDS)}
+
+
+def taq_linear_pair_plan(desc: "WeightDesc", rows: int, out_kind: int, heads: int = 1, n_requests: int = 0) -> dict:
+    """The same where the problem runs on pairs of CTAs ("bn" is 0 where it does not)."""
+    arr = (C.c_int32 * 10)()
+    _check(lib().taq_linear_pair_plan(C.byref(desc), rows, out_kind, heads, n_requests, arr))
     return {k: int(arr[i]) for i, k in enumerate(LINEAR_PLAN_FIELDS)}
 
 

@@ -774,8 +774,8 @@ void taq_dispatch_reset(void) {
     for (int i = 0; i < TAQ_N_KERNEL_FAMILIES; ++i) g_dispatch[i].store(0, std::memory_order_relaxed);
 }
 
-taq_status taq_linear_plan(const taq_weight_desc* d, int64_t rows, int32_t out_kind, int32_t heads, int32_t int8_activations,
-                           int32_t batched, int32_t* plan_out) {
+static taq_status linear_plan(const taq_weight_desc* d, int64_t rows, int32_t out_kind, int32_t heads, int32_t int8_activations,
+                              int32_t batched, int n_z, bool pairs, int32_t* plan_out) {
     taq_status s = check_weight_desc(d);
     if (s != TAQ_OK) return s;
     if (!plan_out) return fail(TAQ_ERR_INVALID_ARG, "plan_out is NULL");
@@ -791,9 +791,19 @@ taq_status taq_linear_plan(const taq_weight_desc* d, int64_t rows, int32_t out_k
     a.heads = out_kind == TAQ_OUT_INT8_HEAD_ROWS ? heads : 1;
     a.epi = out_kind == TAQ_OUT_F16 ? EPI_F16 : out_kind == TAQ_OUT_F32 ? EPI_F32 : EPI_Q8_HEAD;
     int out[10];
-    linear_plan_of(a, out);
+    linear_plan_of(a, n_z, pairs, out);
     for (int i = 0; i < 10; ++i) plan_out[i] = out[i];
     return TAQ_OK;
+}
+
+taq_status taq_linear_plan(const taq_weight_desc* d, int64_t rows, int32_t out_kind, int32_t heads, int32_t int8_activations,
+                           int32_t batched, int32_t* plan_out) {
+    return linear_plan(d, rows, out_kind, heads, int8_activations, batched, 1, false, plan_out);
+}
+
+taq_status taq_linear_pair_plan(const taq_weight_desc* d, int64_t rows, int32_t out_kind, int32_t heads, int32_t n_requests, int32_t* plan_out) {
+    if (n_requests < 0) return fail(TAQ_ERR_INVALID_ARG, "n_requests (%d) must not be negative", n_requests);
+    return linear_plan(d, rows, out_kind, heads, 0, n_requests > 0, n_requests > 0 ? n_requests : 1, true, plan_out);
 }
 
 taq_status taq_selftest_wait_expiry(int64_t limit_cycles, void* stream) {

@@ -2,7 +2,7 @@
 // kernel is in taq_linear_sm100.cuh; every tile width is compiled in a file of its own (taq_linear_sm100_n*.cu).
 #include "taq_prof.cuh"
 TAQ_PROF_DEFINE(linear)
-#include "taq_linear_sm100.cuh"
+#include "taq_linear_pair_sm100.cuh"
 #include <algorithm>
 #include <cmath>
 
@@ -13,6 +13,8 @@ extern template cudaError_t launch_tile<64>(const CUtensorMap&, const LinearArgs
 extern template cudaError_t launch_tile<80>(const CUtensorMap&, const LinearArgs&, const LinearLayout&, int, size_t, cudaStream_t);
 extern template cudaError_t launch_tile<128>(const CUtensorMap&, const LinearArgs&, const LinearLayout&, int, size_t, cudaStream_t);
 extern template cudaError_t launch_tile<160>(const CUtensorMap&, const LinearArgs&, const LinearLayout&, int, size_t, cudaStream_t);
+extern template cudaError_t launch_pair<128>(const CUtensorMap&, const LinearArgs&, const LinearLayout&, const CUtensorMap&, int, size_t, cudaStream_t);
+extern template cudaError_t launch_pair<160>(const CUtensorMap&, const LinearArgs&, const LinearLayout&, const CUtensorMap&, int, size_t, cudaStream_t);
 }  // namespace linear
 
 namespace {
@@ -35,7 +37,7 @@ EncodeTiledFn encode_tiled_fn() {
 }
 
 // How a launch is laid out.
-struct Choice { int bn, grid; LinearLayout lay; int total, ring, staged; };      // grid in CTAs; staged: bytes the epilogue stages in the rings
+struct Choice { int bn, grid; LinearLayout lay; int total, ring, staged; bool pair; };      // grid in CTAs; staged: bytes the epilogue stages in the rings; pair: linear_pair_kernel
 
 struct Problem {                       // what the choice depends on
     int n_groups, group_len, bke, n_kb, d, ncols_factor;
@@ -123,6 +125,19 @@ bool rings_of(const LinearArgs& a, const Problem& p, int bn, int nsplit, int hea
     return false;
 }
 
+// Pairs of CTAs (taq_linear_pair_sm100.cuh): fp16 rows in, fp16 or per-head int8 rows out, scale groups that end with a pair of k-blocks.
+template <int BN>
+bool pair_rings(const LinearArgs& a, const Problem& p, Choice& c) {
+    if (p.i8 || (a.epi != EPI_F16 && a.epi != EPI_Q8_HEAD) || (p.n_groups > 1 && p.group_len / p.bke % 2 != 0)) return false;
+    if (!rings<BN>(a, p, 1, 0, true, c)) return false;                        // (the layout's other fields)
+    Plan& P = c.lay.plan;
+    const int ring = pair_staged_bytes<BN>(), shift = ring - P.ring_bytes;
+    P.ring_bytes = ring; P.off_scales += shift; P.off_bias += shift; P.off_xchg += shift; P.off_bars += shift; P.total += shift;
+    c.lay.nsa = c.lay.nsb = PAIR_STAGES;
+    c.total = P.total; c.ring = ring; c.staged = BM * BN * 2; c.pair = true;          // (behind the stages)
+    return P.total <= SMEM_LIMIT;
+}
+
 constexpr int SMS = 148;                                 // of a B200
 
 // Whether a tile of bn columns can carry the epilogue: per-head outputs want a thread's 80 or 64 columns to be whole heads, or a
@@ -156,31 +171,33 @@ constexpr Pace PACES[4] = {
     {80, 2.49, 0.200, 0.131, 0.52, 0.35, 1.05, 1.04},
     {64, 2.56, 0.192, 0.106, 0.24, 0.18, 1.00, 0.87},
 };
-Choice choose_anew(const LinearArgs& a, int n_z) {
+Choice& finish(Choice& c, const LinearArgs& a, const Problem& p, long long tiles, long long ctas) {
+
+    c.lay.n_tiles = (int)tiles;
+    c.lay.n_cols = a.n_out / c.bn * p.ncols_factor; c.lay.n_rows = (int)p.row_tiles;
+    c.lay.mul_cols = multiplier(c.lay.n_cols, tiles); c.lay.mul_rows = multiplier(c.lay.n_rows, tiles);
+    c.grid = (int)ctas;
+    // Packed weights asked for ahead of time, a share by each of up to 16 CTAs: where all CTAs of the launch find room beside its
+    // predecessor's, at most half the SMs.  Weights of requests are known behind the wait only.
+    if (!a.reqs && ctas <= SMS / 2 && p.L.total < (1u << 31)) {
+        const uint32_t n = (uint32_t)std::min(ctas, 16LL), bytes = (uint32_t)align_up((p.L.total + n - 1) / n, 128);
+        c.lay.blob_bytes = (uint32_t)p.L.total; c.lay.prefetch_bytes = bytes;
+        c.lay.prefetch_ctas = (uint32_t)((p.L.total + bytes - 1) / bytes);
+    }
+    return c;
+}
+
+Choice choose_single(const LinearArgs& a, int n_z, double& best_cost) {
     const Problem p = problem_of(a);
     Choice best{};
-    auto finish = [&](Choice& c, long long tiles, long long ctas) {
-        c.lay.n_tiles = (int)tiles;
-        c.lay.n_cols = a.n_out / c.bn * p.ncols_factor; c.lay.n_rows = (int)p.row_tiles;
-        c.lay.mul_cols = multiplier(c.lay.n_cols, tiles); c.lay.mul_rows = multiplier(c.lay.n_rows, tiles);
-        c.grid = (int)ctas;
-        // Packed weights asked for ahead of time, a share by each of up to 16 CTAs: where all CTAs of the launch find room beside its
-        // predecessor's, at most half the SMs.  Weights of requests are known behind the wait only.
-        if (!a.reqs && ctas <= SMS / 2 && p.L.total < (1u << 31)) {
-            const uint32_t n = (uint32_t)std::min(ctas, 16LL), bytes = (uint32_t)align_up((p.L.total + n - 1) / n, 128);
-            c.lay.blob_bytes = (uint32_t)p.L.total; c.lay.prefetch_bytes = bytes;
-            c.lay.prefetch_ctas = (uint32_t)((p.L.total + bytes - 1) / bytes);
-        }
-        return c;
-    };
+    best_cost = 1e30;
     // Heads of 160 channels in a launch of few rows: two 80-wide tiles per head whose CTAs exchange the rows' absmax, the K loop in
     // halves (with integer activations: halves of the scale groups).
     if (a.epi == EPI_Q8_HEAD && p.d == 160 && a.bits == 4 && (p.n_groups >= 2 || (!p.i8 && p.n_kb >= 2))) {
         const long long tiles = p.row_tiles * (a.n_out / 80) * (long long)n_z;
         Choice c{};
-        if (tiles * 2 <= SMS && rings_of(a, p, 80, 2, 1, false, c)) return finish(c, tiles, tiles * 2);
+        if (tiles * 2 <= SMS && rings_of(a, p, 80, 2, 1, false, c)) { best_cost = 0; return finish(c, a, p, tiles, tiles * 2); }      // (faster than pairs, too)
     }
-    double best_cost = 1e30;
     for (const Pace& m : PACES) {
         const int bn = m.bn;
         if (!tile_carries(a, p, bn)) continue;
@@ -203,10 +220,45 @@ Choice choose_anew(const LinearArgs& a, int n_z) {
             const double groups = p.n_groups == 1 ? 1 : (double)share * p.n_groups / p.n_kb;
             const double cost = (persistent ? 1 : per) * fixed + (double)per * (share * m.kb + groups * m.group + tile + (a.epi == EPI_Q8_HEAD ? m.q8 : 0)) +
                                 (ns > 1 ? m.split + 0.1 * (ns - 2) + m.exchange * (ns - 1) * (double)(tiles * ns) / SMS : 0);
-            if (cost < best_cost) { best_cost = cost; best = finish(c, tiles, ctas); }
+            if (cost < best_cost) { best_cost = cost; best = finish(c, a, p, tiles, ctas); }
         }
     }
     return best;
+}
+
+// Tiles of 256 rows on pairs of CTAs, in rounds of 74.  A fit to 151 measured launches (256 to 32768 rows, 320 to 1280 channels, W4 and
+// W8, fp16 and per-head int8 rows; 6 and 5 % rms).
+Choice choose_pair(const LinearArgs& a, int n_z, double& best_cost) {
+    struct PairPace { int bn; double fixed, pair4, pair8, tile, q8; };
+    constexpr PairPace PAIR_PACES[2] = {{160, 3.70, 0.628, 0.541, 1.25, -0.73}, {128, 3.16, 0.559, 0.504, 0.87, -0.22}};
+    const Problem p = problem_of(a);
+    Choice best{};
+    best_cost = 1e30;
+    for (const PairPace& m : PAIR_PACES) {
+        Choice c{};
+        if (!tile_carries(a, p, m.bn) || !(m.bn == 160 ? pair_rings<160>(a, p, c) : pair_rings<128>(a, p, c))) continue;
+        const long long rows2 = (p.row_tiles + 1) / 2, tiles = rows2 * (a.n_out / m.bn) * (long long)n_z;
+        if (tiles > (1 << 29)) continue;
+        const long long per = (tiles + SMS / 2 - 1) / (SMS / 2), pairs = (tiles + per - 1) / per;
+        const double cost = m.fixed + (double)per * ((p.n_kb + 1) / 2 * (a.bits == 4 ? m.pair4 : m.pair8) + m.tile) + (a.epi == EPI_Q8_HEAD ? m.q8 : 0);
+        if (cost >= best_cost) continue;
+        best_cost = cost;
+        best = finish(c, a, p, tiles, 2 * pairs);
+        best.lay.n_rows = (int)rows2;
+        best.lay.mul_rows = multiplier(best.lay.n_rows, tiles);
+    }
+    return best;
+}
+
+// Pairs or one CTA per tile.  Where a CTA would walk several tiles pairs were faster in every launch measured (by 2 to 45 %).  Elsewhere the
+// cheaper one, the wide tiles of one CTA with 2 us more than their model says: with fp16 rows launches of one wave of 128 or 160
+// columns take 1.4 to 3.2 us more.  So every one of 202 launches gets the faster kernel (with 1.5 us one is 7 % slower, with
+// none eight are 12 to 29 %).
+Choice choose_anew(const LinearArgs& a, int n_z) {
+    double cost, pair_cost;
+    const Choice single = choose_single(a, n_z, cost), pair = choose_pair(a, n_z, pair_cost);
+    if (!pair.bn || (single.bn && !single.lay.persistent && pair_cost >= cost + (single.bn >= 128 ? 2.0 : 0.0))) return single;
+    return pair;
 }
 
 // The last few problems of the calling thread: a program runs the same layers again and again.
@@ -246,16 +298,18 @@ bool sm100_linear_supported(const LinearArgs& a) {
     return choose(a, 1).bn != 0 && encode_tiled_fn() != nullptr;
 }
 
-// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed): tile width, ring depth in k-blocks, CTAs that
+// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed), with one CTA or a cluster's share of the K loop per
+// tile, or on pairs of CTAs (zeros where it does not take that): tile width, ring depth in k-blocks, CTAs that
 // share a tile's K loop, and the byte ranges of shared memory that the rings,
 // the epilogue's staging area in them and the fixed sections occupy.  out: {bn, nstage, split, ring_bytes, staging_bytes,
 // off_raw (the first fixed section), off_bias, off_bars, total, limit}.  bn = 0: the tensor-core kernel does not take it.
-void linear_plan_of(const LinearArgs& a, int out[10]) {
+void linear_plan_of(const LinearArgs& a, int n_z, bool pairs, int out[10]) {
     for (int i = 0; i < 10; ++i) out[i] = 0;
     out[9] = SMEM_LIMIT;
     if (!takes_shape(a)) return;
-    const Choice c = choose(a, 1);
-    if (c.bn == 0) return;
+    double cost;
+    const Choice c = pairs ? choose_anew(a, n_z) : choose_single(a, n_z, cost);
+    if (c.bn == 0 || (pairs && !c.pair)) return;
     const Plan& P = c.lay.plan;
     out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = c.lay.nsplit; out[3] = P.ring_bytes; out[4] = c.staged;
     out[5] = P.off_scales; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;
@@ -277,6 +331,20 @@ cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t strea
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
     const Choice c = choose(a, n_z);
+    if (c.pair) {
+        // the output: boxes of 32 rows, 32 columns of fp16 (64-byte swizzle) or a tile's width of int8 codes (128 columns: swizzled)
+        CUtensorMap tmap_y;
+        const bool q8 = a.epi == EPI_Q8_HEAD;
+        const cuuint64_t osz = q8 ? 1 : 2;
+        const cuuint64_t ydims[3] = {(cuuint64_t)a.n_out, (cuuint64_t)a.rows, (cuuint64_t)n_z};
+        const cuuint64_t ystrides[2] = {(cuuint64_t)a.n_out * osz, (cuuint64_t)a.n_out * osz * (cuuint64_t)a.rows};
+        const cuuint32_t ybox[3] = {(cuuint32_t)(q8 ? c.bn : 32), 32, 1};
+        r = enc(&tmap_y, q8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, a.y, ydims, ystrides, ybox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                !q8 ? CU_TENSOR_MAP_SWIZZLE_64B : c.bn == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        return c.bn == 160 ? launch_pair<160>(tmap, a, c.lay, tmap_y, c.grid, c.total, stream) : launch_pair<128>(tmap, a, c.lay, tmap_y, c.grid, c.total, stream);
+    }
     switch (c.bn) {
         case 64: return launch_tile<64>(tmap, a, c.lay, c.grid, c.total, stream);
         case 80: return launch_tile<80>(tmap, a, c.lay, c.grid, c.total, stream);

@@ -51,6 +51,40 @@ def test_linear_tiles(rows, n_out, k_in, bits, group, heads, dense, per_head):
     layer.test_quantized_linear(rows, n_out, k_in, bits, group, heads)
 
 
+# (tile widths of the launches on pairs of CTAs, 0 where the plan above is taken)
+@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
+    (5633, 640, 640, 4, 128, 8, 128, 160),             # the last tile: one row of the first CTA, none of the second
+    (5505, 640, 640, 8, 0, 10, 128, 128),              # ... one row of the second CTA; accumulators of three and two pairs of k-blocks
+    (9999, 320, 192, 4, 128, 8, 160, 160),             # an odd number of k-blocks, a short last group, heads of 40
+    (20000, 320, 64, 8, 0, 8, 160, 160),               # one k-block
+    (12289, 640, 512, 4, 256, 4, 160, 160),            # groups of two pairs of k-blocks, heads of 160
+    (3000, 1280, 320, 4, 128, 20, 128, 128),
+    (2049, 1280, 1280, 4, 0, 8, 160, 160),             # one group of 4-bit codes
+    (1, 1280, 1280, 8, 0, 8, 0, 160),
+])
+def test_linear_tiles_on_pairs(rows, n_out, k_in, bits, group, heads, dense, per_head):
+    wd = tb.weight_desc(n_out, k_in, bits, group)
+    assert tb.taq_linear_pair_plan(wd, rows, tb.TAQ_OUT_F16)["bn"] == dense
+    assert tb.taq_linear_pair_plan(wd, rows, tb.TAQ_OUT_INT8_HEAD_ROWS, heads)["bn"] == per_head
+    layer.test_quantized_linear(rows, n_out, k_in, bits, group, heads)
+
+
+def test_pairs_write_their_rows_only():
+    """Requests side by side, each with weights of its own: the last tile of one ends inside the rows of the next."""
+    assert tb.taq_linear_pair_plan(tb.weight_desc(640, 640, 4, 128), 520, tb.TAQ_OUT_F16, n_requests=8)["bn"] != 0
+    shape, desc, ckpts, route, reqs_data, packed, y, kv_blocks = layer._serving_case(n_ckpt=3, n_req=8, n_query=520, C_=640, Dc=768)
+    for r, c in enumerate(route):
+        layer._check_request(shape, desc, ckpts[int(c)], reqs_data[r], packed[int(c)], kv_blocks[r], y[r: r + 1], slice(490, 520))
+    n = 5633 * 640
+    for kind, dtype in ((tb.TAQ_OUT_F16, torch.float16), (tb.TAQ_OUT_INT8_HEAD_ROWS, torch.int8)):
+        buf = torch.full((n + 4096,), -7, dtype=dtype, device="cuda")
+        x = torch.randn(5633, 640, device="cuda").half()
+        blob = packed[0]["Wq"]
+        tb.taq_quantized_linear(tb.weight_desc(640, 640, 4, 128), x, blob, kind, heads=8, y=buf[2048: 2048 + n])
+        tb.taq_poll_device_status()
+        assert bool((buf[:2048] == -7).all()) and bool((buf[2048 + n:] == -7).all())
+
+
 @pytest.mark.parametrize("rows,k_in,n_out,bits,group,dense", [
     (1, 320, 320, 4, 128, "64"), (257, 1280, 1280, 4, 128, "64"), (4225, 640, 640, 4, 128, "160"), (300, 656, 640, 8, 0, "64"),
     (1, 1280, 1280, 4, 128, "64x2"), (5505, 64, 320, 4, 128, "64+"), (3000, 320, 1280, 4, 128, "128+"),
