@@ -73,7 +73,7 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
     using TL = Tile<BN>;
     const int n_pair = (share_of(p, nsplit) + 1) / 2;
     int staged = 0;
-    const int tile_bytes = a.epi == EPI_F16 ? BM * BN * 2 : a.epi == EPI_F32 ? BM * BN * 4 : a.epi == EPI_Q8_HEAD ? BM * BN : 128 * (BN + 1) * 4 + BN / p.d * 1024;      // (K~/V~: the fp32 tile and the rows' scales)
+    const int tile_bytes = a.epi == EPI_F16 ? BM * BN * 2 : a.epi == EPI_F32 ? BM * BN * 4 : a.epi == EPI_Q8_HEAD ? BM * BN : kv_tile_bytes(BN) + std::max(1, BN / p.d) * 1024;      // (K~/V~: the fp32 tile and the rows' scales)
     if (persistent) {
         // (stored from the registers)
     } else if (nsplit == 1) {
@@ -81,14 +81,18 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
     } else {
         staged = std::max(TL::NCG * (4 - 4 / nsplit) * TL::PIECE, tile_bytes);                  // (the pieces of the other CTAs, then the output)
     }
+    // (K~/V~ of fp16 contexts: the images' 80 rows and not 128: 0.1 - 0.2 us of every such launch; with int8 contexts W4 lost as much)
+    const int xb = a.epi == EPI_KV && !p.i8 && a.n_ctx <= kOperandKeys ? kOperandKeys * 128 : A_TILE_BYTES;
     int nsa = n_pair < 2 ? 1 : 2, nsb = n_pair < 2 ? 1 : 2;
-    while (make_plan<BN>(p.n_groups, nsa, nsb, persistent).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
-    auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, persistent).total <= SMEM_LIMIT; };
+    while (make_plan<BN>(p.n_groups, nsa, nsb, persistent, xb).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
+    auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, persistent, xb).total <= SMEM_LIMIT; };
+
     while (nsb < (persistent ? MAX_STAGE : n_pair) && nsb < MAX_STAGE && fits(nsa, nsb + 1)) ++nsb;
     while (nsa < 3 && nsa < n_pair && fits(nsa + 1, nsb)) ++nsa;
-    const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, persistent);
+    const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, persistent, xb);
     if (P.total > SMEM_LIMIT || P.ring_bytes < staged) return false;
     c.bn = BN;
+    c.lay.kv.x_bytes = (uint32_t)xb;
     c.lay.nsplit = nsplit; c.lay.nsa = nsa; c.lay.nsb = nsb; c.lay.head_pair = head_pair; c.lay.persistent = persistent;
     c.lay.plan = P;
     c.lay.n_groups = p.n_groups; c.lay.n_kb = p.n_kb; c.lay.mul_groups = multiplier(p.n_groups, (long long)BN * p.n_groups);
@@ -108,8 +112,8 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
         OperandGeom g{};
         G.images = operand_geom(p.d, a.n_ctx, &g);
         G.head_bytes = (uint32_t)g.head_bytes; G.k_bytes = (uint32_t)g.k_bytes; G.vt_bytes = (uint32_t)g.vt_bytes;
-        G.dp = g.dp; G.kbq = g.kbq; G.n_heads = BN / p.d;
-        G.mul_dp = g.dp ? multiplier(g.dp, BN / p.d * g.dp) : 0;
+        G.dp = g.dp; G.kbq = g.kbq; G.n_heads = std::max(1, BN / p.d);
+        G.mul_dp = g.dp ? multiplier(g.dp, G.n_heads * g.dp) : 0;
         G.logit_unit = 1.4426950408889634f / sqrtf((float)p.d);
     }
     c.total = P.total; c.ring = P.ring_bytes; c.staged = staged;
@@ -197,6 +201,13 @@ Choice choose_single(const LinearArgs& a, int n_z, double& best_cost) {
         const long long tiles = p.row_tiles * (a.n_out / 80) * (long long)n_z;
         Choice c{};
         if (tiles * 2 <= SMS && rings_of(a, p, 80, 2, 1, false, c)) { best_cost = 0; return finish(c, a, p, tiles, tiles * 2); }      // (faster than pairs, too)
+    }
+    // K~/V~ with heads of 160 channels: the same, the K loop whole, where the CTAs are one wave (two prompts of 77 x 768, 1280 channels: W4 13.4 ->
+    // 9.5 us, W8 12.8 -> 9.1, against one 160-wide tile per head on half as many).
+    if (a.epi == EPI_KV && p.d == 160 && !(p.i8 && a.bits == 8)) {
+        const long long tiles = p.row_tiles * (a.n_out / 80) * 2 * (long long)n_z;
+        Choice c{};
+        if (tiles <= SMS && rings_of(a, p, 80, 1, 1, false, c)) { best_cost = 0; return finish(c, a, p, tiles, tiles); }
     }
     for (const Pace& m : PACES) {
         const int bn = m.bn;
@@ -319,18 +330,18 @@ cudaError_t launch_linear_sm100(const LinearArgs& a, int n_z, cudaStream_t strea
     if (a.rows == 0 || n_z == 0) return cudaSuccess;
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return cudaErrorNotSupported;
+    const Choice c = choose(a, n_z);
     CUtensorMap tmap;
     const bool i8 = a.xq != nullptr;
     const cuuint64_t esz = i8 ? 1 : 2;
     const cuuint64_t dims[3] = {(cuuint64_t)a.k_in, (cuuint64_t)a.rows, (cuuint64_t)n_z};
     const cuuint64_t strides[2] = {(cuuint64_t)a.k_in * esz, (cuuint64_t)a.k_in * esz * (cuuint64_t)a.rows};
-    const cuuint32_t box[3] = {(cuuint32_t)(i8 ? 2 * BK : BK), BM, 1};       // 128 bytes of K either way; elements beyond k_in read as zero
+    const cuuint32_t box[3] = {(cuuint32_t)(i8 ? 2 * BK : BK), c.lay.kv.x_bytes / 128, 1};       // 128 bytes of K either way; elements beyond k_in read as zero
     const cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(&tmap, i8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3,
                      i8 ? (void*)const_cast<int8_t*>(a.xq) : (void*)const_cast<__half*>(a.x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    const Choice c = choose(a, n_z);
     if (c.pair) {
         // the output: boxes of 32 rows, 32 columns of fp16 (64-byte swizzle) or a tile's width of int8 codes (128 columns: swizzled)
         CUtensorMap tmap_y;

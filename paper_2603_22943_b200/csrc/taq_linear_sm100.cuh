@@ -25,7 +25,7 @@
 // A register spilled in a loop is a round trip to L2, since beside 200 KB of shared memory there is next to no L1 (a first version
 // with 120 bytes of spills ran at half the speed), hence the register split.  What `-Xptxas -v` still reports at 72
 // registers: 4 to 64 bytes stored and up to 108 loaded in most 160-wide kernels and some of the others, none in the rest.  Whether such a
-// kernel pays for them is told by its time only: the unsplit 160-wide K/V kernels went from 8 / 8 bytes to 36 / 84 when their epilogue was
+// kernel pays for them is told by its time only: the unsplit 160-wide K/V kernels went from 8 / 8 bytes to 44 / 100 when their epilogue was
 // shortened, and two prompts at 1280 channels from 15.3 to 14.0 us.
 #pragma once
 #include "taq_ptx.cuh"
@@ -80,6 +80,9 @@ struct Tile {
     static_assert(BN * 16 % (NBUILD / 2) == 0 && HC % 8 == 0 && NSLOT <= MAX_SLOT && NSLOT >= 3, "tile shape");
 };
 
+// The K~/V~ epilogue's fp32 tile in shared memory.
+__host__ __device__ constexpr int kv_tile_bytes(int bn) { return (128 * (bn + 4) + 16 * 8) * 4; }
+
 struct Bars {
     uint64_t full_a[MAX_STAGE], empty_a[MAX_STAGE], full_b[MAX_STAGE], empty_b[MAX_STAGE];
     uint64_t acc_full[MAX_SLOT], acc_free[MAX_SLOT];
@@ -96,9 +99,9 @@ struct Plan { int ring_bytes, off_scales, scale_bytes, off_bias, off_xchg, off_b
 
 // nsa, nsb: pairs of k-blocks in the rings; persistent: a CTA walks several tiles.
 template <int BN>
-inline Plan make_plan(int n_groups, int nsa, int nsb, bool persistent) {
+inline Plan make_plan(int n_groups, int nsa, int nsb, bool persistent, int x_bytes) {
     Plan p;
-    p.ring_bytes = 2 * (nsa * A_TILE_BYTES + nsb * Tile<BN>::B_TILE);
+    p.ring_bytes = 2 * (nsa * x_bytes + nsb * Tile<BN>::B_TILE);
     p.off_scales = p.ring_bytes;                                              // (two buffers of) float [n_groups][BN], then bias [BN]
     p.scale_bytes = (n_groups + 1) * BN * 4;
     p.off_bias = p.off_scales + n_groups * BN * 4;
@@ -129,6 +132,7 @@ struct LinearLayout {
         int images, dp, kbq, n_heads;       // n_heads: of a tile
         uint32_t mul_dp;
         float logit_unit;                   // log2(e) / sqrt(d)
+        uint32_t x_bytes;                   // of an activation tile: 128 rows, or the 80 that images have (the MMA's other rows are whatever lies behind them, and used by nobody)
     } kv;
     uint32_t prefetch_ctas, prefetch_bytes, blob_bytes;      // CTAs that ask for a share of the packed weights each (0: none)
 };
@@ -181,6 +185,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     constexpr bool KV = OUT == Out::KV;
     constexpr bool clustered = CTAS == Ctas::SPLIT;
     constexpr bool persistent = CTAS == Ctas::MANY;
+    const bool head_pair = clustered && (!KV || BN == 80) && lay.head_pair;      // heads of 160 channels on the 80-wide tiles of two CTAs
     using CodeT = typename Code<I8, W8>::T;
     constexpr int HC = TL::HC, NCG = TL::NCG, NSLOT = TL::NSLOT, NCH = TL::NCH;
     constexpr int BKE = I8 ? 2 * BK : BK;             // elements per K block
@@ -195,6 +200,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     const Plan& P = lay.plan;
     static_assert(sizeof(Bars) <= 1024, "barrier block");
     Bars* bars = reinterpret_cast<Bars*>(smem + P.off_bars);
+    const uint32_t XT = KV ? lay.kv.x_bytes : (uint32_t)A_TILE_BYTES;      // an activation tile
     const int n_kb_all = lay.n_kb;                      // (int8: the last block may be ragged; TMA and the expansion zero-fill)
     const int kb_per_group = lay.kb_per_group;          // k-blocks in a full group (the last group may be shorter)
     // this CTA's share of the K loop: a run of whole scale groups, or (one scale per output channel) of k-blocks
@@ -230,7 +236,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
         for (int i = lane; i < N_BARS; i += 32) {
             const int count = i >= FULL_B && i < EMPTY_B ? TL::NB / 2 : i < ACC_FREE ? 1 : i < SCALE_FULL ? TL::NF : i < SCALE_FREE ? 2 : i < SCALE_FREE + 2 ? TL::NF :
-                              i == SCALE_FREE + 3 && clustered ? nsplit - 1 : 1;       // (the last: peer_ready)
+                              i == SCALE_FREE + 3 && clustered ? max(nsplit - 1, 1) : 1;       // (the last: peer_ready)
             ptx::mbar_init(all + i, (uint32_t)count);
         }
         ptx::mbar_fence_init();
@@ -241,7 +247,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const int per_cta = 4 / nsplit;              // lane quarters whose rows a CTA finishes
                 for (int cg = 0; cg < NCG; ++cg)             // the warps of those quarters receive a piece from every other CTA
                     for (int i = 0; i < per_cta; ++i) ptx::mbar_arrive_expect_tx(&bars->part_full[cg * 4 + rank * per_cta + i], (uint32_t)((nsplit - 1) * TL::PIECE));
-                if (lay.head_pair)
+                if (head_pair)
                     for (int i = 0; i < per_cta; ++i) ptx::mbar_arrive_expect_tx(&bars->pair_full[rank * per_cta + i], 128u);
             }
         }
@@ -264,22 +270,24 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // once.  With the eight folder warps alone these loops took 9 000: two warps on a scheduler hide no latency.
     // With the block's layout worked out here, 2 300 cycles went by before the first load; it comes from the host now: two
     // prompts of 77 x 768, W4, 320 channels 10.0 -> 8.6 us, 1280 channels 15.3 -> 14.0.)
-    constexpr int KV_STRIDE = BN + 1;                        // floats (odd: a row per lane is free of bank conflicts)
+    // Row t of the fp32 tile: 16-byte accesses by a row per lane, and reads of eight columns by four groups of eight rows, hit all banks
+    // (with 4-byte accesses and an odd row length 2 prompts, W4, 320 channels took 8.70 us, 8.55 so; 32 prompts, 1280 channels, 52.0 and 50.1).
+    auto kv_row = [](int t) { return t * (BN + 4) + (t >> 3) * 8; };
     auto kv_store = [&](int w) {
         constexpr int NT = TL::NFOLD + TL::NBUILD, NC8 = BN / 8;
         int z, row0, col0, kv_which;
         tile_of(tile0, z, row0, col0, kv_which);
         const auto& G = lay.kv;
-        const int T = a.n_ctx, d = lay.d, head0 = quotient(col0, d, lay.mul_d);
+        const int T = a.n_ctx, d = lay.d, head0 = quotient(col0, d, lay.mul_d), ch0 = head_pair ? col0 - head0 * d : 0;      // (ch0: the second half of a head on two tiles)
         uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * G.block_bytes;
         uint8_t* img0 = blk + G.off_operands + (uint32_t)head0 * G.head_bytes;
         const int* slots = reinterpret_cast<const int*>(smem + P.off_xchg) + 512;
         const float* ys = reinterpret_cast<const float*>(smem);
-        const float2* hs = reinterpret_cast<const float2*>(smem + 128 * KV_STRIDE * 4);
+        const float2* hs = reinterpret_cast<const float2*>(smem + kv_tile_bytes(BN));
         const int own_shift = nsplit == 1 ? 7 : nsplit == 2 ? 6 : 5;         // (CTAs that share the tile finish the rows of some lane quarters each)
         auto own = [&](int key) { return key >> own_shift == rank; };
         {                                                    // codes, trigger rows and K~'s image: 8 channels of a token
-            const int c = (w % NC8) * 8, hl = quotient(c, d, lay.mul_d), ch = c - hl * d, h = head0 + hl;
+            const int c = (w % NC8) * 8, hl = quotient(ch0 + c, d, lay.mul_d), ch = ch0 + c - hl * d, h = head0 + hl;
             uint8_t* codes = blk + (kv_which ? G.off_v_codes : 0u) + (uint32_t)(h * T * d + ch);
             uint8_t* trigs = blk + (kv_which ? G.off_v_trigger : G.off_k_trigger) + (uint32_t)(h * d + ch) * 2;
             uint8_t* k_img = img0 + (uint32_t)hl * G.head_bytes + (ch >> 6) * (kOperandKeys * 128);
@@ -287,9 +295,9 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 if (!own(t)) continue;
                 const int slot = slots[t];
                 const float rs = hs[hl * 128 + t].y;
-                float f[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) f[e] = ys[t * KV_STRIDE + c + e];
+                const float4* row = reinterpret_cast<const float4*>(ys + kv_row(t) + c);
+                const float4 lo = row[0], hi = row[1];
+                const float f[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
                 const uint2 code = slot == -1 ? quant8(f, rs) : make_uint2(0, 0);
                 *reinterpret_cast<uint2*>(codes + t * d) = code;
                 uint4 k8 = codes_w8_to_half(code);
@@ -302,28 +310,28 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
         if (!G.images) return;
         if (!kv_which) {                                     // K~'s padding: keys T..79, and the channels behind the head's last
-            const int ncc = G.kbq * 8;
+            const int cc0 = ch0 >> 3, ncc = head_pair && ch0 == 0 ? NC8 : G.kbq * 8;       // (of a head on two tiles this CTA's)
             for (int line = w >> 3; line < G.n_heads * kOperandKeys; line += NT / 8) {
                 const int hl = line / kOperandKeys, t = line - hl * kOperandKeys;
                 if (!own(t)) continue;
                 for (int cc = (w & 7) + (t >= T || d >= 64 ? 0 : d / 8 & ~7); cc < ncc; cc += 8)
-                    if (t >= T || cc * 8 >= d) *reinterpret_cast<uint4*>(img0 + (uint32_t)hl * G.head_bytes + (cc >> 3) * (kOperandKeys * 128) + ptx::sw128_offset(t, cc & 7)) = make_uint4(0, 0, 0, 0);
+                    if ((t >= T && cc >= cc0) || cc * 8 >= d) *reinterpret_cast<uint4*>(img0 + (uint32_t)hl * G.head_bytes + (cc >> 3) * (kOperandKeys * 128) + ptx::sw128_offset(t, cc & 7)) = make_uint4(0, 0, 0, 0);
             }
         } else {
             // V~^T: 8 keys of a channel per lane; a warp takes 8 channels x 4 chunks of keys (reads of the fp32 tile without bank
             // conflicts, stores of 64 contiguous bytes).  Everything is read first (rows and columns beyond the last token and
             // channel, too: something of the tile, not used), so that a chunk costs one round trip to shared memory.
             const int wl = w & 31;
-            for (int u = w >> 5; u < G.n_heads * (G.dp >> 3) * 4; u += NT / 32) {
-                const int jc = (u & 3) * 4 + (wl >> 3), line = (u >> 2) * 8 + (wl & 7), hl = quotient(line, G.dp, G.mul_dp), ch = line - hl * G.dp;
+            for (int u = w >> 5; u < (head_pair ? BN : G.n_heads * G.dp) / 2; u += NT / 32) {
+                const int jc = (u & 3) * 4 + (wl >> 3), line = ch0 + (u >> 2) * 8 + (wl & 7), hl = quotient(line, G.dp, G.mul_dp), ch = line - hl * G.dp;
                 if (!own(jc * 8)) continue;
-                const float* col = ys + jc * 8 * KV_STRIDE + hl * d + min(ch, d - 1);
+                const float* col = ys + kv_row(jc * 8) + hl * d + min(ch, d - 1) - ch0;
                 const float4* sc4 = reinterpret_cast<const float4*>(hs + hl * 128 + jc * 8);
                 const int n_real = ch < d ? T - jc * 8 : 0;
                 float x[8];
                 float4 sc[4];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] = col[e * KV_STRIDE];
+                for (int e = 0; e < 8; ++e) x[e] = col[e * (BN + 4)];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) sc[e] = sc4[e];
                 __half v[8];
@@ -430,7 +438,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 mine = alive && owner == rank && !padding;
                 if (ft < nsplit && ft != rank) ptx::mbar_arrive_cluster_relaxed(ptx::map_to_cta(ptx::smem_u32(&bars->peer_ready), base + (uint32_t)ft));
                 auto piece = [&](int cta, int from) { return smem + ((cg * per_cta + q - cta * per_cta) * (nsplit - 1) + (from < cta ? from : from - 1)) * TL::PIECE + lane * 16; };
-                if (padding) {
+                if (padding || nsplit == 1) {
                     // nothing to send, nothing comes
                 } else if (owner != rank) {
                     if (alive && ptx::mbar_wait(&bars->peer_ready, 0)) {                 // the other CTAs' rings are free, too
@@ -570,7 +578,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 #pragma unroll
                     for (int k = PARTNERS ? 1 : 0; k < NCG; ++k) if (k < per_head) am = fmaxf(am, xc[(PARTNERS ? cg ^ k : first + k) * 128 + r]);
                     if (persistent) asm volatile("bar.sync %0, %1;" ::"r"(6 + q), "n"(NCG * 32) : "memory");      // (read before the next tile's are written)
-                    if (!KV && lay.head_pair && mine) {
+                    if (head_pair && mine) {
                         // The head's other columns belong to a CTA of the same cluster (same rows, same share of the K loop):
                         // each sends its rows' absmax over.
                         const uint32_t me = ptx::cluster_ctarank();
@@ -605,16 +613,16 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     const auto& G = lay.kv;
                     uint8_t* blk = a.reqs ? (uint8_t*)a.reqs[z].kv : (uint8_t*)a.y + (size_t)z * G.block_bytes;
                     const int head0 = quotient(col0, d, lay.mul_d);
-                    float* ys = reinterpret_cast<float*>(staging);                   // [128][KV_STRIDE]
-                    float2* hs = reinterpret_cast<float2*>(staging + 128 * KV_STRIDE * 4);   // [heads][128] scale and its reciprocal (trigger rows: 0 and -1)
+                    float* ys = reinterpret_cast<float*>(staging);                   // see kv_row
+                    float2* hs = reinterpret_cast<float2*>(staging + kv_tile_bytes(BN));   // [heads][128] scale and its reciprocal (trigger rows: 0 and -1)
                     if (mine) {
                         const int slot = slots[r];           // >= 0: trigger row, -1: ordinary (or padding), -2: a trigger row beyond the capacity
                         const bool plain = r < T && slot == -1;
 #pragma unroll
-                        for (int c = 0; c < HC; ++c) ys[r * KV_STRIDE + cb + c] = y[c];
+                        for (int c = 0; c < HC; c += 4) *reinterpret_cast<float4*>(ys + kv_row(r) + cb + c) = make_float4(y[c], y[c + 1], y[c + 2], y[c + 3]);
+                        const float sk = plain ? s : 0.f;
+                        if (owner || (head_pair && cg == 0)) hs[(h0 - head0) * 128 + r] = make_float2(sk, plain ? rs : slot >= 0 ? -1.f : 0.f);
                         if (owner) {
-                            const float sk = plain ? s : 0.f;
-                            hs[(h0 - head0) * 128 + r] = make_float2(sk, plain ? rs : slot >= 0 ? -1.f : 0.f);
                             if (r < T) reinterpret_cast<float*>(blk + (kv_which ? G.off_v_scales : G.off_k_scales))[(uint32_t)(h0 * T + r)] = sk;
                             if (!kv_which && h0 == 0) reinterpret_cast<int32_t*>(blk + G.off_trig_slot)[r] = slot >= 0 ? slot : -1;
                             if (!kv_which && G.images && r < kOperandKeys) {
@@ -633,7 +641,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     } else if (warp >= TL::W_BUILD && warp < TL::W_BUILD + TL::NB) {
         // ---------------- builders ----------------
         const int bt = (tid - 32 * TL::W_BUILD) & (TL::NBUILD / 2 - 1), group = (warp - TL::W_BUILD) / (TL::NB / 2);
-        unsigned char* b_ring = smem + 2 * nsa * A_TILE_BYTES;
+        unsigned char* b_ring = smem + 2 * nsa * XT;
         // The two halves of the builders take the pairs of k-blocks in turn: a pair costs its warps about 900 cycles of latency
         // (barrier, expansion, proxy fence), half of which is somebody else's turn.  16 chunks per weight row; sixteen
         // consecutive lanes take one row, so that a warp's loads are two runs of 64 (128) consecutive bytes and its stores
@@ -718,11 +726,11 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     tile_of(tile, z, row0, col0, kv_which);
                     for (int i = 0; i < n_kb; i += 2) {
                         if (passed && !ptx::mbar_wait(&bars->empty_a[s], ph)) { give_up(); ok = false; break; }
-                        unsigned char* dst = smem + 2 * s * A_TILE_BYTES;
+                        unsigned char* dst = smem + 2 * s * XT;
                         const bool two = i + 1 < n_kb;
-                        ptx::mbar_arrive_expect_tx(&bars->full_a[s], two ? 2 * A_TILE_BYTES : A_TILE_BYTES);
+                        ptx::mbar_arrive_expect_tx(&bars->full_a[s], two ? 2 * XT : XT);
                         ptx::tma_load_3d(dst, &tmap_x, &bars->full_a[s], (kb_begin + i) * BKE, row0, z);
-                        if (two) ptx::tma_load_3d(dst + A_TILE_BYTES, &tmap_x, &bars->full_a[s], (kb_begin + i + 1) * BKE, row0, z);
+                        if (two) ptx::tma_load_3d(dst + XT, &tmap_x, &bars->full_a[s], (kb_begin + i + 1) * BKE, row0, z);
                         ++issued;
                         if (++s == nsa) { s = 0; ph ^= 1; passed = true; }
                     }
@@ -742,7 +750,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&bars->tmem_base);
                 constexpr uint32_t idesc = I8 ? ptx::idesc_i8_m128(BN) : ptx::idesc_f16_m128(BN);
                 constexpr uint32_t HI = ptx::kDescHiSw128;
-                const uint32_t a_lo0 = ptx::desc_lo(ptx::smem_u32(smem)), b_lo0 = ptx::desc_lo(ptx::smem_u32(smem + 2 * nsa * A_TILE_BYTES));
+                const uint32_t a_lo0 = ptx::desc_lo(ptx::smem_u32(smem)), b_lo0 = ptx::desc_lo(ptx::smem_u32(smem + 2 * nsa * XT));
                 int sa = 0, sb = 0, slot = 0;
                 uint32_t pha = 0, phb = 0, ph_free = 1, a_lo = a_lo0, b_lo = b_lo0;
                 bool ok = true, recycled = false;            // recycled: every accumulator has been used once
@@ -770,7 +778,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                             }
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {    // four 32-byte K slices per 128-byte operand row
-                                const uint64_t da = ptx::desc_join(HI, a_lo + h * (A_TILE_BYTES >> 4) + 2 * k), db = ptx::desc_join(HI, b_lo + h * (TL::B_TILE >> 4) + 2 * k);
+                                const uint64_t da = ptx::desc_join(HI, a_lo + h * (XT >> 4) + 2 * k), db = ptx::desc_join(HI, b_lo + h * (TL::B_TILE >> 4) + 2 * k);
                                 if (I8) ptx::mma_i8_ss(d_tmem, da, db, idesc, acc | k);
                                 else ptx::mma_f16_ss(d_tmem, da, db, idesc, acc | k);
                             }
@@ -784,7 +792,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                         if (todo > nsa) ptx::mma_commit(&bars->empty_a[sa]);
                         if (todo > nsb) ptx::mma_commit(&bars->empty_b[sb]);
                         --todo;
-                        a_lo += 2 * A_TILE_BYTES >> 4;
+                        a_lo += 2 * XT >> 4;
                         b_lo += 2 * TL::B_TILE >> 4;
                         if (++sa == nsa) { sa = 0; pha ^= 1; a_lo = a_lo0; }
                         if (++sb == nsb) { sb = 0; phb ^= 1; b_lo = b_lo0; }
@@ -802,7 +810,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             // Packed weights, on their way to L2 while the previous kernel runs (the builders may read only behind the wait).  Sixteen
             // projections of a prompt 175.5 -> 171.5 us, sixteen layers of a denoising step 317.3 -> 315.4 (in front of the barrier above, which
             // it kept everybody from, 172.1 and 316.5, and 8.99 instead of 8.91 for two prompts at 320 channels).  In the K/V kernels of
-            // every width (the wide ones spill as much without it: 36 bytes stored, 84 loaded in 160-wide tiles, none in the 128- and 64-wide
+            // every width (the wide ones spill as much without it: 44 bytes stored, 100 loaded in 160-wide tiles, none in the 128- and 64-wide
             // ones) and in the 80-wide ones.  Not in the others that are no K/V kernels: the wide ones have no register to spare there (116 bytes of
             // spills, 2048 x 1280 x 1280 1.6 us more), and a layer of 1294 rows x 640, 64-wide tiles on 120 CTAs, which none of
             // them asks for, lost 0.2 us of 20.9 to the code alone.
@@ -897,7 +905,7 @@ template <int BN>
 cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const LinearLayout& lay, int grid, size_t smem_bytes, cudaStream_t stream) {
     using TL = Tile<BN>;
     const bool i8 = a.xq != nullptr, w8 = a.bits == 8;
-    const Ctas ctas = lay.nsplit > 1 ? Ctas::SPLIT : lay.persistent ? Ctas::MANY : Ctas::ONE;
+    const Ctas ctas = lay.nsplit > 1 || lay.head_pair ? Ctas::SPLIT : lay.persistent ? Ctas::MANY : Ctas::ONE;
     using Kernel = void (*)(const CUtensorMap, const LinearArgs, const LinearLayout);
     auto of_types = [&](auto out, auto ctas_c) -> Kernel {
         constexpr Out O = decltype(out)::value;
@@ -919,7 +927,7 @@ cudaError_t launch_tile(const CUtensorMap& tmap, const LinearArgs& a, const Line
     if (!kern) return cudaErrorNotSupported;
     cudaError_t e = allow_shared_memory((const void*)kern, SMEM_LIMIT, limit_set[(a.epi * 3 + (int)ctas) * 4 + i8 * 2 + w8]);
     if (e != cudaSuccess) return e;
-    if (lay.nsplit > 1) return launch_pdl_cluster(kern, dim3(grid), dim3(lay.nsplit * (lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), smem_bytes, stream, tmap, a, lay);
+    if (ctas == Ctas::SPLIT) return launch_pdl_cluster(kern, dim3(grid), dim3(lay.nsplit * (lay.head_pair ? 2 : 1), 1, 1), dim3(TL::NTHREADS), smem_bytes, stream, tmap, a, lay);
     return launch_pdl(kern, dim3(grid), dim3(TL::NTHREADS), smem_bytes, stream, tmap, a, lay);
 }
 

@@ -97,6 +97,7 @@ def test_integer_linear_tiles(rows, k_in, n_out, bits, group, dense):
 @pytest.mark.parametrize("channels,heads,ctx_dim,n_ctx,batch,w_bits", [
     (320, 8, 768, 9, 1, 4), (320, 8, 768, 80, 3, 8), (640, 8, 768, 77, 2, 4), (640, 10, 2048, 20, 1, 4),
     (1280, 20, 2048, 77, 1, 8), (1280, 8, 768, 64, 2, 8), (640, 10, 2048, 77, 9, 4),
+    (1280, 8, 768, 9, 1, 4), (1280, 8, 768, 80, 4, 4), (1280, 8, 768, 77, 5, 4),      # heads on two tiles; more of them than one wave
 ])
 def test_kv_projection(channels, heads, ctx_dim, n_ctx, batch, w_bits):
     shape = replace(synth.config1(), batch=batch, channels=channels, heads=heads, ctx_dim=ctx_dim, n_ctx=n_ctx, w_bits=w_bits, w_group=128 if w_bits == 4 else 0,
