@@ -171,6 +171,12 @@ __device__ __forceinline__ void store_32b(void* gmem_dst, const uint32_t* w) {
                  ::"l"(gmem_dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
 }
 
+// 32 bytes from a 32-byte aligned global address; an ordinary load, which stays behind a pdl_wait() before it.
+__device__ __forceinline__ void load_32b(const void* gmem_src, uint4& lo, uint4& hi) {
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w) : "l"(gmem_src) : "memory");
+}
+
 // ---- TMEM -------------------------------------------------------------------------------------------
 // Whole-warp calls.  ncols: power of two in [32, 512].
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_slot, uint32_t ncols) {

@@ -150,3 +150,31 @@ def test_kv_projections_of_one_shape_and_two_trigger_capacities():
         assert (blocks[2][name] == blocks[5][name]).all(), name
     for name in ("K_trigger", "V_trigger"):
         assert (blocks[2][name] == blocks[5][name][:, :2]).all(), name
+
+
+# (280 channels: rows of Q~ start 8 bytes apart from 16-byte boundaries, too)
+@pytest.mark.parametrize("channels,heads", [(640, 10), (160, 4), (280, 7)])
+@pytest.mark.parametrize("q_bits", [8, 0])
+def test_attention_in_pieces_of_any_alignment(channels, heads, q_bits):
+    """Heads of 64 and 40 channels are read and written in pieces as wide as the address allows: right, and the same bits 16 bytes further."""
+    shape = replace(synth.config1(), batch=2, n_query=130, channels=channels, heads=heads, name=f"pieces_{channels}_{heads}")
+    layer.test_cross_attention_isolated(shape, 130, q_bits)
+    shape = replace(shape, q_bits=q_bits)
+    data = synth.make_layer(shape)
+    desc = tl.gpu_desc(shape)
+    P = tl.pack_layer_weights(shape, data)
+    mask = tl.dev(data["mask"])
+    kv = tb.taq_kv_project(desc, tl.dev(data["ctx"]), P["Wk"], P["Wv"], mask)
+    n = shape.rows * channels
+    gen = torch.Generator("cuda").manual_seed(1)
+    q = torch.randint(-127, 128, (n,), device="cuda", generator=gen).to(torch.int8) if q_bits else torch.randn(n, device="cuda", generator=gen).half()
+    scales = torch.rand(shape.rows * heads, device="cuda", generator=gen) / 30 if q_bits else None
+    outs = []
+    for shift in (0, 16):                                            # bytes
+        qq = torch.zeros(n + 64, dtype=q.dtype, device="cuda")[shift // q.element_size():][:n].copy_(q)
+        o = torch.full((n + 64,), -7.0, dtype=torch.float16, device="cuda")
+        tb.taq_cross_attention(desc, qq, scales, kv, mask, o[shift // 2: shift // 2 + n])
+        tb.taq_poll_device_status()
+        assert bool((o[: shift // 2] == -7.0).all()) and bool((o[shift // 2 + n:] == -7.0).all())
+        outs.append(o[shift // 2: shift // 2 + n].clone())
+    assert torch.equal(outs[0], outs[1])
