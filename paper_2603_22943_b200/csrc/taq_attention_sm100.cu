@@ -35,6 +35,7 @@ namespace {
 using namespace parts;
 
 constexpr int ROWS = 128;
+constexpr int MISC_BYTES = 4608;     // barriers and small tables
 constexpr int ROW_WARPS = 8;         // two threads per query row
 constexpr int MMA_WARP = 8, COPY_WARP = 9, V_WARP = 10;
 // Three warpgroups: two of row warps, and one of the MMA and copy warps with two idle ones, which gives registers to the rows where
@@ -88,12 +89,12 @@ struct Cfg {
     static constexpr int UO_BYTES = ROWS * D * 2;                  // an O tile
     static constexpr int U_BYTES = TMA_IO ? UO_BYTES + ROWS * D : 0; // + a raw int8 Q~ tile
     static constexpr int OFF_MISC = OFF_U + U_BYTES;
-    static constexpr int TOTAL = OFF_MISC + 4096 + 192 + 1024;   // misc block + slack for 1024-byte alignment
+    static constexpr int TOTAL = OFF_MISC + MISC_BYTES + 1024;   // misc block + slack for 1024-byte alignment
     static constexpr uint32_t TMEM_S = 0, TMEM_O = 2 * TP;
     static constexpr uint32_t TMEM_COLS = (2 * TP + OBUF * DP) <= 256 ? 256 : 512;
     static constexpr int CTAS_PER_SM = (2 * (TOTAL + 1024) <= 232448 && TMEM_COLS == 256) ? 2 : 1;
     static_assert(HEAD_BYTES % 1024 == 0 && K_BYTES % 1024 == 0 && VT_BLOCK % 1024 == 0, "operand tiles must keep 1024-byte alignment");
-    static_assert(TOTAL <= 232448, "shared memory budget");
+    static_assert(TOTAL <= 232448 && OFF_MISC % 16 == 0, "shared memory budget");
     static_assert(QTAIL == 0 || QTAIL == 16, "narrow tile of Q~: 32-byte rows");
     static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0 && OFF_U % 128 == 0, "tile alignment");
     // 16-byte chunk cc ^ flip (8 channels; flip 0 or 2) of a row of the Q~ tile; chunk of a row of P (8 keys)
@@ -112,9 +113,10 @@ struct Misc {
     uint32_t tmem_base;
     volatile int abort_flag;
     float2 xchg[2][2][ROWS];     // [head parity][half][row]: (max, sum) of a thread's half of the softmax
+    alignas(16) float pad[TP];   // 0, or kPadLogit for the keys at and beyond T
 };
 constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
-static_assert(sizeof(Misc) <= 4096 + 192 && N_BARS <= 32, "misc block");
+static_assert(sizeof(Misc) <= MISC_BYTES && N_BARS <= 32 && offsetof(Misc, pad) % 16 == 0 && offsetof(Misc, xchg) % 8 == 0, "misc block");
 static_assert(sizeof(OperandConsts) % 16 == 0 && sizeof(OperandConsts) <= 384, "constants slot");
 
 // Half of the query codes (or fp16 values) of one row and head, held in registers between the global load and
@@ -194,6 +196,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(126); }
+    if (tid < TP) misc->pad[tid] = tid < T ? 0.f : kPadLogit;
     if (warp == COPY_WARP) {                          // one lane per barrier
         uint64_t* all = misc->kv_full;
         // one arrival per row warp; q_full of an fp16 tile that TMA loads: one; o_free: one per warp of the O warps
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                     ptx::tc_fence_before_sync();
                     const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT);
                     float m_loc, l_loc;
-                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, sq, T, key0, e, m_loc, l_loc);
+                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? 1e-20f : sq, e, m_loc, l_loc);      // (1e-20: any logit is 0 beside it)
                     trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                      : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
                     misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);
@@ -722,7 +725,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
             float e[HK];
             float m_loc, l_loc;
-            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, sq, T, key0, e, m_loc, l_loc);
+            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? 1e-20f : sq, e, m_loc, l_loc);      // (1e-20: any logit is 0 beside it)
             const unsigned long long trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                                       : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
             misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);

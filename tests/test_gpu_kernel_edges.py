@@ -178,3 +178,31 @@ def test_attention_in_pieces_of_any_alignment(channels, heads, q_bits):
         assert bool((o[: shift // 2] == -7.0).all()) and bool((o[shift // 2 + n:] == -7.0).all())
         outs.append(o[shift // 2: shift // 2 + n].clone())
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("channels,heads", [(640, 10), (160, 4), (640, 8), (1280, 8)])
+@pytest.mark.parametrize("n_ctx", [1, 40, 64, 65, 80])
+def test_attention_of_zero_queries(channels, heads, n_ctx):
+    """A row of zero codes has scale 0: every token weighs the same, and padding keys nothing, as with any other scale."""
+    shape = replace(synth.config1(), n_query=130, channels=channels, heads=heads, n_ctx=n_ctx, trigger=(0,), name=f"zero_{channels}_{heads}_{n_ctx}")
+    data = synth.make_layer(shape)
+    desc = tl.gpu_desc(shape)
+    P = tl.pack_layer_weights(shape, data)
+    mask = tl.dev(data["mask"])
+    kv = tb.taq_kv_project(desc, tl.dev(data["ctx"]), P["Wk"], P["Wv"], mask)
+    q = torch.zeros(shape.rows, channels, dtype=torch.int8, device="cuda")
+    q[::2] = torch.randint(-127, 128, q[::2].shape, device="cuda", generator=torch.Generator("cuda").manual_seed(1)).to(torch.int8)
+    scales = torch.full((shape.rows, heads), 0.02, device="cuda")
+    want = tb.taq_cross_attention(desc, q, scales, kv, mask)
+    scales[1::2] = 0.0
+    got = tb.taq_cross_attention(desc, q, scales, kv, mask)
+    tb.taq_poll_device_status()
+    assert bool(torch.isfinite(got).all()) and torch.equal(got, want)
+    p = tl.parse_kv_block(desc, kv)
+    v = p["V_codes"][0].astype("f8") * p["V_scales"][0][..., None]                   # [H, T, d] of the ordinary tokens
+    v[:, 0] = p["V_trigger"][0][0]
+    prob = torch.full((n_ctx,), float(round(255.0 / n_ctx)), dtype=torch.float64)    # the nearest code, and fp16 for the trigger column
+    prob[0] = torch.tensor(255.0 / n_ctx).half().double()
+    mean = (v * prob.numpy()[None, :, None] / 255.0).sum(1).reshape(-1)
+    # V~ and O are fp16 values: half a unit in the last place each, of a sum of n_ctx products
+    assert abs(got.view(-1, channels)[1].double().cpu().numpy() - mean).max() <= 2.0 ** -11 * (abs(v).max() + abs(mean).max())
