@@ -261,14 +261,16 @@ Choice choose_pair(const LinearArgs& a, int n_z, double& best_cost) {
     return best;
 }
 
-// Pairs or one CTA per tile.  Where a CTA would walk several tiles pairs were faster in every launch measured (by 2 to 45 %).  Elsewhere the
-// cheaper one, the wide tiles of one CTA with 2 us more than their model says: with fp16 rows launches of one wave of 128 or 160
-// columns take 1.4 to 3.2 us more.  So every one of 202 launches gets the faster kernel (with 1.5 us one is 7 % slower, with
-// none eight are 12 to 29 %).
+// Pairs or one CTA per tile: the cheaper one, with two corrections.  Where a CTA would walk several tiles the model of one CTA per tile is 10 to
+// 40 % short (in one problem's launches pairs were always faster there, by 2 to 45 %), but requests of few rows leave half of every
+// 256-row tile empty: 18 requests x 34 rows at 1280 channels, heads of 64, took 46.2 us a layer on pairs and 43.6 so.  In launches of one wave of 128 or
+// 160 columns fp16 rows take 1.4 to 3.2 us more than it says: with 2 us more every one of 202 launches gets the faster kernel (with
+// 1.5 us one is 7 % slower, with none eight are 12 to 29 %).
 Choice choose_anew(const LinearArgs& a, int n_z) {
     double cost, pair_cost;
     const Choice single = choose_single(a, n_z, cost), pair = choose_pair(a, n_z, pair_cost);
-    if (!pair.bn || (single.bn && !single.lay.persistent && pair_cost >= cost + (single.bn >= 128 ? 2.0 : 0.0))) return single;
+    const double limit = single.lay.persistent ? (a.rows <= BM ? 1.1 : 1.4) * cost : cost + (single.bn >= 128 ? 2.0 : 0.0);
+    if (!pair.bn || (single.bn && pair_cost >= limit)) return single;
     return pair;
 }
 

@@ -55,8 +55,9 @@ def test_linear_tiles(rows, n_out, k_in, bits, group, heads, dense, per_head):
 @pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
     (5633, 640, 640, 4, 128, 8, 128, 160),             # the last tile: one row of the first CTA, none of the second
     (5505, 640, 640, 8, 0, 10, 128, 128),              # ... one row of the second CTA; accumulators of three and two pairs of k-blocks
-    (9999, 320, 192, 4, 128, 8, 160, 160),             # an odd number of k-blocks, a short last group, heads of 40
-    (20000, 320, 64, 8, 0, 8, 160, 160),               # one k-block
+    (9999, 640, 192, 4, 128, 16, 128, 160),            # an odd number of k-blocks, a short last group, heads of 40
+    (20000, 640, 64, 8, 0, 16, 128, 160),              # one k-block
+    (9473, 320, 320, 4, 128, 8, 0, 160),
     (12289, 640, 512, 4, 256, 4, 160, 160),            # groups of two pairs of k-blocks, heads of 160
     (3000, 1280, 320, 4, 128, 20, 128, 128),
     (2049, 1280, 1280, 4, 0, 8, 160, 160),             # one group of 4-bit codes
