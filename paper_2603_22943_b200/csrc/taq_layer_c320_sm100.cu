@@ -176,7 +176,7 @@ __device__ __forceinline__ float softmax_row(const uint32_t (&u)[TP], float (&e)
         for (int i = 0; i < 8; ++i) {
             const int j = 8 * j8 + i;
             e[j] = __uint_as_float(u[j]) * f[i];
-            if (j >= TAIL_FROM) { if (j >= T) e[j] = -INFINITY; }
+            if (j >= TAIL_FROM) { if (j >= T) e[j] = kPadLogit; }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) m4[i] = max3(m4[i], e[8 * j8 + i], e[8 * j8 + 4 + i]);
@@ -185,11 +185,7 @@ __device__ __forceinline__ float softmax_row(const uint32_t (&u)[TP], float (&e)
     msq_out = msq;
     // all exponentials first, then the sums: the special-function unit's latency is hidden behind the next arguments
 #pragma unroll
-    for (int j = 0; j < TP; ++j) {
-        float arg = fmaf(e[j], sq, -msq);
-        if (j >= TAIL_FROM) { if (j >= T) arg = -INFINITY; }      // also when sq = 0
-        e[j] = ex2_approx(arg);
-    }
+    for (int j = 0; j < TP; ++j) e[j] = ex2_approx(fmaf(e[j], sq, -msq));
     float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < TP; ++j) sum4[j & 3] += e[j];
@@ -702,6 +698,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             }
             const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + OFF_CST + hi * kOperandConstBytes);
             float msq;
+            // (any logit is 0 beside 1e-20, and padding keys are compared with T once: 64 requests x 4096 rows 401.6 -> 398.5 us; by numbers to add, as in
+            // softmax_half, 409.8, for it spills)
+            if (sq == 0.f) sq = 1e-20f;
             const float l = softmax_row<TAIL_FROM>(u, e, cst->logit_factor, sq, T, msq);
             const float k255 = __fdividef(pmax, l);
             const uint32_t trig[3] = {cst->trig_bits[0], cst->trig_bits[1], cst->trig_bits[2]};

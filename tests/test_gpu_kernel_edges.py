@@ -181,7 +181,7 @@ def test_attention_in_pieces_of_any_alignment(channels, heads, q_bits):
     assert torch.equal(outs[0], outs[1])
 
 
-@pytest.mark.parametrize("channels,heads", [(640, 10), (160, 4), (640, 8), (1280, 8)])
+@pytest.mark.parametrize("channels,heads", [(640, 10), (160, 4), (320, 8), (640, 8), (1280, 8)])
 @pytest.mark.parametrize("n_ctx", [1, 40, 64, 65, 80])
 def test_attention_of_zero_queries(channels, heads, n_ctx):
     """A row of zero codes has scale 0: every token weighs the same, and padding keys nothing, as with any other scale."""
