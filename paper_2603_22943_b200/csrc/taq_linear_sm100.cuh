@@ -18,7 +18,8 @@
 //             and run the epilogue: bias / fp16 conversion, or the per-(row, head) int8 quantization Q_a of Eq. 2, or the
 //             mixed int8 / fp16 K~, V~ of Eq. 2 together with the attention kernel's operand images.
 // Launches of more tiles than SMs are persistent: a CTA walks several tiles, and the epilogue of one runs under the K loop of
-// the next.  The packed weights stay packed in HBM.
+// the next (most of those with fp16 rows in and no fp32 rows out run on pairs of CTAs instead: taq_linear_pair_sm100.cuh).  The packed weights
+// stay packed in HBM.
 //
 // What bounds it.  A 64-wide K block of a 160-column tile is 320 cycles of tensor time; the MMA thread needs 60 cycles per wait
 // on a complete barrier, 60 per commit and 45 per MMA (measured), hence barriers per pair of blocks, looked at one pair ahead.
