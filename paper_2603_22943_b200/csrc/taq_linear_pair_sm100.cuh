@@ -23,7 +23,10 @@ namespace taq {
 namespace linear {
 
 constexpr int PAIR_STAGES = 3;             // ring depth in pairs of k-blocks, activations and weights together
-constexpr int ONE_GROUP_PAIRS = 3;         // (long sums in the tensor core's accumulator lose bits: the scales of 8192 x 640 x 640, W8, are off by 1.5e-6 at most from sums over 640 elements, by 0.9e-6 so)
+// Long sums in the tensor core's accumulator lose bits.  Root mean square error of the scales of per-head rows, W8: 8192 x 640 x 640 7.0e-7 from
+// sums of 640 elements, 3.7e-7 from three pairs, 2.4e-7 from two; 64 x 1280 x 1280 2.8e-7 from a K loop in quarters, 3.3e-7 and 2.2e-7.  (8.47 us
+// with three pairs, 8.67 with two; 8192 x 640 x 640 11.44 and 11.53.)
+constexpr int ONE_GROUP_PAIRS = 2;
 constexpr int PAIR_DONE = 4;               // barriers of finished pairs of k-blocks, taken in turn: at least the accumulators in TMEM
 // The stages (a CTA has half of the weight rows) and, behind them, the output tile on its way out.
 template <int BN> constexpr int pair_ring_bytes() { return PAIR_STAGES * (2 * A_TILE_BYTES + Tile<BN>::B_TILE); }

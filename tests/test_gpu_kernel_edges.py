@@ -54,7 +54,7 @@ def test_linear_tiles(rows, n_out, k_in, bits, group, heads, dense, per_head):
 # (tile widths of the launches on pairs of CTAs, 0 where the plan above is taken)
 @pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
     (5633, 640, 640, 4, 128, 8, 128, 160),             # the last tile: one row of the first CTA, none of the second
-    (5505, 640, 640, 8, 0, 10, 128, 128),              # ... one row of the second CTA; accumulators of three and two pairs of k-blocks
+    (5505, 640, 640, 8, 0, 10, 128, 128),              # ... one row of the second CTA; accumulators of two, two and one pairs of k-blocks
     (9999, 640, 192, 4, 128, 16, 128, 160),            # an odd number of k-blocks, a short last group, heads of 40
     (20000, 640, 64, 8, 0, 16, 128, 160),              # one k-block
     (9473, 320, 320, 4, 128, 8, 0, 160),
