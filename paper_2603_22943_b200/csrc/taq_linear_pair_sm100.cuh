@@ -13,7 +13,7 @@
 // are measured.  At a tile's end the folders are away for 3 200 cycles, of which the accumulators in TMEM cover three groups.
 // Measured, a CTA per tile -> pairs (buffers larger than L2): W4, fp16 rows: 8192 x 640 x 640 16.7 -> 12.1 us, 2048 x 1280 x 1280 13.6 -> 12.0,
 // 8192 x 1280 x 1280 44.6 -> 32.7, 32768 x 640 x 640 45.0 -> 32.8; per-head rows of 80: 8192 x 640 x 640 17.4 -> 11.9, 32768 50.6 -> 33.4, of 64: 16.9 ->
-// 13.5 and 44.5 -> 35.8; W8, fp16 rows: 8192 x 640 x 640 15.3 -> 11.9.
+// 13.5 and 44.5 -> 35.8; W8, fp16 rows: 8192 x 640 x 640 15.3 -> 12.1.
 // Taken back: weights in TMEM as the A operand, channels on its lanes (two accumulators beside them are too few: 33.9 us at 8192 x 1280 x
 // 1280, 18.0 at 640 channels); a warp of its own that sends the output off (one tile per pair 0.3 us more, seven 4 % less).
 #pragma once
