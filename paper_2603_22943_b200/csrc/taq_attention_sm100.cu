@@ -113,7 +113,7 @@ struct Misc {
     uint32_t tmem_base;
     volatile int abort_flag;
     float2 xchg[2][2][ROWS];     // [head parity][half][row]: (max, sum) of a thread's half of the softmax
-    alignas(16) float pad[TP];   // 0, or kPadLogit for the keys at and beyond T
+    alignas(16) float pad[TP];   // 0, or -inf for the keys at and beyond T
 };
 constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
 static_assert(sizeof(Misc) <= MISC_BYTES && N_BARS <= 32 && offsetof(Misc, pad) % 16 == 0 && offsetof(Misc, xchg) % 8 == 0, "misc block");
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
 
     TAQ_PROF_INIT
     if (tid == 0) { TAQ_PROF(0); TAQ_GPROF(126); }
-    if (tid < TP) misc->pad[tid] = tid < T ? 0.f : kPadLogit;
+    if (tid < TP) misc->pad[tid] = tid < T ? 0.f : -INFINITY;
     if (warp == COPY_WARP) {                          // one lane per barrier
         uint64_t* all = misc->kv_full;
         // one arrival per row warp; q_full of an fp16 tile that TMA loads: one; o_free: one per warp of the O warps
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                     ptx::tc_fence_before_sync();
                     const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT);
                     float m_loc, l_loc;
-                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? 1e-20f : sq, e, m_loc, l_loc);      // (1e-20: any logit is 0 beside it)
+                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? __int_as_float(1) : sq, e, m_loc, l_loc);      // (the smallest number above 0: any logit is 0 beside it)
                     trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                      : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
                     misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);
@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
             float e[HK];
             float m_loc, l_loc;
-            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? 1e-20f : sq, e, m_loc, l_loc);      // (1e-20: any logit is 0 beside it)
+            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? __int_as_float(1) : sq, e, m_loc, l_loc);      // (the smallest number above 0: any logit is 0 beside it)
             const unsigned long long trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                                       : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
             misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);

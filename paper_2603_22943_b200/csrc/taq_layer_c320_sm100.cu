@@ -160,6 +160,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
+constexpr float kPadLogit = -1e30f;
+
 // The softmax of one thread's row over all TP keys: raw scores u (integer dot products) -> e_j = 2^(u_j f_j sq - m)
 // with the row's own maximum m (log2 units); returns their sum.  Keys at or beyond T get weight exactly 0.
 // The softmax of one thread's row over all TP keys: raw scores u (integer dot products) -> e_j = 2^(u_j f_j sq - m)

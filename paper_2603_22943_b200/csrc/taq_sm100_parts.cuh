@@ -107,10 +107,9 @@ __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const floa
     l_out = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
 }
 
-// The same with the keys at or beyond T told by numbers to add, pad[j] = 0 or kPadLogit, and sq not zero: their weight is exactly 0 without a
-// comparison and two selections per key and pass, which the pipe that paces the softmax (16 lanes a cycle) would do: 8192 rows x 10 heads of 64
-// 13.3 -> 12.6 us.  (A thread whose keys are all padding has a maximum, halfway between those and any logit, that vanishes beside the other half's.)
-constexpr float kPadLogit = -1e30f;
+// The same with the keys at or beyond T told by numbers to add, pad[j] = 0 or -inf: beside a scale above 0, however small or large, their weight
+// is exactly 0 without a comparison and two selections per key and pass, which the pipe that paces the softmax (16 lanes a cycle) would do:
+// 8192 rows x 10 heads of 64 13.3 -> 12.6 us.
 template <bool TAIL_ONLY>
 __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const float* factor, const float* pad, float sq, float (&e)[HK], float& m_out, float& l_out) {
 #pragma unroll
@@ -129,11 +128,11 @@ __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const floa
             e[4 * j4 + 3] = __uint_as_float(u[4 * j4 + 3]) * f.w;
         }
     }
-    constexpr float FLOOR = 0.5f * kPadLogit;
-    float m4[4] = {FLOOR, FLOOR, FLOOR, FLOOR};
+    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int j = 0; j < HK; ++j) m4[j & 3] = fmaxf(m4[j & 3], e[j]);
-    const float msq = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sq;
+    // (a finite floor for a thread whose keys are all padding, behind the product: no scale takes it to -inf)
+    const float msq = fmaxf(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sq, -3e38f);
     float sum4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int j = 0; j < HK; ++j) {

@@ -207,3 +207,47 @@ def test_attention_of_zero_queries(channels, heads, n_ctx):
     mean = (v * prob.numpy()[None, :, None] / 255.0).sum(1).reshape(-1)
     # V~ and O are fp16 values: half a unit in the last place each, of a sum of n_ctx products
     assert abs(got.view(-1, channels)[1].double().cpu().numpy() - mean).max() <= 2.0 ** -11 * (abs(v).max() + abs(mean).max())
+
+
+@pytest.mark.parametrize("channels,heads", [(640, 10), (160, 4), (640, 8), (1280, 8)])
+@pytest.mark.parametrize("n_ctx", [1, 9, 40, 64, 77])
+def test_attention_of_any_query_scale(channels, heads, n_ctx):
+    """Padding keys weigh nothing beside the smallest and the largest scales, too, and rows of a tile do not depend on their neighbours' scales."""
+    shape = replace(synth.config1(), n_query=130, channels=channels, heads=heads, n_ctx=n_ctx, trigger=(0,), name=f"scale_{channels}_{heads}_{n_ctx}")
+    data = synth.make_layer(shape)
+    desc = tl.gpu_desc(shape)
+    P = tl.pack_layer_weights(shape, data)
+    mask = tl.dev(data["mask"])
+    kv = tb.taq_kv_project(desc, tl.dev(data["ctx"]), P["Wk"], P["Wv"], mask)
+    q = torch.randint(-127, 128, (shape.rows, channels), device="cuda", generator=torch.Generator("cuda").manual_seed(1)).to(torch.int8)
+    d = channels // heads
+
+    def attention(scale, codes=q):
+        scales = torch.full((shape.rows, heads), 0.02, device="cuda")
+        scales[1::2] = scale
+        o = tb.taq_cross_attention(desc, codes, scales, kv, mask).view(-1, channels)
+        tb.taq_poll_device_status()
+        return o
+
+    plain, flat = attention(0.02), attention(0.0)
+    assert torch.equal(flat[::2], plain[::2])
+    # logits of at most 127 * 127 * 160 units, each under 1: beside these scales all are 0
+    for scale in (1e-45, 1e-38, 1e-30, 1e-24):
+        assert torch.equal(attention(scale), flat), scale
+    # A scale at which the largest logit takes all of it, of single codes of 1: logits of about 1e9, whose last place (64) is nothing that the sums
+    # of powers of two could not hold.
+    p = tl.parse_kv_block(desc, kv)
+    k, v = (p[n + "_codes"][0].astype("f8") * p[n + "_scales"][0][..., None] for n in "KV")      # [H, T, d]
+    k[:, 0], v[:, 0] = p["K_trigger"][0][0], p["V_trigger"][0][0]
+    k, v = torch.from_numpy(k), torch.from_numpy(v).half().double()                               # (V~ is an fp16 operand)
+    single = q.view(-1, heads, d).clone()
+    single[1::2] = torch.nn.functional.one_hot(torch.arange(shape.rows, device="cuda") % d, d)[1::2, None]
+    logits = torch.einsum("rhd,htd->rht", single[1::2].cpu().double(), k)
+    top = logits.topk(min(2, n_ctx), dim=-1).values
+    clear = (top[..., 0] - top[..., -1] > 1e-5 * top[..., 0].abs() + 1e-5) | (n_ctx == 1)         # (1e9 / 8 of that: far more than 64 + 24)
+    got = attention(1e9, single.view(-1, channels))
+    assert torch.equal(got[::2], plain[::2])
+    got = got[1::2].view(-1, heads, d).cpu().double()
+    want = v[torch.arange(heads), logits.argmax(-1)]                                              # [rows, H, d]
+    # the one probability is 255 of 255; O = V~ * 255 * (1 / 255) in fp32, rounded to fp16
+    assert bool(clear.any()) and bool(((got - want).abs() <= 2.0 ** -11 * want.abs() + 1e-7)[clear].all())
