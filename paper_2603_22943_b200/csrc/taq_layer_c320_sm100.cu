@@ -160,12 +160,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-constexpr float kPadLogit = -1e30f;
-
 // The softmax of one thread's row over all TP keys: raw scores u (integer dot products) -> e_j = 2^(u_j f_j sq - m)
-// with the row's own maximum m (log2 units); returns their sum.  Keys at or beyond T get weight exactly 0.
-// The softmax of one thread's row over all TP keys: raw scores u (integer dot products) -> e_j = 2^(u_j f_j sq - m)
-// with the row's own maximum m (log2 units); returns their sum.  Keys at or beyond T get weight exactly 0; only keys from
+// with the row's own maximum m (log2 units); returns their sum.  Keys at or beyond T get weight exactly 0 (sq: above 0); only keys from
 // TAIL_FROM on can be such keys (the launcher picks TAIL_FROM <= T).
 template <int TAIL_FROM>
 __device__ __forceinline__ float softmax_row(const uint32_t (&u)[TP], float (&e)[TP], const float* factor, float sq, int T, float& msq_out) {
@@ -178,7 +174,7 @@ __device__ __forceinline__ float softmax_row(const uint32_t (&u)[TP], float (&e)
         for (int i = 0; i < 8; ++i) {
             const int j = 8 * j8 + i;
             e[j] = __uint_as_float(u[j]) * f[i];
-            if (j >= TAIL_FROM) { if (j >= T) e[j] = kPadLogit; }
+            if (j >= TAIL_FROM) { if (j >= T) e[j] = -INFINITY; }
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) m4[i] = max3(m4[i], e[8 * j8 + i], e[8 * j8 + 4 + i]);
@@ -700,9 +696,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) layer_c320_kernel(const __grid_co
             }
             const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + OFF_CST + hi * kOperandConstBytes);
             float msq;
-            // (any logit is 0 beside 1e-20, and padding keys are compared with T once: 64 requests x 4096 rows 401.6 -> 398.5 us; by numbers to add, as in
-            // softmax_half, 409.8, for it spills)
-            if (sq == 0.f) sq = 1e-20f;
+            // (The smallest number above 0 leaves every logit 0, and -inf what it is: padding keys are compared with T once.  64 requests x 4096 rows
+            // 401.6 -> 398.5 us; by numbers to add, as in softmax_half, 409.8, for it spills.)
+            if (sq == 0.f) sq = __int_as_float(1);
             const float l = softmax_row<TAIL_FROM>(u, e, cst->logit_factor, sq, T, msq);
             const float k255 = __fdividef(pmax, l);
             const uint32_t trig[3] = {cst->trig_bits[0], cst->trig_bits[1], cst->trig_bits[2]};

@@ -251,3 +251,15 @@ def test_attention_of_any_query_scale(channels, heads, n_ctx):
     want = v[torch.arange(heads), logits.argmax(-1)]                                              # [rows, H, d]
     # the one probability is 255 of 255; O = V~ * 255 * (1 / 255) in fp32, rounded to fp16
     assert bool(clear.any()) and bool(((got - want).abs() <= 2.0 ** -11 * want.abs() + 1e-7)[clear].all())
+
+
+@pytest.mark.parametrize("channels,n_ctx", [(320, 9), (320, 77), (640, 9), (640, 77)])
+def test_layer_of_tiny_query_projections(channels, n_ctx):
+    """A to_q of tiny weights leaves tiny scales, beside which every logit is 0: the same output as of a to_q of zeros."""
+    shape = replace(synth.config2(), n_query=130, channels=channels, n_ctx=n_ctx, name=f"tiny_q_{channels}_{n_ctx}")
+    data = synth.make_layer(shape)
+    none = dict(data, Wq=0.0 * data["Wq"])
+    want = tl.gpu_layer(shape, none)
+    tl.assert_layer_close(want, tl.oracle_layer(shape, none)["Y"], "zero queries")
+    for size in (1e-35, 1e-30, 1e-25):
+        assert (tl.gpu_layer(shape, dict(data, Wq=(size * data["Wq"]).astype("f4"))) == want).all(), size
