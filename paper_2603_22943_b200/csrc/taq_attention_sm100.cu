@@ -119,6 +119,9 @@ constexpr int N_BARS = (int)(offsetof(Misc, tmem_base) / 8);
 static_assert(sizeof(Misc) <= MISC_BYTES && N_BARS <= 32 && offsetof(Misc, pad) % 16 == 0 && offsetof(Misc, xchg) % 8 == 0, "misc block");
 static_assert(sizeof(OperandConsts) % 16 == 0 && sizeof(OperandConsts) <= 384, "constants slot");
 
+// What the softmax takes for a row's scale: its sign is with the codes (SignOf), and beside the smallest number above 0 any logit is 0.
+__device__ __forceinline__ float size_of(float scale) { return scale == 0.f ? __int_as_float(1) : fabsf(scale); }
+
 // Half of the query codes (or fp16 values) of one row and head, held in registers between the global load and
 // the store into the operand tile: the row's two threads take the lower and the upper half of the 16-byte chunks.
 template <int D, bool Q8>
@@ -169,10 +172,10 @@ struct QRegs {
         }
     }
     // local chunk i (8 channels) as fp16 operands; channels beyond D are zero (a zero int8 code maps to fp16 zero)
-    __device__ __forceinline__ uint4 chunk(int i) const {
+    __device__ __forceinline__ uint4 chunk(int i, const SignOf& sign) const {
         if (Q8) {
             const uint4 w = v[i / 2];
-            return codes_w8_to_half((i & 1) ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y));
+            return codes_w8_to_half((i & 1) ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y), sign);
         }
         return v[i];
     }
@@ -240,8 +243,9 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                 const unsigned char* UQ = smem + C::OFF_U + C::UO_BYTES;
                 const int t = tid - 32 * Q_WARP, swap = D == 160 ? (t >> 2) & 1 : 0;
                 static_assert(D != 160 || (N % 2 == 0 && C::QTAIL == 0), "pairs of chunks");
-                if (t == 0) ptx::pdl_wait();                             // (this thread loads Q~ of the third head and on)
-                __syncwarp();
+                ptx::pdl_wait();                                         // (scales; one thread loads Q~ of the third head and on, too)
+                const float* scales = a.q_scales + ((size_t)zb * a.n_query + min(row0 + t, a.n_query - 1)) * H + h_begin;
+                float scale = HG > 1 ? scales[1] : 0.f;
                 for (int hi = 1; hi < HG; ++hi) {
                     alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(hi), (hi >> 1) & 1));
                     uint4 raw[N];
@@ -254,17 +258,19 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                         ptx::tma_load_3d(smem + C::OFF_U + C::UO_BYTES, &tmap_q, qraw_full(hi + 1), (h_begin + hi + 1) * D, row0, zb);
                     }
                     __syncwarp();
+                    SignOf sign(scale);
                     alive = alive && __all_sync(0xffffffffu, ptx::mbar_wait(&misc->s_full[(hi - 1) & 1], ((hi - 1) >> 1) & 1));
                     if (alive) {
 #pragma unroll
                         for (int i = 0; i < N; ++i) {
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].x, raw[i].y));
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i + 1, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].z, raw[i].w));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].x, raw[i].y), sign);
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(t, 2 * i + 1, 2 * swap)) = codes_w8_to_half(make_uint2(raw[i].z, raw[i].w), sign);
                         }
                         ptx::fence_proxy_async_smem();
                     }
                     __syncwarp();
                     if (alive && lane < ROW_WARPS / 4) ptx::mbar_arrive(&misc->q_full);      // (two lanes of each of four warps: as many as row warps)
+                    if (hi + 1 < HG) scale = scales[hi + 1];
                 }
             } else if (warp == Q_WARP && lane == 0) {
                 // (channels behind the head's last in its last 64-wide block are never multiplied)
@@ -509,7 +515,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             unsigned char* U = smem + C::OFF_U;
             auto all256 = [&]() { asm volatile("bar.sync 5, 256;" ::: "memory"); };
             // raw tile of the first head -> fp16 operand tile: half a row per thread
-            auto stage_q_u = [&]() {
+            auto stage_q_u = [&](float scale) {
                 constexpr int N = D / 16, N2 = (N + 1) / 2;  // sixteen codes at a time
                 unsigned char* UQ = U + C::UO_BYTES;
                 auto load_q = [&](int hi) {                  // one thread: raw Q~ tile of head hi (rows beyond n_query read as zero)
@@ -519,12 +525,13 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                 if (tid == 0) load_q(0);
                 alive = __all_sync(0xffffffffu, ptx::mbar_wait(qraw_full(0), 0));
                 if (alive) {
+                    const SignOf sign(scale);
 #pragma unroll
                     for (int i = 0; i < N2; ++i) {
                         if (half * N2 + i < N) {
                             const uint4 raw = *reinterpret_cast<const uint4*>(UQ + r * D + (half * N2 + i) * 16);
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i))) = codes_w8_to_half(make_uint2(raw.x, raw.y));
-                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i) + 1)) = codes_w8_to_half(make_uint2(raw.z, raw.w));
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i))) = codes_w8_to_half(make_uint2(raw.x, raw.y), sign);
+                            *reinterpret_cast<uint4*>(smem + C::OFF_Q + C::q_offset(r, 2 * (half * N2 + i) + 1)) = codes_w8_to_half(make_uint2(raw.z, raw.w), sign);
                         }
                     }
                     ptx::fence_proxy_async_smem();
@@ -566,7 +573,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             float sq = 1.0f, sq_next = 1.0f;
             if (Q8) {
                 sq = valid ? a.q_scales[grow * H + h_begin] : 0.f;
-                stage_q_u();
+                stage_q_u(sq);
             }
 
             for (int hi = 0; hi < HG; ++hi) {
@@ -593,7 +600,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
                     ptx::tc_fence_before_sync();
                     const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_CST + (hi % C::CST_SLOTS) * C::CST_SLOT);
                     float m_loc, l_loc;
-                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? __int_as_float(1) : sq, e, m_loc, l_loc);      // (the smallest number above 0: any logit is 0 beside it)
+                    softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, size_of(sq), e, m_loc, l_loc);
                     trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                      : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
                     misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);
@@ -681,11 +688,12 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             }
             ptx::tc_fence_before_sync();
         };
-        auto stage_q = [&](const QRegs<D, Q8>& qr) {
+        auto stage_q = [&](const QRegs<D, Q8>& qr, float scale) {
+            const SignOf sign(scale);
 #pragma unroll
             for (int i = 0; i < CH2; ++i) {
                 const int cc = half * CH2 + i;
-                if (cc < DP / 8) *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(r, cc & 7)) = qr.chunk(i);
+                if (cc < DP / 8) *reinterpret_cast<uint4*>(smem + C::OFF_Q + (cc >> 3) * C::A_BLOCK + ptx::sw128_offset(r, cc & 7)) = qr.chunk(i, sign);
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();
@@ -696,7 +704,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
         qr.load(a.q, grow * Cch + (size_t)h_begin * D, valid, half);
         float sq = 1.0f, sq_next = 1.0f;
         if (Q8) sq = valid ? a.q_scales[grow * H + h_begin] : 0.f;
-        stage_q(qr);
+        stage_q(qr, sq);
 
         for (int hi = 0; hi < HG; ++hi) {
             const uint32_t ph = hi & 1;
@@ -725,7 +733,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
             const OperandConsts* cst = reinterpret_cast<const OperandConsts*>(smem + C::OFF_KV + (hi % C::KVBUF) * C::HEAD_BYTES + C::K_BYTES + C::VT_BYTES);
             float e[HK];
             float m_loc, l_loc;
-            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, sq == 0.f ? __int_as_float(1) : sq, e, m_loc, l_loc);      // (the smallest number above 0: any logit is 0 beside it)
+            softmax_half<TAIL_ONLY>(u, cst->logit_factor + key0, misc->pad + key0, size_of(sq), e, m_loc, l_loc);
             const unsigned long long trig = half == 0 ? ((unsigned long long)cst->trig_bits[0] | ((unsigned long long)(cst->trig_bits[1] & 0xFFu) << 32))
                                                       : ((unsigned long long)(cst->trig_bits[1] >> 8) | ((unsigned long long)cst->trig_bits[2] << 24));
             misc->xchg[ph][half][r] = make_float2(m_loc, l_loc);
@@ -737,7 +745,7 @@ __global__ void __launch_bounds__(Cfg<D, Q8>::THREADS, Cfg<D, Q8>::CTAS_PER_SM) 
 
             // S of this head is complete, so the Q~ tile is free again; the next head's codes, asked for at the top of this
             // iteration, have had the softmax to arrive
-            if (more) stage_q(qr);
+            if (more) stage_q(qr, sq_next);
             if (tid == 0 && hi < 8) TAQ_PROF(32 + hi);
             // the P tile is free once the previous head's PV has completed
             if (hi > 0) {

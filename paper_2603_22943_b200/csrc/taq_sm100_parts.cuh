@@ -41,6 +41,27 @@ __device__ __forceinline__ uint4 codes_w8_to_half(uint2 raw) {
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// The same times 1 or -1, the sign of a row's scale (exact: an FMA takes the difference's place).  Turned in the softmax, by a branch or by flipping
+// scores, signs cost every row 1 to 4 %: its loop fills the instruction cache.
+struct SignOf {
+    __half2 one, off;
+    __device__ __forceinline__ explicit SignOf(float scale) : one(__float2half2_rn(scale < 0.f ? -1.f : 1.f)), off(__float2half2_rn(scale < 0.f ? 1152.f : -1152.f)) {}
+};
+__device__ __forceinline__ uint4 codes_w8_to_half(uint2 raw, const SignOf& sign) {
+    const uint32_t w[2] = {raw.x ^ 0x80808080u, raw.y ^ 0x80808080u};
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        uint32_t lo = __byte_perm(w[i], 0x64646464u, 0x5140);
+        uint32_t hi = __byte_perm(w[i], 0x64646464u, 0x5342);
+        __half2 a = __hfma2(*reinterpret_cast<__half2*>(&lo), sign.one, sign.off);
+        __half2 b = __hfma2(*reinterpret_cast<__half2*>(&hi), sign.one, sign.off);
+        o[2 * i] = *reinterpret_cast<uint32_t*>(&a);
+        o[2 * i + 1] = *reinterpret_cast<uint32_t*>(&b);
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // Eight 4-bit codes of one word -> eight int8 codes in fan-in order (the integer-activation GEMM's weight operand).
 __device__ __forceinline__ uint2 codes_w4_to_i8(uint32_t p) {
     const uint32_t even = p & 0x0F0F0F0Fu;              // bytes: elements 0, 4, 1, 5 (+8)
@@ -109,7 +130,7 @@ __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const floa
 
 // The same with the keys at or beyond T told by numbers to add, pad[j] = 0 or -inf: beside a scale above 0, however small or large, their weight
 // is exactly 0 without a comparison and two selections per key and pass, which the pipe that paces the softmax (16 lanes a cycle) would do:
-// 8192 rows x 10 heads of 64 13.3 -> 12.6 us.
+// 8192 rows x 10 heads of 64 13.3 -> 12.7 us.
 template <bool TAIL_ONLY>
 __device__ __forceinline__ void softmax_half(const uint32_t (&u)[HK], const float* factor, const float* pad, float sq, float (&e)[HK], float& m_out, float& l_out) {
 #pragma unroll

@@ -234,6 +234,8 @@ def test_attention_of_any_query_scale(channels, heads, n_ctx):
     # logits of at most 127 * 127 * 160 units, each under 1: beside these scales all are 0
     for scale in (1e-45, 1e-38, 1e-30, 1e-24):
         assert torch.equal(attention(scale), flat), scale
+    # the sign of scale and codes together does not matter (the maximum taken off the logits does, hence ties)
+    tl.assert_same_up_to_code_ties(attention(-0.02, torch.where(torch.arange(shape.rows, device="cuda")[:, None] % 2 == 1, -q, q)), plain, "negative scales")
     # A scale at which the largest logit takes all of it, of single codes of 1: logits of about 1e9, whose last place (64) is nothing that the sums
     # of powers of two could not hold.
     p = tl.parse_kv_block(desc, kv)
