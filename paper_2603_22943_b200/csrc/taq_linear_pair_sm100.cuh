@@ -354,6 +354,11 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
                         if (++j == n_pair) j = 0;
                     }
                 }
+                // The last arrivals on acc_free, half of them the other CTA's, are seen here, too: nothing may arrive in a CTA that has left.  (Release
+                // instead of relaxed in the barrier below would do, and wait for the stores of every thread: 0.2 to 0.6 us a launch.)
+                if (rank == 0)
+                    for (int s = 0; s < NSLOT && ok; ++s)
+                        if (s < slot || recycled) ok = ptx::mbar_wait(&bars->acc_free[s], s < slot ? ph_free ^ 1 : ph_free);
                 if (!ok) give_up();
             }
             __syncwarp();

@@ -190,3 +190,26 @@ def test_rows_that_several_warps_staged_are_stored_only_if_none_of_them_gave_up(
         at = src.index(store)
         between = src[src.rindex(barrier, 0, at): at]
         assert "!misc->abort_flag" in between, (name, barrier)
+
+
+def test_pairs_of_ctas_see_the_last_arrivals_before_they_leave():
+    """An accumulator's last two arrivals come from both CTAs of a pair and let no MMA go on; the issuing thread waits for them all the same, so
+    that none arrives in a CTA that has left.  (Read from the source; and the parities it waits for, on every count of groups.)"""
+    src = open(os.path.join(tbuild.CSRC, "taq_linear_pair_sm100.cuh")).read()
+    last_commit, teardown = src.rindex("mma_commit_pair("), src.index("// ---------------- teardown")
+    loop = "for (int s = 0; s < NSLOT && ok; ++s)"
+    assert loop in src[last_commit:teardown]
+    assert "if (s < slot || recycled) ok = ptx::mbar_wait(&bars->acc_free[s], s < slot ? ph_free ^ 1 : ph_free);" in src[last_commit:teardown]
+    for n_slots in (3, 4):
+        for n_groups in range(1, 40):
+            slot, recycled, ph_free, used = 0, False, 1, [0] * n_slots
+            for _ in range(n_groups):                      # the issuing thread's walk
+                used[slot] += 1
+                slot += 1
+                if slot == n_slots:
+                    slot, recycled, ph_free = 0, True, ph_free ^ 1
+            for s in range(n_slots):
+                if s < slot or recycled:                   # completion number used[s] has this parity, the one before has not
+                    assert (used[s] - 1) & 1 == (ph_free ^ 1 if s < slot else ph_free)
+                else:
+                    assert used[s] == 0
