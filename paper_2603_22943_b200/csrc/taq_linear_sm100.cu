@@ -203,8 +203,10 @@ Choice choose_single(const LinearArgs& a, int n_z, double& best_cost) {
         if (tiles * 2 <= SMS && rings_of(a, p, 80, 2, 1, false, c)) { best_cost = 0; return finish(c, a, p, tiles, tiles * 2); }      // (faster than pairs, too)
     }
     // K~/V~ with heads of 160 channels: the same, the K loop whole, where the CTAs are one wave (two prompts of 77 x 768, 1280 channels: W4 13.4 ->
-    // 9.5 us, W8 12.8 -> 9.1, against one 160-wide tile per head on half as many).
-    if (a.epi == EPI_KV && p.d == 160 && !(p.i8 && a.bits == 8)) {
+    // 9.5 us, W8 12.8 -> 9.1, against one 160-wide tile per head on half as many).  Wider contexts are split below, and their sums stay as short as
+    // that makes them: whole, the scales' root mean square error of W8 rises from 3.4e-7 to 8.1e-7 at 1024 (12.9 -> 10.2 us) and from 3.1e-7 to
+    // 1.8e-6 at 2048 (13.8 -> 13.3), and 4096 takes 21.1 us instead of 19.1.
+    if (a.epi == EPI_KV && p.d == 160 && a.k_in < 1024 && !(p.i8 && a.bits == 8)) {
         const long long tiles = p.row_tiles * (a.n_out / 80) * 2 * (long long)n_z;
         Choice c{};
         if (tiles <= SMS && rings_of(a, p, 80, 1, 1, false, c)) { best_cost = 0; return finish(c, a, p, tiles, tiles); }
