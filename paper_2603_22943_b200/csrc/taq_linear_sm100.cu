@@ -267,10 +267,13 @@ Choice choose_pair(const LinearArgs& a, int n_z, double& best_cost) {
 // 40 % short (in one problem's launches pairs were always faster there, by 2 to 45 %), but requests of few rows leave half of every
 // 256-row tile empty: 18 requests x 34 rows at 1280 channels, heads of 64, took 46.2 us a layer on pairs and 43.6 so.  In launches of one wave of 128 or
 // 160 columns fp16 rows take 1.4 to 3.2 us more than it says: with 2 us more every one of 202 launches gets the faster kernel (with
-// 1.5 us one is 7 % slower, with none eight are 12 to 29 %).
+// 1.5 us one is 7 % slower, with none eight are 12 to 29 %).  Scale groups that a cluster would share stay shared (heads of 160 channels, 600 to
+// 1150 rows): sums of all groups in a row lose bits that two halves keep.  1100 x 1280 x 1280, W4: scales' root mean square error 5.3e-8,
+// on pairs 6.3e-8 (12.9 and 10.8 us); x 2560 5.8e-8 and 7.9e-8 (18.0 and 19.6 us).
 Choice choose_anew(const LinearArgs& a, int n_z) {
     double cost, pair_cost;
     const Choice single = choose_single(a, n_z, cost), pair = choose_pair(a, n_z, pair_cost);
+    if (single.lay.nsplit > 1 && single.lay.n_groups > 1) return single;
     const double limit = single.lay.persistent ? (a.rows <= BM ? 1.1 : 1.4) * cost : cost + (single.bn >= 128 ? 2.0 : 0.0);
     if (!pair.bn || (single.bn && pair_cost >= limit)) return single;
     return pair;

@@ -213,3 +213,16 @@ def test_pairs_of_ctas_see_the_last_arrivals_before_they_leave():
                     assert (used[s] - 1) & 1 == (ph_free ^ 1 if s < slot else ph_free)
                 else:
                     assert used[s] == 0
+
+
+def test_scale_groups_that_a_cluster_shares_do_not_go_to_pairs(L):
+    """Heads of 160 channels, 600 to 1150 rows, 4-bit weights: the sums of all groups in a row, as pairs of CTAs take them, are less exact than the
+    two halves of a cluster.  (8-bit weights have one group, which pairs sum over 256 elements at a time.)"""
+    for rows in (600, 700, 1024, 1152):
+        for group in (128, 256):
+            for k_in in (1280, 2560):
+                wd = tb.weight_desc(1280, k_in, 4, group)
+                assert tb.taq_linear_pair_plan(wd, rows, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["bn"] == 0
+                assert tb.taq_linear_plan(wd, rows, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["split"] == 2
+    assert tb.taq_linear_pair_plan(tb.weight_desc(1280, 1280, 8, 0), 1024, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["bn"] == 160
+    assert tb.taq_linear_pair_plan(tb.weight_desc(1280, 1280, 4, 128), 2048, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["bn"] == 160
