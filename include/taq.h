@@ -358,19 +358,19 @@ enum {
 taq_status taq_dispatch_counts(int64_t* counts_out, int32_t n);
 void taq_dispatch_reset(void);
 
-/* The launch plan the tensor-core dequant-GEMM with one CTA, or a cluster, per tile would take for a problem (host arithmetic only; nothing is launched
- * and no GPU is needed).  plan_out: int32 [10] = {tile width BN (0: the tensor-core kernel does not take the
+/* The launch plan the tensor-core dequant-GEMM takes for a problem (host arithmetic only; nothing is launched
+ * and no GPU is needed).  plan_out: int32 [10] = {tile width BN (0: the tensor-core kernels do not take the
  * problem), ring stages in k-blocks, CTAs that share the K loop of a tile (1, 2 or 4), bytes of the ring, bytes of the
  * ring the epilogue reuses as its staging area, offset of the scales (the first section behind the ring), offset of the
  * bias, offset of the barriers, total shared memory, shared-memory limit}.  Every region must lie inside `total`, the
- * staging area inside the ring.  int8_activations / batched select the variant as taq_quantized_linear_i8 and the
- * per-request calls do. */
+ * staging area inside the ring (on pairs of CTAs it lies behind the stages and is counted with them).  Tiles have 128 rows,
+ * on pairs of CTAs 256.  int8_activations / batched select the variant as taq_quantized_linear_i8 and the
+ * per-request calls do, with one request. */
 taq_status taq_linear_plan(const taq_weight_desc* desc, int64_t rows, int32_t out_kind, int32_t heads,
                            int32_t int8_activations, int32_t batched, int32_t* plan_out);
 
-/* Launches of many rows of fp16 activations with fp16 or per-head int8 outputs run on pairs of CTAs instead, which compute
- * tiles of 256 rows together.  The same plan for those (tile width 0: the problem runs as taq_linear_plan says); the staging area lies
- * inside the bytes counted as the ring.  n_requests: requests of a batched call, 0 for a single problem. */
+/* The same where the problem runs on pairs of CTAs, tile width 0 where it does not.  Launches of many rows of fp16 activations with
+ * fp16 or per-head int8 outputs do.  n_requests: requests of a batched call, 0 for a single problem. */
 taq_status taq_linear_pair_plan(const taq_weight_desc* desc, int64_t rows, int32_t out_kind, int32_t heads,
                                 int32_t n_requests, int32_t* plan_out);
 

@@ -467,7 +467,7 @@ LINEAR_PLAN_FIELDS = ("bn", "nstage", "split", "ring_bytes", "staging_bytes", "o
 
 
 def taq_linear_plan(desc: "WeightDesc", rows: int, out_kind: int, heads: int = 1, int8_activations: bool = False, batched: bool = False) -> dict:
-    """Shared-memory plan of the tensor-core dequant-GEMM for a problem (host arithmetic; needs no GPU)."""
+    """Shared-memory plan of the tensor-core dequant-GEMM for a problem, as it is launched (host arithmetic; needs no GPU)."""
     arr = (C.c_int32 * 10)()
     _check(lib().taq_linear_plan(C.byref(desc), rows, out_kind, heads, int(int8_activations), int(batched), arr))
     return {k: int(arr[i]) for i, k in enumerate(LINEAR_PLAN_FIELDS)}

@@ -775,7 +775,7 @@ void taq_dispatch_reset(void) {
 }
 
 static taq_status linear_plan(const taq_weight_desc* d, int64_t rows, int32_t out_kind, int32_t heads, int32_t int8_activations,
-                              int32_t batched, int n_z, bool pairs, int32_t* plan_out) {
+                              int32_t batched, int n_z, bool pairs_only, int32_t* plan_out) {
     taq_status s = check_weight_desc(d);
     if (s != TAQ_OK) return s;
     if (!plan_out) return fail(TAQ_ERR_INVALID_ARG, "plan_out is NULL");
@@ -791,7 +791,7 @@ static taq_status linear_plan(const taq_weight_desc* d, int64_t rows, int32_t ou
     a.heads = out_kind == TAQ_OUT_INT8_HEAD_ROWS ? heads : 1;
     a.epi = out_kind == TAQ_OUT_F16 ? EPI_F16 : out_kind == TAQ_OUT_F32 ? EPI_F32 : EPI_Q8_HEAD;
     int out[10];
-    linear_plan_of(a, n_z, pairs, out);
+    linear_plan_of(a, n_z, pairs_only, out);
     for (int i = 0; i < 10; ++i) plan_out[i] = out[i];
     return TAQ_OK;
 }

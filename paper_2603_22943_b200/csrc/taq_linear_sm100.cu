@@ -316,18 +316,16 @@ bool sm100_linear_supported(const LinearArgs& a) {
     return choose(a, 1).bn != 0 && encode_tiled_fn() != nullptr;
 }
 
-// The launch plan of a dequant-GEMM as the launcher would take it (no GPU needed), with one CTA or a cluster's share of the K loop per
-// tile, or on pairs of CTAs (zeros where it does not take that): tile width, ring depth in k-blocks, CTAs that
-// share a tile's K loop, and the byte ranges of shared memory that the rings,
-// the epilogue's staging area in them and the fixed sections occupy.  out: {bn, nstage, split, ring_bytes, staging_bytes,
-// off_raw (the first fixed section), off_bias, off_bars, total, limit}.  bn = 0: the tensor-core kernel does not take it.
-void linear_plan_of(const LinearArgs& a, int n_z, bool pairs, int out[10]) {
+// The launch plan of a dequant-GEMM as the launcher takes it (no GPU needed): tile width, ring depth in k-blocks, CTAs that share a tile's K
+// loop, and the byte ranges of shared memory that the rings, the epilogue's staging area in them and the fixed sections occupy.  out: {bn,
+// nstage, split, ring_bytes, staging_bytes, off_raw (the first fixed section), off_bias, off_bars, total, limit}.  bn = 0: the tensor-core
+// kernels do not take it (pairs_only: it does not run on pairs of CTAs).
+void linear_plan_of(const LinearArgs& a, int n_z, bool pairs_only, int out[10]) {
     for (int i = 0; i < 10; ++i) out[i] = 0;
     out[9] = SMEM_LIMIT;
     if (!takes_shape(a)) return;
-    double cost;
-    const Choice c = pairs ? choose_anew(a, n_z) : choose_single(a, n_z, cost);
-    if (c.bn == 0 || (pairs && !c.pair)) return;
+    const Choice c = choose_anew(a, n_z);
+    if (c.bn == 0 || (pairs_only && !c.pair)) return;
     const Plan& P = c.lay.plan;
     out[0] = c.bn; out[1] = 2 * (c.lay.nsa < c.lay.nsb ? c.lay.nsa : c.lay.nsb); out[2] = c.lay.nsplit; out[3] = P.ring_bytes; out[4] = c.staged;
     out[5] = P.off_scales; out[6] = P.off_bias; out[7] = P.off_bars; out[8] = P.total;

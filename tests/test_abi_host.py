@@ -226,3 +226,16 @@ def test_scale_groups_that_a_cluster_shares_do_not_go_to_pairs(L):
                 assert tb.taq_linear_plan(wd, rows, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["split"] == 2
     assert tb.taq_linear_pair_plan(tb.weight_desc(1280, 1280, 8, 0), 1024, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["bn"] == 160
     assert tb.taq_linear_pair_plan(tb.weight_desc(1280, 1280, 4, 128), 2048, tb.TAQ_OUT_INT8_HEAD_ROWS, heads=8)["bn"] == 160
+
+
+def test_linear_plan_is_the_launch_s(L):
+    """Where a problem runs on pairs of CTAs both calls say so; elsewhere the one about pairs says that it does not."""
+    for n_out, k_in, bits, group, rows, kind, heads, on_pairs in (
+            (640, 640, 4, 128, 8192, tb.TAQ_OUT_F16, 1, True), (640, 640, 4, 128, 8192, tb.TAQ_OUT_INT8_HEAD_ROWS, 8, True),
+            (640, 640, 4, 64, 8192, tb.TAQ_OUT_F16, 1, False), (640, 640, 4, 128, 8192, tb.TAQ_OUT_F32, 1, False),
+            (640, 640, 4, 128, 77, tb.TAQ_OUT_F16, 1, False), (1280, 1280, 8, 0, 2048, tb.TAQ_OUT_INT8_HEAD_ROWS, 20, True)):
+        wd = tb.weight_desc(n_out, k_in, bits, group)
+        plan, pairs = tb.taq_linear_plan(wd, rows, kind, heads), tb.taq_linear_pair_plan(wd, rows, kind, heads)
+        assert plan["bn"] != 0 and (pairs["bn"] != 0) == on_pairs
+        if on_pairs:
+            assert plan == pairs

@@ -17,41 +17,58 @@ pytestmark = pytest.mark.gpu
 
 
 def layout(rows, n_out, k_in, bits, group, kind, heads=1, int8_activations=False):
-    """Tile width of a launch, "x2" or "x4" where so many CTAs share a tile, "+" where a CTA walks several tiles (148 SMs)."""
-    plan = tb.taq_linear_plan(tb.weight_desc(n_out, k_in, bits, group), rows, kind, heads=heads, int8_activations=int8_activations)
+    """Tile width of a launch, "p" on pairs of CTAs, "x2" or "x4" where so many CTAs share a tile, "+" where a CTA walks several tiles (148 SMs)."""
+    wd = tb.weight_desc(n_out, k_in, bits, group)
+    plan = tb.taq_linear_plan(wd, rows, kind, heads=heads, int8_activations=int8_activations)
+    if not int8_activations and kind != tb.TAQ_OUT_F32 and tb.taq_linear_pair_plan(wd, rows, kind, heads)["bn"]:
+        return f"{plan['bn']}p"
     ctas = (rows + 127) // 128 * (n_out // plan["bn"]) * plan["split"] if plan["bn"] else 0
     return f"{plan['bn']}" + (f"x{plan['split']}" if plan["split"] > 1 else "") + ("+" if ctas > 148 else "")
 
 
-# (the layouts of the fp16 and fp32 outputs and of the per-head int8 output: a change of the rule that chooses them says here which
-# of them is no longer run)
-@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
-    (1, 640, 640, 4, 128, 8, "64", "80"),              # one row
-    (129, 640, 640, 8, 0, 10, "64", "64"),             # a second row tile of one row
-    (2047, 640, 640, 4, 128, 10, "80", "128"),
-    (5616, 640, 640, 4, 128, 10, "64+", "64+"),
-    (5505, 640, 640, 8, 0, 8, "64+", "80+"),           # a last row tile of one row
-    (4225, 640, 640, 4, 128, 8, "160", "160"),
-    (64, 1280, 1280, 4, 128, 20, "64x2", "64x2"),      # shares of whole groups
-    (300, 1280, 1280, 8, 0, 20, "64x2", "64x2"),       # ... and of k-blocks
-    (129, 1280, 1280, 4, 0, 8, "64x2", "80x2"),        # heads over two tiles
-    (129, 1280, 1280, 8, 0, 8, "64x2", "160x2"),
-    (1100, 1280, 1280, 8, 0, 8, "80", "160x2"),
-    (97, 320, 192, 4, 128, 8, "64", "80"),             # an odd number of k-blocks, a short last group
-    (200, 320, 64, 8, 0, 8, "80", "80"),               # one k-block
-    (64, 1280, 1280, 8, 0, 8, "64x2", "160x4"),
-    (3000, 1280, 320, 4, 128, 20, "128+", "128+"),
-    (4300, 1280, 1280, 4, 128, 8, "160+", "160+"),
-    (1, 640, 768, 4, 128, 8, "64x2", "80x2"),
+# (the layouts of the fp16, the fp32 and the per-head int8 output: a change of the rule that chooses them says here which of them is no
+# longer run.  Scale groups of 64 do not go to pairs, nor do some shapes with 8-bit weights.)
+@pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,half,single,per_head", [
+    (1, 640, 640, 4, 128, 8, "64", "64", "80"),              # one row
+    (129, 640, 640, 8, 0, 10, "64", "64", "64"),             # a second row tile of one row
+    (2047, 640, 640, 4, 128, 10, "80", "80", "128p"),
+    (2047, 640, 640, 4, 64, 10, "80", "80", "128"),
+    (5616, 640, 640, 4, 128, 10, "128p", "64+", "128p"),
+    (5616, 640, 640, 4, 64, 10, "64+", "64+", "128+"),
+    (5505, 640, 640, 8, 0, 8, "128p", "64+", "160p"),        # a last row tile of one row
+    (5505, 640, 640, 4, 64, 8, "64+", "64+", "80+"),
+    (4225, 640, 640, 4, 128, 8, "160p", "160", "160p"),
+    (4225, 640, 640, 4, 64, 8, "160", "160", "160"),
+    (64, 1280, 1280, 4, 128, 20, "64x2", "64x2", "64x2"),    # shares of whole groups
+    (300, 1280, 1280, 8, 0, 20, "64x2", "64x2", "64x2"),     # ... and of k-blocks
+    (129, 1280, 1280, 4, 0, 8, "64x2", "64x2", "80x2"),      # heads over two tiles
+    (129, 1280, 1280, 8, 0, 8, "64x2", "64x2", "160p"),
+    (1100, 1280, 1280, 4, 128, 8, "80", "80", "160x2"),
+    (1100, 1280, 1280, 8, 0, 8, "80", "80", "160p"),
+    (1, 3840, 2048, 8, 0, 24, "64x2", "64x2", "160x2"),
+    (1, 1600, 1600, 8, 0, 10, "64x2", "64x2", "160x4"),
+    (97, 320, 192, 4, 128, 8, "64", "64", "80"),             # an odd number of k-blocks, a short last group
+    (200, 320, 64, 8, 0, 8, "80", "80", "80"),               # one k-block
+    (64, 1280, 1280, 8, 0, 8, "64x2", "64x2", "160p"),
+    (3000, 1280, 320, 4, 128, 20, "128p", "128+", "128p"),
+    (3000, 1280, 320, 4, 64, 20, "128+", "128+", "128+"),
+    (4300, 1280, 1280, 4, 128, 8, "160p", "160+", "160p"),
+    (4300, 1280, 1280, 4, 64, 8, "160+", "160+", "160+"),
+    (20000, 64, 64, 8, 0, 1, "64+", "64+", "64+"),
+    (20000, 80, 64, 8, 0, 2, "80+", "80+", "80+"),
+    (1100, 2048, 64, 8, 0, 32, "128", "128", "128"),
+    (7000, 2048, 64, 8, 0, 32, "128+", "128+", "128+"),
+    (1100, 2400, 64, 8, 0, 60, "160", "160", "160"),
+    (1, 640, 768, 4, 128, 8, "64x2", "64x2", "80x2"),
 ])
-def test_linear_tiles(rows, n_out, k_in, bits, group, heads, dense, per_head):
-    for kind in (tb.TAQ_OUT_F16, tb.TAQ_OUT_F32):
-        assert layout(rows, n_out, k_in, bits, group, kind) == dense
+def test_linear_tiles(rows, n_out, k_in, bits, group, heads, half, single, per_head):
+    assert layout(rows, n_out, k_in, bits, group, tb.TAQ_OUT_F16) == half
+    assert layout(rows, n_out, k_in, bits, group, tb.TAQ_OUT_F32) == single
     assert layout(rows, n_out, k_in, bits, group, tb.TAQ_OUT_INT8_HEAD_ROWS, heads) == per_head
     layer.test_quantized_linear(rows, n_out, k_in, bits, group, heads)
 
 
-# (tile widths of the launches on pairs of CTAs, 0 where the plan above is taken)
+# (tile widths of the launches on pairs of CTAs, 0 where they do not run there)
 @pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,dense,per_head", [
     (5633, 640, 640, 4, 128, 8, 128, 160),             # the last tile: one row of the first CTA, none of the second
     (5505, 640, 640, 8, 0, 10, 128, 128),              # ... one row of the second CTA; accumulators of two, two and one pairs of k-blocks
