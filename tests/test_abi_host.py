@@ -157,6 +157,34 @@ def test_linear_plan_keeps_every_region_inside_shared_memory(L):
     assert plan["bn"] == 160 and plan["staging_bytes"] == 128 * 160 * 4 and plan["ring_bytes"] >= plan["staging_bytes"]
 
 
+def test_pair_plan_keeps_every_region_inside_shared_memory(L):
+    """The same for launches on pairs of CTAs, whose output tile lies behind the stages: three of them, of two activation tiles of 128 rows and, in
+    each CTA, half of two weight tiles."""
+    seen = 0
+    for n_out in (128, 160, 320, 640, 1280, 1920):
+        for k_in in (64, 128, 192, 320, 640, 768, 1280, 2048, 5120):
+            for bits, group in ((4, 128), (4, 0), (4, 256), (4, 64), (8, 0)):
+                for rows in (34, 300, 2048, 8192, 65536):
+                    for kind, heads in ((tb.TAQ_OUT_F16, 1), (tb.TAQ_OUT_INT8_HEAD_ROWS, n_out // 40), (tb.TAQ_OUT_INT8_HEAD_ROWS, n_out // 64),
+                                        (tb.TAQ_OUT_INT8_HEAD_ROWS, max(1, n_out // 160))):
+                        for n_requests in (0, 8, 64):
+                            if n_out % heads:
+                                continue
+                            plan = tb.taq_linear_pair_plan(tb.weight_desc(n_out, k_in, bits, group), rows, kind, heads, n_requests)
+                            if plan["bn"] == 0:
+                                continue
+                            seen += 1
+                            what = (n_out, k_in, bits, group, rows, kind, heads, n_requests, plan)
+                            assert plan["bn"] in (128, 160) and plan["nstage"] == 6 and plan["split"] == 1, what
+                            assert plan["staging_bytes"] == 128 * plan["bn"] * 2, what
+                            assert plan["ring_bytes"] == 3 * 2 * (128 * 128 + plan["bn"] // 2 * 128) + plan["staging_bytes"], what
+                            groups = 1 if group == 0 else -(-k_in // group)
+                            scale_bytes = (groups + 1) * plan["bn"] * 4            # of a tile, with its biases: two buffers of them
+                            assert plan["ring_bytes"] == plan["off_raw"] and plan["off_bias"] == plan["off_raw"] + groups * plan["bn"] * 4, what
+                            assert plan["off_raw"] + 2 * scale_bytes <= plan["off_bars"] < plan["total"] <= plan["limit"], what
+    assert seen > 1000
+
+
 def test_linear_plan_of_heads_of_160_channels(L):
     """Per-head Q_a over heads of 160 channels: up to one wave of split tiles the projection runs on 80-wide tiles (two
     per head); beyond that on one 160-wide tile per head."""

@@ -12,6 +12,7 @@ import test_gpu_int8_activations as int8_activations
 from paper_2603_22943_b200 import binding as tb
 from paper_2603_22943_b200 import synth
 import taq_testlib as tl
+from oracle import taq_oracle as orc
 
 pytestmark = pytest.mark.gpu
 
@@ -27,7 +28,7 @@ def layout(rows, n_out, k_in, bits, group, kind, heads=1, int8_activations=False
 
 
 # (the layouts of the fp16, the fp32 and the per-head int8 output: a change of the rule that chooses them says here which of them is no
-# longer run.  Scale groups of 64 do not go to pairs, nor do some shapes with 8-bit weights.)
+# longer run.  Scale groups of 64 do not go to pairs, nor do some shapes with 8-bit weights; see also test_requests_of_few_rows.)
 @pytest.mark.parametrize("rows,n_out,k_in,bits,group,heads,half,single,per_head", [
     (1, 640, 640, 4, 128, 8, "64", "64", "80"),              # one row
     (129, 640, 640, 8, 0, 10, "64", "64", "64"),             # a second row tile of one row
@@ -92,15 +93,49 @@ def test_pairs_write_their_rows_only():
     assert tb.taq_linear_pair_plan(tb.weight_desc(640, 640, 4, 128), 520, tb.TAQ_OUT_F16, n_requests=8)["bn"] != 0
     shape, desc, ckpts, route, reqs_data, packed, y, kv_blocks = layer._serving_case(n_ckpt=3, n_req=8, n_query=520, C_=640, Dc=768)
     for r, c in enumerate(route):
-        layer._check_request(shape, desc, ckpts[int(c)], reqs_data[r], packed[int(c)], kv_blocks[r], y[r: r + 1], slice(490, 520))
-    n = 5633 * 640
+        layer._check_request(shape, desc, ckpts[int(c)], reqs_data[r], packed[int(c)], kv_blocks[r], y[r: r + 1])
+    rows, heads = 5633, 8
+    n = rows * 640
+    wd, blob = tb.weight_desc(640, 640, 4, 128), packed[0]["Wq"]
+    x = torch.randn(rows, 640, device="cuda", generator=torch.Generator("cuda").manual_seed(1)).half()
+    codes, group_scales = tb.taq_unpack_weights(wd, blob)
+    want = x.double() @ (codes.double() * group_scales.view(640, -1).repeat_interleave(128, 1).double()).T
+    want_scales = want.view(rows, heads, -1).abs().amax(-1) / 127
+
+    def guarded(count, dtype):
+        buf = torch.full((count + 4096,), -7, dtype=dtype, device="cuda")
+        return buf, buf[2048: 2048 + count]
+
     for kind, dtype in ((tb.TAQ_OUT_F16, torch.float16), (tb.TAQ_OUT_INT8_HEAD_ROWS, torch.int8)):
-        buf = torch.full((n + 4096,), -7, dtype=dtype, device="cuda")
-        x = torch.randn(5633, 640, device="cuda").half()
-        blob = packed[0]["Wq"]
-        tb.taq_quantized_linear(tb.weight_desc(640, 640, 4, 128), x, blob, kind, heads=8, y=buf[2048: 2048 + n])
+        per_head = kind == tb.TAQ_OUT_INT8_HEAD_ROWS
+        (buf, out), (scale_buf, scales) = guarded(n, dtype), guarded(rows * heads, torch.float32)
+        tb.taq_quantized_linear(wd, x, blob, kind, heads=heads, y=out, scales=scales if per_head else None)
         tb.taq_poll_device_status()
-        assert bool((buf[:2048] == -7).all()) and bool((buf[2048 + n:] == -7).all())
+        for b in (buf, scale_buf):
+            assert bool((b[:2048] == -7).all()) and bool((b[-2048:] == -7).all())
+        if per_head:
+            assert bool(((scales.view(rows, heads).double() - want_scales).abs() <= 2e-5 * want_scales).all())
+            layer._code_agreement(out.view(rows, heads, -1).cpu().numpy(), (want.view(rows, heads, -1) / want_scales[..., None]).round().cpu().numpy(), "codes")
+        else:                                        # half a unit in the last place of an fp16 value, and fp32 sums of 640 products
+            assert bool(((out.view(rows, 640).double() - want).abs() <= 2.0 ** -11 * want.abs() + 2e-5 * want.abs().max()).all())
+
+
+# (none of these goes to pairs.  fp16 rows on 160-wide tiles, the first two one per CTA, the others several; per-head rows on 128, 128, 80, 128 and
+# 160 columns, several per CTA)
+@pytest.mark.parametrize("channels,heads,n_req,w_bits", [(1280, 20, 18, 4), (1280, 20, 18, 8), (640, 8, 64, 8), (640, 10, 64, 4), (1280, 16, 33, 8)])
+def test_requests_of_few_rows(channels, heads, n_req, w_bits):
+    """Batched layers whose requests fill a quarter of a row tile: tiles of several requests in one CTA's walk.  Sums of to_q are of whole numbers, so
+    that the query codes are those of the single projection, whatever its layout, and the oracle starts from them."""
+    wd = tb.weight_desc(channels, channels, w_bits, 128 if w_bits == 4 else 0)
+    assert tb.taq_linear_pair_plan(wd, 34, tb.TAQ_OUT_F16, n_requests=n_req)["bn"] == 0
+    assert tb.taq_linear_pair_plan(wd, 34, tb.TAQ_OUT_INT8_HEAD_ROWS, heads, n_requests=n_req)["bn"] == 0
+    shape, desc, ckpts, route, reqs_data, packed, y, kv_blocks = layer._serving_case(n_ckpt=3, n_req=n_req, n_query=34, C_=channels, Dc=768, heads=heads, w_bits=w_bits, whole=True)
+    cfg = tl.oracle_cfg(shape)
+    for r, c in enumerate(route):
+        ck, rd = ckpts[int(c)], reqs_data[r]
+        g = tl.gpu_decisions(shape, {**ck.weights, **rd}, {"desc": desc, "packed": packed[int(c)], "kv": kv_blocks[r]})
+        O = orc.taq_attention(g["Q_tilde"], g["K_tilde"], g["V_tilde"], rd["mask"], cfg)
+        tl.assert_layer_close(y[r: r + 1], orc.taq_out(O, ck.weights["Wout"], ck.weights["bout"], cfg), f"request {r}")
 
 
 @pytest.mark.parametrize("rows,k_in,n_out,bits,group,dense", [

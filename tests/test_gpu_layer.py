@@ -291,18 +291,27 @@ def test_empty_inputs():
 # ---------------------------------------------------------------------------------------------------------
 # Batched serving: every request carries its own checkpoint (weights, trigger mask) and its own K~/V~
 # ---------------------------------------------------------------------------------------------------------
-def _serving_case(n_ckpt, n_req, n_query, C_, Dc, T=77, seed=0):
+def _serving_case(n_ckpt, n_req, n_query, C_, Dc, T=77, seed=0, heads=8, w_bits=4, whole=False):
+    # whole: to_q and X of whole numbers, whose sums do not depend on their order
     ckpts = [synth.make_checkpoint(c, C_, Dc, T) for c in range(n_ckpt)]
     route = synth.make_request_batch(n_req, n_ckpt, seed)
-    shape = synth.LayerShape(1, n_query, C_, 8, T, Dc, 4, 128, (), seed=0)
+    shape = synth.LayerShape(1, n_query, C_, heads, T, Dc, w_bits, 128 if w_bits == 4 else 0, (), seed=0)
     desc = tl.gpu_desc(shape, max_trigger=3)
     packed = []
     for ck in ckpts:
+        if whole:
+            m = 127 if w_bits == 8 else 7
+            w = np.random.default_rng(ck.ckpt_id).integers(-m, m + 1, (C_, C_))
+            w[:, ::128] = m                                          # (every group's largest: scales are powers of two)
+            ck.weights["Wq"] = (w / (m + 1) / 32).astype(np.float32)
         d = dict(ck.weights)
         packed.append(tl.pack_layer_weights(shape, d))
     lay = tb.taq_kv_layout_of(desc)
     kv_arena = torch.zeros(n_req * lay.block_bytes, dtype=torch.uint8, device="cuda")
     reqs_data = [synth.make_request_activations(ckpts[int(c)], n_query, C_, Dc, T, seed=1000 * seed + r) for r, c in enumerate(route)]
+    if whole:
+        for r, rd in enumerate(reqs_data):
+            rd["X"] = np.random.default_rng(r).integers(-8, 9, rd["X"].shape).astype(np.float16)
     X = dev(np.concatenate([rd["X"] for rd in reqs_data], axis=0))
     ctx = dev(np.concatenate([rd["ctx"] for rd in reqs_data], axis=0))
     masks = [dev(rd["mask"][0]) for rd in reqs_data]
