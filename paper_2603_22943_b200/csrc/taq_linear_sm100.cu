@@ -86,7 +86,6 @@ bool rings(const LinearArgs& a, const Problem& p, int nsplit, int head_pair, boo
     int nsa = n_pair < 2 ? 1 : 2, nsb = n_pair < 2 ? 1 : 2;
     while (make_plan<BN>(p.n_groups, nsa, nsb, persistent, xb).ring_bytes < staged) { if (nsa < nsb) ++nsa; else ++nsb; if (nsb > MAX_STAGE) return false; }
     auto fits = [&](int na, int nb) { return make_plan<BN>(p.n_groups, na, nb, persistent, xb).total <= SMEM_LIMIT; };
-
     while (nsb < (persistent ? MAX_STAGE : n_pair) && nsb < MAX_STAGE && fits(nsa, nsb + 1)) ++nsb;
     while (nsa < 3 && nsa < n_pair && fits(nsa + 1, nsb)) ++nsa;
     const Plan P = make_plan<BN>(p.n_groups, nsa, nsb, persistent, xb);
@@ -176,7 +175,6 @@ constexpr Pace PACES[4] = {
     {64, 2.56, 0.192, 0.106, 0.24, 0.18, 1.00, 0.87},
 };
 Choice& finish(Choice& c, const LinearArgs& a, const Problem& p, long long tiles, long long ctas) {
-
     c.lay.n_tiles = (int)tiles;
     c.lay.n_cols = a.n_out / c.bn * p.ncols_factor; c.lay.n_rows = (int)p.row_tiles;
     c.lay.mul_cols = multiplier(c.lay.n_cols, tiles); c.lay.mul_rows = multiplier(c.lay.n_rows, tiles);
@@ -240,7 +238,8 @@ Choice choose_single(const LinearArgs& a, int n_z, double& best_cost) {
 }
 
 // Tiles of 256 rows on pairs of CTAs, in rounds of 74.  A fit to 151 measured launches (256 to 32768 rows, 320 to 1280 channels, W4 and
-// W8, fp16 and per-head int8 rows; 6 and 5 % rms).
+// W8, fp16 and per-head int8 rows; 6 and 5 % rms).  The per-head terms, below 0, are what the fit leaves between the two outputs, whose other
+// parts are one number each, and no step's cost.
 Choice choose_pair(const LinearArgs& a, int n_z, double& best_cost) {
     struct PairPace { int bn; double fixed, pair4, pair8, tile, q8; };
     constexpr PairPace PAIR_PACES[2] = {{160, 3.70, 0.628, 0.541, 1.25, -0.73}, {128, 3.16, 0.559, 0.504, 0.87, -0.22}};
@@ -263,13 +262,14 @@ Choice choose_pair(const LinearArgs& a, int n_z, double& best_cost) {
     return best;
 }
 
-// Pairs or one CTA per tile: the cheaper one, with two corrections.  Where a CTA would walk several tiles the model of one CTA per tile is 10 to
-// 40 % short (in one problem's launches pairs were always faster there, by 2 to 45 %), but requests of few rows leave half of every
-// 256-row tile empty: 18 requests x 34 rows at 1280 channels, heads of 64, took 46.2 us a layer on pairs and 43.6 so.  In launches of one wave of 128 or
-// 160 columns fp16 rows take 1.4 to 3.2 us more than it says: with 2 us more every one of 202 launches gets the faster kernel (with
-// 1.5 us one is 7 % slower, with none eight are 12 to 29 %).  Scale groups that a cluster would share stay shared (heads of 160 channels, 600 to
-// 1150 rows): sums of all groups in a row lose bits that two halves keep.  1100 x 1280 x 1280, W4: scales' root mean square error 5.3e-8,
-// on pairs 6.3e-8 (12.9 and 10.8 us); x 2560 5.8e-8 and 7.9e-8 (18.0 and 19.6 us).
+// Pairs or one CTA per tile: the cheaper one, with three corrections.  Where a CTA would walk several tiles the model of one CTA per tile is 10 to
+// 40 % short (in one problem's launches pairs were always faster there, by 2 to 45 %).  But requests of up to 128 rows leave half of every 256-row
+// tile empty, and of 160 measured layers of such requests none is faster on pairs (18 requests x 34 rows, 1280 channels, heads of 64: 52.4 us, 43.4
+// so).  In launches of one wave of 128 or 160 columns fp16 rows take 1.4 to 3.2 us more than the model says.  Of 248 single launches (16 to 32768
+// rows) all but two get the kernel that is faster, or within 1.5 % of it, and of 224 layers of requests all within 2.6 %.  The two are of the
+// third correction: scale groups that a cluster would share stay shared (heads of 160 channels, 600 to 1150 rows), for sums of all groups in a
+// row lose bits that two halves keep.  1100 x 1280 x 1280, W4: scales' root mean square error 5.3e-8, on pairs 6.3e-8 (12.9 and 10.8 us); x 2560
+// 5.8e-8 and 7.9e-8 (18.0 and 19.6 us).
 Choice choose_anew(const LinearArgs& a, int n_z) {
     double cost, pair_cost;
     const Choice single = choose_single(a, n_z, cost), pair = choose_pair(a, n_z, pair_cost);

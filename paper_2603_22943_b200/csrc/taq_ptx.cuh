@@ -90,7 +90,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// Arrival on a barrier of another CTA, behind what this thread has seen (release at CTA scope: at cluster scope it took 1 500 cycles).
+// Arrival on a barrier of another CTA, with release at CTA scope (at cluster scope it took 1 500 cycles).  That suffices for what it hands over here,
+// which no thread of the other CTA reads: operands of an MMA, which their writers have fenced to the async proxy on their own SM, and seen complete
+// on a barrier there, before this arrival, and accumulators, whose reads tcgen05.fence::before_thread_sync has put in front of it.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
